@@ -189,6 +189,7 @@ tj_status ensure_device() {
   TJ_CUDA(join_init_attributes());
   TJ_CUDA(mlp_init_attributes());
   TJ_CUDA(fused_init_attributes());
+  TJ_CUDA(word_init_attributes());
   g_inited[dev] = true;
   return TJ_OK;
 }
@@ -508,6 +509,109 @@ void set_job_buffers(RadixJob<K>& j, const K* in_k, const K* in_v, K* ak, K* av,
   *res_v = cv;
 }
 
+// ---- folded rows (tj_word.cu) -------------------------------------------------------
+// A row is one 64-bit word, (key - wlo) << ib | (id - ilo), when the bits of
+// the key range and of the ids fit together; then every pass but the first and
+// the last moves 8 bytes a row.  32-bit rows always fit (ib = 32).  64-bit
+// rows: the ids' range is known from a sample (two rows a tile), so the window
+// the spare bits allow is centred on it; the folding pass checks every row, and
+// one outside sends the call back to separate columns (kErrFold).
+struct Fold {
+  bool on = false;
+  uint64_t wlo = 0, ilo = 0;
+  int ib = 0;
+};
+
+template <typename K>
+Fold make_fold(uint64_t lo, int key_bits, unsigned long long id_min_u,
+               unsigned long long id_max_u) {
+  Fold f;
+  f.wlo = lo;
+  if (sizeof(K) == 4) {
+    f.ib = 32;
+    f.on = true;
+    return f;
+  }
+  const int avail = 64 - key_bits;
+  if (avail < 1 || avail > 63 || id_max_u < id_min_u) return f;
+  const uint64_t range = id_max_u - id_min_u;
+  if (bitlen(range) > avail) return f;
+  const uint64_t window = ((uint64_t)1 << avail) - 1;
+  f.ib = avail;
+  f.ilo = (uint64_t)key_of<int64_t>(id_min_u) - (window - range) / 2;
+  f.on = true;
+  return f;
+}
+
+// Rows below which a word pass takes the small tile: the large one would
+// leave most of the chip without a CTA.
+constexpr int64_t kWSmallRows = (int64_t)1 << 22;
+int word_items(int64_t rows) { return rows < kWSmallRows ? kWItemsSmall : kWItems; }
+
+// Time of one word pass by digit width, relative to one of at most 7 bits
+// (GB300, 10^8 words: 500, 538, 618 and 770 us for 7 to 10 bits), and the plan
+// of fewest such units: 27 bits take 3 passes of 9 instead of 4 of 7.
+double word_pass_cost(int w) { return w <= 7 ? 1.0 : w == 8 ? 1.08 : w == 9 ? 1.24 : 1.55; }
+
+Plan make_word_plan(uint64_t lo, uint64_t range, bool even, int max_digit, int min_passes) {
+  const int kb = bitlen(range);
+  int best = -1;
+  double cost = 0;
+  for (int P = std::max(min_passes, (kb + max_digit - 1) / max_digit); P <= kMaxPasses; ++P) {
+    if (even && (P & 1)) continue;
+    const double c = P * word_pass_cost((kb + P - 1) / P);
+    if (best < 0 || c < cost) {
+      best = P;
+      cost = c;
+    }
+  }
+  return make_plan(lo, range, false, max_digit, kb == 0 ? 0 : best);
+}
+
+// A plan's digits as positions within words whose keys start at bit ib,
+// relative to the offset `lo` (already shifted into word position).
+template <typename K>
+void set_word_plan(RadixJob<K>& j, const Plan& p, const Fold& f, uint64_t lo) {
+  set_job_plan(j, p);
+  for (int i = 0; i < p.passes; ++i) j.shift[i] += f.ib;
+  j.lo = lo;
+  j.wlo = f.wlo;
+  j.ilo = f.ilo;
+  j.ib = f.ib;
+  j.dst_rows = j.n;
+}
+
+// One word pass: from columns into words, or words to words (8 bytes a row
+// whatever K: the 64-bit instantiation over the same job layout).
+template <typename K>
+cudaError_t word_pass(const RadixJob<K>* d_jobs, int nj, int64_t tiles, int p, int max_bits,
+                      bool fold_in, const Fold& f, int items, uint32_t* d_counter, int* d_err,
+                      cudaStream_t st, const int32_t* d_tile_job = nullptr) {
+  if (fold_in)
+    return launch_wsweep<K>(d_jobs, nj, tiles, p, max_bits, kModeSort, true, false, f.ib >= 32,
+                            items, false, d_counter, d_err, st, d_tile_job);
+  static_assert(sizeof(RadixJob<K>) == sizeof(RadixJob<int64_t>), "one job layout");
+  return launch_wsweep<int64_t>(reinterpret_cast<const RadixJob<int64_t>*>(d_jobs), nj, tiles, p,
+                                max_bits, kModeSort, false, false, f.ib >= 32, items, false,
+                                d_counter, d_err, st, d_tile_job);
+}
+
+// Ping-pong of a word job: pass 0 reads the columns (fold_in) or the words
+// `in`, pass p writes `a` when p is even, `b` when odd.  Returns where the
+// words end up.
+template <typename K>
+uint64_t* set_word_buffers(RadixJob<K>& j, const K* in_k, const K* in_v, uint64_t* a, uint64_t* b) {
+  const K* src = in_k;
+  for (int p = 0; p < j.passes; ++p) {
+    j.src_k[p] = src;
+    if (p == 0) j.fold_v[0] = in_v;
+    j.dst_k[p] = reinterpret_cast<K*>((p & 1) ? b : a);
+    j.dst_v[p] = nullptr;
+    src = j.dst_k[p];
+  }
+  return reinterpret_cast<uint64_t*>(const_cast<K*>(src));
+}
+
 // ---- inner join -------------------------------------------------------------------
 struct Opts {
   int router = TJ_ROUTE_AUTO;
@@ -521,11 +625,14 @@ struct Opts {
   double radix_judge = 1.25;  // < 0: the learned model is always kept
   bool fused = true;          // the partition-resident phase for narrow batches
   bool exact_route = false;  // size the batch regions by a histogram, not the sample
+  bool fold = true;          // folded rows where they fit (partitioned join)
 };
 
 // part_join_impl's request to be run again with exact batch sizes (a batch
 // outgrew the region its sample estimate gave it)
 constexpr tj_status kRouteAgain = (tj_status)100;
+// ... or on separate columns (a row did not fold)
+constexpr tj_status kColumnsAgain = (tj_status)kErrFold;
 
 Opts make_opts(const tj_join_opts* o) {
   Opts x;
@@ -601,6 +708,10 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
   hj[1].keys = ks;
   hj[1].n = ns;
   hj[1].tile0 = tiles_r;
+  if (sizeof(K) == 8) {
+    hj[0].ids = ir;
+    hj[1].ids = is;
+  }
   TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
   TJ_CUDA(cudaMemsetAsync(d_stats, 0xFF, 2 * sizeof(KeyStats), st));
   TJ_CUDA(put_small(d_jobs, hj, sizeof(hj), st));
@@ -612,14 +723,18 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     stats.learned = router;
     Opts po = opts;
     po.router = router;
-    tj_status ps = part_join_impl<K>(kr, ir, nr, ks, is, ns, lo, hi, range_known, budget, po,
-                                     out, cap, out_count, stats, tr, st);
-    if (ps == kRouteAgain) {
-      po.exact_route = true;
+    tj_status ps = TJ_OK;
+    while (true) {
       ps = part_join_impl<K>(kr, ir, nr, ks, is, ns, lo, hi, range_known, budget, po, out, cap,
                              out_count, stats, tr, st);
-      stats.route_regions = 3;
+      if (ps == kRouteAgain && !po.exact_route)
+        po.exact_route = true;
+      else if (ps == kColumnsAgain && po.fold)
+        po.fold = false;
+      else
+        break;
     }
+    if (po.exact_route) stats.route_regions = 3;
     if (ps == TJ_OK || ps == TJ_ERR_CAPACITY) {
       stats.out_count = *out_count;
       g_stats = stats;
@@ -697,6 +812,107 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
   if (budget != 0 && need > budget)
     return set_err(TJ_ERR_BUDGET,
                    "join needs %zu bytes of scratch in one pass, budget is %zu", need, budget);
+  // Folded rows (at most the memory of the column passes, so a budget that
+  // admits those admits these)
+  const Fold fold = P > 0 ? make_fold<K>(plan.lo, plan.key_bits,
+                                         std::min(hs[0].id_min_u, hs[1].id_min_u),
+                                         std::max(~hs[0].id_max_u, ~hs[1].id_max_u))
+                          : Fold();
+  while (fold.on) {
+    const Plan wp = nr + ns >= kCostRows
+                        ? make_word_plan(plan.lo, range_of<K>(lo, hi), false,
+                                         max_digit_bits<K>(), 1)
+                        : plan;
+    const int items = word_items(nr + ns);
+    const int64_t wtile = (int64_t)kWThreads * items;
+    const int64_t wt_r = ceil_div(nr, wtile), wt = wt_r + ceil_div(ns, wtile);
+    const int64_t lb_words = wt << wp.max_bits;
+    const bool regions = (int64_t)wp.passes * lb_words * 4 <= (int64_t)1 << 20;
+    Carve wc;
+    const size_t o_a = wc.add<uint64_t>((size_t)(nr + ns));
+    const size_t o_b = wc.add<uint64_t>(wp.passes > 1 ? (size_t)(nr + ns) : 0);
+    const size_t o_wt = wc.add<JTile<K>>(jtiles);
+    const size_t o_whist = wc.add<uint32_t>((size_t)2 * wp.passes << wp.max_bits);
+    const size_t o_wjlb = wc.add<uint64_t>(jtiles);
+    const size_t o_wlb = wc.add<uint32_t>((size_t)(regions ? wp.passes : 1) * lb_words);
+    const size_t wneed = wc.off + cc.off;
+    if (wneed > need) break;
+    Block big;
+    TJ_CUDA(big.alloc(wc.off, st));
+    RadixJob<K> hw[4] = {hj[0], hj[1], hj[0], hj[1]};
+    uint64_t* res[2];
+    for (int i = 0; i < 2; ++i) {
+      RadixJob<K>& h = hw[i];
+      RadixJob<K>& x = hw[2 + i];
+      set_job_plan(h, wp);
+      h.hist_stride = 1 << wp.max_bits;
+      h.hist = big.at<uint32_t>(o_whist) + ((size_t)i * wp.passes << wp.max_bits);
+      x.hist_stride = h.hist_stride;
+      x.hist = h.hist;
+      set_word_plan(x, wp, fold, 0);
+      x.tile0 = i ? wt_r : 0;
+      x.lookback = big.at<uint32_t>(o_wlb) + ((i ? wt_r : 0) << wp.max_bits);
+      x.lb_stride = regions ? lb_words : 0;
+      uint64_t* a = big.at<uint64_t>(o_a) + (i ? nr : 0);
+      uint64_t* b = big.at<uint64_t>(o_b) + (i ? nr : 0);
+      res[i] = set_word_buffers(x, i ? ks : kr, i ? is : ir, a, b);
+    }
+    JoinJob<K> jj;
+    jj.rk = reinterpret_cast<const K*>(res[0]);
+    jj.rv = nullptr;
+    jj.nr = nr;
+    jj.sk = reinterpret_cast<const K*>(res[1]);
+    jj.sv = nullptr;
+    jj.ns = ns;
+    jj.tile0 = 0;
+    TJ_CUDA(put_small(d_jobs, hw, sizeof(hw), st));
+    TJ_CUDA(put_small(d_jj, &jj, sizeof(jj), st));
+    TJ_CUDA(cudaMemsetAsync(big.p + o_whist, 0,
+                            (regions ? o_wlb + (size_t)wp.passes * lb_words * 4 : o_wlb) - o_whist,
+                            st));
+    tr.begin("histogram", w * (nr + ns));
+    TJ_CUDA(launch_histogram<K>(d_jobs, 2, tiles_r + tiles_s, st));
+    tr.end();
+    TJ_CUDA(launch_digit_scan<K>(d_jobs, 2, wp.passes, st));
+    for (int p = 0; p < wp.passes; ++p) {
+      if (!regions) TJ_CUDA(cudaMemsetAsync(big.p + o_wlb, 0, (size_t)lb_words * 4, st));
+      tr.begin("onesweep", ((p ? 8.0 : 2.0 * w) + 8.0) * (nr + ns));
+      TJ_CUDA(word_pass<K>(d_jobs + 2, 2, wt, p, wp.max_bits, p == 0, fold, items,
+                           d_counters + p, d_err, st));
+      tr.end();
+    }
+    WordFmt fmt;
+    fmt.ib = fold.ib;
+    fmt.ilo = fold.ilo;
+    JTile<K>* d_tiles = big.at<JTile<K>>(o_wt);
+    TJ_CUDA(launch_tile_ranges<K>(d_jj, 1, jtiles, d_tiles, st, nullptr, fmt, d_err));
+    tr.begin("join", 8.0 * (nr + ns));
+    TJ_CUDA(launch_join<K>(jtiles, d_tiles, big.at<uint64_t>(o_wjlb), d_counters + kMaxPasses,
+                           out, cap, nullptr, nullptr, d_total, d_err, st, fmt));
+    tr.end();
+    int64_t h_total = 0;
+    int h_err = 0;
+    TJ_CUDA(get_small(&h_total, d_total, sizeof(int64_t), st));
+    TJ_CUDA(get_small(&h_err, d_err, sizeof(int), st));
+    TJ_CUDA(sync_stream(st));
+    if (h_err == kErrFold) {  // an id outside the window of the sampled ones
+      TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
+      break;
+    }
+    stats.scratch_peak = (int64_t)wneed;
+    stats.radix_passes = wp.passes;
+    stats.digit_bits = wp.max_bits;
+    if (h_total <= cap) tr.add_bytes("join", 2.0 * w * (double)h_total);
+    tr.flush();
+    if (h_err) return set_err((tj_status)h_err, "device reported %d", h_err);
+    *out_count = h_total;
+    stats.out_count = h_total;
+    g_stats = stats;
+    if (h_total > cap)
+      return set_err(TJ_ERR_CAPACITY, "result has %lld pairs, capacity %lld", (long long)h_total,
+                     (long long)cap);
+    return TJ_OK;
+  }
   Block big;
   TJ_CUDA(big.alloc(bc.off, st));
   stats.scratch_peak = (int64_t)need;
@@ -858,6 +1074,18 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
                          cudaStream_t st) {
   const double w = (double)sizeof(K);
   const int maxd = max_digit_bits<K>();
+  // range of sampled ids (for folded rows): read with the next synchronisation
+  unsigned long long id_min_u = ~0ull, id_max_u = 0ull;
+  KeyStats idst;
+  memset(&idst, 0xFF, sizeof(idst));
+  Block idb;
+  const bool ask_ids = sizeof(K) == 8 && o.fused && o.fold;
+  if (ask_ids) {
+    TJ_CUDA(idb.alloc(sizeof(KeyStats), st));
+    TJ_CUDA(cudaMemsetAsync(idb.p, 0xFF, sizeof(KeyStats), st));
+    TJ_CUDA(launch_id_range<K>(ir, nr, is, ns, idb.at<KeyStats>(0), st));
+    TJ_CUDA(get_small(&idst, idb.p, sizeof(idst), st));
+  }
   // batches: as asked, else from the key range (the sample's when the range
   // is not known yet)
   int parts = o.partitions > 0 ? std::max(2, std::min(o.partitions, kMaxCuts))
@@ -1068,6 +1296,41 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     stats.heavy_keys = heavy;
   }
 
+  // Folded rows (tj_word.cu) from the route pass on.  A range read off the
+  // sample gets a thirty-second of slack on either side; a row outside sends the
+  // call back to separate columns.
+  Fold fold;
+  if (ask_ids) {
+    if (!g_reads.empty()) TJ_CUDA(sync_stream(st));  // (a router that sampled has waited)
+    id_min_u = idst.id_min_u;
+    id_max_u = ~idst.id_max_u;
+  }
+  if (o.fused && o.fold) {
+    if (sizeof(K) == 4) {
+      fold = make_fold<K>(lo_bits<K>(std::numeric_limits<K>::min()), 32, 0, 0);
+    } else {
+      const uint64_t range = range_of<K>(lo, hi);
+      const uint64_t slack = range_known ? 0 : range / 32 + 1024;
+      if (range + 2 * slack >= range && range + 2 * slack < ((uint64_t)1 << 62)) {
+        const int kw = std::max(1, bitlen(range + 2 * slack));
+        const uint64_t spare = range_known ? 0 : ((((uint64_t)1 << kw) - 1) - range) / 2;
+        fold = make_fold<K>(lo_bits<K>(lo) - spare, kw, id_min_u, id_max_u);
+      }
+    }
+  }
+  const bool words = fold.on;
+  const int ib = fold.ib;
+  WordFmt fmt;
+  if (words) {
+    fmt.ib = fold.ib;
+    fmt.ilo = fold.ilo;
+  }
+  // offset of a key from the words' first key (exact for keys within the window)
+  auto off = [&](K k) -> uint64_t {
+    return (uint64_t)(typename UnsignedOf<K>::type)(lo_bits<K>(k) - fold.wlo);
+  };
+  const double rowb = words ? 8.0 : 2.0 * w;  // bytes of a routed row
+
   // ---- 2. route pass into staging, in chunks whose look-back fits the budget ----
   // log-scale index over the cuts (see RadixJob::route_tab): tab[b] = number of
   // cuts below the first key of bucket b
@@ -1126,15 +1389,19 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   // batches the 9-row tile measured 1.4x slower)
   // equal-width batches: batch = (clamp(key) - lo) >> rshift, rbits wide
   const int rshift = radix_route ? std::max(0, bitlen(krange) - rbits) : 0;
-  const int ritems = radix_route ? (rbits <= kWideBits ? kItemsWide : kItems)
+  const int citems = radix_route ? (rbits <= kWideBits ? kItemsWide : kItems)
                                  : (rbits <= kWideBits ? kItemsRoute : kItems);
-  const int64_t rtile = (int64_t)kSortThreads * ritems;
+  const int ritems = words ? kWItems : citems;
+  const int64_t rtile = (int64_t)(words ? kWThreads : kSortThreads) * ritems;
+  // chunks, look-back room and regions are sized for the columns' tile either
+  // way, so a budget admits and refuses the same joins
+  const int64_t ctile = (int64_t)kSortThreads * citems;
   const int64_t lb_per_tile = ((int64_t)1 << rbits) * 4;
   const int64_t route_lb = budget ? std::max<int64_t>((int64_t)budget / 4, 16 * lb_per_tile)
                                   : INT64_MAX;
-  const int64_t all_tiles = ceil_div(std::max(nr, ns), rtile);
+  const int64_t all_tiles = ceil_div(std::max(nr, ns), ctile);
   const int64_t chunk_tiles = std::max<int64_t>(1, std::min(all_tiles, route_lb / lb_per_tile));
-  const int64_t chunk_rows = chunk_tiles * rtile;  // <= max(n_r, n_s) rounded up to a tile
+  const int64_t chunk_rows = chunk_tiles * ctile;  // <= max(n_r, n_s) rounded up to a tile
   if ((int64_t)nr + ns >= ((int64_t)1 << 32))
     return set_err(TJ_ERR_INVALID, "partitioned join needs n_r + n_s < 2^32");
   // Batch regions in the routed copies: sized from the sample when the router
@@ -1153,7 +1420,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       int64_t acc = 0;
       for (int p2 = 0; p2 < nparts; ++p2) {
         const double c = (double)sample_cnt[(size_t)side * kMaxBins + p2];
-        const int64_t k = (int64_t)std::ceil((c + 6.0 * std::sqrt(c) + 8.0) * scale) + rtile;
+        const int64_t k = (int64_t)std::ceil((c + 6.0 * std::sqrt(c) + 8.0) * scale) + ctile;
         rcap[(size_t)side * nparts + p2] = k;
         rstart[(size_t)side * nparts + p2] = acc;
         acc += k;
@@ -1179,18 +1446,27 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   for (int i = 0; i < nch;) {
     int j = i;
     int64_t acc = 0;
-    while (j < nch && (j == i || (!est && acc + ceil_div(chunks[(size_t)j].n, rtile) * lb_per_tile <=
+    while (j < nch && (j == i || (!est && acc + ceil_div(chunks[(size_t)j].n, ctile) * lb_per_tile <=
                                                route_lb)))
-      acc += ceil_div(chunks[(size_t)j].n, rtile) * lb_per_tile, ++j;
+      acc += ceil_div(chunks[(size_t)j].n, ctile) * lb_per_tile, ++j;
     cgroups.push_back({i, j});
     lb_max = std::max(lb_max, acc);
     i = j;
   }
   Carve cc;
-  const size_t o_rk = cc.add<K>((size_t)side_rows[0]), o_rv = cc.add<K>((size_t)side_rows[0]);
-  const size_t o_sk = cc.add<K>((size_t)side_rows[1]), o_sv = cc.add<K>((size_t)side_rows[1]);
+  // (folded rows: o_rk and o_sk hold the words)
+  const size_t o_rk = words ? cc.add<uint64_t>((size_t)side_rows[0]) : cc.add<K>((size_t)side_rows[0]);
+  const size_t o_rv = words ? 0 : cc.add<K>((size_t)side_rows[0]);
+  const size_t o_sk = words ? cc.add<uint64_t>((size_t)side_rows[1]) : cc.add<K>((size_t)side_rows[1]);
+  const size_t o_sv = words ? 0 : cc.add<K>((size_t)side_rows[1]);
   const size_t staging = cc.off;
+  // a side's routed rows from row r on
+  auto routed = [&](const Block& b, int side, int64_t r) -> K* {
+    return words ? reinterpret_cast<K*>(b.at<uint64_t>(side ? o_sk : o_rk) + r)
+                 : b.at<K>(side ? o_sk : o_rk) + r;
+  };
   const size_t o_cuts = cc.add<K>(kMaxCuts);
+  const size_t o_wcuts = words ? cc.add<uint64_t>(kMaxCuts) : 0;  // cuts as offsets
   const size_t o_tab = cc.add<uint16_t>(kRouteBuckets + 1);
   const size_t o_hist = cc.add<uint32_t>((size_t)nch * kMaxBins);
   const size_t o_rend = cc.add<uint32_t>(2 * (size_t)kMaxBins);  // regions' ends (est)
@@ -1207,6 +1483,11 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   std::vector<K> hc(kMaxCuts, std::numeric_limits<K>::max());
   std::copy(cuts.begin(), cuts.end(), hc.begin());
   TJ_CUDA(put_small(stg.at<K>(o_cuts), hc.data(), kMaxCuts * sizeof(K), st));
+  if (words) {
+    std::vector<uint64_t> wc(kMaxCuts, ~0ull);
+    for (int i = 0; i < ncuts; ++i) wc[(size_t)i] = off(cuts[(size_t)i]);
+    TJ_CUDA(put_small(stg.at<uint64_t>(o_wcuts), wc.data(), kMaxCuts * sizeof(uint64_t), st));
+  }
   TJ_CUDA(put_small(stg.at<uint16_t>(o_tab), tab.data(), tab.size() * sizeof(uint16_t), st));
   // histogram jobs (global tile numbering) then per-launch route jobs (tile0
   // rebased to their launch); the route jobs' hist slots receive the bases
@@ -1230,9 +1511,9 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     x.hist_stride = kMaxBins;
     x.hist = stg.at<uint32_t>(o_hist) + (size_t)c * kMaxBins;
     x.src_k[0] = kb + ch.r0;
-    x.src_v[0] = vb + ch.r0;
-    x.dst_k[0] = ch.side ? stg.at<K>(o_sk) : stg.at<K>(o_rk);
-    x.dst_v[0] = ch.side ? stg.at<K>(o_sv) : stg.at<K>(o_rv);
+    x.src_v[0] = vb + ch.r0;  // (folded rows: fold_v[0])
+    x.dst_k[0] = routed(stg, ch.side, 0);
+    x.dst_v[0] = words ? nullptr : ch.side ? stg.at<K>(o_sv) : stg.at<K>(o_rv);
     x.cuts = radix_route ? nullptr : stg.at<K>(o_cuts);  // radix: the digit path
     x.ncuts = ncuts;
     x.route_tab = stg.at<uint16_t>(o_tab);
@@ -1251,6 +1532,15 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       route_lbw[(size_t)c] = lbw;
       t += ceil_div(x.n, rtile);
       lbw += ceil_div(x.n, rtile) << rbits;
+      if (words) {  // the route's view: offsets within words
+        x.lo = off(lo);
+        x.route_hi = range_of<K>(lo, hi);
+        x.wlo = fold.wlo;
+        x.ilo = fold.ilo;
+        x.ib = fold.ib;
+        x.dst_rows = side_rows[chunks[(size_t)c].side];
+        if (!radix_route) x.cuts = reinterpret_cast<const K*>(stg.at<uint64_t>(o_wcuts));
+      }
       hj[(size_t)nch + c] = x;
     }
   }
@@ -1316,9 +1606,12 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   // histograms, the groups' output bases).  The budget bounds control + the
   // larger of the two blocks + tables.
   const int64_t control = (int64_t)(cc.off - staging);
-  if (budget && control + lb_max + 4096 > (int64_t)budget)
+  // what separate columns would need decides whether the budget suffices
+  const int64_t ask_control = control - (words ? (int64_t)(kMaxCuts * sizeof(uint64_t)) : 0);
+  if (budget && ask_control + lb_max + 4096 > (int64_t)budget)
     return set_err(TJ_ERR_BUDGET, "budget %zu below the route pass's %lld bytes", budget,
-                   (long long)(control + lb_max + 4096));
+                   (long long)(ask_control + lb_max + 4096));
+  if (budget && control + lb_max > (int64_t)budget) return kColumnsAgain;
   Block rlb;
   TJ_CUDA(rlb.alloc((size_t)std::max<int64_t>(lb_max, 256), st));
   for (int c = 0; c < nch; ++c)
@@ -1331,10 +1624,15 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     TJ_CUDA(cudaMemsetAsync(d_counters + kMaxPasses, 0, sizeof(uint32_t), st));
     double rows = 0;
     for (int c = g.first; c < g.second; ++c) rows += (double)chunks[(size_t)c].n;
-    tr.begin("route", 4.0 * w * rows);
-    TJ_CUDA(launch_onesweep<K>(d_rj + nch + g.first, g.second - g.first, t, 0, rbits,
-                               radix_route ? kModeRadix : kModeCuts, d_counters + kMaxPasses,
-                               d_err, st, nullptr, ritems, est));
+    tr.begin("route", (2.0 * w + rowb) * rows);
+    if (words)
+      TJ_CUDA(launch_wsweep<K>(d_rj + nch + g.first, g.second - g.first, t, 0, rbits,
+                               radix_route ? kModeRadix : kModeCuts, true, false, ib >= 32, kWItems,
+                               est, d_counters + kMaxPasses, d_err, st));
+    else
+      TJ_CUDA(launch_onesweep<K>(d_rj + nch + g.first, g.second - g.first, t, 0, rbits,
+                                 radix_route ? kModeRadix : kModeCuts, d_counters + kMaxPasses,
+                                 d_err, st, nullptr, ritems, est));
     tr.end();
     if (est) {  // where this chunk ended: the next chunk's bases, or the side's end
       const int c = g.first, side = chunks[(size_t)c].side;
@@ -1351,12 +1649,20 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     TJ_CUDA(get_small(&h_err, d_err, sizeof(int), st));
     TJ_CUDA(sync_stream(st));
     if (h_err == TJ_ERR_CAPACITY) return kRouteAgain;
+    if (h_err == kErrFold) return kColumnsAgain;
     if (h_err) return set_err((tj_status)h_err, "device reported %d during the route pass", h_err);
     for (int side = 0; side < 2; ++side)
       for (int p2 = 0; p2 < nparts; ++p2) {
         const size_t i = (size_t)side * nparts + p2;
         pcount[i] = (int64_t)rfin[(size_t)side * kMaxBins + p2] - rstart[i];
       }
+  }
+  if (!est && words) {  // rows that did not fold: nothing may read them
+    int h_err = 0;
+    TJ_CUDA(get_small(&h_err, d_err, sizeof(int), st));
+    TJ_CUDA(sync_stream(st));
+    if (h_err == kErrFold || h_err == TJ_ERR_CAPACITY) return kColumnsAgain;
+    if (h_err) return set_err((tj_status)h_err, "device reported %d during the route pass", h_err);
   }
   if (!range_known) {
     // the smallest key is in the first non-empty batch, the largest in the
@@ -1375,7 +1681,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
         const size_t i = (size_t)side * nparts + p2;
         RadixJob<K> x;
         memset(&x, 0, sizeof(x));
-        x.keys = (side ? stg.at<K>(o_sk) : stg.at<K>(o_rk)) + rstart[i];
+        x.keys = routed(stg, side, rstart[i]);
         x.n = pcount[i];
         x.tile0 = rtiles;
         rtiles += ceil_div(x.n, kTile);
@@ -1384,7 +1690,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     TJ_CUDA(put_small(stg.at<RadixJob<K>>(o_rjobs), rj.data(), rj.size() * sizeof(RadixJob<K>), st));
     TJ_CUDA(cudaMemsetAsync(stg.at<KeyStats>(o_range), 0xFF, 4 * sizeof(KeyStats), st));
     tr.begin("stats", w * (double)rtiles * kTile);
-    TJ_CUDA(launch_stats<K>(stg.at<RadixJob<K>>(o_rjobs), 4, rtiles, stg.at<KeyStats>(o_range), st));
+    TJ_CUDA(launch_stats<K>(stg.at<RadixJob<K>>(o_rjobs), 4, rtiles, stg.at<KeyStats>(o_range), st,
+                            kTile, words));
     tr.end();
     KeyStats hr[4];
     TJ_CUDA(get_small(hr, stg.at<KeyStats>(o_range), sizeof(hr), st));
@@ -1394,8 +1701,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       mn = std::min(mn, hr[i].min_u);
       mx = std::max(mx, ~hr[i].max_u);
     }
-    lo = key_of<K>(mn);
-    hi = key_of<K>(mx);
+    lo = words ? (K)((mn >> ib) + fold.wlo) : key_of<K>(mn);
+    hi = words ? (K)((mx >> ib) + fold.wlo) : key_of<K>(mx);
     stats.key_bits = bitlen(range_of<K>(lo, hi));
   }
   {
@@ -1431,6 +1738,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     int64_t ws;   // working set without the look-back words
     int64_t lb;   // look-back bytes of one pass
     int np;       // passes (at least 1)
+    int64_t ask;  // working set as separate columns: what a budget must hold
     size_t hist_at;  // its histograms in the tables block (R side, then S side)
     int fj;          // fused: index of its FusedJob
   };
@@ -1494,8 +1802,11 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     const int64_t rtiles = ceil_div(q.nr, kTile) + ceil_div(q.ns, kTile);
     q.np = std::max(1, q.plan.passes);
     q.lb = rtiles * bins * 4;
-    q.ws = (int64_t)std::min(q.plan.passes, 1) * (q.nr + q.ns) * 2 * (int64_t)sizeof(K) +
-           ceil_div(q.ns, kJTile) * (int64_t)(sizeof(JTile<K>) + 12) + rtiles * 4 + 4096;
+    const int64_t buf = (int64_t)std::min(q.plan.passes, 1) * (q.nr + q.ns);
+    const int64_t rest =
+        ceil_div(q.ns, kJTile) * (int64_t)(sizeof(JTile<K>) + 12) + rtiles * 4 + 4096;
+    q.ask = buf * 2 * (int64_t)sizeof(K) + rest + q.lb * q.np;
+    q.ws = buf * (words ? 8 : 2 * (int64_t)sizeof(K)) + rest;
   };
   // ... and on the fused path: the MSD pass's output, its look-back words and
   // tile map, the items (descriptor and chained word), the multi-tile count
@@ -1506,9 +1817,12 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     q.lb = q.m > 0 ? rtiles * ((int64_t)1 << q.m) * 4 : 0;
     // (+ the layout's minimum of one count vector and one totals slot and its
     // 256-byte alignment of each of about a dozen arrays)
-    q.ws = (q.m > 0 ? (q.nr + q.ns) * 2 * (int64_t)sizeof(K) + rtiles * 4 : 0) +
-           q.items * (int64_t)(sizeof(FItem) + 8) +
-           (q.kbt + q.kbs + 2) * (int64_t)kFKeys * 4 + (int64_t)sizeof(FusedJob<K>) + 8192;
+    const int64_t rest = (q.m > 0 ? rtiles * 4 : 0) + q.items * (int64_t)(sizeof(FItem) + 8) +
+                         (q.kbt + q.kbs + 2) * (int64_t)kFKeys * 4 +
+                         (int64_t)sizeof(FusedJob<K>) + 8192;
+    const int64_t buf = q.m > 0 ? q.nr + q.ns : 0;
+    q.ask = buf * 2 * (int64_t)sizeof(K) + rest + q.lb * q.np;
+    q.ws = buf * (words ? 8 : 2 * (int64_t)sizeof(K)) + rest;
   };
   for (auto& q : P)
     if (!q.fused) plan_lsd(q);
@@ -1518,6 +1832,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       q.ws = 4096;
       q.lb = 0;
       q.np = 1;
+      q.ask = 4096;
     }
   // tables: histogram-pass jobs and group jobs (radix), join jobs, fused jobs
   // and their counts, histograms, output bases (one more than groups; at most
@@ -1532,8 +1847,9 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
                         ~(size_t)255;
   const size_t t_base = (t_hist + hist_words_all * 4 + 255) & ~(size_t)255;
   const size_t tbl_bytes = t_base + (P.size() + 1) * sizeof(int64_t);
-  const int64_t fixed = control + (int64_t)tbl_bytes + 4096;
-  const int64_t room = budget ? (int64_t)budget - fixed : INT64_MAX;
+  const int64_t fixed = ask_control + (int64_t)tbl_bytes + 4096;
+  const int64_t room = budget ? (int64_t)budget - fixed : INT64_MAX;  // to admit a batch
+  const int64_t use = budget ? room - (control - ask_control) : INT64_MAX;  // to group them
   if (room <= 0)
     return set_err(TJ_ERR_BUDGET, "budget %zu below the join's tables and control (%lld bytes)",
                    budget, (long long)fixed);
@@ -1553,8 +1869,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   // ---- 5. digit histograms of every batch in one launch ----
   // (the routed copies: LSD digits, or the MSD digit of a fused batch)
   auto batch_side = [&](const Part& q, int side, K** k0, K** v0) {
-    *k0 = side ? stg.at<K>(o_sk) + q.s0 : stg.at<K>(o_rk) + q.r0;
-    *v0 = side ? stg.at<K>(o_sv) + q.s0 : stg.at<K>(o_rv) + q.r0;
+    *k0 = routed(stg, side, side ? q.s0 : q.r0);
+    *v0 = words ? *k0 : side ? stg.at<K>(o_sv) + q.s0 : stg.at<K>(o_rv) + q.r0;
     return side ? q.ns : q.nr;
   };
   auto hist_jobs = [&](bool fused_only_lsd, std::vector<RadixJob<K>>& out, int64_t* tiles) {
@@ -1570,7 +1886,10 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
         K* v0;
         x.n = batch_side(q, side, &k0, &v0);
         x.keys = k0;
-        set_job_plan(x, q.plan);
+        if (words)
+          set_word_plan(x, q.plan, fold, off(q.lo) << ib);
+        else
+          set_job_plan(x, q.plan);
         x.hist_stride = 1 << q.plan.max_bits;
         x.hist = d_hist_all + q.hist_at + (side ? hist_half(q) : 0);
         x.tile0 = *tiles;
@@ -1578,6 +1897,11 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
         out.push_back(x);
       }
     }
+  };
+  auto batch_histogram = [&](const RadixJob<K>* jobs, int nj, int64_t tiles) -> cudaError_t {
+    return words ? launch_histogram<int64_t>(reinterpret_cast<const RadixJob<int64_t>*>(jobs), nj,
+                                             tiles, st)
+                 : launch_histogram<K>(jobs, nj, tiles, st);
   };
   int maxp = 0;
   for (auto& q : P) maxp = std::max(maxp, q.plan.passes);
@@ -1587,7 +1911,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   if (!all_rjh.empty()) {
     TJ_CUDA(put_small(d_rjh_all, all_rjh.data(), all_rjh.size() * sizeof(RadixJob<K>), st));
     tr.begin("histogram", w * (double)(nr + ns));
-    TJ_CUDA(launch_histogram<K>(d_rjh_all, (int)all_rjh.size(), htiles, st));
+    TJ_CUDA(batch_histogram(d_rjh_all, (int)all_rjh.size(), htiles));
     tr.end();
     TJ_CUDA(launch_digit_scan<K>(d_rjh_all, (int)all_rjh.size(), maxp, st));
   }
@@ -1602,7 +1926,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       f.hs = q.m > 0 ? d_hist_all + q.hist_at + hist_half(q) : nullptr;
       f.nr = q.nr;
       f.ns = q.ns;
-      f.lo = lo_bits<K>(q.lo);
+      f.lo = words ? off(q.lo) : lo_bits<K>(q.lo);
       f.m = q.m;
     }
     TJ_CUDA(put_small(d_fj_all, fj.data(), fj.size() * sizeof(FusedJob<K>), st));
@@ -1637,7 +1961,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
         for (auto& q : P)
           if (!q.fused && q.fj >= 0) dmaxp = std::max(dmaxp, q.plan.passes);
         TJ_CUDA(put_small(d_dj, dj.data(), dj.size() * sizeof(RadixJob<K>), st));
-        TJ_CUDA(launch_histogram<K>(d_dj, (int)dj.size(), dt, st));
+        TJ_CUDA(batch_histogram(d_dj, (int)dj.size(), dt));
         TJ_CUDA(launch_digit_scan<K>(d_dj, (int)dj.size(), dmaxp, st));
         maxp = std::max(maxp, dmaxp);
       }
@@ -1682,19 +2006,22 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     return -1;
   };
   {
-    const int64_t bad = make_groups(room);
+    int64_t bad = -1;
+    for (size_t i = 0; i < P.size() && bad < 0; ++i)
+      if (P[i].ask > room) bad = (int64_t)i;
+    if (bad < 0 && make_groups(use) >= 0) return kColumnsAgain;  // (words always fit, but for 8 KB)
     if (bad >= 0)
       return set_err(TJ_ERR_BUDGET,
                      "batch of keys [%lld, %lld] needs %lld bytes of working set, budget "
                      "leaves %lld (raise the budget or the number of batches)",
                      (long long)P[(size_t)bad].lo, (long long)P[(size_t)bad].hi,
-                     (long long)need_of((size_t)bad), (long long)room);
+                     (long long)P[(size_t)bad].ask, (long long)room);
   }
   int lanes = 1;
   if (groups.size() > 1) {
     const auto one = groups;
     const int64_t one_max = ws_max;
-    if (make_groups(room / 2) < 0) {
+    if (make_groups(use / 2) < 0) {
       lanes = 2;
     } else {
       groups = one;
@@ -1771,7 +2098,10 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     std::vector<size_t> o_buf(nj * 4, 0);
     for (size_t i = 0; i < nj; ++i) {
       const Part& q = P[g.first + i];
-      if (q.plan.passes > 0) {
+      if (q.plan.passes > 0 && words) {
+        o_buf[i * 4 + 0] = gc.add<uint64_t>((size_t)q.nr);
+        o_buf[i * 4 + 2] = gc.add<uint64_t>((size_t)q.ns);
+      } else if (q.plan.passes > 0) {
         o_buf[i * 4 + 0] = gc.add<K>((size_t)q.nr);
         o_buf[i * 4 + 1] = gc.add<K>((size_t)q.nr);
         o_buf[i * 4 + 2] = gc.add<K>((size_t)q.ns);
@@ -1787,9 +2117,10 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       else
         gp.maxbits = std::max(gp.maxbits, q.plan.max_bits);
     }
-    gp.ipt = gp.maxbits <= kWideBits ? kItemsWide : kItems;
-    gp.iptm = gp.maxbitsm <= kWideBits ? kItemsWide : kItems;
-    const int64_t otile = (int64_t)kSortThreads * gp.ipt, otilem = (int64_t)kSortThreads * gp.iptm;
+    gp.ipt = words ? kWItems : gp.maxbits <= kWideBits ? kItemsWide : kItems;
+    gp.iptm = words ? kWItems : gp.maxbitsm <= kWideBits ? kItemsWide : kItems;
+    const int64_t othreads = words ? kWThreads : kSortThreads;
+    const int64_t otile = othreads * gp.ipt, otilem = othreads * gp.iptm;
     std::vector<size_t> lb_at(nj * 2);
     for (size_t i = 0; i < nj; ++i) {
       const Part& q = P[g.first + i];
@@ -1865,18 +2196,25 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
         memset(&x, 0, sizeof(x));
         x.keys = k0;
         x.n = n;
-        set_job_plan(x, q.plan);
+        if (words)
+          set_word_plan(x, q.plan, fold, off(q.lo) << ib);
+        else
+          set_job_plan(x, q.plan);
         x.hist_stride = 1 << q.plan.max_bits;
         x.hist = d_hist_all + q.hist_at + (side ? hist_half(q) : 0);
         K* ak = lw.at<K>(o_buf[i * 4 + 2 * side]);
-        K* av = lw.at<K>(o_buf[i * 4 + 2 * side + 1]);
+        K* av = words ? ak : lw.at<K>(o_buf[i * 4 + 2 * side + 1]);
         const K** rk = &res[i * 4 + 2 * side];
         const K** rv = &res[i * 4 + 2 * side + 1];
         if (q.fused) {
           // the MSD pass: routed copy -> the batch's MSD output
           x.lookback = lw.at<uint32_t>(gp.o_lbm) + lb_at[i * 2 + side];
           x.lb_stride = (int64_t)gp.lbm_words;
-          set_job_buffers(x, k0, v0, ak, av, ak, av, rk, rv);
+          if (words)
+            *rk = *rv = reinterpret_cast<const K*>(
+                set_word_buffers<K>(x, k0, nullptr, reinterpret_cast<uint64_t*>(ak), nullptr));
+          else
+            set_job_buffers(x, k0, v0, ak, av, ak, av, rk, rv);
           x.tile0 = gp.tilesm;
           gp.tilesm += ceil_div(n, otilem);
           rj_msd.push_back(x);
@@ -1884,7 +2222,12 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
           // LSD passes alternate: routed copy -> buffer -> routed copy -> ...
           x.lookback = lw.at<uint32_t>(gp.o_lb) + lb_at[i * 2 + side];
           x.lb_stride = (int64_t)gp.lb_words;
-          set_job_buffers(x, k0, v0, ak, av, k0, v0, rk, rv);
+          if (words)
+            *rk = *rv = reinterpret_cast<const K*>(
+                set_word_buffers<K>(x, k0, nullptr, reinterpret_cast<uint64_t*>(ak),
+                                 reinterpret_cast<uint64_t*>(k0)));
+          else
+            set_job_buffers(x, k0, v0, ak, av, k0, v0, rk, rv);
           x.tile0 = gp.tiles;
           gp.tiles += ceil_div(n, otile);
           rj_lsd.push_back(x);
@@ -2009,8 +2352,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     // joins, launches counted) with two events instead of two per kernel.
     const bool whole = lanes > 1;
     if (whole) {
-      double by = 2.0 * w * gp.rows + 4.0 * w * gp.msd_rows;  // join input, MSD pass
-      for (int p = 0; p < gp.P; ++p) by += 4.0 * w * gp.prow[p];
+      double by = rowb * gp.rows + 2.0 * rowb * gp.msd_rows;  // join input, MSD pass
+      for (int p = 0; p < gp.P; ++p) by += 2.0 * rowb * gp.prow[p];
       tr.begin("group/lanes", by, gs, gp.P + 2 + 2 * (int)gp.runs.size());
     }
     TJ_CUDA(cudaMemsetAsync(lw.p + gp.o_zero, 0, gp.zero_bytes, gs));
@@ -2026,10 +2369,15 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     if (gp.nrj_lsd > 0) {
       RadixJob<K>* d_gj = d_rj_all + gp.rj_lsd_at;
       TJ_CUDA(launch_group_maps<K>(d_gj, gp.nrj_lsd, lw.at<int32_t>(gp.o_tmap), d_gjj, lsd_jobs,
-                                   lw.at<int32_t>(gp.o_jmap), gs, kSortThreads * gp.ipt));
+                                   lw.at<int32_t>(gp.o_jmap), gs,
+                                   (words ? kWThreads : kSortThreads) * gp.ipt));
       for (int p = 0; p < gp.P; ++p) {
-        if (!whole) tr.begin("onesweep", 4.0 * w * gp.prow[p], gs);
-        TJ_CUDA(launch_onesweep<K>(d_gj, gp.nrj_lsd, gp.tiles, p, gp.maxbits, kModeSort,
+        if (!whole) tr.begin("onesweep", 2.0 * rowb * gp.prow[p], gs);
+        if (words)
+          TJ_CUDA(word_pass<K>(d_gj, gp.nrj_lsd, gp.tiles, p, gp.maxbits, false, fold, gp.ipt,
+                               d_gcnt + p, d_err, gs, lw.at<int32_t>(gp.o_tmap)));
+        else
+          TJ_CUDA(launch_onesweep<K>(d_gj, gp.nrj_lsd, gp.tiles, p, gp.maxbits, kModeSort,
                                    d_gcnt + p, d_err, gs, lw.at<int32_t>(gp.o_tmap), gp.ipt));
         if (!whole) tr.end();
       }
@@ -2040,31 +2388,35 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     if (gp.nrj_msd > 0) {
       RadixJob<K>* d_gm = d_rj_all + gp.rj_msd_at;
       TJ_CUDA(launch_group_maps<K>(d_gm, gp.nrj_msd, lw.at<int32_t>(gp.o_tmapm), nullptr, 0,
-                                   nullptr, gs, kSortThreads * gp.iptm));
-      if (!whole) tr.begin("msd", 4.0 * w * gp.msd_rows, gs);
-      TJ_CUDA(launch_onesweep<K>(d_gm, gp.nrj_msd, gp.tilesm, 0, gp.maxbitsm, kModeSort,
+                                   nullptr, gs, (words ? kWThreads : kSortThreads) * gp.iptm));
+      if (!whole) tr.begin("msd", 2.0 * rowb * gp.msd_rows, gs);
+      if (words)
+        TJ_CUDA(word_pass<K>(d_gm, gp.nrj_msd, gp.tilesm, 0, gp.maxbitsm, false, fold, gp.iptm,
+                             d_gcnt + kMaxPasses, d_err, gs, lw.at<int32_t>(gp.o_tmapm)));
+      else
+        TJ_CUDA(launch_onesweep<K>(d_gm, gp.nrj_msd, gp.tilesm, 0, gp.maxbitsm, kModeSort,
                                  d_gcnt + kMaxPasses, d_err, gs, lw.at<int32_t>(gp.o_tmapm),
                                  gp.iptm));
       if (!whole) tr.end();
     }
     if (gp.jtiles > 0)
       TJ_CUDA(launch_tile_ranges<K>(d_gjj, lsd_jobs, gp.jtiles, lw.at<JTile<K>>(gp.o_jt), gs,
-                                    lw.at<int32_t>(gp.o_jmap)));
+                                    lw.at<int32_t>(gp.o_jmap), fmt));
     for (auto& r : gp.runs)
       if (r.fused)
         TJ_CUDA(launch_fused_prep<K>(d_fj_all + r.jj_at, (int)r.nj, lw.at<FItem>(r.o_items),
-                                     r.items, r.any_multi, lw.at<uint32_t>(r.o_kbt), gs));
+                                     r.items, r.any_multi, lw.at<uint32_t>(r.o_kbt), gs, fmt));
     if (lanes > 1 && g > 0) TJ_CUDA(cudaStreamWaitEvent(gs, side->ev[1], 0));
     for (size_t ri = 0; ri < gp.runs.size(); ++ri) {
       const RunPlan& r = gp.runs[ri];
       uint32_t* cnt = d_gcnt + kMaxPasses + 1 + ri;
       if (r.fused) {
-        if (!whole) tr.begin("fused", 2.0 * w * r.rows, gs);
+        if (!whole) tr.begin("fused", rowb * r.rows, gs);
         if (r.items > 0) {
           TJ_CUDA(launch_fused_join<K>(d_fj_all + r.jj_at, lw.at<FItem>(r.o_items), r.items, cnt,
                                        lw.at<uint64_t>(r.o_ilb), lw.at<uint32_t>(r.o_kbl),
                                        lw.at<uint32_t>(r.o_kbt), out, cap, d_gbase + r.base,
-                                       d_gbase + r.base + 1, d_err, gs));
+                                       d_gbase + r.base + 1, d_err, gs, fmt));
         } else {  // no pairs in this run: the next one starts where it did
           TJ_CUDA(launch_copy_bytes(d_gbase + r.base + 1, d_gbase + r.base, sizeof(int64_t), gs));
         }
@@ -2072,13 +2424,13 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       } else if (r.cross) {
         if (!whole) tr.begin("cross", w * (double)r.rows + 2.0 * w * (double)r.pairs, gs);
         TJ_CUDA(launch_cross<K>(d_cj_all + r.jj_at, (int)r.nj, r.xblocks, out, cap,
-                                d_gbase + r.base, d_gbase + r.base + 1, r.pairs, gs));
+                                d_gbase + r.base, d_gbase + r.base + 1, r.pairs, gs, fmt));
         if (!whole) tr.end();
       } else {
-        if (!whole) tr.begin("join", 2.0 * w * r.rows, gs);
+        if (!whole) tr.begin("join", rowb * r.rows, gs);
         TJ_CUDA(launch_join<K>(r.jtiles, lw.at<JTile<K>>(gp.o_jt) + r.jt0,
                                lw.at<uint64_t>(r.o_jlb), cnt, out, cap, d_gbase + r.base, nullptr,
-                               d_gbase + r.base + 1, d_err, gs));
+                               d_gbase + r.base + 1, d_err, gs, fmt));
         if (!whole) tr.end();
       }
     }
@@ -2107,6 +2459,71 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
 }
 
 // ---- sort ---------------------------------------------------------------------------
+// The passes over folded rows.  64-bit rows: columns -> words -> ... -> columns,
+// the words alternating between two scratch arrays, so the caller's columns
+// stay as they are until the last pass (which does not run if a row failed to
+// fold).  32-bit rows always fold and a word is no smaller than a row: their
+// passes alternate between one array of words and the caller's columns.
+template <typename K>
+tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f,
+                     RadixJob<K>* d_jobs, uint32_t* d_counters, int* d_err, size_t ctl_bytes,
+                     tj_stats& stats, Tracer& tr, cudaStream_t st) {
+  const double w = (double)sizeof(K);
+  const int P = plan.passes;
+  const int items = word_items(n);
+  const int64_t otiles = ceil_div(n, (int64_t)kWThreads * items);
+  const int64_t lb_words = otiles << plan.max_bits;
+  // one cleared look-back region per pass while they are small, else one
+  // cleared before every pass
+  const bool regions = (int64_t)P * lb_words * 4 <= (int64_t)1 << 20;
+  Carve bc;
+  const size_t o_a = bc.add<uint64_t>((size_t)n);
+  const size_t o_b = bc.add<uint64_t>(sizeof(K) == 8 && P > 2 ? (size_t)n : 0);
+  const size_t o_hist = bc.add<uint32_t>((size_t)P << plan.max_bits);
+  const size_t o_lb = bc.add<uint32_t>((size_t)(regions ? P : 1) * lb_words);
+  Block big;
+  TJ_CUDA(big.alloc(bc.off, st));
+  stats.scratch_peak = (int64_t)(bc.off + ctl_bytes);
+  RadixJob<K> hj[2];  // the histogram's view (columns), the passes' view (words)
+  memset(hj, 0, sizeof(hj));
+  hj[0].keys = keys;
+  hj[0].n = n;
+  set_job_plan(hj[0], plan);
+  hj[0].hist_stride = 1 << plan.max_bits;
+  hj[0].hist = big.at<uint32_t>(o_hist);
+  hj[1] = hj[0];
+  set_word_plan(hj[1], plan, f, 0);
+  hj[1].lookback = big.at<uint32_t>(o_lb);
+  hj[1].lb_stride = regions ? lb_words : 0;
+  auto folds = [&](int p) { return p == 0 || (sizeof(K) == 4 && (p & 1) == 0); };
+  auto unfolds = [&](int p) { return p == P - 1 || (sizeof(K) == 4 && (p & 1) == 1); };
+  uint64_t* a = big.at<uint64_t>(o_a);
+  uint64_t* b = big.at<uint64_t>(o_b);
+  for (int p = 0; p < P; ++p) {
+    K* in = reinterpret_cast<K*>(sizeof(K) == 4 || (p & 1) ? a : b);
+    K* to = reinterpret_cast<K*>(sizeof(K) == 4 || !(p & 1) ? a : b);
+    hj[1].src_k[p] = folds(p) ? keys : in;
+    if (folds(p)) hj[1].fold_v[p] = ids;
+    hj[1].dst_k[p] = unfolds(p) ? keys : to;
+    hj[1].dst_v[p] = unfolds(p) ? ids : nullptr;
+  }
+  TJ_CUDA(put_small(d_jobs, hj, sizeof(hj), st));
+  TJ_CUDA(cudaMemsetAsync(big.p + o_hist, 0,
+                          (regions ? o_lb + (size_t)P * lb_words * 4 : o_lb) - o_hist, st));
+  tr.begin("histogram", w * n);
+  TJ_CUDA(launch_histogram<K>(d_jobs, 1, ceil_div(n, kTile), st));
+  tr.end();
+  TJ_CUDA(launch_digit_scan<K>(d_jobs, 1, P, st));
+  for (int p = 0; p < P; ++p) {
+    if (!regions) TJ_CUDA(cudaMemsetAsync(big.p + o_lb, 0, (size_t)lb_words * 4, st));
+    tr.begin("onesweep", (2.0 * ((folds(p) ? w : 4.0) + (unfolds(p) ? w : 4.0))) * n);
+    TJ_CUDA(launch_wsweep<K>(d_jobs + 1, 1, otiles, p, plan.max_bits, kModeSort, folds(p),
+                             unfolds(p), f.ib >= 32, items, false, d_counters + p, d_err, st));
+    tr.end();
+  }
+  return TJ_OK;
+}
+
 template <typename K>
 tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
   tj_stats stats = {};
@@ -2119,7 +2536,7 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
   if (s != TJ_OK) return s;
   const int64_t tiles = ceil_div(n, kTile);
   Carve cc;
-  const size_t o_jobs = cc.add<RadixJob<K>>(1);
+  const size_t o_jobs = cc.add<RadixJob<K>>(2);
   const size_t o_stats = cc.add<KeyStats>(1);
   const size_t o_misc = cc.add<int64_t>(32);
   Block ctl;
@@ -2132,6 +2549,7 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
   RadixJob<K> hj;
   memset(&hj, 0, sizeof(hj));
   hj.keys = keys;
+  hj.ids = sizeof(K) == 8 ? ids : nullptr;
   hj.n = n;
   TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
   TJ_CUDA(cudaMemsetAsync(d_stats, 0xFF, sizeof(KeyStats), st));
@@ -2154,6 +2572,32 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
   if (plan.passes == 0) {  // all keys equal: already sorted
     g_stats = stats;
     return TJ_OK;
+  }
+  const Fold fold = make_fold<K>(plan.lo, plan.key_bits, hs.id_min_u, ~hs.id_max_u);
+  if (fold.on) {
+    // (below kCostRows a pass's fixed cost decides: the fewest passes)
+    const Plan wplan = n >= kCostRows
+                           ? make_word_plan(plan.lo, range_of<K>(lo, hi), sizeof(K) == 4,
+                                            max_digit_bits<K>(), 2)
+                           : plan;
+    stats.radix_passes = wplan.passes;
+    stats.digit_bits = wplan.max_bits;
+    s = sort_words<K>(keys, ids, n, wplan, fold, d_jobs, d_counters, d_err, cc.off, stats, tr2,
+                      st);
+    if (s != TJ_OK) return s;
+    int h_err = 0;
+    TJ_CUDA(get_small(&h_err, d_err, sizeof(int), st));
+    TJ_CUDA(sync_stream(st));
+    if (h_err == 0) {
+      tr2.flush();
+      g_stats = stats;
+      return TJ_OK;
+    }
+    if (h_err != kErrFold) return set_err((tj_status)h_err, "device reported %d", h_err);
+    // an id outside the window of the sampled ones: the columns are untouched
+    stats.radix_passes = plan.passes;
+    stats.digit_bits = plan.max_bits;
+    TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
   }
   const int64_t bins_max = (int64_t)1 << plan.max_bits;
   // onesweep tiles (narrow digits: the wider tile); the histogram keeps kTile

@@ -31,6 +31,8 @@
 //   k_fused_items : the item list of a group in key order;
 //   k_fused_hist  : per-key totals of the multi-tile sub-batches;
 //   k_fused_join  : the join of one item.
+#include <type_traits>
+
 #include "tj_internal.cuh"
 #include "tj_warp.cuh"
 
@@ -39,22 +41,28 @@ namespace tj {
 namespace {
 
 constexpr int kFWarps = kFThreads / 32;
-constexpr int kFItemsS = kFCapS / kFThreads;  // S rows per thread (9)
+constexpr int kFItemsS = kFCapS / kFThreads;  // S rows per thread (18)
 static_assert(kFItemsS * kFThreads == kFCapS, "S tile = threads x rows per thread");
-constexpr int kFItemsR = kFCapR / kFThreads;  // R rows per thread (4)
+constexpr int kFItemsR = kFCapR / kFThreads;  // R rows per thread (8)
+constexpr int kFKeysT = kFKeys / kFThreads;   // key offsets per thread in the scans (4)
 constexpr int kFDigit = kFKeyBits / 2;        // bits per in-smem sort pass (5)
 constexpr int kFBins = 1 << kFDigit;          // 32
 static_assert(kFDigit * 2 == kFKeyBits, "two in-smem passes cover the key offset");
-static_assert(kFKeys == 2 * kFThreads, "two key offsets per thread in the scans");
+static_assert(kFKeysT == 4, "four key offsets per thread in the scans: 16-byte words");
 static_assert(kFCapS <= 65536 && kFCapR <= 65536, "16-bit row indices");
 
-__device__ __forceinline__ uint32_t ld_vol_u32(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.volatile.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+__device__ __forceinline__ uint4 ld_vol_v4(const uint32_t* p) {
+  uint4 v;
+  asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p)
+               : "memory");
   return v;
 }
-__device__ __forceinline__ void st_vol_u32(uint32_t* p, uint32_t v) {
-  asm volatile("st.volatile.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void st_vol_v4(uint32_t* p, uint4 v) {
+  asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y),
+               "r"(v.z), "r"(v.w)
+               : "memory");
 }
 __device__ __forceinline__ uint64_t ld_vol_u64(const uint64_t* p) {
   uint64_t v;
@@ -215,7 +223,7 @@ __global__ void __launch_bounds__(kFThreads) k_fused_items(const FusedJob<K>* __
 template <typename K>
 __global__ void __launch_bounds__(256) k_fused_hist(const FusedJob<K>* __restrict__ jobs,
                                                     const FItem* __restrict__ items,
-                                                    uint32_t* __restrict__ tot) {
+                                                    uint32_t* __restrict__ tot, int ib) {
   __shared__ uint32_t h[kFKeys];
   const FItem it = items[blockIdx.x];
   if (it.kbt < 0) return;
@@ -226,7 +234,7 @@ __global__ void __launch_bounds__(256) k_fused_hist(const FusedJob<K>* __restric
   const int n = it.ns;
   const K* __restrict__ sk = reinterpret_cast<const K*>(it.sk);
   for (int i = threadIdx.x; i < n; i += 256)
-    atomicAdd(&h[(uint32_t)((U)sk[i] - sublo) & (kFKeys - 1)], 1u);
+    atomicAdd(&h[(uint32_t)(((U)sk[i] >> ib) - sublo) & (kFKeys - 1)], 1u);
   __syncthreads();
   uint32_t* T = tot + (size_t)it.kbs * kFKeys;
   for (int i = threadIdx.x; i < kFKeys; i += 256)
@@ -298,8 +306,8 @@ __device__ __forceinline__ void sort_offsets(const uint16_t* __restrict__ koff, 
 // word) and lane-mask tables of the ranking | per key offset: the
 // sub-batch's R rows (two 16-bit counters a word) and the entry a row reads
 // to write its pairs | the R rows' key offsets, sorted by key offset
-// (stably) when a key has several R rows.  About 75 KB: three CTAs a
-// multiprocessor.
+// (stably) when a key has several R rows.  About 48 KB: four CTAs a
+// multiprocessor, which their 64 registers a thread allow too.
 // What a row of key offset k needs to write its pairs, in one 16-byte load:
 // the position of the key's first pair for this tile's rows within the
 // sub-batch's output (~0: no R row has the key), and the key's R id (one R
@@ -312,13 +320,17 @@ struct alignas(16) KeyEnt {
 
 template <typename K>
 struct FusedSmem {
-  uint32_t wh[kFWarps][kFKeys / 2];
-  uint32_t wm[kFWarps][128];
+  uint16_t wh[kFWarps][kFKeys];
+  union {
+    uint32_t wm[kFWarps][128 * kWMaskItems];  // dead before the R rows are sorted
+    struct {
+      uint16_t r_pa[kFCapR];
+      uint16_t r_pb[kFCapR];
+    };
+  };
   uint32_t cR[kFKeys / 2];
   KeyEnt<K> ent[kFKeys];
   uint16_t r_koff[kFCapR];
-  uint16_t r_pa[kFCapR];
-  uint16_t r_pb[kFCapR];
   uint32_t wcnt[kFWarps * (kFBins / 2)];
   uint16_t wexcl[kFWarps * kFBins];
   uint32_t dbase[kFBins];
@@ -339,149 +351,189 @@ size_t fused_smem_bytes() {
 //   1. R rows: count per key offset; a key's first R id goes to a table (a
 //      key with several R rows sets a flag: then the R rows are sorted by key
 //      offset, stably, and each key's run is used);
-//   2. S rows into registers (warp w owns rows [w 256, (w + 1) 256), item u
-//      of a lane is row w 256 + 32 u + lane), counted per key offset, ranked
-//      stably within the warp by key offset (rank_items_or);
+//   2. S rows (warp w owns 32 kFItemsS consecutive ones, item u of a lane is
+//      the warp's row 32 u + lane) counted per key offset and ranked stably
+//      within the warp by key offset (wrank); the rows are read again (from
+//      L2) when their pairs are written, so only ranks stay in registers;
 //   3. per key offset: the S rows of earlier warps (prefix over the warps'
 //      counters), of earlier tiles of the sub-batch (look-back over count
 //      vectors), and the key's first pair, Sum_{k' < k} |S_k'| |R_k'|;
 //   4. the chained scan over the group's items gives the tile's first pair;
 //   5. each S row's pairs go to their final position straight from registers.
+// Eight warps a CTA, four CTAs a multiprocessor: the per-warp counter tables
+// are cleared and summed for every item, so few warps with many rows each pay
+// less for them, and four items in different phases hide each other's waits.
 #ifndef TJ_FUSED_MINB
-#define TJ_FUSED_MINB 2
+#define TJ_FUSED_MINB 4
 #endif
-template <typename K>
+// WORDS: the rows are folded (tj_word.cu), R and S words at it.rk and it.sk.
+template <typename K, bool WORDS>
 __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
-    k_fused_join(const FItem* __restrict__ items,
+    k_fused_join(const FItem* __restrict__ items, WordFmt f,
                  int64_t n_items, uint32_t* __restrict__ item_counter,
                  uint64_t* __restrict__ item_lb, uint32_t* __restrict__ kb_lb,
                  const uint32_t* __restrict__ kb_tot, K* __restrict__ out, int64_t capacity,
                  const int64_t* __restrict__ out_base, int64_t* __restrict__ total,
                  int* __restrict__ err) {
-  using U = typename UnsignedOf<K>::type;
+  using Elem = typename std::conditional<WORDS, uint64_t, K>::type;
+  const uint64_t idm = (1ull << f.ib) - 1ull;
+  // key offset within the sub-batch, id of a word
+  auto koff = [&](Elem e, uint32_t sublo) -> uint32_t {
+    return ((WORDS ? (uint32_t)((uint64_t)e >> f.ib) : (uint32_t)e) - sublo) & (kFKeys - 1);
+  };
+  auto word_id = [&](uint64_t e) -> K { return (K)((e & idm) + f.ilo); };
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FusedSmem<K>& S = *reinterpret_cast<FusedSmem<K>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) S.s_item = atomicAdd(item_counter, 1u);
   // counters and tables start at zero
-  for (int i = tid; i < kFWarps * (kFKeys / 2); i += kFThreads) (&S.wh[0][0])[i] = 0u;
-  for (int i = tid; i < kFWarps * 128; i += kFThreads) (&S.wm[0][0])[i] = 0u;
-  for (int i = tid; i < kFKeys / 2; i += kFThreads) S.cR[i] = 0u;
+  {
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < (int)(sizeof(S.wh) / 16); i += kFThreads)
+      reinterpret_cast<uint4*>(S.wh)[i] = z;
+    for (int i = tid; i < (int)(sizeof(S.wm) / 16); i += kFThreads)
+      reinterpret_cast<uint4*>(S.wm)[i] = z;
+    for (int i = tid; i < (int)(sizeof(S.cR) / 16); i += kFThreads)
+      reinterpret_cast<uint4*>(S.cR)[i] = z;
+  }
   __syncthreads();
   const int64_t ii = S.s_item;
   if (ii >= n_items) return;
   const FItem it = items[ii];
   const int t = (int)(it.dt >> 11);
   const bool multi_tile = it.kbt >= 0;
-  const U sublo = (U)it.sublo;
+  const uint32_t sublo = (uint32_t)it.sublo;  // offsets below 2^10: 32 bits suffice
   const int nr = it.nr;  // <= kFCapR (the host checked)
   const int ns = it.ns;
   const K* __restrict__ g_rv = reinterpret_cast<const K*>(it.rv);
   const K* __restrict__ g_sv = reinterpret_cast<const K*>(it.sv);
 
-  // 1. the tile's global loads in flight at once: S keys, R keys and ids
-  //    (the S ids are loaded when the pairs are written)
+  // 1. the tile's global loads in flight at once: S keys (the S ids are loaded
+  //    when the pairs are written), half of the R rows there is room for
   const int wrow = warp * 32 * kFItemsS;
-  K rkey[kFItemsR], rid_v[kFItemsR], skey[kFItemsS];
-  {
-    const K* __restrict__ rk = reinterpret_cast<const K*>(it.rk);
-    const K* __restrict__ rv = g_rv;
-    const K* __restrict__ sk = reinterpret_cast<const K*>(it.sk);
+  const Elem* __restrict__ g_rk = reinterpret_cast<const Elem*>(it.rk);
+  const Elem* __restrict__ g_sk = reinterpret_cast<const Elem*>(it.sk);
+  // a row past the end takes the last key offset: it ranks after all rows
+  const Elem pad = WORDS ? (Elem)((it.sublo + (kFKeys - 1)) << f.ib)
+                         : (Elem)(it.sublo + (kFKeys - 1));
+  Elem skey[kFItemsS];
 #pragma unroll
-    for (int u = 0; u < kFItemsS; ++u) {
-      const int row = wrow + u * 32 + lane;
-      skey[u] = row < ns ? sk[row] : K(0);
-    }
-#pragma unroll
-    for (int u = 0; u < kFItemsR; ++u) {
-      const int i = tid + u * kFThreads;
-      rkey[u] = i < nr ? rk[i] : K(0);
-      rid_v[u] = i < nr ? rv[i] : K(0);
-    }
+  for (int u = 0; u < kFItemsS; ++u) {
+    const int row = wrow + u * 32 + lane;
+    skey[u] = row < ns ? g_sk[row] : pad;
   }
   // R rows: counts per key offset, a key's first R id in the table
   bool dup = false;
+#pragma unroll 1
+  for (int u0 = 0; u0 * kFThreads < nr; u0 += kFItemsR / 2) {
+    Elem rkey[kFItemsR / 2];
+    K rid_v[WORDS ? 1 : kFItemsR / 2];
 #pragma unroll
-  for (int u = 0; u < kFItemsR; ++u) {
-    const int i = tid + u * kFThreads;
-    if (i < nr) {
-      const uint32_t o = (uint32_t)((U)rkey[u] - sublo) & (kFKeys - 1);
-      S.r_koff[i] = (uint16_t)o;
-      const uint32_t sh = (o & 1u) * 16u;  // counts <= kFCapR: the halves never carry
-      if (((atomicAdd(&S.cR[o >> 1], 1u << sh) >> sh) & 0xFFFFu) == 0u)
-        S.ent[o].r = rid_v[u];  // the key's R id, kept unless the key has several
-      else
-        dup = true;
+    for (int u = 0; u < kFItemsR / 2; ++u) {
+      const int i = tid + (u0 + u) * kFThreads;
+      rkey[u] = i < nr ? g_rk[i] : Elem(0);
+      if constexpr (!WORDS) rid_v[u] = i < nr ? g_rv[i] : K(0);
+    }
+#pragma unroll
+    for (int u = 0; u < kFItemsR / 2; ++u) {
+      const int i = tid + (u0 + u) * kFThreads;
+      if (i < nr) {
+        const uint32_t o = koff(rkey[u], sublo);
+        K rid;
+        if constexpr (WORDS) rid = word_id(rkey[u]);
+        else rid = rid_v[u];
+        S.r_koff[i] = (uint16_t)o;
+        const uint32_t sh = (o & 1u) * 16u;  // counts <= kFCapR: the halves never carry
+        if (((atomicAdd(&S.cR[o >> 1], 1u << sh) >> sh) & 0xFFFFu) == 0u)
+          S.ent[o].r = rid;  // the key's R id, kept unless the key has several
+        else
+          dup = true;
+      }
     }
   }
   // 2. S rows counted and ranked
-  uint32_t dr[kFItemsS];
+  Half<kFItemsS> rank, dig;
+  if constexpr (!WORDS) {  // folded rows give the offset again when they are read again
 #pragma unroll
-  for (int u = 0; u < kFItemsS; ++u) dr[u] = (uint32_t)((U)skey[u] - sublo) & (kFKeys - 1);
-  rank_items_or<kFKeyBits - 7, kFItemsS>(dr, ns - wrow, &S.wh[warp][0], &S.wm[warp][0]);
+    for (int u = 0; u < kFItemsS; ++u) dig.set(u, koff(skey[u], sublo));
+  }
+  auto row_digit = [&](int u) -> uint32_t {
+    if constexpr (WORDS) return koff(skey[u], sublo);
+    else return dig.get(u);
+  };
+  wrank<kFKeyBits, kFItemsS>(row_digit, rank, S.wh[warp], S.wm[warp], ns - wrow);
   dup = __syncthreads_or(dup) != 0;  // also: counts complete, ranks done
 
-  // 3. per key offset (two per thread: word tid of the warps' counters):
-  //    the S rows of earlier warps, and the tile's count
-  const int k0 = 2 * tid;
-  uint32_t cs[2];
+  // 3. per key offset (four per thread, two 16-bit counters a word): the S rows
+  //    of earlier warps, and the tile's count
+  const int k0 = kFKeysT * tid;
+  uint32_t cs[kFKeysT];
   {
-    uint32_t run = 0;  // the two 16-bit halves never carry (counts <= kFCapS)
+    uint2 run = make_uint2(0u, 0u);  // the 16-bit halves never carry (counts <= kFCapS)
 #pragma unroll
     for (int w = 0; w < kFWarps; ++w) {
-      const uint32_t c = S.wh[w][tid];
-      S.wh[w][tid] = run;
-      run += c;
+      uint2* c = reinterpret_cast<uint2*>(&S.wh[w][k0]);
+      const uint2 v = *c;
+      *c = run;
+      run.x += v.x;
+      run.y += v.y;
     }
-    cs[0] = run & 0xFFFFu;
-    cs[1] = run >> 16;
+    cs[0] = run.x & 0xFFFFu;
+    cs[1] = run.x >> 16;
+    cs[2] = run.y & 0xFFFFu;
+    cs[3] = run.y >> 16;
+    if (tid == kFThreads - 1) {
+      // the last warp with rows ranked its last group whole: those past the
+      // end were counted as the last key offset
+      constexpr int kGroup = 32 * wrank_group<kFItemsS>();
+      const int local = (ns - 1) % (32 * kFItemsS) + 1;
+      cs[3] -= (uint32_t)((local + kGroup - 1) / kGroup * kGroup - local);
+    }
   }
   // multi-tile sub-batches: publish this tile's counts (look-back over the
   // sub-batch's tiles, one word per key offset)
   uint32_t* lb_mine = multi_tile ? kb_lb + (size_t)it.kbt * kFKeys : nullptr;
-  if (multi_tile)
-#pragma unroll
-    for (int e = 0; e < 2; ++e) st_vol_u32(lb_mine + k0 + e, (t == 0 ? kFlagInc : kFlagAgg) | cs[e]);
+  if (multi_tile) {
+    const uint32_t fl = t == 0 ? kFlagInc : kFlagAgg;
+    st_vol_v4(lb_mine + k0, make_uint4(fl | cs[0], fl | cs[1], fl | cs[2], fl | cs[3]));
+  }
   // keys with several R rows: their R rows sorted by key offset
   if (dup) sort_offsets<kFItemsR>(S.r_koff, nr, S.r_pa, S.r_pb, S.wcnt, S.wexcl, S.dbase);
-  uint32_t pr[2] = {0u, 0u};
+  uint32_t pr[kFKeysT] = {0u, 0u, 0u, 0u};
   if (multi_tile && t > 0) {
     // decoupled look-back over the earlier tiles of the sub-batch (a window
-    // of kLB predecessors per round trip, both key offsets together; tile 0
-    // publishes inclusive counts, so the walk ends there at the latest;
-    // bounded wait)
-    constexpr int kLB = 8;
+    // of kLB predecessors per round trip, the four key offsets in lockstep;
+    // tile 0 publishes inclusive counts, so the walk ends there at the
+    // latest; bounded wait)
+    constexpr int kLB = 4;
     const int64_t first = it.kbt - t;  // a sub-batch's tiles have consecutive slots
-    int64_t p[2] = {it.kbt - 1, it.kbt - 1};
-    bool done[2] = {false, false};
+    int64_t p = it.kbt - 1;
+    uint32_t open = 0xFu;  // key offsets without an inclusive word yet
     int spins = 0;
-    while (!(done[0] && done[1])) {
-      uint32_t v[2][kLB];
+    while (open != 0u) {
+      uint4 v[kLB];
 #pragma unroll
-      for (int e = 0; e < 2; ++e)
+      for (int q = 0; q < kLB; ++q)
+        v[q] = p - q >= first ? ld_vol_v4(kb_lb + (size_t)(p - q) * kFKeys + k0)
+                              : make_uint4(kFlagInc, kFlagInc, kFlagInc, kFlagInc);
+      int used = 0;
 #pragma unroll
-        for (int q = 0; q < kLB; ++q)
-          v[e][q] = (!done[e] && p[e] - q >= first)
-                        ? ld_vol_u32(kb_lb + (size_t)(p[e] - q) * kFKeys + k0 + e)
-                        : kFlagInc;
-      bool progress = false;
+      for (int q = 0; q < kLB; ++q) {
+        const uint32_t x[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+        bool ready = true;
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        if (done[e]) continue;
+        for (int e = 0; e < kFKeysT; ++e) ready &= (x[e] & ~kValMask) != 0u;
+        if (used != q || !ready) continue;  // an earlier one is not published yet
+        ++used;
 #pragma unroll
-        for (int q = 0; q < kLB; ++q) {
-          const uint32_t f = v[e][q] & ~kValMask;
-          if (f == 0u) break;  // not published yet: wait for it
-          pr[e] += v[e][q] & kValMask;
-          --p[e];
-          progress = true;
-          if (f == kFlagInc) {
-            done[e] = true;
-            break;
+        for (int e = 0; e < kFKeysT; ++e)
+          if ((open >> e) & 1u) {
+            pr[e] += x[e] & kValMask;
+            if ((x[e] & ~kValMask) == kFlagInc) open &= ~(1u << e);
           }
-        }
       }
-      if (!progress) {
+      p -= used;
+      if (used == 0) {
         if (++spins > kSpinLimit) {
           atomicExch(err, (int)TJ_ERR_TIMEOUT);
           break;
@@ -489,31 +541,40 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
         __nanosleep(32);
       }
     }
-#pragma unroll
-    for (int e = 0; e < 2; ++e)
-      st_vol_u32(lb_mine + k0 + e, kFlagInc | ((pr[e] + cs[e]) & kValMask));
+    st_vol_v4(lb_mine + k0, make_uint4(kFlagInc | ((pr[0] + cs[0]) & kValMask),
+                                       kFlagInc | ((pr[1] + cs[1]) & kValMask),
+                                       kFlagInc | ((pr[2] + cs[2]) & kValMask),
+                                       kFlagInc | ((pr[3] + cs[3]) & kValMask)));
   }
-  uint32_t cr[2];
-  uint64_t tot[2];
+  uint32_t cr[kFKeysT], tot[kFKeysT];
   {
-    const uint32_t c2 = S.cR[tid];
-    cr[0] = c2 & 0xFFFFu;
-    cr[1] = c2 >> 16;
-  }
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    tot[e] = multi_tile ? (uint64_t)kb_tot[(size_t)it.kbs * kFKeys + k0 + e] : (uint64_t)cs[e];
+    const uint2 c4 = *reinterpret_cast<const uint2*>(&S.cR[2 * tid]);
+    cr[0] = c4.x & 0xFFFFu;
+    cr[1] = c4.x >> 16;
+    cr[2] = c4.y & 0xFFFFu;
+    cr[3] = c4.y >> 16;
+    uint4 t4 = make_uint4(cs[0], cs[1], cs[2], cs[3]);
+    if (multi_tile)
+      t4 = *reinterpret_cast<const uint4*>(kb_tot + (size_t)it.kbs * kFKeys + k0);
+    tot[0] = t4.x;
+    tot[1] = t4.y;
+    tot[2] = t4.z;
+    tot[3] = t4.w;
   }
   // one pass over the key offsets: the exclusive scan of the keys' pairs in
   // the sub-batch (the first pair of each key) and of their R rows (run
   // starts), with the sums of this tile's pairs and of earlier tiles' pairs
   uint64_t total_sub, cnt_tile, before;
   {
-    const uint64_t p0 = tot[0] * cr[0], p1 = tot[1] * cr[1];
-    uint64_t a = p0 + p1;                                              // scanned
-    uint64_t b = (uint64_t)cs[0] * cr[0] + (uint64_t)cs[1] * cr[1];   // summed
-    uint64_t c = (uint64_t)pr[0] * cr[0] + (uint64_t)pr[1] * cr[1];   // summed
-    uint32_t r = cr[0] + cr[1];                                        // scanned
+    uint64_t a = 0, b = 0, c = 0;  // scanned, summed, summed
+    uint32_t r = 0;                // scanned
+#pragma unroll
+    for (int e = 0; e < kFKeysT; ++e) {
+      a += (uint64_t)tot[e] * cr[e];
+      b += (uint64_t)cs[e] * cr[e];
+      c += (uint64_t)pr[e] * cr[e];
+      r += cr[e];
+    }
     uint64_t xa = a;
     uint32_t xr = r;
 #pragma unroll
@@ -552,31 +613,33 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
       tb += S.s_wb[w];
       tc += S.s_wc[w];
     }
-    const uint64_t eo = pa + xa - a;  // first pair of key k0 in the sub-batch
-    const uint32_t er = pr32 + xr - r;  // first sorted R row of key k0
-    const uint64_t first[2] = {eo, eo + p0};
-    const uint32_t rstart[2] = {er, er + cr[0]};
+    uint64_t eo = pa + xa - a;     // first pair of key k0 in the sub-batch
+    uint32_t er = pr32 + xr - r;  // first sorted R row of key k0
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < kFKeysT; ++e) {
       // the key's first pair for this tile's rows: after the earlier tiles';
       // with several R rows a key's run start replaces its R id
-      S.ent[k0 + e].a = cr[e] ? first[e] + (uint64_t)pr[e] * cr[e] : ~0ull;
-      if (dup) S.ent[k0 + e].r = (K)rstart[e];
+      S.ent[k0 + e].a = cr[e] ? eo + (uint64_t)pr[e] * cr[e] : ~0ull;
+      if (dup) S.ent[k0 + e].r = (K)er;
+      eo += (uint64_t)tot[e] * cr[e];
+      er += cr[e];
     }
     total_sub = ta;
     cnt_tile = tb;
     before = tc;
   }
 
-  // the S ids (read when the pairs are written): their loads in flight while
-  // warp 0 runs the chained scan (the S keys' registers are free by now)
-  K sid[kFItemsS];
+  // the S ids (folded rows: the words again, from L2), needed when the pairs
+  // are written: their loads in flight while warp 0 runs the chained scan
+  using SRow = typename std::conditional<WORDS, uint64_t, K>::type;
+  SRow srow[kFItemsS];
   {
-    const K* __restrict__ sv = g_sv;
+    const SRow* __restrict__ src =
+        WORDS ? reinterpret_cast<const SRow*>(it.sk) : reinterpret_cast<const SRow*>(g_sv);
 #pragma unroll
     for (int u = 0; u < kFItemsS; ++u) {
       const int row = wrow + u * 32 + lane;
-      sid[u] = row < ns ? sv[row] : K(0);
+      srow[u] = row < ns ? src[row] : SRow(0);
     }
   }
   // 4. chained scan over the group's items (warp 0): the tile's first pair
@@ -632,26 +695,34 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
   // 5. every S row's pairs, in key order, then S position, then R position
   using P = typename PairOf<K>::type;
   const bool vec = (((uintptr_t)out) & (2 * sizeof(K) - 1)) == 0;
-  const uint32_t* wx = &S.wh[warp][0];
+  const uint16_t* wx = S.wh[warp];
 #pragma unroll
   for (int u = 0; u < kFItemsS; ++u) {
     if (wrow + u * 32 + lane >= ns) continue;
-    const uint32_t k = dr[u] & 0xFFFFu;
+    uint32_t k;
+    K s_id;
+    if constexpr (WORDS) {
+      k = koff(srow[u], sublo);
+      s_id = word_id(srow[u]);
+    } else {
+      k = dig.get(u);
+      s_id = srow[u];
+    }
     const KeyEnt<K> en = S.ent[k];
     if (en.a == ~0ull) continue;  // no R row has the key
     // S rows of the key before this one in the tile: earlier warps, earlier
     // lanes and items of this warp
-    const uint32_t within = ((wx[k >> 1] >> ((k & 1u) * 16u)) & 0xFFFFu) + (dr[u] >> 16);
+    const uint32_t within = wx[k] + rank.get(u);
     if (!dup) {
       const uint64_t pos = base + en.a + within;
       if (vec) {
         P pr2;
         pr2.x = en.r;
-        pr2.y = sid[u];
+        pr2.y = s_id;
         *reinterpret_cast<P*>(out + 2 * pos) = pr2;
       } else {
         out[2 * pos] = en.r;
-        out[2 * pos + 1] = sid[u];
+        out[2 * pos + 1] = s_id;
       }
     } else {
       const uint32_t c = (S.cR[k >> 1] >> ((k & 1u) * 16u)) & 0xFFFFu;
@@ -659,8 +730,10 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
       const uint32_t r0 = (uint32_t)en.r;
       const K* __restrict__ rv = g_rv;  // R ids in the order of the key's run
       for (uint32_t j = 0; j < c; ++j) {
-        out[2 * (pos + j)] = rv[S.r_pb[r0 + j]];
-        out[2 * (pos + j) + 1] = sid[u];
+        const uint32_t row = S.r_pb[r0 + j];
+        if constexpr (WORDS) out[2 * (pos + j)] = word_id(g_rk[row]);
+        else out[2 * (pos + j)] = rv[row];
+        out[2 * (pos + j) + 1] = s_id;
       }
     }
   }
@@ -677,12 +750,20 @@ cudaError_t launch_fused_info(const FusedJob<K>* d_jobs, int nj, int64_t* d_info
 
 template <typename K>
 cudaError_t launch_fused_prep(const FusedJob<K>* d_jobs, int nj, FItem* d_items, int64_t n_items,
-                              bool any_multi, uint32_t* d_kb_tot, cudaStream_t st) {
+                              bool any_multi, uint32_t* d_kb_tot, cudaStream_t st, WordFmt f) {
   if (nj <= 0 || n_items <= 0) return cudaSuccess;
-  k_fused_items<K><<<nj, kFThreads, 0, st>>>(d_jobs, d_items);
+  // folded rows: the pointers step 8 bytes a row whatever K
+  const auto* w_jobs = reinterpret_cast<const FusedJob<int64_t>*>(d_jobs);
+  if (f.ib)
+    k_fused_items<int64_t><<<nj, kFThreads, 0, st>>>(w_jobs, d_items);
+  else
+    k_fused_items<K><<<nj, kFThreads, 0, st>>>(d_jobs, d_items);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || !any_multi) return e;
-  k_fused_hist<K><<<(unsigned)n_items, 256, 0, st>>>(d_jobs, d_items, d_kb_tot);
+  if (f.ib)
+    k_fused_hist<int64_t><<<(unsigned)n_items, 256, 0, st>>>(w_jobs, d_items, d_kb_tot, f.ib);
+  else
+    k_fused_hist<K><<<(unsigned)n_items, 256, 0, st>>>(d_jobs, d_items, d_kb_tot, 0);
   return cudaGetLastError();
 }
 
@@ -691,32 +772,42 @@ cudaError_t launch_fused_join(const FusedJob<K>* d_jobs, const FItem* d_items, i
                               uint32_t* d_item_counter, uint64_t* d_item_lb, uint32_t* d_kb_lb,
                               const uint32_t* d_kb_tot, K* out, int64_t capacity,
                               const int64_t* d_out_base, int64_t* d_total, int* d_err,
-                              cudaStream_t st) {
+                              cudaStream_t st, WordFmt f) {
   (void)d_jobs;  // the items carry what the join needs
   if (n_items <= 0) return cudaSuccess;
-  k_fused_join<K><<<(unsigned)n_items, kFThreads, fused_smem_bytes<K>(), st>>>(
-      d_items, n_items, d_item_counter, d_item_lb, d_kb_lb, d_kb_tot, out, capacity,
-      d_out_base, d_total, d_err);
+  if (f.ib)
+    k_fused_join<K, true><<<(unsigned)n_items, kFThreads, fused_smem_bytes<K>(), st>>>(
+        d_items, f, n_items, d_item_counter, d_item_lb, d_kb_lb, d_kb_tot, out, capacity,
+        d_out_base, d_total, d_err);
+  else
+    k_fused_join<K, false><<<(unsigned)n_items, kFThreads, fused_smem_bytes<K>(), st>>>(
+        d_items, f, n_items, d_item_counter, d_item_lb, d_kb_lb, d_kb_tot, out, capacity,
+        d_out_base, d_total, d_err);
   return cudaGetLastError();
 }
 
+template <typename K, bool WORDS>
+cudaError_t fused_attr() {
+  return cudaFuncSetAttribute(k_fused_join<K, WORDS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)fused_smem_bytes<K>());
+}
+
 cudaError_t fused_init_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(k_fused_join<int32_t>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fused_smem_bytes<int32_t>());
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_fused_join<int64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)fused_smem_bytes<int64_t>());
+  cudaError_t e = fused_attr<int32_t, false>();
+  if (e == cudaSuccess) e = fused_attr<int32_t, true>();
+  if (e == cudaSuccess) e = fused_attr<int64_t, false>();
+  if (e == cudaSuccess) e = fused_attr<int64_t, true>();
+  return e;
 }
 
 #define TJ_INSTANTIATE_FUSED(K)                                                                 \
   template cudaError_t launch_fused_info<K>(const FusedJob<K>*, int, int64_t*, cudaStream_t);   \
   template cudaError_t launch_fused_prep<K>(const FusedJob<K>*, int, FItem*, int64_t, bool,     \
-                                            uint32_t*, cudaStream_t);                           \
+                                            uint32_t*, cudaStream_t, WordFmt);                  \
   template cudaError_t launch_fused_join<K>(const FusedJob<K>*, const FItem*, int64_t,          \
                                             uint32_t*, uint64_t*, uint32_t*, const uint32_t*,   \
                                             K*, int64_t, const int64_t*, int64_t*, int*,        \
-                                            cudaStream_t);
+                                            cudaStream_t, WordFmt);
 TJ_INSTANTIATE_FUSED(int32_t)
 TJ_INSTANTIATE_FUSED(int64_t)
 

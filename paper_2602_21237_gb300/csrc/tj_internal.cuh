@@ -41,6 +41,23 @@ constexpr int kTileWide = kSortThreads * kItemsWide;
 #endif
 constexpr int kItemsRoute = TJ_ROUTE_ITEMS;
 constexpr int kTileRoute = kSortThreads * kItemsRoute;
+// onesweep passes over folded rows (tj_word.cu): words a thread holds in
+// registers, and fewer for arrays too small to fill the chip with big tiles
+#ifndef TJ_W_THREADS
+#define TJ_W_THREADS 512
+#endif
+#ifndef TJ_W_ITEMS
+#define TJ_W_ITEMS 16
+#endif
+#ifndef TJ_W_MINB
+#define TJ_W_MINB 2
+#endif
+constexpr int kWThreads = TJ_W_THREADS;
+constexpr int kWWarps = kWThreads / 32;
+constexpr int kWMinB = TJ_W_MINB;
+constexpr int kWItems = TJ_W_ITEMS;
+constexpr int kWItemsSmall = 6;
+constexpr int kWMaskItems = 2;  // of four items ranked by the lane-mask tables
 constexpr int kMaxDigitBits = 10;           // widest radix digit
 constexpr int kMaxBins = 1 << kMaxDigitBits;
 constexpr int kMaxPasses = 8;               // 64-bit keys at 8 bits per pass
@@ -84,6 +101,10 @@ template <typename K> struct UnsignedOf;
 template <> struct UnsignedOf<int32_t> { using type = uint32_t; };
 template <> struct UnsignedOf<int64_t> { using type = uint64_t; };
 
+// passes of a word job that may read columns: 32-bit rows take at most 4 passes
+// and fold in every other one, 64-bit rows only in the first
+constexpr int kFoldPasses = 4;
+
 // ---- per-array radix job ---------------------------------------------------
 // One array being sorted by (key - lo) over `passes` LSD digits.  Pass p reads
 // src_k/src_v[p] and writes dst_k/dst_v[p] (ping-pong buffers).
@@ -102,13 +123,27 @@ struct RadixJob {
   int64_t lb_stride;    // words between the look-back regions of consecutive
                         // passes (0: one region, cleared before every pass)
   const K* src_k[kMaxPasses];
-  const K* src_v[kMaxPasses];
+  // Folded rows (tj_word.cu): a row is the word (key - wlo) << ib | (id - ilo).
+  // Word passes read `lo` and `shift` as offsets and positions within words
+  // (route passes: lo = the range's first key - wlo, route_hi = its width,
+  // cuts = offsets from wlo); src_k / dst_k are words except where a pass reads
+  // or writes columns, which only passes below kFoldPasses read.
+  union {
+    const K* src_v[kMaxPasses];
+    struct {
+      const K* fold_v[kFoldPasses];
+      uint64_t wlo, ilo;
+      int64_t dst_rows;  // room at dst_k (rows) of a pass that folds
+      const K* ids;      // statistics: ids sampled beside the keys (may be null)
+    };
+  };
   K* dst_k[kMaxPasses];
   K* dst_v[kMaxPasses];
   // Route digit (pass 0 only, when cuts != nullptr): the digit of a key is the
   // number of cut keys <= key, i.e. the index of its key-range partition.
   const K* cuts;        // sorted cut keys, padded to kMaxCuts with the key type's max
   int32_t ncuts;        // real cuts (<= kMaxCuts - 1); partitions = ncuts + 1
+  int32_t ib;           // id bits of folded rows (0: separate columns)
   // Log-scale index over the cuts: with x = key - lo, bucket b(x) = x for
   // x < 32, else 32 * bitlen(x) + the 5 bits below x's leading one; bucket b
   // holds cuts [route_tab[b], route_tab[b + 1]).  Fine-grained at every
@@ -132,6 +167,10 @@ struct RadixJob {
   uint64_t route_hi;
 };
 
+// A row's key offset or id did not fit its word: the call runs again on
+// separate columns.
+constexpr int kErrFold = 101;
+
 // Kinds of onesweep pass: a sort digit of key - lo, a route by the cut table
 // (batch = number of cuts <= key), a route by equal-width ranges.
 constexpr int kModeSort = 0;
@@ -139,9 +178,20 @@ constexpr int kModeCuts = 1;
 constexpr int kModeRadix = 2;
 
 // Per-array min/max, stored as order-preserving unsigned (key ^ sign bit).
+// (maxima inverted, so that one fill and one atomic serve all four), and the
+// same of a sample of the ids.
 struct KeyStats {
   unsigned long long min_u;
   unsigned long long max_u;
+  unsigned long long id_min_u;
+  unsigned long long id_max_u;
+};
+
+// Layout of the rows a join kernel reads: separate key and id columns (ib = 0)
+// or folded rows, whose job and tile pointers (rk, sk) are words.
+struct WordFmt {
+  int32_t ib = 0;
+  uint64_t ilo = 0;
 };
 
 // ---- join job ---------------------------------------------------------------
@@ -204,8 +254,8 @@ constexpr int kFKeyBits = 10;               // key offsets within a sub-batch
 // whole batch is one sub-batch, no MSD pass)
 constexpr int kFMinBits = TJ_FUSED_MIN_BITS;
 constexpr int kFKeys = 1 << kFKeyBits;
-constexpr int kFThreads = 512;              // threads of a fused CTA
-constexpr int kFCapS = 4608;                // S rows of one item (9 per thread)
+constexpr int kFThreads = 256;              // threads of a fused CTA
+constexpr int kFCapS = 4608;                // S rows of one item (18 per thread)
 constexpr int kFCapR = 2048;                // R rows of a sub-batch (on chip)
 #ifndef TJ_FUSED_MAX_MSD
 #define TJ_FUSED_MAX_MSD 10
@@ -255,7 +305,8 @@ cudaError_t launch_fused_info(const FusedJob<K>* d_jobs, int nj, int64_t* d_info
 // sub-batches (d_kb_tot zeroed beforehand)
 template <typename K>
 cudaError_t launch_fused_prep(const FusedJob<K>* d_jobs, int nj, FItem* d_items, int64_t n_items,
-                              bool any_multi, uint32_t* d_kb_tot, cudaStream_t st);
+                              bool any_multi, uint32_t* d_kb_tot, cudaStream_t st,
+                              WordFmt f = WordFmt());
 // the joins of the group's items (item and count-vector look-back zeroed);
 // pairs from *d_out_base on, *d_total = the end of the group's pairs
 template <typename K>
@@ -263,7 +314,7 @@ cudaError_t launch_fused_join(const FusedJob<K>* d_jobs, const FItem* d_items, i
                               uint32_t* d_item_counter, uint64_t* d_item_lb, uint32_t* d_kb_lb,
                               const uint32_t* d_kb_tot, K* out, int64_t capacity,
                               const int64_t* d_out_base, int64_t* d_total, int* d_err,
-                              cudaStream_t st);
+                              cudaStream_t st, WordFmt f = WordFmt());
 
 // ---- late materialisation (tj_gather.cu) ------------------------------------
 constexpr int kGatherCols = 16;  // columns per gather launch
@@ -307,7 +358,8 @@ cudaError_t radix_init_attributes();
 // of a smaller onesweep tile); jobs' tile0 counts tiles of that size.
 template <typename K>
 cudaError_t launch_stats(const RadixJob<K>* d_jobs, int num_jobs, int64_t total_tiles,
-                         KeyStats* d_stats, cudaStream_t st, int tile = kTile);
+                         KeyStats* d_stats, cudaStream_t st, int tile = kTile,
+                         bool words = false);
 template <typename K>
 cudaError_t launch_histogram(const RadixJob<K>* d_jobs, int num_jobs, int64_t total_tiles,
                              cudaStream_t st, const int32_t* d_tile_job = nullptr,
@@ -328,24 +380,38 @@ cudaError_t launch_onesweep(const RadixJob<K>* d_jobs, int num_jobs, int64_t tot
                             int* d_err, cudaStream_t st, const int32_t* d_tile_job = nullptr,
                             int items = kItems, bool guard = false);
 
+// ---- launchers (tj_word.cu) -------------------------------------------------
+cudaError_t word_init_attributes();
+// One onesweep pass over folded rows; tiles of kWThreads * items rows (items =
+// kWItems or, sort digits only, kWItemsSmall).  raw_in: reads key and id
+// columns and folds them; raw_out: writes columns; hi: every job's shift is at
+// least 32 and its lo a multiple of 2^32 (always so for 32-bit keys).
+template <typename K>
+cudaError_t launch_wsweep(const RadixJob<K>* d_jobs, int num_jobs, int64_t total_tiles, int pass,
+                          int max_bits, int mode, bool raw_in, bool raw_out, bool hi, int items,
+                          bool guard, uint32_t* d_tile_counter, int* d_err, cudaStream_t st,
+                          const int32_t* d_tile_job = nullptr);
+
 // ---- launchers (tj_join.cu) -------------------------------------------------
 cudaError_t join_init_attributes();
+// d_err (optional): if the word there is set, the tiles come out empty
 template <typename K>
 cudaError_t launch_tile_ranges(const JoinJob<K>* d_jobs, int num_jobs, int64_t total_tiles,
                                JTile<K>* d_tiles, cudaStream_t st,
-                               const int32_t* d_tile_job = nullptr);
+                               const int32_t* d_tile_job = nullptr, WordFmt f = WordFmt(),
+                               const int* d_err = nullptr);
 template <typename K>
 cudaError_t launch_join(int64_t total_tiles, const JTile<K>* d_tiles, uint64_t* d_lookback,
                         uint32_t* d_tile_counter, K* out, int64_t capacity,
                         const int64_t* d_out_base, int64_t* d_job_out, int64_t* d_total,
-                        int* d_err, cudaStream_t st);
+                        int* d_err, cudaStream_t st, WordFmt f = WordFmt());
 // k_cross over a run of single-key batches: reads the run's base, writes
 // base + run_pairs for the next run (CTA 0), and writes a batch's pairs only
 // if all of them fit `capacity`.
 template <typename K>
 cudaError_t launch_cross(const CrossJob<K>* d_jobs, int num_jobs, int64_t blocks, K* out,
                          int64_t capacity, const int64_t* d_base, int64_t* d_next,
-                         int64_t run_pairs, cudaStream_t st);
+                         int64_t run_pairs, cudaStream_t st, WordFmt f = WordFmt());
 // tile -> job maps of a group's radix jobs (tile of kTile rows) and join jobs
 template <typename K>
 cudaError_t launch_group_maps(const RadixJob<K>* d_rjobs, int nr, int32_t* d_rmap,
@@ -356,6 +422,10 @@ cudaError_t launch_group_maps(const RadixJob<K>* d_rjobs, int nr, int32_t* d_rma
 template <typename K>
 cudaError_t launch_sample_gather(const K* a, int64_t ma, int64_t off_a, const K* b, int64_t mb,
                                  int64_t off_b, int stride, K* out_k, K* out_v, cudaStream_t st);
+// *out's id fields: the range of about 8000 ids of each side (out filled with 0xFF before)
+template <typename K>
+cudaError_t launch_id_range(const K* a, int64_t na, const K* b, int64_t nb, KeyStats* out,
+                            cudaStream_t st);
 template <typename K>
 cudaError_t launch_quantiles(const K* sorted, int64_t m, int G, int first, int last, int step,
                              K* out, cudaStream_t st);

@@ -46,6 +46,36 @@ __device__ __forceinline__ uint32_t ht_hash(int32_t k) {
 __device__ __forceinline__ uint32_t ht_hash(int64_t k) {
   return (uint32_t)(((uint64_t)k * 0x9E3779B97F4A7C15ull) >> (64 - kHTBits));
 }
+__device__ __forceinline__ uint32_t ht_hash(uint64_t k) { return ht_hash((int64_t)k); }
+__device__ __forceinline__ uint32_t ht_hash(uint32_t k) { return ht_hash((int32_t)k); }
+
+// How a join kernel reads rows: W = 0, separate columns (an element is a key);
+// W = 1, folded rows (tj_word.cu), keys of up to 63 bits; W = 2, folded rows
+// whose key offset lies in the word's upper half (compared in 32 bits).
+template <typename K, int W>
+struct RowOf {
+  using E = uint64_t;
+  using Key = uint64_t;
+  static __device__ __forceinline__ Key key(E e, int ib) { return e >> ib; }
+};
+template <typename K>
+struct RowOf<K, 0> {
+  using E = K;
+  using Key = K;
+  static __device__ __forceinline__ Key key(E e, int) { return e; }
+};
+template <typename K>
+struct RowOf<K, 2> {
+  using E = uint64_t;
+  using Key = uint32_t;
+  static __device__ __forceinline__ Key key(E e, int ib) {
+    return (uint32_t)(e >> 32) >> (ib & 31);
+  }
+};
+template <typename K>
+__device__ __forceinline__ K word_id(uint64_t w, const WordFmt& f) {
+  return (K)((w & ((1ull << f.ib) - 1ull)) + f.ilo);
+}
 static_assert(kRCap < 0xFFFF, "run bounds are packed in 16 bits");
 
 constexpr uint32_t kHTEmpty = 0xFFFFFFFFu;
@@ -70,10 +100,13 @@ __device__ __forceinline__ void st_volatile_u64(uint64_t* p, uint64_t v) {
 // key >= the tile's first key, lanes 16-31 the first R row with key > the
 // tile's last key, each by a 16-ary search (16 probes per round trip); lane 0
 // writes the tile's descriptor, so a join tile needs one load to start.
-template <typename K>
+template <typename K, bool WORDS>
 __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
                               int64_t total_tiles, JTile<K>* __restrict__ tiles,
-                              const int32_t* __restrict__ tile_job) {
+                              const int32_t* __restrict__ tile_job, int ib,
+                              const int* __restrict__ err) {
+  using Row = RowOf<K, WORDS ? 1 : 0>;
+  using E = typename Row::E;
   const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (t >= total_tiles) return;  // whole warps leave together
   const int lane = threadIdx.x & 31, sub = lane & 15;
@@ -81,10 +114,26 @@ __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
   const uint32_t half = upper ? 0xFFFF0000u : 0x0000FFFFu;
   const int j = tile_job ? tile_job[t] : find_job_j(jobs, num_jobs, t);
   const JoinJob<K>* J = jobs + j;
+  if (err && *err != 0) {  // the rows did not fold: empty tiles, nothing is joined
+    if (lane == 0) {
+      JTile<K> d = {};
+      d.sk = J->sk;
+      d.rk = J->rk;
+      d.lt = t - J->tile0;
+      d.j = j;
+      tiles[t] = d;
+    }
+    return;
+  }
   const int64_t row0 = (t - J->tile0) * kJTile;
   const int64_t row1 = min(J->ns, row0 + kJTile);
-  const K key = upper ? J->sk[row1 - 1] : J->sk[row0];
-  const K* __restrict__ r = J->rk;
+  const E* __restrict__ s = reinterpret_cast<const E*>(J->sk);
+  const E* __restrict__ r = reinterpret_cast<const E*>(J->rk);
+  const auto key = Row::key(upper ? s[row1 - 1] : s[row0], ib);
+  auto below = [&](int64_t i) {
+    const auto x = Row::key(r[i], ib);
+    return upper ? !(key < x) : (x < key);
+  };
   // invariant: every row before lo satisfies the predicate, none from hi on
   // (predicate: r[i] < key for the lower bound, r[i] <= key for the upper)
   int64_t lo = 0, hi = J->nr;
@@ -94,7 +143,7 @@ __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
     const int64_t step = (len + 15) / 16;
     const int64_t p = lo + sub * step;
     bool pred = false;
-    if (len > 16 && p < hi) pred = upper ? !(key < r[p]) : (r[p] < key);
+    if (len > 16 && p < hi) pred = below(p);
     const int c = __popc(__ballot_sync(0xFFFFFFFFu, pred) & half);
     if (len > 16) {
       // probes 0..c-1 satisfy the predicate, probe c (if any) does not
@@ -104,7 +153,7 @@ __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
     }
   }
   const int64_t p = lo + sub;
-  const bool pred = p < hi && (upper ? !(key < r[p]) : (r[p] < key));
+  const bool pred = p < hi && below(p);
   const int64_t res = lo + __popc(__ballot_sync(0xFFFFFFFFu, pred) & half);
   const int64_t b = __shfl_sync(0xFFFFFFFFu, res, 16);
   if (lane == 0) {
@@ -135,7 +184,7 @@ constexpr int kJItems = kJTile / kJThreads;     // S rows per thread
 static_assert(kJItems * kJThreads == kJTile, "join tile = threads x items");
 
 // Shared memory: S keys | S ids (kJTile + kPad each) | R keys | R ids (kRCap +
-// kPad each) | hash table[kHTSlots] u32.  Each staged array starts up to kPad
+// kPad each) | hash table[kHTSlots] u32; folded rows: S words | R words | table.  Each staged array starts up to kPad
 // elements into its area (its first element keeps the source's address modulo
 // 16, so that all but a head and a tail move in 16-byte copies).  After the
 // probe the many-matches write path (which reads ids from global memory)
@@ -144,11 +193,15 @@ template <typename K>
 __host__ __device__ constexpr int join_pad() {
   return 16 / (int)sizeof(K);
 }
-template <typename K>
+template <typename K, int W>
 constexpr size_t join_smem_bytes() {
-  return sizeof(K) * (size_t)(2 * (kJTile + join_pad<K>()) + 2 * (kRCap + join_pad<K>())) +
+  using E = typename RowOf<K, W>::E;
+  return sizeof(E) * (size_t)(W ? 1 : 2) *
+             (size_t)(kJTile + join_pad<E>() + kRCap + join_pad<E>()) +
          sizeof(uint32_t) * kHTSlots;
 }
+static_assert(sizeof(uint64_t) * (kJTile + kRCap) >= (sizeof(uint64_t) + sizeof(uint32_t)) * kJTile,
+              "offsets and run starts fit in the folded rows' shared memory");
 static_assert(sizeof(int32_t) * (2 * kJTile + 2 * kRCap) >=
                   (sizeof(uint64_t) + sizeof(uint32_t)) * kJTile,
               "offsets and run starts fit in the join's shared memory");
@@ -199,19 +252,24 @@ __device__ __forceinline__ K* join_copy_async(K* dst, const K* __restrict__ src,
 //      comes from ballots over the warp and the warps' totals; otherwise the
 //      tile's counts are scanned and each output index finds its S row.
 // Output order: key, then S position, then R position.
-template <typename K>
+template <typename K, int W>
 __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
-    k_join(int64_t total_tiles, const JTile<K>* __restrict__ tiles,
+    k_join(int64_t total_tiles, const JTile<K>* __restrict__ tiles, WordFmt f,
            uint64_t* __restrict__ lookback, uint32_t* __restrict__ tile_counter,
            K* __restrict__ out, int64_t capacity, const int64_t* __restrict__ out_base,
            int64_t* __restrict__ job_out, int64_t* __restrict__ total, int* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int kPad = join_pad<K>();
-  K* const b_sk = reinterpret_cast<K*>(smem);  // staging areas (16-byte aligned)
-  K* const b_sv = b_sk + kJTile + kPad;
-  K* const b_rk = b_sv + kJTile + kPad;
-  K* const b_rv = b_rk + kRCap + kPad;
-  uint32_t* s_ht = reinterpret_cast<uint32_t*>(b_rv + kRCap + kPad);
+  using Row = RowOf<K, W>;
+  using E = typename Row::E;
+  using Key = typename Row::Key;
+  const int ib = f.ib;
+  constexpr int kPad = join_pad<E>();
+  constexpr int kCols = W ? 1 : 2;  // arrays a relation's rows take
+  E* const b_sk = reinterpret_cast<E*>(smem);  // staging areas (16-byte aligned)
+  E* const b_sv = b_sk + kJTile + kPad;        // (W == 0 only)
+  E* const b_rk = b_sk + kCols * (kJTile + kPad);
+  E* const b_rv = b_rk + kRCap + kPad;  // (W == 0 only)
+  uint32_t* s_ht = reinterpret_cast<uint32_t*>(b_rk + kCols * (kRCap + kPad));
   __shared__ uint64_t s_wsum[kJWarps];
   __shared__ uint64_t s_base;
   __shared__ uint32_t s_t;
@@ -226,20 +284,26 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   const int64_t nrr = T.nrr;
   const int64_t lt = T.lt;
   const int nv = T.nv;
-  const K* __restrict__ rk_g = T.rk;
+  const E* __restrict__ rk_g = reinterpret_cast<const E*>(T.rk);
   const K* __restrict__ rv_g = T.rv;
+  // id of R row i of the tile's range, read from global memory
+  auto rid_g = [&](int64_t i) -> K {
+    if constexpr (W != 0) return word_id<K>(rk_g[i], f);
+    else return rv_g[i];
+  };
   const int64_t nchunks = (nrr + kRCap - 1) / kRCap;
   const bool onchip = nchunks <= kMaxChunks;
 
   // 1. stage S and the first R chunk
-  const K* s_sk = join_copy_async<K>(b_sk, T.sk, nv);
-  const K* s_sv = join_copy_async<K>(b_sv, T.sv, nv);
-  K* s_rk = b_rk;  // the staged R chunk (where its copy starts)
-  K* s_rv = b_rv;
+  const E* s_sk = join_copy_async<E>(b_sk, reinterpret_cast<const E*>(T.sk), nv);
+  const E* s_sv = b_sv;
+  E* s_rk = b_rk;  // the staged R chunk (where its copy starts)
+  E* s_rv = b_rv;
+  if constexpr (W == 0) s_sv = join_copy_async<E>(b_sv, T.sv, nv);
   if (onchip && nchunks > 0) {
     const int nc0 = (int)min((int64_t)kRCap, nrr);
-    s_rk = join_copy_async<K>(b_rk, rk_g, nc0);
-    s_rv = join_copy_async<K>(b_rv, rv_g, nc0);
+    s_rk = join_copy_async<E>(b_rk, rk_g, nc0);
+    if constexpr (W == 0) s_rv = join_copy_async<E>(b_rv, rv_g, nc0);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 
@@ -254,8 +318,8 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
       const int nc = (int)min((int64_t)kRCap, nrr - c0);
       if (c > 0) {
         __syncthreads();  // the previous chunk's probes are done
-        s_rk = join_copy_async<K>(b_rk, rk_g + c0, nc);
-        s_rv = join_copy_async<K>(b_rv, rv_g + c0, nc);
+        s_rk = join_copy_async<E>(b_rk, rk_g + c0, nc);
+        if constexpr (W == 0) s_rv = join_copy_async<E>(b_rv, rv_g + c0, nc);
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
       for (int i = tid; i < kHTSlots; i += kJThreads) s_ht[i] = kHTEmpty;
@@ -264,8 +328,9 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
       // insert the first row of every run of equal keys; keys are distinct, so
       // an occupied slot is never this key and insertion needs no comparison
       for (int i = tid; i < nc; i += kJThreads) {
-        if (i == 0 || s_rk[i] != s_rk[i - 1]) {
-          uint32_t h = ht_hash(s_rk[i]);
+        const Key key = Row::key(s_rk[i], ib);
+        if (i == 0 || key != Row::key(s_rk[i - 1], ib)) {
+          uint32_t h = ht_hash(key);
           while (atomicCAS(&s_ht[h], kHTEmpty, (uint32_t)i | 0xFFFF0000u) != kHTEmpty)
             h = (h + 1) & (kHTSlots - 1);
         }
@@ -273,12 +338,12 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
       __syncthreads();
       // the last row of every run records the run's end
       for (int i = tid; i < nc; i += kJThreads) {
-        if (i == nc - 1 || s_rk[i] != s_rk[i + 1]) {
-          const K key = s_rk[i];
+        const Key key = Row::key(s_rk[i], ib);
+        if (i == nc - 1 || key != Row::key(s_rk[i + 1], ib)) {
           uint32_t h = ht_hash(key);
           while (true) {
             const uint32_t w = s_ht[h];
-            if (s_rk[w & 0xFFFFu] == key) {
+            if (Row::key(s_rk[w & 0xFFFFu], ib) == key) {
               s_ht[h] = (w & 0xFFFFu) | ((uint32_t)(i + 1) << 16);
               break;
             }
@@ -287,21 +352,21 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         }
       }
       __syncthreads();
-      const K cf = s_rk[0], cl = s_rk[nc - 1];
+      const Key cf = Row::key(s_rk[0], ib), cl = Row::key(s_rk[nc - 1], ib);
 #pragma unroll
       for (int u = 0; u < kJItems; ++u) {
         const int q = wbase + u * 32 + lane;
         if (q >= nv) continue;
-        const K key = s_sk[q];
+        const Key key = Row::key(s_sk[q], ib);
         if (key < cf || cl < key) continue;
         uint32_t h = ht_hash(key);
         while (true) {
           const uint32_t w = s_ht[h];
           if (w == kHTEmpty) break;
-          const uint32_t f = w & 0xFFFFu;
-          if (s_rk[f] == key) {
-            if (cnt[u] == 0u) start[u] = (uint32_t)c0 + f;
-            cnt[u] += (w >> 16) - f;
+          const uint32_t r0 = w & 0xFFFFu;
+          if (Row::key(s_rk[r0], ib) == key) {
+            if (cnt[u] == 0u) start[u] = (uint32_t)c0 + r0;
+            cnt[u] += (w >> 16) - r0;
             break;
           }
           h = (h + 1) & (kHTSlots - 1);
@@ -321,11 +386,11 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
     __syncthreads();
     int steps = 0;  // halvings that empty a range of `stride` rows
     while (((int64_t)1 << steps) <= stride) ++steps;
-    K key[kJItems];
+    Key key[kJItems];
 #pragma unroll
     for (int u = 0; u < kJItems; ++u) {
       const int q = wbase + u * 32 + lane;
-      key[u] = q < nv ? s_sk[q] : K(0);
+      key[u] = q < nv ? Row::key(s_sk[q], ib) : Key(0);
     }
     // bound 0: first R row with key >= the row's key; 1: first with key >
     // (offsets into the range: nrr < 2^30)
@@ -338,7 +403,8 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         int a = 0, c = m;
         while (a < c) {
           const int mid = (a + c) >> 1;
-          const bool pr = bound ? !(key[u] < s_rk[mid]) : (s_rk[mid] < key[u]);
+          const Key x = Row::key(s_rk[mid], ib);
+          const bool pr = bound ? !(key[u] < x) : (x < key[u]);
           a = pr ? mid + 1 : a;
           c = pr ? c : mid;
         }
@@ -351,7 +417,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
 #pragma unroll
         for (int u = 0; u < kJItems; ++u) {
           const int half = n[u] >> 1;
-          const K r = rk_g[min(lo[u] + half, nr32 - 1)];  // in range even when n == 0
+          const Key r = Row::key(rk_g[min(lo[u] + half, nr32 - 1)], ib);  // in range even when n == 0
           const bool go = n[u] > 0 && (bound ? !(key[u] < r) : (r < key[u]));
           lo[u] = go ? lo[u] + half + 1 : lo[u];
           n[u] = go ? n[u] - half - 1 : half;
@@ -366,8 +432,8 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
 #pragma unroll
     for (int u = 0; u < kJItems; ++u) {
       const bool valid = wbase + u * 32 + lane < nv;
-      const K r0 = rk_g[min(lo[u], nr32 - 1)];
-      const K r1 = rk_g[min(lo[u] + 1, nr32 - 1)];
+      const Key r0 = Row::key(rk_g[min(lo[u], nr32 - 1)], ib);
+      const Key r1 = Row::key(rk_g[min(lo[u] + 1, nr32 - 1)], ib);
       const bool e0 = valid && lo[u] < nr32 && r0 == key[u];
       const bool e1 = e0 && lo[u] + 1 < nr32 && r1 == key[u];
       start[u] = (uint32_t)lo[u];
@@ -451,8 +517,8 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   __syncthreads();
   // output index of this tile's first pair: the group's base (the partitioned
   // join writes several groups one after another) plus the chained prefix
-  const uint64_t E = s_base + (out_base ? (uint64_t)*out_base : 0ull);
-  if (E + C > (uint64_t)capacity) return;  // the host reports TJ_ERR_CAPACITY
+  const uint64_t first = s_base + (out_base ? (uint64_t)*out_base : 0ull);
+  if (first + C > (uint64_t)capacity) return;  // the host reports TJ_ERR_CAPACITY
 
   // 4. write
   if (!multi) {
@@ -462,15 +528,21 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
     // R rows of the chunk still in shared memory (the last one) are read
     // there, earlier ones from global memory
     const int64_t cres = onchip && nchunks > 0 ? (nchunks - 1) * kRCap : INT64_MAX;
-    uint64_t off = E + wpre;
+    uint64_t off = first + wpre;
 #pragma unroll
     for (int u = 0; u < kJItems; ++u) {
       const uint32_t m = __ballot_sync(0xFFFFFFFFu, cnt[u] != 0u);
       if (cnt[u] != 0u) {
         const uint64_t o = off + __popc(m & ltm);
         const int64_t st0 = (int64_t)start[u];
-        const K sid = s_sv[wbase + u * 32 + lane];
-        const K rid = st0 >= cres ? s_rv[st0 - cres] : rv_g[st0];
+        K sid, rid;
+        if constexpr (W != 0) {
+          sid = word_id<K>(s_sk[wbase + u * 32 + lane], f);
+          rid = st0 >= cres ? word_id<K>(s_rk[st0 - cres], f) : rid_g(st0);
+        } else {
+          sid = s_sv[wbase + u * 32 + lane];
+          rid = st0 >= cres ? s_rv[st0 - cres] : rid_g(st0);
+        }
         if (vec) {
           P pr;
           pr.x = rid;
@@ -530,7 +602,8 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
     }
     __syncthreads();
     const K* __restrict__ sv_g = T.sv;
-    K* __restrict__ o = out + 2 * E;
+    const E* __restrict__ sk_g = reinterpret_cast<const E*>(T.sk);
+    K* __restrict__ o = out + 2 * first;
     for (uint64_t x = tid; x < C; x += kJThreads) {
       int lo = 0, hi = nv - 1;  // last q with s_off[q] <= x
       while (lo < hi) {
@@ -541,8 +614,9 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
           hi = mid - 1;
       }
       const uint64_t r = s_rs[lo] + (x - s_off[lo]);
-      o[2 * x] = rv_g[r];
-      o[2 * x + 1] = sv_g[lo];
+      o[2 * x] = rid_g((int64_t)r);
+      if constexpr (W != 0) o[2 * x + 1] = word_id<K>(sk_g[lo], f);
+      else o[2 * x + 1] = sv_g[lo];
     }
   }
 }
@@ -550,11 +624,17 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
 // ---------------------------------------------------------------------------
 template <typename K>
 cudaError_t launch_tile_ranges(const JoinJob<K>* d_jobs, int num_jobs, int64_t total_tiles,
-                               JTile<K>* d_tiles, cudaStream_t st, const int32_t* d_tile_job) {
+                               JTile<K>* d_tiles, cudaStream_t st, const int32_t* d_tile_job,
+                               WordFmt f, const int* d_err) {
   if (total_tiles <= 0) return cudaSuccess;
-  const int64_t grid = (total_tiles * 32 + kThreads - 1) / kThreads;
-  k_tile_ranges<K><<<(unsigned)grid, kThreads, 0, st>>>(d_jobs, num_jobs, total_tiles, d_tiles,
-                                                        d_tile_job);
+  const unsigned grid = (unsigned)((total_tiles * 32 + kThreads - 1) / kThreads);
+  if (f.ib)  // words: the pointers step 8 bytes a row whatever K
+    k_tile_ranges<int64_t, true><<<grid, kThreads, 0, st>>>(
+        reinterpret_cast<const JoinJob<int64_t>*>(d_jobs), num_jobs, total_tiles,
+        reinterpret_cast<JTile<int64_t>*>(d_tiles), d_tile_job, f.ib, d_err);
+  else
+    k_tile_ranges<K, false><<<grid, kThreads, 0, st>>>(d_jobs, num_jobs, total_tiles, d_tiles,
+                                                       d_tile_job, 0, d_err);
   return cudaGetLastError();
 }
 
@@ -607,12 +687,20 @@ template <typename K>
 cudaError_t launch_join(int64_t total_tiles, const JTile<K>* d_tiles, uint64_t* d_lookback,
                         uint32_t* d_tile_counter, K* out, int64_t capacity,
                         const int64_t* d_out_base, int64_t* d_job_out, int64_t* d_total,
-                        int* d_err, cudaStream_t st) {
+                        int* d_err, cudaStream_t st, WordFmt f) {
   if (total_tiles <= 0) return cudaSuccess;
-  const size_t smem = join_smem_bytes<K>();
-  k_join<K><<<(unsigned)total_tiles, kJThreads, smem, st>>>(
-      total_tiles, d_tiles, d_lookback, d_tile_counter, out, capacity, d_out_base, d_job_out,
-      d_total, d_err);
+#define TJ_JOIN(W)                                                                            \
+  k_join<K, W><<<(unsigned)total_tiles, kJThreads, join_smem_bytes<K, W>(), st>>>(            \
+      total_tiles, d_tiles, f, d_lookback, d_tile_counter, out, capacity, d_out_base,         \
+      d_job_out, d_total, d_err)
+  if (f.ib >= 32) {
+    TJ_JOIN(2);
+  } else if (f.ib > 0) {
+    if constexpr (sizeof(K) == 8) TJ_JOIN(1);  // 32-bit rows always have ib = 32
+  } else {
+    TJ_JOIN(0);
+  }
+#undef TJ_JOIN
   return cudaGetLastError();
 }
 
@@ -652,9 +740,9 @@ cudaError_t launch_fix_job_out(const JoinJob<K>* d_jobs, int num_jobs, int64_t t
 // consecutive pairs of a batch): pair p = i * nr + j of a batch is (R id j,
 // S id i), so for nr = 1 (a foreign key's heavy value) a CTA reads 4096
 // consecutive S ids and writes 4096 consecutive pairs.
-template <typename K>
+template <typename K, bool WORDS>
 __global__ void __launch_bounds__(kXThreads)
-    k_cross(const CrossJob<K>* __restrict__ jobs, int num_jobs, K* __restrict__ out,
+    k_cross(const CrossJob<K>* __restrict__ jobs, int num_jobs, WordFmt f, K* __restrict__ out,
             int64_t capacity, const int64_t* __restrict__ base_in, int64_t* __restrict__ base_out,
             int64_t run_pairs) {
   const int64_t b = blockIdx.x;
@@ -667,6 +755,10 @@ __global__ void __launch_bounds__(kXThreads)
       hi = mid - 1;
   }
   const CrossJob<K> J = jobs[lo];
+  auto id = [&](const K* p, int64_t i) -> K {
+    if constexpr (WORDS) return word_id<K>(reinterpret_cast<const uint64_t*>(p)[i], f);
+    else return p[i];
+  };
   const int64_t base = *base_in;
   if (b == 0 && threadIdx.x == 0) *base_out = base + run_pairs;
   const int64_t np = J.nr * J.ns;
@@ -677,9 +769,9 @@ __global__ void __launch_bounds__(kXThreads)
   using P = typename PairOf<K>::type;
   const bool vec = (((uintptr_t)out) & (2 * sizeof(K) - 1)) == 0;
   if (J.nr == 1) {
-    const K r = J.rv[0];
+    const K r = id(J.rv, 0);
     for (int64_t p = p0 + threadIdx.x; p < p1; p += kXThreads) {
-      const K sid = J.sv[p];
+      const K sid = id(J.sv, p);
       if (vec) {
         P v;
         v.x = r;
@@ -693,8 +785,8 @@ __global__ void __launch_bounds__(kXThreads)
   } else {
     for (int64_t p = p0 + threadIdx.x; p < p1; p += kXThreads) {
       const int64_t i = p / J.nr, j = p - i * J.nr;
-      out[2 * (o + p)] = J.rv[j];
-      out[2 * (o + p) + 1] = J.sv[i];
+      out[2 * (o + p)] = id(J.rv, j);
+      out[2 * (o + p) + 1] = id(J.sv, i);
     }
   }
 }
@@ -702,31 +794,43 @@ __global__ void __launch_bounds__(kXThreads)
 template <typename K>
 cudaError_t launch_cross(const CrossJob<K>* d_jobs, int num_jobs, int64_t blocks, K* out,
                          int64_t capacity, const int64_t* d_base, int64_t* d_next,
-                         int64_t run_pairs, cudaStream_t st) {
+                         int64_t run_pairs, cudaStream_t st, WordFmt f) {
   if (num_jobs <= 0 || blocks <= 0) return cudaErrorInvalidValue;
-  k_cross<K><<<(unsigned)blocks, kXThreads, 0, st>>>(d_jobs, num_jobs, out, capacity, d_base,
-                                                     d_next, run_pairs);
+  if (f.ib)
+    k_cross<K, true><<<(unsigned)blocks, kXThreads, 0, st>>>(d_jobs, num_jobs, f, out, capacity,
+                                                             d_base, d_next, run_pairs);
+  else
+    k_cross<K, false><<<(unsigned)blocks, kXThreads, 0, st>>>(d_jobs, num_jobs, f, out, capacity,
+                                                              d_base, d_next, run_pairs);
   return cudaGetLastError();
 }
 
+template <typename K, int W>
+cudaError_t join_attr() {
+  return cudaFuncSetAttribute(k_join<K, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)join_smem_bytes<K, W>());
+}
+
 cudaError_t join_init_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(k_join<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)join_smem_bytes<int32_t>());
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_join<int64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)join_smem_bytes<int64_t>());
+  cudaError_t e = join_attr<int32_t, 0>();
+  if (e == cudaSuccess) e = join_attr<int32_t, 2>();
+  if (e == cudaSuccess) e = join_attr<int64_t, 0>();
+  if (e == cudaSuccess) e = join_attr<int64_t, 1>();
+  if (e == cudaSuccess) e = join_attr<int64_t, 2>();
+  return e;
 }
 
 #define TJ_INSTANTIATE_JOIN(K)                                                                  \
   template cudaError_t launch_tile_ranges<K>(const JoinJob<K>*, int, int64_t, JTile<K>*,        \
-                                             cudaStream_t, const int32_t*);                     \
+                                             cudaStream_t, const int32_t*, WordFmt, const int*); \
   template cudaError_t launch_fill_join_tile_job<K>(const JoinJob<K>*, int, int32_t*,            \
                                                     cudaStream_t);                              \
   template cudaError_t launch_join<K>(int64_t, const JTile<K>*, uint64_t*, uint32_t*, K*,        \
                                       int64_t, const int64_t*, int64_t*, int64_t*, int*,          \
-                                      cudaStream_t);                                              \
+                                      cudaStream_t, WordFmt);                                     \
   template cudaError_t launch_cross<K>(const CrossJob<K>*, int, int64_t, K*, int64_t,            \
-                                       const int64_t*, int64_t*, int64_t, cudaStream_t);        \
+                                       const int64_t*, int64_t*, int64_t, cudaStream_t,         \
+                                       WordFmt);                                                  \
   template cudaError_t launch_fix_job_out<K>(const JoinJob<K>*, int, int64_t, int64_t*,          \
                                              const int64_t*, cudaStream_t);                     \
   template cudaError_t launch_group_maps<K>(const RadixJob<K>*, int, int32_t*, const JoinJob<K>*, \

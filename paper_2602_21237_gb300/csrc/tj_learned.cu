@@ -29,6 +29,50 @@ __global__ void k_sample_gather(const K* __restrict__ a, int64_t ma, int64_t off
   }
 }
 
+// Ids sampled evenly over both sides (and the last row of each): their least
+// and greatest, in order_u form, the greatest inverted (as KeyStats).
+template <typename K>
+__global__ void __launch_bounds__(256)
+    k_id_range(const K* __restrict__ a, int64_t na, const K* __restrict__ b, int64_t nb,
+               KeyStats* __restrict__ out) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t m = (int64_t)gridDim.x * blockDim.x;
+  unsigned long long mn = ~0ull, mx = ~0ull;
+  for (int side = 0; side < 2; ++side) {
+    const K* __restrict__ p = side ? b : a;
+    const int64_t n = side ? nb : na;
+    const int64_t i = t == m - 1 ? n - 1 : (int64_t)((double)n / (double)m * (double)t);
+    if (n > 0 && i < n) {
+      const unsigned long long u =
+          (unsigned long long)(long long)p[i] ^ 0x8000000000000000ull;
+      mn = u < mn ? u : mn;
+      mx = ~u < mx ? ~u : mx;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xFFFFFFFFu, mn, o);
+    const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
+    mn = x < mn ? x : mn;
+    mx = y < mx ? y : mx;
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&out->id_min_u, mn);
+    atomicMin(&out->id_max_u, mx);
+  }
+}
+
+template <typename K>
+cudaError_t launch_id_range(const K* a, int64_t na, const K* b, int64_t nb, KeyStats* out,
+                            cudaStream_t st) {
+  k_id_range<K><<<32, 256, 0, st>>>(a, na, b, nb, out);
+  return cudaGetLastError();
+}
+template cudaError_t launch_id_range<int32_t>(const int32_t*, int64_t, const int32_t*, int64_t,
+                                              KeyStats*, cudaStream_t);
+template cudaError_t launch_id_range<int64_t>(const int64_t*, int64_t, const int64_t*, int64_t,
+                                              KeyStats*, cudaStream_t);
+
 // out[i] = sorted[floor(i * (m - 1) / G) ] for i in [first, last]
 template <typename K>
 __global__ void k_quantiles(const K* __restrict__ sorted, int64_t m, int G, int first, int last,

@@ -16,6 +16,9 @@
 //
 // Every kernel takes an array of jobs so that one launch serves any number of
 // arrays (both sides of a join, or thousands of joins of a batch).
+#include <algorithm>
+#include <type_traits>
+
 #include "tj_internal.cuh"
 #include "tj_warp.cuh"
 
@@ -122,43 +125,66 @@ __device__ __forceinline__ void block_excl_scan_bins(const uint32_t* in, uint32_
 // ---------------------------------------------------------------------------
 // K1: min / max of every array's keys
 // ---------------------------------------------------------------------------
-template <typename K>
-__global__ void __launch_bounds__(kThreads) k_stats(const RadixJob<K>* __restrict__ jobs,
-                                                    int num_jobs, int64_t total_tiles,
-                                                    KeyStats* __restrict__ stats, int tile) {
+// WORDS: the "keys" are folded rows, compared unsigned.  (Eight CTAs a
+// multiprocessor at 32 registers: the read needs the loads in flight.)
+template <typename K, bool WORDS>
+__global__ void __launch_bounds__(kThreads, 8) k_stats(const RadixJob<K>* __restrict__ jobs,
+                                                       int num_jobs, int64_t total_tiles,
+                                                       KeyStats* __restrict__ stats, int tile) {
+  using T = typename std::conditional<WORDS, unsigned long long, K>::type;
+  constexpr unsigned long long kFlip = WORDS ? 0ull : 1ull << (8 * sizeof(K) - 1);
+  auto order = [](T k) -> unsigned long long {
+    return (unsigned long long)(typename UnsignedOf<K>::type)k ^ kFlip;
+  };
   __shared__ unsigned long long s_mn[kWarps], s_mx[kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // a contiguous run of tiles per CTA: one reduction and one pair of atomics
   // per job the run touches
   const int64_t per = (total_tiles + gridDim.x - 1) / gridDim.x;
   const int64_t t0 = (int64_t)blockIdx.x * per, t1 = min(total_tiles, t0 + per);
+  if (threadIdx.x == 0 && t0 < t1) {
+    // a sample of the ids' range: the run's first and last row (and the last
+    // row of the job it starts in)
+    auto sample = [&](int j, int64_t r) {
+      if (!jobs[j].ids) return;
+      const unsigned long long u = order_u(jobs[j].ids[r]);
+      atomicMin(&stats[j].id_min_u, u);
+      atomicMin(&stats[j].id_max_u, ~u);
+    };
+    const int j0 = find_job(jobs, num_jobs, t0), j1 = find_job(jobs, num_jobs, t1 - 1);
+    sample(j0, (t0 - jobs[j0].tile0) * tile);
+    sample(j1, min(jobs[j1].n, (t1 - jobs[j1].tile0) * tile) - 1);
+    if (j0 != j1) sample(j0, jobs[j0].n - 1);
+  }
   int cur = -1;
   int64_t cur_end = 0;  // first tile after the current job
-  unsigned long long mn = ~0ull, mx = 0ull;
+  const T kLeast = WORDS ? T(0) : (T)((typename UnsignedOf<K>::type)1 << (8 * sizeof(K) - 1));
+  T mn = ~kLeast, mx = kLeast;
   auto flush = [&]() {
+    unsigned long long a = order(mn), b = order(mx);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      unsigned long long a = __shfl_xor_sync(0xFFFFFFFFu, mn, o);
-      unsigned long long b = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
-      mn = a < mn ? a : mn;
-      mx = b > mx ? b : mx;
+      const unsigned long long x = __shfl_xor_sync(0xFFFFFFFFu, a, o);
+      const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, b, o);
+      a = x < a ? x : a;
+      b = y > b ? y : b;
     }
     if (lane == 0) {
-      s_mn[warp] = mn;
-      s_mx[warp] = mx;
+      s_mn[warp] = a;
+      s_mx[warp] = b;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int w = 1; w < kWarps; ++w) {
-        mn = s_mn[w] < mn ? s_mn[w] : mn;
-        mx = s_mx[w] > mx ? s_mx[w] : mx;
+        a = s_mn[w] < a ? s_mn[w] : a;
+        b = s_mx[w] > b ? s_mx[w] : b;
       }
-      atomicMin(&stats[cur].min_u, mn);
-      atomicMin(&stats[cur].max_u, ~mx);  // stored inverted so both fields use atomicMin
+      atomicMin(&stats[cur].min_u, a);
+      atomicMin(&stats[cur].max_u, ~b);  // stored inverted so both fields use atomicMin
     }
     __syncthreads();
-    mn = ~0ull;
-    mx = 0ull;
+    mn = ~kLeast;
+    mx = kLeast;
   };
   for (int64_t t = t0; t < t1; ++t) {
     if (cur < 0 || t >= cur_end) {
@@ -166,14 +192,14 @@ __global__ void __launch_bounds__(kThreads) k_stats(const RadixJob<K>* __restric
       cur = find_job(jobs, num_jobs, t);
       cur_end = jobs[cur].tile0 + (jobs[cur].n + tile - 1) / tile;
     }
-    const K* __restrict__ keys = jobs[cur].keys;
+    const T* __restrict__ keys = reinterpret_cast<const T*>(jobs[cur].keys);
     const int64_t row0 = (t - jobs[cur].tile0) * tile;
     const int64_t row1 = min(jobs[cur].n, row0 + tile);
 #pragma unroll 4
     for (int64_t r = row0 + threadIdx.x; r < row1; r += kThreads) {
-      const unsigned long long u = order_u(keys[r]);
-      mn = u < mn ? u : mn;
-      mx = u > mx ? u : mx;
+      const T k = keys[r];
+      mn = k < mn ? k : mn;
+      mx = k > mx ? k : mx;
     }
   }
   if (cur >= 0) flush();
@@ -187,8 +213,9 @@ __global__ void __launch_bounds__(kThreads) k_stats(const RadixJob<K>* __restric
 constexpr int kHistWords = 4096;
 
 // Counts of every pass's digit for the rows a thread loaded (P passes known at
-// compile time; NARROW: all digits lie in the low 32 bits of key - lo).
-template <typename K, int P, bool NARROW, int N>
+// compile time; HALF: 1, all digits lie in the low 32 bits of key - lo; 2, all
+// in the high 32 bits, of which lo has only high ones; 0, anywhere).
+template <typename K, int P, int HALF, int N>
 __device__ __forceinline__ void hist_rows(const K (&kv)[N], int row1,
                                           typename UnsignedOf<K>::type lo, const int (&sh)[kMaxPasses],
                                           const uint32_t (&mk)[kMaxPasses], uint32_t* s_h, int hs) {
@@ -196,10 +223,11 @@ __device__ __forceinline__ void hist_rows(const K (&kv)[N], int row1,
 #pragma unroll
   for (int u = 0; u < N; ++u) {
     if ((int)threadIdx.x + u * kThreads < row1) {
-      if (NARROW) {
-        const uint32_t x = (uint32_t)kv[u] - (uint32_t)lo;
+      if (HALF != 0) {
+        const uint32_t x = HALF == 1 ? (uint32_t)kv[u] - (uint32_t)lo
+                                     : (uint32_t)((uint64_t)kv[u] >> 32) - (uint32_t)((uint64_t)lo >> 32);
 #pragma unroll
-        for (int p = 0; p < P; ++p) atomicAdd(&s_h[p * hs + ((x >> sh[p]) & mk[p])], 1u);
+        for (int p = 0; p < P; ++p) atomicAdd(&s_h[p * hs + ((x >> (sh[p] & 31)) & mk[p])], 1u);
       } else {
         const U x = (U)kv[u] - lo;
 #pragma unroll
@@ -222,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_histogram(const RadixJob<K>* __
   __shared__ K s_cuts[kMaxCuts];
   __shared__ uint16_t s_tab[kRouteBuckets + 1];
   int cur = -1, passes = 0, ncuts = -1, hs = 0, rsteps = 0, rshift = -1;
-  bool narrow = false;
+  int half = 0;
   U lo = 0;
   int sh[kMaxPasses];
   uint32_t mk[kMaxPasses];
@@ -270,7 +298,8 @@ __global__ void __launch_bounds__(kThreads, 6) k_histogram(const RadixJob<K>* __
         sh[p] = p < passes ? jobs[j].shift[p] : 0;
         mk[p] = p < passes ? (1u << jobs[j].bits[p]) - 1u : 0u;
       }
-      narrow = passes > 0 && jobs[j].shift[passes - 1] + jobs[j].bits[passes - 1] <= 32;
+      half = passes > 0 && jobs[j].shift[passes - 1] + jobs[j].bits[passes - 1] <= 32 ? 1 : 0;
+      if (sizeof(K) == 8 && passes > 0 && jobs[j].shift[0] >= 32 && (uint32_t)lo == 0u) half = 2;
       for (int i = threadIdx.x; i < passes * hs; i += kThreads) s_h[i] = 0;
       __syncthreads();
     }
@@ -293,10 +322,12 @@ __global__ void __launch_bounds__(kThreads, 6) k_histogram(const RadixJob<K>* __
     } else {
 #define TJ_HIST_CASE(P)                                                   \
   case P:                                                                 \
-    if (narrow)                                                           \
-      hist_rows<K, P, true>(kv, row1, lo, sh, mk, s_h, hs);               \
+    if (half == 1)                                                        \
+      hist_rows<K, P, 1>(kv, row1, lo, sh, mk, s_h, hs);                  \
+    else if (half == 2)                                                   \
+      hist_rows<K, P, 2>(kv, row1, lo, sh, mk, s_h, hs);                  \
     else                                                                  \
-      hist_rows<K, P, false>(kv, row1, lo, sh, mk, s_h, hs);              \
+      hist_rows<K, P, 0>(kv, row1, lo, sh, mk, s_h, hs);                  \
     break;
       switch (passes) {
         TJ_HIST_CASE(1)
@@ -815,10 +846,14 @@ cudaError_t launch_route_chain(const uint32_t* base, const uint32_t* lookback, i
 // ---------------------------------------------------------------------------
 template <typename K>
 cudaError_t launch_stats(const RadixJob<K>* d_jobs, int num_jobs, int64_t total_tiles,
-                         KeyStats* d_stats, cudaStream_t st, int tile) {
+                         KeyStats* d_stats, cudaStream_t st, int tile, bool words) {
   if (total_tiles <= 0) return cudaSuccess;
-  const int64_t grid = total_tiles < 152 * 8 ? total_tiles : 152 * 8;
-  k_stats<K><<<(unsigned)grid, kThreads, 0, st>>>(d_jobs, num_jobs, total_tiles, d_stats, tile);
+  const unsigned grid = (unsigned)std::min<int64_t>(total_tiles, 152 * 8);
+  if (words)  // 8 bytes a row whatever K
+    k_stats<int64_t, true><<<grid, kThreads, 0, st>>>(
+        reinterpret_cast<const RadixJob<int64_t>*>(d_jobs), num_jobs, total_tiles, d_stats, tile);
+  else
+    k_stats<K, false><<<grid, kThreads, 0, st>>>(d_jobs, num_jobs, total_tiles, d_stats, tile);
   return cudaGetLastError();
 }
 
@@ -940,7 +975,7 @@ cudaError_t radix_init_attributes() {
 
 #define TJ_INSTANTIATE_RADIX(K)                                                                 \
   template cudaError_t launch_stats<K>(const RadixJob<K>*, int, int64_t, KeyStats*,             \
-                                       cudaStream_t, int);                                      \
+                                       cudaStream_t, int, bool);                                \
   template cudaError_t launch_histogram<K>(const RadixJob<K>*, int, int64_t, cudaStream_t,      \
                                            const int32_t*, int);                                \
   template cudaError_t launch_fill_tile_job<K>(const RadixJob<K>*, int, int32_t*, cudaStream_t, \

@@ -1,11 +1,13 @@
-// Warp-level ranking shared by the onesweep passes (tj_radix.cu) and the
-// fused partition-resident join (tj_fused.cu): stable ranks of a warp's rows
-// by a small digit, found with one ballot per digit bit (rank_items) or with a
+// Warp-level ranking shared by the onesweep passes (tj_radix.cu, tj_word.cu) and
+// the partition-resident join (tj_fused.cu): stable ranks of a warp's rows by a
+// small digit, found with one ballot per digit bit (rank_items), with a
 // per-warp table of lane masks for the low 7 bits and one ballot per higher
-// bit (rank_items_or).
+// bit (rank_items_or), or some rows each way (wrank).
 #pragma once
 
 #include <stdint.h>
+
+#include "tj_internal.cuh"
 
 namespace tj {
 
@@ -98,6 +100,97 @@ __device__ __forceinline__ void rank_items_or(uint32_t (&dr)[ITEMS], int nv, uin
     __syncwarp();
     base = __shfl_sync(0xFFFFFFFFu, base, leader);
     dr[i] |= (base + __popc(peers & ltm)) << 16;
+  }
+}
+
+__device__ __forceinline__ uint32_t lanemask_gt() {
+  uint32_t m;
+  asm volatile("mov.u32 %0, %%lanemask_gt;" : "=r"(m));
+  return m;
+}
+
+// 16-bit values, two a register.
+template <int N>
+struct Half {
+  uint32_t v[(N + 1) / 2];
+  __device__ __forceinline__ uint32_t get(int i) const {
+    return (i & 1) ? v[i >> 1] >> 16 : v[i >> 1] & 0xFFFFu;
+  }
+  // i in ascending order: the even one sets the register, the odd one adds
+  __device__ __forceinline__ void set(int i, uint32_t x) {
+    if (i & 1)
+      v[i >> 1] |= x << 16;
+    else
+      v[i >> 1] = x;
+  }
+  __device__ __forceinline__ void put(int i, uint32_t x) {
+    v[i >> 1] = __byte_perm(v[i >> 1], x, (i & 1) ? 0x5410 : 0x3254);
+  }
+};
+
+// items ranked together by wrank
+template <int ITEMS>
+__host__ __device__ constexpr int wrank_group() {
+  return ITEMS % 4 == 0 ? 4 : (ITEMS % 3 == 0 ? 3 : (ITEMS % 2 == 0 ? 2 : 1));
+}
+
+// Stable ranks of a warp's words, item i of the warp being 32 consecutive
+// rows with digit(i) (NB bits): rows of the digit earlier in the warp (`cnt`,
+// of 16 or 32 bits, and `masks` zero on entry; groups of items at or beyond row
+// nv are skipped, rows beyond it in the last group counted).  All
+// lanes read the warp's count of their digit and the digit's highest lane
+// stores the new one.  The lanes of equal digit are found for kWMaskItems of
+// every G items through a table of lane masks by the digit's low 7 bits (each
+// lane ORs its bit in, reads the word back, and the group's highest lane
+// clears it) with a ballot per higher bit, for the others by a ballot per
+// digit bit.  Ballots cost issue slots, the table conflicting shared-memory
+// accesses, and each alone bounds the pass: 10^8 words by a 7-bit digit take
+// 526 us with ballots only, 527 with the table only, 500 with two of four
+// items each way (GB300, 512 threads x 16 words).
+template <int NB, int ITEMS, typename C, typename D>
+__device__ __forceinline__ void wrank(const D& digit, Half<ITEMS>& rank, C* cnt, uint32_t* masks,
+                                      int nv = 32 * ITEMS) {
+  const uint32_t bit = 1u << (threadIdx.x & 31), ltm = lanemask_lt(), gtm = lanemask_gt();
+  constexpr int G = wrank_group<ITEMS>();
+  constexpr int MX = kWMaskItems < G ? kWMaskItems : G;
+#pragma unroll
+  for (int i0 = 0; i0 < ITEMS; i0 += G) {
+    if (nv < 32 * ITEMS && i0 * 32 >= nv) break;
+    uint32_t d[G], peers[G];
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      d[h] = digit(i0 + h);
+      peers[h] = 0xFFFFFFFFu;
+    }
+#pragma unroll
+    for (int h = 0; h < MX; ++h) atomicOr(&masks[h * 128 + (d[h] & 127u)], bit);
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < MX; ++h) peers[h] = masks[h * 128 + (d[h] & 127u)];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        if (h < MX && b < 7) continue;
+        const bool p = (d[h] & (1u << b)) != 0u;
+        const uint32_t x = __ballot_sync(0xFFFFFFFFu, p);
+        peers[h] &= p ? x : ~x;  // lanes whose bit b equals this lane's
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < MX; ++h)
+      if ((peers[h] & gtm) == 0u) masks[h * 128 + (d[h] & 127u)] = 0u;
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      C* c = cnt + d[h];
+      const uint32_t base = *c;
+      __syncwarp();
+      if ((peers[h] & gtm) == 0u) *c = (C)(base + __popc(peers[h]));
+      rank.set(i0 + h, base + __popc(peers[h] & ltm));
+      __syncwarp();
+    }
   }
 }
 

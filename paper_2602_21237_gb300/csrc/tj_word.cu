@@ -1,0 +1,538 @@
+// Radix passes over folded rows: the tensor-path sort (paper Sec. 4.2) and the
+// route / MSD passes of the join, on rows of one 64-bit word.
+//
+// A row (key, id) whose key offset and id fit 64 bits together is one word,
+//   w = (key - wlo) << ib | (id - ilo),
+// made by the first pass as it reads the caller's columns and taken apart
+// again only where ids (or keys) are written.  Against separate key and id
+// arrays every pass in between moves 8 bytes a row instead of 16 (64-bit
+// rows), and a row is one load, one shared-memory slot and one store instead
+// of two of each plus an index.
+//
+// k_wsweep is one onesweep pass (decoupled look-back, as k_onesweep in
+// tj_radix.cu) over a tile of kWThreads * ITEMS words held in registers:
+// rank inside the warp, move the words to their
+// tile-sorted slots in shared memory, write the slots out in order.
+#include <algorithm>
+
+#include "tj_internal.cuh"
+#include "tj_warp.cuh"
+
+namespace tj {
+
+namespace {
+
+__device__ __forceinline__ uint32_t wld_volatile(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.volatile.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void wst_volatile(uint32_t* p, uint32_t v) {
+  asm volatile("st.volatile.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+template <typename Job>
+__device__ __forceinline__ int find_job_w(const Job* jobs, int num_jobs, int64_t t) {
+  int lo = 0, hi = num_jobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs[mid].tile0 <= t)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  return lo;
+}
+
+// Digit of a word: bits [shift, shift + n) of w - lo.  HI: shift >= 32 and lo
+// is a multiple of 2^32 (keys of at most 32 bits sit in the word's upper
+// half), so one 32-bit subtract and shift give it.
+template <bool HI>
+__device__ __forceinline__ uint32_t wdigit(uint64_t w, uint64_t lo, int shift, uint32_t mask) {
+  if (HI) return (((uint32_t)(w >> 32) - (uint32_t)(lo >> 32)) >> (shift & 31)) & mask;
+  return (uint32_t)((w - lo) >> shift) & mask;
+}
+
+// Batch of a word under equal-width ranges: (clamp(key) - lo) >> shift, all
+// as offsets from the words' first key (rlo: the range's first key, span: its
+// width).  HI as above: the key offset lies in the upper 32 bits.
+template <bool HI>
+__device__ __forceinline__ uint32_t wroute_radix(uint64_t w, int ib, uint64_t rlo, uint64_t span,
+                                                 int shift) {
+  if (HI) {
+    const uint32_t x = (uint32_t)(w >> 32) >> (ib & 31), l = (uint32_t)rlo;
+    const uint32_t y = x < l ? 0u : min(x - l, (uint32_t)span);
+    return y >> shift;
+  }
+  const uint64_t x = w >> ib;
+  uint64_t y = x < rlo ? 0ull : x - rlo;
+  y = y < span ? y : span;
+  return (uint32_t)(y >> shift);
+}
+
+// Batch of a word under the cut table: the number of cuts <= key (offsets from
+// the words' first key), through the radix index over the cuts (the same
+// number of halvings on every lane; see RadixJob::route_tab).
+__device__ __forceinline__ uint32_t wroute_cuts(uint64_t w, int ib, uint64_t rlo,
+                                                const uint64_t* s_cuts, const uint16_t* s_tab,
+                                                int steps, int ushift) {
+  const uint64_t key = w >> ib;
+  const uint64_t x = key < rlo ? 0ull : key - rlo;
+  uint32_t b;
+  if (ushift >= 0) {
+    const uint64_t u = x >> ushift;
+    b = u < (uint64_t)(kRouteBuckets - 1) ? (uint32_t)u : (uint32_t)(kRouteBuckets - 1);
+  } else {
+    const int nb = 64 - __clzll((long long)x);
+    b = nb < 6 ? (uint32_t)x : (uint32_t)((nb << 5) | ((x >> (nb - 6)) & 31ull));
+  }
+  int a = s_tab[b];
+  int n = (int)s_tab[b + 1] - a;
+  for (int i = 0; i < steps; ++i) {
+    const int half = n >> 1;
+    const bool go = n > 0 && s_cuts[a + half] <= key;
+    a = go ? a + half + 1 : a;
+    n = go ? n - half - 1 : half;
+  }
+  return (uint32_t)a;
+}
+
+// Per-warp ranking tables of a pass: digit counts, lane masks.
+__host__ __device__ constexpr size_t wtable_bytes(int nbits) {
+  return (size_t)kWWarps * 4u * (((size_t)1 << (nbits < 2 ? 2 : nbits)) + 128u * kWMaskItems);
+}
+
+// Shared memory: the tile's words in tile-sorted order, overlaid with the
+// ranking tables (dead before the words move) | global base and tile
+// count per digit | end of each batch's region (guarded route passes) | cut
+// keys, radix index and slot digits (route passes by the cut table).
+template <int ITEMS>
+__host__ __device__ constexpr size_t wsweep_smem_bytes(int nbits, int mode, bool guard) {
+  const size_t stage = 8u * (size_t)kWThreads * ITEMS;
+  const size_t bins = (size_t)1 << nbits;
+  return (stage > wtable_bytes(nbits) ? stage : wtable_bytes(nbits)) + 8u * bins +
+         (mode != kModeSort && guard ? 4u * bins : 0u) +
+         (mode == kModeCuts ? 8u * bins + 2u * (kRouteBuckets + 8) +
+                                  (size_t)(nbits <= 8 ? 1 : 2) * kWThreads * ITEMS
+                            : 0u);
+}
+
+template <int ITEMS, typename D>
+__device__ __forceinline__ void wrank_bits(const D& digit, int nbits, Half<ITEMS>& rank,
+                                           uint32_t* cnt, uint32_t* masks) {
+  switch (nbits) {
+    case 0:  // one digit value
+    case 1: wrank<1, ITEMS>(digit, rank, cnt, masks); break;
+    case 2: wrank<2, ITEMS>(digit, rank, cnt, masks); break;
+    case 3: wrank<3, ITEMS>(digit, rank, cnt, masks); break;
+    case 4: wrank<4, ITEMS>(digit, rank, cnt, masks); break;
+    case 5: wrank<5, ITEMS>(digit, rank, cnt, masks); break;
+    case 6: wrank<6, ITEMS>(digit, rank, cnt, masks); break;
+    case 7: wrank<7, ITEMS>(digit, rank, cnt, masks); break;
+    case 8: wrank<8, ITEMS>(digit, rank, cnt, masks); break;
+    case 9: wrank<9, ITEMS>(digit, rank, cnt, masks); break;
+    default: wrank<10, ITEMS>(digit, rank, cnt, masks); break;
+  }
+}
+
+// Sum look-back words (newest predecessor first) into `prefix` up to the first
+// inclusive one, stopping at one not published yet; returns the words used.
+template <int W>
+__device__ __forceinline__ int wlookback(const uint32_t (&v)[W], uint32_t& prefix, bool& done) {
+  int used = 0;
+  uint32_t acc = 0;
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    if (used != k) break;
+    const uint32_t f = v[k] & ~kValMask;
+    if (f == 0u) break;
+    acc += v[k] & kValMask;
+    ++used;
+    if (f == kFlagInc) {
+      done = true;
+      break;
+    }
+  }
+  prefix += acc;
+  return used;
+}
+
+}  // namespace
+
+// One pass over a tile of kWThreads * ITEMS rows:
+//   1. words into registers (RAW_IN: folded from the key and id columns; a row
+//      whose key offset or id does not fit sets *err = kErrFold), digits,
+//      stable ranks inside each warp;
+//   2. per digit: sum over the warps, publish to the look-back chain, scan;
+//   3. the words move to their tile-sorted slots in shared memory while the
+//      digits' threads finish the look-back (bounded wait);
+//   4. slots in order -> global: each digit's run lands contiguously (RAW_OUT:
+//      as key and id columns).
+// Rows beyond the tile's end carry the largest digit, so they rank last and
+// need no test before step 4.
+// MODE: kModeSort (a digit of w - lo), kModeRadix or kModeCuts (route passes:
+// the batch under equal-width ranges or the cut table).  HI: see wdigit.
+// After rows failed to fold, the later passes return at once, so a RAW_OUT
+// pass never overwrites the caller's columns with them.
+template <typename K, bool RAW_IN, bool RAW_OUT, int MODE, bool HI, int ITEMS>
+__global__ void __launch_bounds__(kWThreads, kWMinB)
+    k_wsweep(const RadixJob<K>* __restrict__ jobs, int num_jobs, int64_t total_tiles, int pass,
+             uint32_t* __restrict__ tile_counter, int* __restrict__ err,
+             const int32_t* __restrict__ tile_job) {
+  using U = typename UnsignedOf<K>::type;
+  constexpr int TILE = kWThreads * ITEMS;
+  static_assert(TILE <= 65536, "16-bit positions within a tile");
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ uint32_t s_warp[kWWarps];
+  __shared__ uint32_t s_t;
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) {
+    // (only passes that fold set kErrFold, so all tiles of a pass agree)
+    const bool stop = !RAW_IN && wld_volatile(reinterpret_cast<const uint32_t*>(err)) ==
+                                     (uint32_t)kErrFold;
+    const uint32_t ticket = atomicAdd(tile_counter, 1u);
+    s_t = stop ? 0xFFFFFFFFu : ticket;
+  }
+  __syncthreads();
+  const int64_t t = s_t;
+  if (t >= total_tiles) return;
+  const int j = tile_job ? tile_job[t] : find_job_w(jobs, num_jobs, t);
+  const RadixJob<K>* J = jobs + j;
+  if (pass >= J->passes) return;
+  // tiles of a job are numbered in 32 bits (n < 2^30 rows)
+  const int lt = (int)(t - J->tile0);
+  const int64_t row0 = (int64_t)lt * TILE;
+  const int nvalid = (int)min((int64_t)TILE, J->n - row0);
+  const int shift = J->shift[pass], nbits = J->bits[pass];
+  const int bins = 1 << nbits;
+  const uint32_t mask = (uint32_t)bins - 1u;
+  const uint64_t lo = J->lo;
+  const int ib = J->ib;
+  const uint64_t idm = (1ull << ib) - 1ull;
+
+  uint64_t* const stage = reinterpret_cast<uint64_t*>(smem);
+  const size_t tab_bytes = wtable_bytes(nbits);
+  const size_t area = 8u * (size_t)TILE > tab_bytes ? 8u * (size_t)TILE : tab_bytes;
+  uint32_t* const s_gbase = reinterpret_cast<uint32_t*>(smem + area);
+  uint32_t* const s_cnt = s_gbase + bins;
+  uint32_t* const s_rend = s_cnt + bins;
+  const bool guard = MODE != kModeSort && J->route_end != nullptr;
+  uint64_t* const s_cuts =
+      reinterpret_cast<uint64_t*>(smem + area + 8u * bins + (guard ? 4u * bins : 0u));
+  uint16_t* const s_tab = reinterpret_cast<uint16_t*>(s_cuts + bins);
+  uint16_t* const s_dig = s_tab + (kRouteBuckets + 8);
+  uint8_t* const s_dig8 = reinterpret_cast<uint8_t*>(s_dig);
+  const bool dig8 = nbits <= 8;
+  const uint64_t span = J->route_hi;  // route passes: the range's width
+  const int rsteps = J->route_steps, rshift = J->route_shift;
+
+  auto digit = [&](uint64_t w) -> uint32_t {
+    if (MODE == kModeRadix) return wroute_radix<HI>(w, ib, lo, span, shift);
+    if (MODE == kModeCuts) return wroute_cuts(w, ib, lo, s_cuts, s_tab, rsteps, rshift);
+    return wdigit<HI>(w, lo, shift, mask);
+  };
+
+  // 1. words
+  const int wbase = warp * 32 * ITEMS + lane;
+  // a row past the end takes the largest digit any row can have
+  const uint64_t pad = MODE == kModeCuts ? ~0ull
+                       : MODE == kModeRadix ? (lo + span) << ib
+                                            : lo + ((uint64_t)mask << shift);
+  uint64_t w[ITEMS];
+  if (RAW_IN) {
+    const K* __restrict__ kp = J->src_k[pass] + row0;
+    const K* __restrict__ vp = J->fold_v[pass] + row0;
+    const U wlo = (U)J->wlo, ilo = (U)J->ilo;
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+      const int r = wbase + i * 32;
+      w[i] = pad;
+      if (r < nvalid) {
+        const uint64_t ko = (uint64_t)(U)((U)kp[r] - wlo), io = (uint64_t)(U)((U)vp[r] - ilo);
+        if (sizeof(K) == 8) bad |= ((io >> ib) | (ko >> (64 - ib))) != 0ull;
+        w[i] = (ko << ib) | (io & idm);
+      }
+    }
+    if (sizeof(K) == 8 && bad && wld_volatile(reinterpret_cast<const uint32_t*>(err)) == 0u)
+      atomicCAS(err, 0, kErrFold);
+  } else {
+    const uint64_t* __restrict__ wp =
+        reinterpret_cast<const uint64_t*>(J->src_k[pass]) + row0;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+      const int r = wbase + i * 32;
+      w[i] = r < nvalid ? wp[r] : pad;
+    }
+  }
+  {
+    uint4* z = reinterpret_cast<uint4*>(smem);
+    for (int i = tid; i < (int)(tab_bytes / 16); i += kWThreads) z[i] = make_uint4(0, 0, 0, 0);
+  }
+  if (MODE == kModeCuts) {
+    const uint64_t* __restrict__ cuts = reinterpret_cast<const uint64_t*>(J->cuts);
+    for (int i = tid; i < bins; i += kWThreads) s_cuts[i] = cuts[i];
+    for (int i = tid; i <= kRouteBuckets; i += kWThreads) s_tab[i] = J->route_tab[i];
+  }
+  if (guard)
+    for (int i = tid; i < bins; i += kWThreads) s_rend[i] = J->route_end[i];
+  __syncthreads();
+  // sort digits are taken from the word again when needed (two instructions),
+  // batch indices are kept
+  constexpr bool KEEP = MODE != kModeSort;
+  Half<ITEMS> dig, rank;
+  if (KEEP) {
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) dig.set(i, digit(w[i]));
+  }
+  int sh = shift;  // opaque to the compiler from phase to phase, see below
+  auto item_digit = [&](int i) -> uint32_t {
+    return KEEP ? dig.get(i) : wdigit<HI>(w[i], lo, sh, mask);
+  };
+  uint32_t* const t_cnt = reinterpret_cast<uint32_t*>(smem);  // [warp][digit]
+  uint32_t* const t_mask = t_cnt + kWWarps * bins;
+  wrank_bits<ITEMS>(item_digit, nbits, rank, t_cnt + warp * bins,
+                    t_mask + warp * 128 * kWMaskItems);
+  __syncthreads();
+
+  // 2. per digit (`per` consecutive ones a thread): the tile's count,
+  //    published, and its exclusive prefix over (digit, warp), left in the
+  //    tables
+  const int per = (bins + kWThreads - 1) / kWThreads;
+  const int d0 = tid * per, d1 = min(bins, d0 + per);
+  uint32_t sum = 0;
+  {
+    const uint32_t npad = (uint32_t)(TILE - nvalid);
+    uint32_t* const lb_mine = J->lookback + pass * J->lb_stride + (int64_t)lt * bins;
+    const uint32_t dpad = npad ? (MODE == kModeCuts ? (uint32_t)J->ncuts : digit(pad)) : ~0u;
+#pragma unroll 1
+    for (int d = d0; d < d1; ++d) {
+      uint32_t c = 0;
+#pragma unroll
+      for (int q = 0; q < kWWarps; ++q) c += t_cnt[q * bins + d];
+      sum += c;
+      s_gbase[d] = c;
+      if ((uint32_t)d == dpad) c -= npad;
+      s_cnt[d] = c;
+      wst_volatile(lb_mine + d, (lt == 0 ? kFlagInc : kFlagAgg) | c);
+    }
+    uint32_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    uint32_t run = x - sum;
+#pragma unroll
+    for (int q = 0; q < kWWarps; ++q)
+      if (q < warp) run += s_warp[q];
+#pragma unroll 1
+    for (int d = d0; d < d1; ++d) {
+      const uint32_t c = s_gbase[d];
+      s_gbase[d] = run;
+      uint32_t p = run;
+#pragma unroll
+      for (int q = 0; q < kWWarps; ++q) {
+        const uint32_t v = t_cnt[q * bins + d];
+        t_cnt[q * bins + d] = p;
+        p += v;
+      }
+      run += c;
+    }
+  }
+  __syncthreads();
+
+  // 3. positions (the tables die here), the look-back, the move
+  // (the digits are computed again, not carried in registers, which spilled)
+  asm volatile("" : "+r"(sh));
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i)
+    rank.put(i, rank.get(i) + t_cnt[warp * bins + item_digit(i)]);
+  __syncthreads();
+  const uint32_t* __restrict__ hist = J->hist + pass * J->hist_stride;
+  uint32_t* const lb_base = J->lookback + pass * J->lb_stride;
+#pragma unroll 1
+  for (int d = d0; d < d1; ++d) {
+    uint32_t prefix = 0;
+    if (lt > 0) {
+      int k = lt - 1;  // newest predecessor not yet summed
+      bool done = false;
+      int spins = 0;
+      while (!done) {
+        uint32_t v[kLookWide];
+#pragma unroll
+        for (int q = 0; q < kLookWide; ++q)
+          v[q] = (k - q >= 0) ? wld_volatile(lb_base + (int64_t)(k - q) * bins + d) : kFlagInc;
+        const int used = wlookback<kLookWide>(v, prefix, done);
+        k -= used;
+        if (used == 0) {
+          if (++spins > kSpinLimit) {
+            atomicExch(err, (int)TJ_ERR_TIMEOUT);
+            break;
+          }
+          __nanosleep(32);
+        }
+      }
+      wst_volatile(lb_base + (int64_t)lt * bins + d, kFlagInc | ((prefix + s_cnt[d]) & kValMask));
+    }
+    s_gbase[d] = hist[d] + prefix - s_gbase[d];  // minus the digit's first slot
+  }
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) {
+    const uint32_t pos = rank.get(i);
+    stage[pos] = w[i];
+    if (MODE == kModeCuts) {
+      if (dig8)
+        s_dig8[pos] = (uint8_t)dig.get(i);
+      else
+        s_dig[pos] = (uint16_t)dig.get(i);
+    }
+  }
+  __syncthreads();
+
+  // 4. slots in order -> global
+  uint64_t* __restrict__ dst_w = reinterpret_cast<uint64_t*>(J->dst_k[pass]);
+  K* __restrict__ dst_k = J->dst_k[pass];
+  K* __restrict__ dst_v = J->dst_v[pass];
+  const U wlo = (U)J->wlo, ilo = (U)J->ilo;
+  const uint32_t room = RAW_IN ? (uint32_t)J->dst_rows : 0u;
+  bool over = false;
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    const int q = tid + it * kWThreads;
+    if (q < nvalid) {
+      const uint64_t x = stage[q];
+      const uint32_t d = MODE == kModeCuts ? (dig8 ? (uint32_t)s_dig8[q] : (uint32_t)s_dig[q])
+                                           : digit(x);
+      const uint32_t g = s_gbase[d] + (uint32_t)q;
+      if (RAW_OUT) {
+        dst_k[g] = (K)((U)(x >> ib) + wlo);
+        dst_v[g] = (K)((U)(x & idm) + ilo);
+      } else {
+        // batch regions sized in advance: a row past its region's end is
+        // dropped and reported (the caller then routes again); rows that did
+        // not fold may miscount, so a folding pass keeps to its destination
+        const bool in = MODE != kModeSort && guard ? g < s_rend[d] : !RAW_IN || g < room;
+        over |= !in;
+        if (in) dst_w[g] = x;
+      }
+    }
+  }
+  if (MODE != kModeSort && over) atomicCAS(err, 0, (int)TJ_ERR_CAPACITY);
+}
+
+// ---------------------------------------------------------------------------
+// launchers
+// ---------------------------------------------------------------------------
+template <typename K, bool RI, bool RO, int MODE, bool HI, int ITEMS>
+cudaError_t wsweep_attr() {
+  size_t m = 0;
+  for (int b = 1; b <= kMaxDigitBits; ++b)
+    m = std::max(m, wsweep_smem_bytes<ITEMS>(b, MODE, MODE != kModeSort));
+  return cudaFuncSetAttribute(k_wsweep<K, RI, RO, MODE, HI, ITEMS>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m);
+}
+
+template <typename K, bool RI, bool RO, int MODE, bool HI, int ITEMS>
+cudaError_t wsweep_go(const RadixJob<K>* d_jobs, int num_jobs, int64_t tiles, int pass,
+                      int max_bits, bool guard, uint32_t* d_counter, int* d_err, cudaStream_t st,
+                      const int32_t* d_tile_job) {
+  if (tiles <= 0) return cudaSuccess;
+  // a launch over jobs of several digit widths takes the widest one's layout
+  size_t smem = 0;
+  for (int b = 1; b <= max_bits; ++b)
+    smem = std::max(smem, wsweep_smem_bytes<ITEMS>(b, MODE, guard));
+  k_wsweep<K, RI, RO, MODE, HI, ITEMS><<<(unsigned)tiles, kWThreads, smem, st>>>(
+      d_jobs, num_jobs, tiles, pass, d_counter, d_err, d_tile_job);
+  return cudaGetLastError();
+}
+
+template <typename K, int MODE, int ITEMS>
+cudaError_t wsweep_pick(const RadixJob<K>* d_jobs, int num_jobs, int64_t tiles, int pass,
+                        int max_bits, bool raw_in, bool raw_out, bool hi, bool guard,
+                        uint32_t* d_counter, int* d_err, cudaStream_t st,
+                        const int32_t* d_tile_job) {
+#define TJ_GO(RI, RO, H)                                                                        \
+  return wsweep_go<K, RI, RO, MODE, H, ITEMS>(d_jobs, num_jobs, tiles, pass, max_bits, guard,  \
+                                              d_counter, d_err, st, d_tile_job)
+  constexpr bool wide = sizeof(K) == 8;  // 32-bit keys always sit in the upper half
+  if (raw_in) {
+    if constexpr (wide && MODE != kModeCuts)
+      if (!hi) TJ_GO(true, false, false);
+    TJ_GO(true, false, true);
+  }
+  if constexpr (MODE == kModeSort) {
+    if (raw_out) {
+      if constexpr (wide)
+        if (!hi) TJ_GO(false, true, false);
+      TJ_GO(false, true, true);
+    }
+    if constexpr (wide) {
+      if (!hi) TJ_GO(false, false, false);
+      TJ_GO(false, false, true);
+    }
+  }
+  return cudaErrorInvalidValue;
+#undef TJ_GO
+}
+
+template <typename K>
+cudaError_t launch_wsweep(const RadixJob<K>* d_jobs, int num_jobs, int64_t total_tiles, int pass,
+                          int max_bits, int mode, bool raw_in, bool raw_out, bool hi, int items,
+                          bool guard, uint32_t* d_tile_counter, int* d_err, cudaStream_t st,
+                          const int32_t* d_tile_job) {
+#define TJ_PICK(M, I)                                                                           \
+  return wsweep_pick<K, M, I>(d_jobs, num_jobs, total_tiles, pass, max_bits, raw_in, raw_out,  \
+                              hi, guard, d_tile_counter, d_err, st, d_tile_job)
+  if (items == kWItems) {
+    if (mode == kModeSort) TJ_PICK(kModeSort, kWItems);
+    if (mode == kModeRadix) TJ_PICK(kModeRadix, kWItems);
+    if (mode == kModeCuts) TJ_PICK(kModeCuts, kWItems);
+  } else if (items == kWItemsSmall && mode == kModeSort) {
+    TJ_PICK(kModeSort, kWItemsSmall);
+  }
+  return cudaErrorInvalidValue;
+#undef TJ_PICK
+}
+
+template <typename K, int MODE, int ITEMS>
+cudaError_t wsweep_attrs_mode() {
+  constexpr bool wide = sizeof(K) == 8;
+  cudaError_t e = wsweep_attr<K, true, false, MODE, true, ITEMS>();
+  if constexpr (wide && MODE != kModeCuts)
+    if (e == cudaSuccess) e = wsweep_attr<K, true, false, MODE, false, ITEMS>();
+  if constexpr (MODE == kModeSort) {
+    if (e == cudaSuccess) e = wsweep_attr<K, false, true, MODE, true, ITEMS>();
+    if constexpr (wide) {
+      if (e == cudaSuccess) e = wsweep_attr<K, false, true, MODE, false, ITEMS>();
+      if (e == cudaSuccess) e = wsweep_attr<K, false, false, MODE, false, ITEMS>();
+      if (e == cudaSuccess) e = wsweep_attr<K, false, false, MODE, true, ITEMS>();
+    }
+  }
+  return e;
+}
+
+template <typename K>
+cudaError_t wsweep_attrs() {
+  cudaError_t e = wsweep_attrs_mode<K, kModeSort, kWItems>();
+  if (e == cudaSuccess) e = wsweep_attrs_mode<K, kModeSort, kWItemsSmall>();
+  if (e == cudaSuccess) e = wsweep_attrs_mode<K, kModeRadix, kWItems>();
+  if (e == cudaSuccess) e = wsweep_attrs_mode<K, kModeCuts, kWItems>();
+  return e;
+}
+
+cudaError_t word_init_attributes() {
+  cudaError_t e = wsweep_attrs<int32_t>();
+  return e != cudaSuccess ? e : wsweep_attrs<int64_t>();
+}
+
+#define TJ_INSTANTIATE_WORD(K)                                                                  \
+  template cudaError_t launch_wsweep<K>(const RadixJob<K>*, int, int64_t, int, int, int, bool, \
+                                        bool, bool, int, bool, uint32_t*, int*, cudaStream_t,  \
+                                        const int32_t*);
+TJ_INSTANTIATE_WORD(int32_t)
+TJ_INSTANTIATE_WORD(int64_t)
+
+}  // namespace tj
