@@ -10,10 +10,11 @@
 // of two of each plus an index.
 //
 // k_wsweep is one onesweep pass (decoupled look-back, as k_onesweep in
-// tj_radix.cu) over a tile of kWThreads * ITEMS words held in registers:
-// rank inside the warp, move the words to their
-// tile-sorted slots in shared memory, write the slots out in order.
+// tj_radix.cu) over a tile of kWThreads * ITEMS rows: take the digits, rank
+// them inside the warp, move the words to their tile-sorted slots in shared
+// memory, write the slots out in order.
 #include <algorithm>
+#include <type_traits>
 
 #include "tj_internal.cuh"
 #include "tj_warp.cuh"
@@ -159,14 +160,22 @@ __device__ __forceinline__ int wlookback(const uint32_t (&v)[W], uint32_t& prefi
 }  // namespace
 
 // One pass over a tile of kWThreads * ITEMS rows:
-//   1. words into registers (RAW_IN: folded from the key and id columns; a row
-//      whose key offset or id does not fit sets *err = kErrFold), digits,
-//      stable ranks inside each warp;
+//   1. digits, 16 bits a row in registers (from the key column, or the words'
+//      upper halves when the key is there), and stable ranks inside each warp;
 //   2. per digit: sum over the warps, publish to the look-back chain, scan;
-//   3. the words move to their tile-sorted slots in shared memory while the
-//      digits' threads finish the look-back (bounded wait);
+//   3. the rows are read again, from L2 (RAW_IN: keys and ids, folded; a row
+//      whose key offset or id does not fit sets *err = kErrFold), and move to
+//      their tile-sorted slots in shared memory, after the digits' threads have
+//      finished the look-back (bounded wait);
 //   4. slots in order -> global: each digit's run lands contiguously (RAW_OUT:
 //      as key and id columns).
+// Reading a row twice, L2's bandwidth being idle, keeps only its digit and rank
+// in registers while the tile is ranked. Holding the words there spilled at
+// 512 threads x 16 rows, two CTAs a multiprocessor (64 registers), above all
+// where columns are folded: 5x10^8 rows by an 8-bit batch digit took 4.44 ms,
+// now 3.08 ms (12 GB); 10^8 words take 491 / 535 / 594 us by 7 / 8 / 9 bits
+// against 500 / 538 / 618. What bounds the pass is the ranking (see wrank):
+// without it and the look-back the same tiles move at the copy rate.
 // Rows beyond the tile's end carry the largest digit, so they rank last and
 // need no test before step 4.
 // MODE: kModeSort (a digit of w - lo), kModeRadix or kModeCuts (route passes:
@@ -232,38 +241,25 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
     return wdigit<HI>(w, lo, shift, mask);
   };
 
-  // 1. words
+  // 1. digits.  A row past the end takes the largest digit any row can have.
   const int wbase = warp * 32 * ITEMS + lane;
-  // a row past the end takes the largest digit any row can have
   const uint64_t pad = MODE == kModeCuts ? ~0ull
                        : MODE == kModeRadix ? (lo + span) << ib
                                             : lo + ((uint64_t)mask << shift);
-  uint64_t w[ITEMS];
-  if (RAW_IN) {
-    const K* __restrict__ kp = J->src_k[pass] + row0;
-    const K* __restrict__ vp = J->fold_v[pass] + row0;
-    const U wlo = (U)J->wlo, ilo = (U)J->ilo;
-    bool bad = false;
+  const uint64_t* __restrict__ wp = reinterpret_cast<const uint64_t*>(J->src_k[pass]) + row0;
+  const K* __restrict__ kp = J->src_k[pass] + row0;
+  using Part = typename std::conditional<RAW_IN, K,
+                                         typename std::conditional<HI, uint32_t, uint64_t>::type>::type;
+  Part part[ITEMS];
 #pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-      const int r = wbase + i * 32;
-      w[i] = pad;
-      if (r < nvalid) {
-        const uint64_t ko = (uint64_t)(U)((U)kp[r] - wlo), io = (uint64_t)(U)((U)vp[r] - ilo);
-        if (sizeof(K) == 8) bad |= ((io >> ib) | (ko >> (64 - ib))) != 0ull;
-        w[i] = (ko << ib) | (io & idm);
-      }
-    }
-    if (sizeof(K) == 8 && bad && wld_volatile(reinterpret_cast<const uint32_t*>(err)) == 0u)
-      atomicCAS(err, 0, kErrFold);
-  } else {
-    const uint64_t* __restrict__ wp =
-        reinterpret_cast<const uint64_t*>(J->src_k[pass]) + row0;
-#pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-      const int r = wbase + i * 32;
-      w[i] = r < nvalid ? wp[r] : pad;
-    }
+  for (int i = 0; i < ITEMS; ++i) {
+    const int r = wbase + i * 32;
+    if constexpr (RAW_IN)
+      part[i] = r < nvalid ? kp[r] : K(0);
+    else if constexpr (HI)
+      part[i] = r < nvalid ? reinterpret_cast<const uint32_t*>(wp)[2 * r + 1] : (uint32_t)(pad >> 32);
+    else
+      part[i] = r < nvalid ? wp[r] : pad;
   }
   {
     uint4* z = reinterpret_cast<uint4*>(smem);
@@ -277,18 +273,22 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
   if (guard)
     for (int i = tid; i < bins; i += kWThreads) s_rend[i] = J->route_end[i];
   __syncthreads();
-  // sort digits are taken from the word again when needed (two instructions),
-  // batch indices are kept
-  constexpr bool KEEP = MODE != kModeSort;
   Half<ITEMS> dig, rank;
-  if (KEEP) {
+  {
+    const U wlo = (U)J->wlo;
 #pragma unroll
-    for (int i = 0; i < ITEMS; ++i) dig.set(i, digit(w[i]));
+    for (int i = 0; i < ITEMS; ++i) {
+      uint64_t x;
+      if constexpr (RAW_IN)
+        x = wbase + i * 32 < nvalid ? (uint64_t)(U)((U)part[i] - wlo) << ib : pad;
+      else if constexpr (HI)
+        x = (uint64_t)part[i] << 32;
+      else
+        x = part[i];
+      dig.set(i, digit(x));
+    }
   }
-  int sh = shift;  // opaque to the compiler from phase to phase, see below
-  auto item_digit = [&](int i) -> uint32_t {
-    return KEEP ? dig.get(i) : wdigit<HI>(w[i], lo, sh, mask);
-  };
+  auto item_digit = [&](int i) -> uint32_t { return dig.get(i); };
   uint32_t* const t_cnt = reinterpret_cast<uint32_t*>(smem);  // [warp][digit]
   uint32_t* const t_mask = t_cnt + kWWarps * bins;
   wrank_bits<ITEMS>(item_digit, nbits, rank, t_cnt + warp * bins,
@@ -345,8 +345,6 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
   __syncthreads();
 
   // 3. positions (the tables die here), the look-back, the move
-  // (the digits are computed again, not carried in registers, which spilled)
-  asm volatile("" : "+r"(sh));
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i)
     rank.put(i, rank.get(i) + t_cnt[warp * bins + item_digit(i)]);
@@ -379,16 +377,50 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
     }
     s_gbase[d] = hist[d] + prefix - s_gbase[d];  // minus the digit's first slot
   }
+  {
+    const K* __restrict__ vp = RAW_IN ? J->fold_v[pass] + row0 : nullptr;
+    const U wlo = (U)J->wlo, ilo = (U)J->ilo;
+    uint64_t out = 0;
+    constexpr int G = RAW_IN && sizeof(K) == 8 ? (ITEMS % 8 == 0 ? 8 : ITEMS % 6 == 0 ? 6 : ITEMS / 2) : ITEMS;
 #pragma unroll
-  for (int i = 0; i < ITEMS; ++i) {
-    const uint32_t pos = rank.get(i);
-    stage[pos] = w[i];
-    if (MODE == kModeCuts) {
-      if (dig8)
-        s_dig8[pos] = (uint8_t)dig.get(i);
-      else
-        s_dig[pos] = (uint16_t)dig.get(i);
+    for (int i0 = 0; i0 < ITEMS; i0 += G) {
+      uint64_t w[G];
+      if constexpr (RAW_IN) {
+        K v[G], k[G];
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+          const int r = wbase + (i0 + i) * 32;
+          k[i] = r < nvalid ? kp[r] : K(0);
+          v[i] = r < nvalid ? vp[r] : K(0);
+        }
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+          const uint64_t ko = (uint64_t)(U)((U)k[i] - wlo), io = (uint64_t)(U)((U)v[i] - ilo);
+          if (sizeof(K) == 8 && wbase + (i0 + i) * 32 < nvalid) out |= (io >> ib) | (ko >> (64 - ib));
+          w[i] = (ko << ib) | (io & idm);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+          const int r = wbase + (i0 + i) * 32;
+          w[i] = r < nvalid ? wp[r] : 0ull;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        const uint32_t pos = rank.get(i0 + i);
+        stage[pos] = w[i];
+        if (MODE == kModeCuts) {
+          if (dig8)
+            s_dig8[pos] = (uint8_t)dig.get(i0 + i);
+          else
+            s_dig[pos] = (uint16_t)dig.get(i0 + i);
+        }
+      }
     }
+    if (RAW_IN && sizeof(K) == 8 && out != 0ull &&
+        wld_volatile(reinterpret_cast<const uint32_t*>(err)) == 0u)
+      atomicCAS(err, 0, kErrFold);
   }
   __syncthreads();
 
