@@ -510,6 +510,7 @@ void set_job_buffers(RadixJob<K>& j, const K* in_k, const K* in_v, K* ak, K* av,
 }
 
 // ---- folded rows (tj_word.cu) -------------------------------------------------------
+// (Rows that do not fit may still travel as a key and a 32-bit id, `wide_too`.)
 // A row is one 64-bit word, (key - wlo) << ib | (id - ilo), when the bits of
 // the key range and of the ids fit together; then every pass but the first and
 // the last moves 8 bytes a row.  32-bit rows always fit (ib = 32).  64-bit
@@ -518,13 +519,14 @@ void set_job_buffers(RadixJob<K>& j, const K* in_k, const K* in_v, K* ak, K* av,
 // one outside sends the call back to separate columns (kErrFold).
 struct Fold {
   bool on = false;
+  bool wide = false;  // wide rows instead: the key as it is and a 32-bit id
   uint64_t wlo = 0, ilo = 0;
   int ib = 0;
 };
 
 template <typename K>
 Fold make_fold(uint64_t lo, int key_bits, unsigned long long id_min_u,
-               unsigned long long id_max_u) {
+               unsigned long long id_max_u, bool wide_too) {
   Fold f;
   f.wlo = lo;
   if (sizeof(K) == 4) {
@@ -532,14 +534,18 @@ Fold make_fold(uint64_t lo, int key_bits, unsigned long long id_min_u,
     f.on = true;
     return f;
   }
-  const int avail = 64 - key_bits;
-  if (avail < 1 || avail > 63 || id_max_u < id_min_u) return f;
+  if (id_max_u < id_min_u) return f;
   const uint64_t range = id_max_u - id_min_u;
-  if (bitlen(range) > avail) return f;
+  int avail = 64 - key_bits;
+  if (avail < 1 || avail > 63 || bitlen(range) > avail) {
+    if (!wide_too || bitlen(range) > 32) return f;
+    f.wide = true;
+    avail = 32;
+  }
   const uint64_t window = ((uint64_t)1 << avail) - 1;
   f.ib = avail;
   f.ilo = (uint64_t)key_of<int64_t>(id_min_u) - (window - range) / 2;
-  f.on = true;
+  f.on = !f.wide;
   return f;
 }
 
@@ -573,12 +579,13 @@ Plan make_word_plan(uint64_t lo, uint64_t range, bool even, int max_digit, int m
 template <typename K>
 void set_word_plan(RadixJob<K>& j, const Plan& p, const Fold& f, uint64_t lo) {
   set_job_plan(j, p);
-  for (int i = 0; i < p.passes; ++i) j.shift[i] += f.ib;
-  j.lo = lo;
-  j.wlo = f.wlo;
   j.ilo = f.ilo;
   j.ib = f.ib;
+  j.wlo = f.wlo;
   j.dst_rows = j.n;
+  if (f.wide) return;  // digits of the keys as they are
+  for (int i = 0; i < p.passes; ++i) j.shift[i] += f.ib;
+  j.lo = lo;
 }
 
 // One word pass: from columns into words, or words to words (8 bytes a row
@@ -589,11 +596,11 @@ cudaError_t word_pass(const RadixJob<K>* d_jobs, int nj, int64_t tiles, int p, i
                       cudaStream_t st, const int32_t* d_tile_job = nullptr) {
   if (fold_in)
     return launch_wsweep<K>(d_jobs, nj, tiles, p, max_bits, kModeSort, true, false, f.ib >= 32,
-                            items, false, d_counter, d_err, st, d_tile_job);
+                            f.wide, items, false, d_counter, d_err, st, d_tile_job);
   static_assert(sizeof(RadixJob<K>) == sizeof(RadixJob<int64_t>), "one job layout");
   return launch_wsweep<int64_t>(reinterpret_cast<const RadixJob<int64_t>*>(d_jobs), nj, tiles, p,
-                                max_bits, kModeSort, false, false, f.ib >= 32, items, false,
-                                d_counter, d_err, st, d_tile_job);
+                                max_bits, kModeSort, false, false, f.ib >= 32, f.wide, items,
+                                false, d_counter, d_err, st, d_tile_job);
 }
 
 // Ping-pong of a word job: pass 0 reads the columns (fold_in) or the words
@@ -604,7 +611,7 @@ uint64_t* set_word_buffers(RadixJob<K>& j, const K* in_k, const K* in_v, uint64_
   const K* src = in_k;
   for (int p = 0; p < j.passes; ++p) {
     j.src_k[p] = src;
-    if (p == 0) j.fold_v[0] = in_v;
+    if (p == 0) j.fold_v = in_v;
     j.dst_k[p] = reinterpret_cast<K*>((p & 1) ? b : a);
     j.dst_v[p] = nullptr;
     src = j.dst_k[p];
@@ -816,9 +823,9 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
   // admits those admits these)
   const Fold fold = P > 0 ? make_fold<K>(plan.lo, plan.key_bits,
                                          std::min(hs[0].id_min_u, hs[1].id_min_u),
-                                         std::max(~hs[0].id_max_u, ~hs[1].id_max_u))
+                                         std::max(~hs[0].id_max_u, ~hs[1].id_max_u), true)
                           : Fold();
-  while (fold.on) {
+  while (fold.on || fold.wide) {
     const Plan wp = nr + ns >= kCostRows
                         ? make_word_plan(plan.lo, range_of<K>(lo, hi), false,
                                          max_digit_bits<K>(), 1)
@@ -831,6 +838,8 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     Carve wc;
     const size_t o_a = wc.add<uint64_t>((size_t)(nr + ns));
     const size_t o_b = wc.add<uint64_t>(wp.passes > 1 ? (size_t)(nr + ns) : 0);
+    const size_t o_ai = wc.add<uint32_t>(fold.wide ? (size_t)(nr + ns) : 0);
+    const size_t o_bi = wc.add<uint32_t>(fold.wide && wp.passes > 1 ? (size_t)(nr + ns) : 0);
     const size_t o_wt = wc.add<JTile<K>>(jtiles);
     const size_t o_whist = wc.add<uint32_t>((size_t)2 * wp.passes << wp.max_bits);
     const size_t o_wjlb = wc.add<uint64_t>(jtiles);
@@ -841,6 +850,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     TJ_CUDA(big.alloc(wc.off, st));
     RadixJob<K> hw[4] = {hj[0], hj[1], hj[0], hj[1]};
     uint64_t* res[2];
+    const K* res_i[2] = {nullptr, nullptr};
     for (int i = 0; i < 2; ++i) {
       RadixJob<K>& h = hw[i];
       RadixJob<K>& x = hw[2 + i];
@@ -856,13 +866,17 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
       uint64_t* a = big.at<uint64_t>(o_a) + (i ? nr : 0);
       uint64_t* b = big.at<uint64_t>(o_b) + (i ? nr : 0);
       res[i] = set_word_buffers(x, i ? ks : kr, i ? is : ir, a, b);
+      for (int p = 0; fold.wide && p < wp.passes; ++p) {
+        x.dst_v[p] = reinterpret_cast<K*>(big.at<uint32_t>((p & 1) ? o_bi : o_ai) + (i ? nr : 0));
+        res_i[i] = x.dst_v[p];
+      }
     }
     JoinJob<K> jj;
     jj.rk = reinterpret_cast<const K*>(res[0]);
-    jj.rv = nullptr;
+    jj.rv = res_i[0];
     jj.nr = nr;
     jj.sk = reinterpret_cast<const K*>(res[1]);
-    jj.sv = nullptr;
+    jj.sv = res_i[1];
     jj.ns = ns;
     jj.tile0 = 0;
     TJ_CUDA(put_small(d_jobs, hw, sizeof(hw), st));
@@ -874,19 +888,21 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     TJ_CUDA(launch_histogram<K>(d_jobs, 2, tiles_r + tiles_s, st));
     tr.end();
     TJ_CUDA(launch_digit_scan<K>(d_jobs, 2, wp.passes, st));
+    const double rowb = fold.wide ? 12.0 : 8.0;
     for (int p = 0; p < wp.passes; ++p) {
       if (!regions) TJ_CUDA(cudaMemsetAsync(big.p + o_wlb, 0, (size_t)lb_words * 4, st));
-      tr.begin("onesweep", ((p ? 8.0 : 2.0 * w) + 8.0) * (nr + ns));
+      tr.begin("onesweep", ((p ? rowb : 2.0 * w) + rowb) * (nr + ns));
       TJ_CUDA(word_pass<K>(d_jobs + 2, 2, wt, p, wp.max_bits, p == 0, fold, items,
                            d_counters + p, d_err, st));
       tr.end();
     }
     WordFmt fmt;
-    fmt.ib = fold.ib;
+    fmt.ib = fold.wide ? 0 : fold.ib;
+    fmt.wide = fold.wide;
     fmt.ilo = fold.ilo;
     JTile<K>* d_tiles = big.at<JTile<K>>(o_wt);
     TJ_CUDA(launch_tile_ranges<K>(d_jj, 1, jtiles, d_tiles, st, nullptr, fmt, d_err));
-    tr.begin("join", 8.0 * (nr + ns));
+    tr.begin("join", rowb * (nr + ns));
     TJ_CUDA(launch_join<K>(jtiles, d_tiles, big.at<uint64_t>(o_wjlb), d_counters + kMaxPasses,
                            out, cap, nullptr, nullptr, d_total, d_err, st, fmt));
     tr.end();
@@ -1307,14 +1323,14 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   }
   if (o.fused && o.fold) {
     if (sizeof(K) == 4) {
-      fold = make_fold<K>(lo_bits<K>(std::numeric_limits<K>::min()), 32, 0, 0);
+      fold = make_fold<K>(lo_bits<K>(std::numeric_limits<K>::min()), 32, 0, 0, false);
     } else {
       const uint64_t range = range_of<K>(lo, hi);
       const uint64_t slack = range_known ? 0 : range / 32 + 1024;
       if (range + 2 * slack >= range && range + 2 * slack < ((uint64_t)1 << 62)) {
         const int kw = std::max(1, bitlen(range + 2 * slack));
         const uint64_t spare = range_known ? 0 : ((((uint64_t)1 << kw) - 1) - range) / 2;
-        fold = make_fold<K>(lo_bits<K>(lo) - spare, kw, id_min_u, id_max_u);
+        fold = make_fold<K>(lo_bits<K>(lo) - spare, kw, id_min_u, id_max_u, false);
       }
     }
   }
@@ -1511,7 +1527,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     x.hist_stride = kMaxBins;
     x.hist = stg.at<uint32_t>(o_hist) + (size_t)c * kMaxBins;
     x.src_k[0] = kb + ch.r0;
-    x.src_v[0] = vb + ch.r0;  // (folded rows: fold_v[0])
+    x.src_v[0] = vb + ch.r0;  // (folded rows: fold_v)
     x.dst_k[0] = routed(stg, ch.side, 0);
     x.dst_v[0] = words ? nullptr : ch.side ? stg.at<K>(o_sv) : stg.at<K>(o_rv);
     x.cuts = radix_route ? nullptr : stg.at<K>(o_cuts);  // radix: the digit path
@@ -1627,8 +1643,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     tr.begin("route", (2.0 * w + rowb) * rows);
     if (words)
       TJ_CUDA(launch_wsweep<K>(d_rj + nch + g.first, g.second - g.first, t, 0, rbits,
-                               radix_route ? kModeRadix : kModeCuts, true, false, ib >= 32, kWItems,
-                               est, d_counters + kMaxPasses, d_err, st));
+                               radix_route ? kModeRadix : kModeCuts, true, false, ib >= 32, false,
+                               kWItems, est, d_counters + kMaxPasses, d_err, st));
     else
       TJ_CUDA(launch_onesweep<K>(d_rj + nch + g.first, g.second - g.first, t, 0, rbits,
                                  radix_route ? kModeRadix : kModeCuts, d_counters + kMaxPasses,
@@ -2463,7 +2479,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
 // the words alternating between two scratch arrays, so the caller's columns
 // stay as they are until the last pass (which does not run if a row failed to
 // fold).  32-bit rows always fold and a word is no smaller than a row: their
-// passes alternate between one array of words and the caller's columns.
+// passes alternate between one array of words and the caller's columns, and so
+// do wide rows (a pass that unfolds does not run after a row failed to fold).
 template <typename K>
 tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f,
                      RadixJob<K>* d_jobs, uint32_t* d_counters, int* d_err, size_t ctl_bytes,
@@ -2477,8 +2494,10 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
   // cleared before every pass
   const bool regions = (int64_t)P * lb_words * 4 <= (int64_t)1 << 20;
   Carve bc;
+  const bool turns = sizeof(K) == 4 || f.wide;  // columns, one scratch array, columns, ...
   const size_t o_a = bc.add<uint64_t>((size_t)n);
-  const size_t o_b = bc.add<uint64_t>(sizeof(K) == 8 && P > 2 ? (size_t)n : 0);
+  const size_t o_ai = bc.add<uint32_t>(f.wide ? (size_t)n : 0);
+  const size_t o_b = bc.add<uint64_t>(!turns && P > 2 ? (size_t)n : 0);
   const size_t o_hist = bc.add<uint32_t>((size_t)P << plan.max_bits);
   const size_t o_lb = bc.add<uint32_t>((size_t)(regions ? P : 1) * lb_words);
   Block big;
@@ -2495,18 +2514,18 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
   set_word_plan(hj[1], plan, f, 0);
   hj[1].lookback = big.at<uint32_t>(o_lb);
   hj[1].lb_stride = regions ? lb_words : 0;
-  auto folds = [&](int p) { return p == 0 || (sizeof(K) == 4 && (p & 1) == 0); };
-  auto unfolds = [&](int p) { return p == P - 1 || (sizeof(K) == 4 && (p & 1) == 1); };
+  auto folds = [&](int p) { return p == 0 || (turns && (p & 1) == 0); };
+  auto unfolds = [&](int p) { return p == P - 1 || (turns && (p & 1) == 1); };
   uint64_t* a = big.at<uint64_t>(o_a);
   uint64_t* b = big.at<uint64_t>(o_b);
   for (int p = 0; p < P; ++p) {
-    K* in = reinterpret_cast<K*>(sizeof(K) == 4 || (p & 1) ? a : b);
-    K* to = reinterpret_cast<K*>(sizeof(K) == 4 || !(p & 1) ? a : b);
+    K* in = reinterpret_cast<K*>(turns || (p & 1) ? a : b);
+    K* to = reinterpret_cast<K*>(turns || !(p & 1) ? a : b);
     hj[1].src_k[p] = folds(p) ? keys : in;
-    if (folds(p)) hj[1].fold_v[p] = ids;
     hj[1].dst_k[p] = unfolds(p) ? keys : to;
-    hj[1].dst_v[p] = unfolds(p) ? ids : nullptr;
+    hj[1].dst_v[p] = unfolds(p) ? ids : f.wide ? reinterpret_cast<K*>(big.at<uint32_t>(o_ai)) : nullptr;
   }
+  hj[1].fold_v = ids;  // (the columns any pass that folds reads)
   TJ_CUDA(put_small(d_jobs, hj, sizeof(hj), st));
   TJ_CUDA(cudaMemsetAsync(big.p + o_hist, 0,
                           (regions ? o_lb + (size_t)P * lb_words * 4 : o_lb) - o_hist, st));
@@ -2516,9 +2535,11 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
   TJ_CUDA(launch_digit_scan<K>(d_jobs, 1, P, st));
   for (int p = 0; p < P; ++p) {
     if (!regions) TJ_CUDA(cudaMemsetAsync(big.p + o_lb, 0, (size_t)lb_words * 4, st));
-    tr.begin("onesweep", (2.0 * ((folds(p) ? w : 4.0) + (unfolds(p) ? w : 4.0))) * n);
+    const double rowb = f.wide ? 12.0 : 8.0;
+    tr.begin("onesweep", ((folds(p) ? 2.0 * w : rowb) + (unfolds(p) ? 2.0 * w : rowb)) * n);
     TJ_CUDA(launch_wsweep<K>(d_jobs + 1, 1, otiles, p, plan.max_bits, kModeSort, folds(p),
-                             unfolds(p), f.ib >= 32, items, false, d_counters + p, d_err, st));
+                             unfolds(p), f.ib >= 32, f.wide, items, false, d_counters + p, d_err,
+                             st));
     tr.end();
   }
   return TJ_OK;
@@ -2573,12 +2594,12 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
     g_stats = stats;
     return TJ_OK;
   }
-  const Fold fold = make_fold<K>(plan.lo, plan.key_bits, hs.id_min_u, ~hs.id_max_u);
-  if (fold.on) {
+  const Fold fold = make_fold<K>(plan.lo, plan.key_bits, hs.id_min_u, ~hs.id_max_u, true);
+  if (fold.on || fold.wide) {
     // (below kCostRows a pass's fixed cost decides: the fewest passes)
     const Plan wplan = n >= kCostRows
-                           ? make_word_plan(plan.lo, range_of<K>(lo, hi), sizeof(K) == 4,
-                                            max_digit_bits<K>(), 2)
+                           ? make_word_plan(plan.lo, range_of<K>(lo, hi),
+                                            sizeof(K) == 4 || fold.wide, max_digit_bits<K>(), 2)
                            : plan;
     stats.radix_passes = wplan.passes;
     stats.digit_bits = wplan.max_bits;

@@ -101,10 +101,6 @@ template <typename K> struct UnsignedOf;
 template <> struct UnsignedOf<int32_t> { using type = uint32_t; };
 template <> struct UnsignedOf<int64_t> { using type = uint64_t; };
 
-// passes of a word job that may read columns: 32-bit rows take at most 4 passes
-// and fold in every other one, 64-bit rows only in the first
-constexpr int kFoldPasses = 4;
-
 // ---- per-array radix job ---------------------------------------------------
 // One array being sorted by (key - lo) over `passes` LSD digits.  Pass p reads
 // src_k/src_v[p] and writes dst_k/dst_v[p] (ping-pong buffers).
@@ -127,11 +123,11 @@ struct RadixJob {
   // Word passes read `lo` and `shift` as offsets and positions within words
   // (route passes: lo = the range's first key - wlo, route_hi = its width,
   // cuts = offsets from wlo); src_k / dst_k are words except where a pass reads
-  // or writes columns, which only passes below kFoldPasses read.
+  // or writes columns.
   union {
     const K* src_v[kMaxPasses];
     struct {
-      const K* fold_v[kFoldPasses];
+      const K* fold_v;  // the id column of passes that fold
       uint64_t wlo, ilo;
       int64_t dst_rows;  // room at dst_k (rows) of a pass that folds
       const K* ids;      // statistics: ids sampled beside the keys (may be null)
@@ -191,6 +187,7 @@ struct KeyStats {
 // or folded rows, whose job and tile pointers (rk, sk) are words.
 struct WordFmt {
   int32_t ib = 0;
+  bool wide = false;  // separate columns whose ids are 32-bit offsets from ilo
   uint64_t ilo = 0;
 };
 
@@ -385,12 +382,13 @@ cudaError_t word_init_attributes();
 // One onesweep pass over folded rows; tiles of kWThreads * items rows (items =
 // kWItems or, sort digits only, kWItemsSmall).  raw_in: reads key and id
 // columns and folds them; raw_out: writes columns; hi: every job's shift is at
-// least 32 and its lo a multiple of 2^32 (always so for 32-bit keys).
+// least 32 and its lo a multiple of 2^32 (always so for 32-bit keys); wide: rows
+// of a 64-bit key and a 32-bit id (sort digits of 64-bit keys only).
 template <typename K>
 cudaError_t launch_wsweep(const RadixJob<K>* d_jobs, int num_jobs, int64_t total_tiles, int pass,
-                          int max_bits, int mode, bool raw_in, bool raw_out, bool hi, int items,
-                          bool guard, uint32_t* d_tile_counter, int* d_err, cudaStream_t st,
-                          const int32_t* d_tile_job = nullptr);
+                          int max_bits, int mode, bool raw_in, bool raw_out, bool hi, bool wide,
+                          int items, bool guard, uint32_t* d_tile_counter, int* d_err,
+                          cudaStream_t st, const int32_t* d_tile_job = nullptr);
 
 // ---- launchers (tj_join.cu) -------------------------------------------------
 cudaError_t join_init_attributes();

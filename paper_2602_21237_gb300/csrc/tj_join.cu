@@ -51,22 +51,33 @@ __device__ __forceinline__ uint32_t ht_hash(uint32_t k) { return ht_hash((int32_
 
 // How a join kernel reads rows: W = 0, separate columns (an element is a key);
 // W = 1, folded rows (tj_word.cu), keys of up to 63 bits; W = 2, folded rows
-// whose key offset lies in the word's upper half (compared in 32 bits).
+// whose key offset lies in the word's upper half (compared in 32 bits); W = 3,
+// separate columns with 32-bit ids.  V: an element of the id column.
 template <typename K, int W>
 struct RowOf {
   using E = uint64_t;
+  using V = uint64_t;  // (no id column)
   using Key = uint64_t;
   static __device__ __forceinline__ Key key(E e, int ib) { return e >> ib; }
 };
 template <typename K>
 struct RowOf<K, 0> {
   using E = K;
+  using V = K;
+  using Key = K;
+  static __device__ __forceinline__ Key key(E e, int) { return e; }
+};
+template <typename K>
+struct RowOf<K, 3> {
+  using E = K;
+  using V = uint32_t;
   using Key = K;
   static __device__ __forceinline__ Key key(E e, int) { return e; }
 };
 template <typename K>
 struct RowOf<K, 2> {
   using E = uint64_t;
+  using V = uint64_t;
   using Key = uint32_t;
   static __device__ __forceinline__ Key key(E e, int ib) {
     return (uint32_t)(e >> 32) >> (ib & 31);
@@ -100,13 +111,14 @@ __device__ __forceinline__ void st_volatile_u64(uint64_t* p, uint64_t v) {
 // key >= the tile's first key, lanes 16-31 the first R row with key > the
 // tile's last key, each by a 16-ary search (16 probes per round trip); lane 0
 // writes the tile's descriptor, so a join tile needs one load to start.
-template <typename K, bool WORDS>
+template <typename K, int W>
 __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
                               int64_t total_tiles, JTile<K>* __restrict__ tiles,
                               const int32_t* __restrict__ tile_job, int ib,
                               const int* __restrict__ err) {
-  using Row = RowOf<K, WORDS ? 1 : 0>;
+  using Row = RowOf<K, W>;
   using E = typename Row::E;
+  using V = typename Row::V;
   const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (t >= total_tiles) return;  // whole warps leave together
   const int lane = threadIdx.x & 31, sub = lane & 15;
@@ -159,9 +171,9 @@ __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
   if (lane == 0) {
     JTile<K> d;
     d.sk = J->sk + row0;
-    d.sv = J->sv + row0;
+    d.sv = reinterpret_cast<const K*>(reinterpret_cast<const V*>(J->sv) + row0);
     d.rk = J->rk + res;
-    d.rv = J->rv + res;
+    d.rv = reinterpret_cast<const K*>(reinterpret_cast<const V*>(J->rv) + res);
     d.lt = t - J->tile0;
     d.nrr = b - res;
     d.nv = (int32_t)(row1 - row0);
@@ -183,8 +195,9 @@ constexpr int kJWarps = kJThreads / 32;
 constexpr int kJItems = kJTile / kJThreads;     // S rows per thread
 static_assert(kJItems * kJThreads == kJTile, "join tile = threads x items");
 
-// Shared memory: S keys | S ids (kJTile + kPad each) | R keys | R ids (kRCap +
-// kPad each) | hash table[kHTSlots] u32; folded rows: S words | R words | table.  Each staged array starts up to kPad
+// Shared memory: S keys | R keys | S ids | R ids (kJTile or kRCap elements and
+// kPad more each) | hash table[kHTSlots] u32; folded rows: S words | R words |
+// table.  Each staged array starts up to kPad
 // elements into its area (its first element keeps the source's address modulo
 // 16, so that all but a head and a tail move in 16-byte copies).  After the
 // probe the many-matches write path (which reads ids from global memory)
@@ -196,8 +209,10 @@ __host__ __device__ constexpr int join_pad() {
 template <typename K, int W>
 constexpr size_t join_smem_bytes() {
   using E = typename RowOf<K, W>::E;
-  return sizeof(E) * (size_t)(W ? 1 : 2) *
-             (size_t)(kJTile + join_pad<E>() + kRCap + join_pad<E>()) +
+  using V = typename RowOf<K, W>::V;
+  constexpr bool ids = W == 0 || W == 3;
+  return sizeof(E) * (size_t)(kJTile + join_pad<E>() + kRCap + join_pad<E>()) +
+         (ids ? sizeof(V) * (size_t)(kJTile + join_pad<V>() + kRCap + join_pad<V>()) : 0) +
          sizeof(uint32_t) * kHTSlots;
 }
 static_assert(sizeof(uint64_t) * (kJTile + kRCap) >= (sizeof(uint64_t) + sizeof(uint32_t)) * kJTile,
@@ -263,13 +278,17 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   using E = typename Row::E;
   using Key = typename Row::Key;
   const int ib = f.ib;
-  constexpr int kPad = join_pad<E>();
-  constexpr int kCols = W ? 1 : 2;  // arrays a relation's rows take
+  using V = typename Row::V;
+  constexpr bool kIds = W == 0 || W == 3;  // an id column beside the keys
+  constexpr int kPad = join_pad<E>(), kPadV = join_pad<V>();
   E* const b_sk = reinterpret_cast<E*>(smem);  // staging areas (16-byte aligned)
-  E* const b_sv = b_sk + kJTile + kPad;        // (W == 0 only)
-  E* const b_rk = b_sk + kCols * (kJTile + kPad);
-  E* const b_rv = b_rk + kRCap + kPad;  // (W == 0 only)
-  uint32_t* s_ht = reinterpret_cast<uint32_t*>(b_rk + kCols * (kRCap + kPad));
+  E* const b_rk = b_sk + kJTile + kPad;
+  V* const b_sv = reinterpret_cast<V*>(b_rk + kRCap + kPad);  // (kIds only)
+  V* const b_rv = b_sv + kJTile + kPadV;
+  uint32_t* s_ht = kIds ? reinterpret_cast<uint32_t*>(b_rv + kRCap + kPadV)
+                        : reinterpret_cast<uint32_t*>(b_sv);
+  // an id column's element as the caller's id
+  auto id_of = [&](V v) -> K { return W == 3 ? (K)((uint64_t)v + f.ilo) : (K)v; };
   __shared__ uint64_t s_wsum[kJWarps];
   __shared__ uint64_t s_base;
   __shared__ uint32_t s_t;
@@ -285,25 +304,25 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   const int64_t lt = T.lt;
   const int nv = T.nv;
   const E* __restrict__ rk_g = reinterpret_cast<const E*>(T.rk);
-  const K* __restrict__ rv_g = T.rv;
+  const V* __restrict__ rv_g = reinterpret_cast<const V*>(T.rv);
   // id of R row i of the tile's range, read from global memory
   auto rid_g = [&](int64_t i) -> K {
-    if constexpr (W != 0) return word_id<K>(rk_g[i], f);
-    else return rv_g[i];
+    if constexpr (!kIds) return word_id<K>(rk_g[i], f);
+    else return id_of(rv_g[i]);
   };
   const int64_t nchunks = (nrr + kRCap - 1) / kRCap;
   const bool onchip = nchunks <= kMaxChunks;
 
   // 1. stage S and the first R chunk
   const E* s_sk = join_copy_async<E>(b_sk, reinterpret_cast<const E*>(T.sk), nv);
-  const E* s_sv = b_sv;
+  const V* s_sv = b_sv;
   E* s_rk = b_rk;  // the staged R chunk (where its copy starts)
-  E* s_rv = b_rv;
-  if constexpr (W == 0) s_sv = join_copy_async<E>(b_sv, T.sv, nv);
+  V* s_rv = b_rv;
+  if constexpr (kIds) s_sv = join_copy_async<V>(b_sv, reinterpret_cast<const V*>(T.sv), nv);
   if (onchip && nchunks > 0) {
     const int nc0 = (int)min((int64_t)kRCap, nrr);
     s_rk = join_copy_async<E>(b_rk, rk_g, nc0);
-    if constexpr (W == 0) s_rv = join_copy_async<E>(b_rv, rv_g, nc0);
+    if constexpr (kIds) s_rv = join_copy_async<V>(b_rv, rv_g, nc0);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 
@@ -319,7 +338,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
       if (c > 0) {
         __syncthreads();  // the previous chunk's probes are done
         s_rk = join_copy_async<E>(b_rk, rk_g + c0, nc);
-        if constexpr (W == 0) s_rv = join_copy_async<E>(b_rv, rv_g + c0, nc);
+        if constexpr (kIds) s_rv = join_copy_async<V>(b_rv, rv_g + c0, nc);
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
       for (int i = tid; i < kHTSlots; i += kJThreads) s_ht[i] = kHTEmpty;
@@ -536,12 +555,12 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         const uint64_t o = off + __popc(m & ltm);
         const int64_t st0 = (int64_t)start[u];
         K sid, rid;
-        if constexpr (W != 0) {
+        if constexpr (!kIds) {
           sid = word_id<K>(s_sk[wbase + u * 32 + lane], f);
           rid = st0 >= cres ? word_id<K>(s_rk[st0 - cres], f) : rid_g(st0);
         } else {
-          sid = s_sv[wbase + u * 32 + lane];
-          rid = st0 >= cres ? s_rv[st0 - cres] : rid_g(st0);
+          sid = id_of(s_sv[wbase + u * 32 + lane]);
+          rid = st0 >= cres ? id_of(s_rv[st0 - cres]) : rid_g(st0);
         }
         if (vec) {
           P pr;
@@ -601,7 +620,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
       }
     }
     __syncthreads();
-    const K* __restrict__ sv_g = T.sv;
+    const V* __restrict__ sv_g = reinterpret_cast<const V*>(T.sv);
     const E* __restrict__ sk_g = reinterpret_cast<const E*>(T.sk);
     K* __restrict__ o = out + 2 * first;
     for (uint64_t x = tid; x < C; x += kJThreads) {
@@ -615,8 +634,8 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
       }
       const uint64_t r = s_rs[lo] + (x - s_off[lo]);
       o[2 * x] = rid_g((int64_t)r);
-      if constexpr (W != 0) o[2 * x + 1] = word_id<K>(sk_g[lo], f);
-      else o[2 * x + 1] = sv_g[lo];
+      if constexpr (!kIds) o[2 * x + 1] = word_id<K>(sk_g[lo], f);
+      else o[2 * x + 1] = id_of(sv_g[lo]);
     }
   }
 }
@@ -629,12 +648,15 @@ cudaError_t launch_tile_ranges(const JoinJob<K>* d_jobs, int num_jobs, int64_t t
   if (total_tiles <= 0) return cudaSuccess;
   const unsigned grid = (unsigned)((total_tiles * 32 + kThreads - 1) / kThreads);
   if (f.ib)  // words: the pointers step 8 bytes a row whatever K
-    k_tile_ranges<int64_t, true><<<grid, kThreads, 0, st>>>(
+    k_tile_ranges<int64_t, 1><<<grid, kThreads, 0, st>>>(
         reinterpret_cast<const JoinJob<int64_t>*>(d_jobs), num_jobs, total_tiles,
         reinterpret_cast<JTile<int64_t>*>(d_tiles), d_tile_job, f.ib, d_err);
+  else if (f.wide)
+    k_tile_ranges<K, 3><<<grid, kThreads, 0, st>>>(d_jobs, num_jobs, total_tiles, d_tiles,
+                                                   d_tile_job, 0, d_err);
   else
-    k_tile_ranges<K, false><<<grid, kThreads, 0, st>>>(d_jobs, num_jobs, total_tiles, d_tiles,
-                                                       d_tile_job, 0, d_err);
+    k_tile_ranges<K, 0><<<grid, kThreads, 0, st>>>(d_jobs, num_jobs, total_tiles, d_tiles,
+                                                   d_tile_job, 0, d_err);
   return cudaGetLastError();
 }
 
@@ -693,7 +715,9 @@ cudaError_t launch_join(int64_t total_tiles, const JTile<K>* d_tiles, uint64_t* 
   k_join<K, W><<<(unsigned)total_tiles, kJThreads, join_smem_bytes<K, W>(), st>>>(            \
       total_tiles, d_tiles, f, d_lookback, d_tile_counter, out, capacity, d_out_base,         \
       d_job_out, d_total, d_err)
-  if (f.ib >= 32) {
+  if (f.wide) {
+    if constexpr (sizeof(K) == 8) TJ_JOIN(3);
+  } else if (f.ib >= 32) {
     TJ_JOIN(2);
   } else if (f.ib > 0) {
     if constexpr (sizeof(K) == 8) TJ_JOIN(1);  // 32-bit rows always have ib = 32
@@ -817,6 +841,7 @@ cudaError_t join_init_attributes() {
   if (e == cudaSuccess) e = join_attr<int64_t, 0>();
   if (e == cudaSuccess) e = join_attr<int64_t, 1>();
   if (e == cudaSuccess) e = join_attr<int64_t, 2>();
+  if (e == cudaSuccess) e = join_attr<int64_t, 3>();
   return e;
 }
 

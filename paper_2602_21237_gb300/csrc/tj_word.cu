@@ -9,6 +9,10 @@
 // rows), and a row is one load, one shared-memory slot and one store instead
 // of two of each plus an index.
 //
+// Rows too wide for one word (64-bit keys whose range and ids need more than 64
+// bits) travel as "wide" rows, the key as it is beside a 32-bit id, when their
+// ids' range fits 32 bits.
+//
 // k_wsweep is one onesweep pass (decoupled look-back, as k_onesweep in
 // tj_radix.cu) over a tile of kWThreads * ITEMS rows: take the digits, rank
 // them inside the warp, move the words to their tile-sorted slots in shared
@@ -103,12 +107,13 @@ __host__ __device__ constexpr size_t wtable_bytes(int nbits) {
 }
 
 // Shared memory: the tile's words in tile-sorted order, overlaid with the
-// ranking tables (dead before the words move) | global base and tile
+// ranking tables (dead before the words move; wide rows: keys, then ids) |
+// global base and tile
 // count per digit | end of each batch's region (guarded route passes) | cut
 // keys, radix index and slot digits (route passes by the cut table).
 template <int ITEMS>
-__host__ __device__ constexpr size_t wsweep_smem_bytes(int nbits, int mode, bool guard) {
-  const size_t stage = 8u * (size_t)kWThreads * ITEMS;
+__host__ __device__ constexpr size_t wsweep_smem_bytes(int nbits, int mode, bool guard, bool wide) {
+  const size_t stage = (wide ? 12u : 8u) * (size_t)kWThreads * ITEMS;
   const size_t bins = (size_t)1 << nbits;
   return (stage > wtable_bytes(nbits) ? stage : wtable_bytes(nbits)) + 8u * bins +
          (mode != kModeSort && guard ? 4u * bins : 0u) +
@@ -182,7 +187,9 @@ __device__ __forceinline__ int wlookback(const uint32_t (&v)[W], uint32_t& prefi
 // the batch under equal-width ranges or the cut table).  HI: see wdigit.
 // After rows failed to fold, the later passes return at once, so a RAW_OUT
 // pass never overwrites the caller's columns with them.
-template <typename K, bool RAW_IN, bool RAW_OUT, int MODE, bool HI, int ITEMS>
+// WIDE: rows are a key and a 32-bit id (src / dst columns of 8 and 4 bytes; a
+// pass after the first reads the ids where the one before wrote them).
+template <typename K, bool RAW_IN, bool RAW_OUT, int MODE, bool HI, bool WIDE, int ITEMS>
 __global__ void __launch_bounds__(kWThreads, kWMinB)
     k_wsweep(const RadixJob<K>* __restrict__ jobs, int num_jobs, int64_t total_tiles, int pass,
              uint32_t* __restrict__ tile_counter, int* __restrict__ err,
@@ -190,6 +197,7 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
   using U = typename UnsignedOf<K>::type;
   constexpr int TILE = kWThreads * ITEMS;
   static_assert(TILE <= 65536, "16-bit positions within a tile");
+  static_assert(!WIDE || (sizeof(K) == 8 && !HI && MODE == kModeSort), "wide rows: 64-bit sorts");
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ uint32_t s_warp[kWWarps];
   __shared__ uint32_t s_t;
@@ -221,7 +229,9 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
 
   uint64_t* const stage = reinterpret_cast<uint64_t*>(smem);
   const size_t tab_bytes = wtable_bytes(nbits);
-  const size_t area = 8u * (size_t)TILE > tab_bytes ? 8u * (size_t)TILE : tab_bytes;
+  constexpr size_t kStage = (WIDE ? 12u : 8u) * (size_t)TILE;
+  const size_t area = kStage > tab_bytes ? kStage : tab_bytes;
+  uint32_t* const stage_v = reinterpret_cast<uint32_t*>(smem + 8u * (size_t)TILE);  // WIDE
   uint32_t* const s_gbase = reinterpret_cast<uint32_t*>(smem + area);
   uint32_t* const s_cnt = s_gbase + bins;
   uint32_t* const s_rend = s_cnt + bins;
@@ -279,7 +289,9 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
       uint64_t x;
-      if constexpr (RAW_IN)
+      if constexpr (RAW_IN && WIDE)
+        x = wbase + i * 32 < nvalid ? (uint64_t)part[i] : pad;
+      else if constexpr (RAW_IN)
         x = wbase + i * 32 < nvalid ? (uint64_t)(U)((U)part[i] - wlo) << ib : pad;
       else if constexpr (HI)
         x = (uint64_t)part[i] << 32;
@@ -378,14 +390,33 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
     s_gbase[d] = hist[d] + prefix - s_gbase[d];  // minus the digit's first slot
   }
   {
-    const K* __restrict__ vp = RAW_IN ? J->fold_v[pass] + row0 : nullptr;
+    const K* __restrict__ vp = RAW_IN ? J->fold_v + row0 : nullptr;
     const U wlo = (U)J->wlo, ilo = (U)J->ilo;
     uint64_t out = 0;
-    constexpr int G = RAW_IN && sizeof(K) == 8 ? (ITEMS % 8 == 0 ? 8 : ITEMS % 6 == 0 ? 6 : ITEMS / 2) : ITEMS;
+    // (pairs of 64-bit columns: half of the rows at a time, to spare registers)
+    constexpr int G = (RAW_IN && sizeof(K) == 8) || WIDE ? ITEMS / 2 : ITEMS;
+    static_assert(ITEMS % G == 0, "whole groups");
+    const uint32_t* __restrict__ ip =
+        WIDE && !RAW_IN ? reinterpret_cast<const uint32_t*>(J->dst_v[pass - 1]) + row0 : nullptr;
 #pragma unroll
     for (int i0 = 0; i0 < ITEMS; i0 += G) {
       uint64_t w[G];
-      if constexpr (RAW_IN) {
+      uint32_t id[WIDE ? G : 1];
+      if constexpr (RAW_IN && WIDE) {
+        K v[G];
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+          const int r = wbase + (i0 + i) * 32;
+          w[i] = r < nvalid ? (uint64_t)kp[r] : 0ull;
+          v[i] = r < nvalid ? vp[r] : (K)ilo;
+        }
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+          const uint64_t io = (uint64_t)(U)((U)v[i] - ilo);
+          out |= io >> 32;
+          id[i] = (uint32_t)io;
+        }
+      } else if constexpr (RAW_IN) {
         K v[G], k[G];
 #pragma unroll
         for (int i = 0; i < G; ++i) {
@@ -404,12 +435,14 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
         for (int i = 0; i < G; ++i) {
           const int r = wbase + (i0 + i) * 32;
           w[i] = r < nvalid ? wp[r] : 0ull;
+          if constexpr (WIDE) id[i] = r < nvalid ? ip[r] : 0u;
         }
       }
 #pragma unroll
       for (int i = 0; i < G; ++i) {
         const uint32_t pos = rank.get(i0 + i);
         stage[pos] = w[i];
+        if constexpr (WIDE) stage_v[pos] = id[i];
         if (MODE == kModeCuts) {
           if (dig8)
             s_dig8[pos] = (uint8_t)dig.get(i0 + i);
@@ -439,7 +472,10 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
       const uint32_t d = MODE == kModeCuts ? (dig8 ? (uint32_t)s_dig8[q] : (uint32_t)s_dig[q])
                                            : digit(x);
       const uint32_t g = s_gbase[d] + (uint32_t)q;
-      if (RAW_OUT) {
+      if constexpr (RAW_OUT && WIDE) {
+        dst_k[g] = (K)x;
+        dst_v[g] = (K)((U)stage_v[q] + ilo);
+      } else if constexpr (RAW_OUT) {
         dst_k[g] = (K)((U)(x >> ib) + wlo);
         dst_v[g] = (K)((U)(x & idm) + ilo);
       } else {
@@ -448,7 +484,10 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
         // not fold may miscount, so a folding pass keeps to its destination
         const bool in = MODE != kModeSort && guard ? g < s_rend[d] : !RAW_IN || g < room;
         over |= !in;
-        if (in) dst_w[g] = x;
+        if (in) {
+          dst_w[g] = x;
+          if constexpr (WIDE) reinterpret_cast<uint32_t*>(dst_v)[g] = stage_v[q];
+        }
       }
     }
   }
@@ -458,16 +497,16 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-template <typename K, bool RI, bool RO, int MODE, bool HI, int ITEMS>
+template <typename K, bool RI, bool RO, int MODE, bool HI, bool WIDE, int ITEMS>
 cudaError_t wsweep_attr() {
   size_t m = 0;
   for (int b = 1; b <= kMaxDigitBits; ++b)
-    m = std::max(m, wsweep_smem_bytes<ITEMS>(b, MODE, MODE != kModeSort));
-  return cudaFuncSetAttribute(k_wsweep<K, RI, RO, MODE, HI, ITEMS>,
+    m = std::max(m, wsweep_smem_bytes<ITEMS>(b, MODE, MODE != kModeSort, WIDE));
+  return cudaFuncSetAttribute(k_wsweep<K, RI, RO, MODE, HI, WIDE, ITEMS>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m);
 }
 
-template <typename K, bool RI, bool RO, int MODE, bool HI, int ITEMS>
+template <typename K, bool RI, bool RO, int MODE, bool HI, bool WIDE, int ITEMS>
 cudaError_t wsweep_go(const RadixJob<K>* d_jobs, int num_jobs, int64_t tiles, int pass,
                       int max_bits, bool guard, uint32_t* d_counter, int* d_err, cudaStream_t st,
                       const int32_t* d_tile_job) {
@@ -475,75 +514,105 @@ cudaError_t wsweep_go(const RadixJob<K>* d_jobs, int num_jobs, int64_t tiles, in
   // a launch over jobs of several digit widths takes the widest one's layout
   size_t smem = 0;
   for (int b = 1; b <= max_bits; ++b)
-    smem = std::max(smem, wsweep_smem_bytes<ITEMS>(b, MODE, guard));
-  k_wsweep<K, RI, RO, MODE, HI, ITEMS><<<(unsigned)tiles, kWThreads, smem, st>>>(
+    smem = std::max(smem, wsweep_smem_bytes<ITEMS>(b, MODE, guard, WIDE));
+  k_wsweep<K, RI, RO, MODE, HI, WIDE, ITEMS><<<(unsigned)tiles, kWThreads, smem, st>>>(
       d_jobs, num_jobs, tiles, pass, d_counter, d_err, d_tile_job);
   return cudaGetLastError();
 }
 
-template <typename K, int MODE, int ITEMS>
-cudaError_t wsweep_pick(const RadixJob<K>* d_jobs, int num_jobs, int64_t tiles, int pass,
-                        int max_bits, bool raw_in, bool raw_out, bool hi, bool guard,
-                        uint32_t* d_counter, int* d_err, cudaStream_t st,
-                        const int32_t* d_tile_job) {
-#define TJ_GO(RI, RO, H)                                                                        \
-  return wsweep_go<K, RI, RO, MODE, H, ITEMS>(d_jobs, num_jobs, tiles, pass, max_bits, guard,  \
-                                              d_counter, d_err, st, d_tile_job)
-  constexpr bool wide = sizeof(K) == 8;  // 32-bit keys always sit in the upper half
+// Calls f<RAW_IN, RAW_OUT, HI, WIDE>() for the layout asked for, if this key
+// type and mode have it.  32-bit keys always sit in the upper half, and words
+// to words go through the 64-bit instantiation.
+template <typename K, int MODE, typename F>
+cudaError_t wsweep_layout(bool raw_in, bool raw_out, bool hi, bool wide, const F& f) {
+  constexpr bool k64 = sizeof(K) == 8;
+  if constexpr (k64 && MODE == kModeSort) {
+    if (wide) {
+      if (raw_in) return f.template operator()<true, false, false, true>();
+      if (raw_out) return f.template operator()<false, true, false, true>();
+      return f.template operator()<false, false, false, true>();
+    }
+  }
+  if (wide) return cudaErrorInvalidValue;
   if (raw_in) {
-    if constexpr (wide && MODE != kModeCuts)
-      if (!hi) TJ_GO(true, false, false);
-    TJ_GO(true, false, true);
+    if constexpr (k64 && MODE != kModeCuts)
+      if (!hi) return f.template operator()<true, false, false, false>();
+    return f.template operator()<true, false, true, false>();
   }
   if constexpr (MODE == kModeSort) {
     if (raw_out) {
-      if constexpr (wide)
-        if (!hi) TJ_GO(false, true, false);
-      TJ_GO(false, true, true);
+      if constexpr (k64)
+        if (!hi) return f.template operator()<false, true, false, false>();
+      return f.template operator()<false, true, true, false>();
     }
-    if constexpr (wide) {
-      if (!hi) TJ_GO(false, false, false);
-      TJ_GO(false, false, true);
+    if constexpr (k64) {
+      if (!hi) return f.template operator()<false, false, false, false>();
+      return f.template operator()<false, false, true, false>();
     }
   }
   return cudaErrorInvalidValue;
-#undef TJ_GO
 }
 
 template <typename K>
-cudaError_t launch_wsweep(const RadixJob<K>* d_jobs, int num_jobs, int64_t total_tiles, int pass,
-                          int max_bits, int mode, bool raw_in, bool raw_out, bool hi, int items,
-                          bool guard, uint32_t* d_tile_counter, int* d_err, cudaStream_t st,
-                          const int32_t* d_tile_job) {
-#define TJ_PICK(M, I)                                                                           \
-  return wsweep_pick<K, M, I>(d_jobs, num_jobs, total_tiles, pass, max_bits, raw_in, raw_out,  \
-                              hi, guard, d_tile_counter, d_err, st, d_tile_job)
-  if (items == kWItems) {
-    if (mode == kModeSort) TJ_PICK(kModeSort, kWItems);
-    if (mode == kModeRadix) TJ_PICK(kModeRadix, kWItems);
-    if (mode == kModeCuts) TJ_PICK(kModeCuts, kWItems);
-  } else if (items == kWItemsSmall && mode == kModeSort) {
-    TJ_PICK(kModeSort, kWItemsSmall);
+struct WordLaunch {
+  const RadixJob<K>* jobs;
+  int num_jobs;
+  int64_t tiles;
+  int pass, max_bits;
+  bool guard;
+  uint32_t* counter;
+  int* err;
+  cudaStream_t st;
+  const int32_t* tile_job;
+};
+template <typename K, int MODE, int ITEMS>
+struct WordGo {
+  const WordLaunch<K>& a;
+  template <bool RI, bool RO, bool HI, bool WIDE>
+  cudaError_t operator()() const {
+    return wsweep_go<K, RI, RO, MODE, HI, WIDE, ITEMS>(a.jobs, a.num_jobs, a.tiles, a.pass,
+                                                       a.max_bits, a.guard, a.counter, a.err,
+                                                       a.st, a.tile_job);
   }
+};
+template <typename K, int MODE, int ITEMS>
+struct WordAttr {
+  template <bool RI, bool RO, bool HI, bool WIDE>
+  cudaError_t operator()() const {
+    return wsweep_attr<K, RI, RO, MODE, HI, WIDE, ITEMS>();
+  }
+};
+
+template <typename K>
+cudaError_t launch_wsweep(const RadixJob<K>* d_jobs, int num_jobs, int64_t total_tiles, int pass,
+                          int max_bits, int mode, bool raw_in, bool raw_out, bool hi, bool wide,
+                          int items, bool guard, uint32_t* d_tile_counter, int* d_err,
+                          cudaStream_t st, const int32_t* d_tile_job) {
+  const WordLaunch<K> a = {d_jobs, num_jobs, total_tiles, pass, max_bits, guard, d_tile_counter,
+                           d_err, st, d_tile_job};
+  if (items == kWItems && mode == kModeSort)
+    return wsweep_layout<K, kModeSort>(raw_in, raw_out, hi, wide, WordGo<K, kModeSort, kWItems>{a});
+  if (items == kWItems && mode == kModeRadix)
+    return wsweep_layout<K, kModeRadix>(raw_in, raw_out, hi, wide,
+                                        WordGo<K, kModeRadix, kWItems>{a});
+  if (items == kWItems && mode == kModeCuts)
+    return wsweep_layout<K, kModeCuts>(raw_in, raw_out, hi, wide, WordGo<K, kModeCuts, kWItems>{a});
+  if (items == kWItemsSmall && mode == kModeSort)
+    return wsweep_layout<K, kModeSort>(raw_in, raw_out, hi, wide,
+                                       WordGo<K, kModeSort, kWItemsSmall>{a});
   return cudaErrorInvalidValue;
-#undef TJ_PICK
 }
 
+// every layout of a mode (raw_in, raw_out, hi, wide in turn)
 template <typename K, int MODE, int ITEMS>
 cudaError_t wsweep_attrs_mode() {
-  constexpr bool wide = sizeof(K) == 8;
-  cudaError_t e = wsweep_attr<K, true, false, MODE, true, ITEMS>();
-  if constexpr (wide && MODE != kModeCuts)
-    if (e == cudaSuccess) e = wsweep_attr<K, true, false, MODE, false, ITEMS>();
-  if constexpr (MODE == kModeSort) {
-    if (e == cudaSuccess) e = wsweep_attr<K, false, true, MODE, true, ITEMS>();
-    if constexpr (wide) {
-      if (e == cudaSuccess) e = wsweep_attr<K, false, true, MODE, false, ITEMS>();
-      if (e == cudaSuccess) e = wsweep_attr<K, false, false, MODE, false, ITEMS>();
-      if (e == cudaSuccess) e = wsweep_attr<K, false, false, MODE, true, ITEMS>();
-    }
+  const WordAttr<K, MODE, ITEMS> f;
+  for (int m = 0; m < 12; ++m) {
+    const bool ri = m % 3 == 1, ro = m % 3 == 2, hi = (m / 3) & 1, wide = m / 6;
+    const cudaError_t e = wsweep_layout<K, MODE>(ri, ro, hi, wide, f);
+    if (e != cudaSuccess && e != cudaErrorInvalidValue) return e;  // (a layout the mode has not)
   }
-  return e;
+  return cudaSuccess;
 }
 
 template <typename K>
@@ -562,8 +631,8 @@ cudaError_t word_init_attributes() {
 
 #define TJ_INSTANTIATE_WORD(K)                                                                  \
   template cudaError_t launch_wsweep<K>(const RadixJob<K>*, int, int64_t, int, int, int, bool, \
-                                        bool, bool, int, bool, uint32_t*, int*, cudaStream_t,  \
-                                        const int32_t*);
+                                        bool, bool, bool, int, bool, uint32_t*, int*,          \
+                                        cudaStream_t, const int32_t*);
 TJ_INSTANTIATE_WORD(int32_t)
 TJ_INSTANTIATE_WORD(int64_t)
 

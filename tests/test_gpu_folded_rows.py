@@ -23,25 +23,28 @@ def sorted_as_oracle(keys, ids):
 
 @pytest.mark.parametrize("n", [SMALL - 1, SMALL, SMALL + 1, 5 * SMALL + 7, (1 << 22) - 1,
                                513 * LARGE, 513 * LARGE + 1])
-@pytest.mark.parametrize("bits", [3, 27, 33])
+@pytest.mark.parametrize("bits", [3, 27, 33, 64])
 def test_tile_edges(n, bits):
     # at 2^22 rows the large tile and the plan of fewest pass units take over;
-    # 33 key bits leave the key in both halves of the word
+    # 33 key bits leave the key in both halves of the word, 64 do not fold: the
+    # key travels beside a 32-bit id
     g = torch.Generator().manual_seed(n + bits)
-    keys = torch.randint(-(1 << (bits - 1)), 1 << (bits - 1), (n,), generator=g)
+    keys = torch.randint(-(1 << (bits - 1)), (1 << (bits - 1)) - 1, (n,), generator=g)
     sorted_as_oracle(keys, torch.arange(n))
 
 
 @pytest.mark.parametrize("dtype", [torch.int32, torch.int64])
 @pytest.mark.parametrize("ids", ["full", "one_far", "offset", "negative"])
-def test_ids_that_fit_and_that_do_not(dtype, ids):
+@pytest.mark.parametrize("bits", [40, 63])
+def test_ids_that_fit_and_that_do_not(dtype, ids, bits):
     # 40 key bits leave 24 id bits: positions of 2^17 rows fit, wherever they
-    # start; one id far from the sampled ones does not, nor do full-range ids
+    # start; one id far from the sampled ones does not, nor do full-range ids.
+    # 63 key bits leave the key beside a 32-bit id, or a full one.
     n = 1 << 17
     info = torch.iinfo(dtype)
     g = torch.Generator().manual_seed(4)
-    top = 40 if dtype == torch.int64 else 30
-    keys = torch.randint(0, 1 << top, (n,), generator=g, dtype=torch.int64).to(dtype)
+    top = bits if dtype == torch.int64 else 30
+    keys = torch.randint(0, (1 << top) - 1, (n,), generator=g, dtype=torch.int64).to(dtype)
     v = torch.arange(n, dtype=torch.int64)
     if ids == "full":
         v = torch.randint(info.min, info.max, (n,), generator=g, dtype=torch.int64)
