@@ -834,20 +834,32 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     const int64_t wtile = (int64_t)kWThreads * items;
     const int64_t wt_r = ceil_div(nr, wtile), wt = wt_r + ceil_div(ns, wtile);
     const int64_t lb_words = wt << wp.max_bits;
-    const bool regions = (int64_t)wp.passes * lb_words * 4 <= (int64_t)1 << 20;
-    Carve wc;
-    const size_t o_a = wc.add<uint64_t>((size_t)(nr + ns));
-    const size_t o_b = wc.add<uint64_t>(wp.passes > 1 ? (size_t)(nr + ns) : 0);
-    const size_t o_ai = wc.add<uint32_t>(fold.wide ? (size_t)(nr + ns) : 0);
-    const size_t o_bi = wc.add<uint32_t>(fold.wide && wp.passes > 1 ? (size_t)(nr + ns) : 0);
-    const size_t o_wt = wc.add<JTile<K>>(jtiles);
-    const size_t o_whist = wc.add<uint32_t>((size_t)2 * wp.passes << wp.max_bits);
-    const size_t o_wjlb = wc.add<uint64_t>(jtiles);
-    const size_t o_wlb = wc.add<uint32_t>((size_t)(regions ? wp.passes : 1) * lb_words);
-    const size_t wneed = wc.off + cc.off;
+    size_t o_a, o_b, o_ai, o_bi, o_wt, o_whist, o_wjlb, o_wlb;
+    auto lay_out = [&](bool per_pass) -> size_t {
+      Carve wc;
+      o_a = wc.add<uint64_t>((size_t)(nr + ns));
+      o_b = wc.add<uint64_t>(wp.passes > 1 ? (size_t)(nr + ns) : 0);
+      o_ai = wc.add<uint32_t>(fold.wide ? (size_t)(nr + ns) : 0);
+      o_bi = wc.add<uint32_t>(fold.wide && wp.passes > 1 ? (size_t)(nr + ns) : 0);
+      o_wt = wc.add<JTile<K>>(jtiles);
+      o_whist = wc.add<uint32_t>((size_t)2 * wp.passes << wp.max_bits);
+      o_wjlb = wc.add<uint64_t>(jtiles);
+      o_wlb = wc.add<uint32_t>((size_t)(per_pass ? wp.passes : 1) * lb_words);
+      return wc.off;
+    };
+    // a look-back region per pass (one memset in all) while they are small and
+    // the column passes' memory has room for them, as it has for one: 32-bit
+    // rows, whose words are no smaller than the columns, need the second try
+    bool regions = (int64_t)wp.passes * lb_words * 4 <= (int64_t)1 << 20;
+    size_t wbytes = lay_out(regions);
+    if (regions && wbytes + cc.off > need) {
+      regions = false;
+      wbytes = lay_out(false);
+    }
+    const size_t wneed = wbytes + cc.off;
     if (wneed > need) break;
     Block big;
-    TJ_CUDA(big.alloc(wc.off, st));
+    TJ_CUDA(big.alloc(wbytes, st));
     RadixJob<K> hw[4] = {hj[0], hj[1], hj[0], hj[1]};
     uint64_t* res[2];
     const K* res_i[2] = {nullptr, nullptr};
@@ -2783,11 +2795,17 @@ tj_status sort_multi_impl(K* const* cols, int ncols, K* ids, int64_t n, int path
 // Radix jobs are laid out R_0, S_0, R_1, S_1, ...; every pair shares its own
 // (lo, bits) and all pairs use the same pass count with per-pair digit widths.
 // Everything after the statistics is captured into one CUDA graph.
+// Folded rows (`words`): ids' window and id bits are the batch's, the first key
+// of a word each pair's own, and each pair takes the passes that suit its key
+// bits (kernels skip a pair that has no such pass); one pass at least, which
+// folds. 1024 pairs of 10^3 to 10^6 int32 rows (2.9x10^8 rows, up to 21 key
+// bits): three column passes took 5.8 ms, the word passes 3.8.
+// A row that does not fold makes the call return kColumnsAgain.
 template <typename K>
 tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, const K* kr,
                      const K* ir, const K* ks, const K* is, K* out, int64_t cap,
                      int64_t* d_out_off, int64_t* out_count, cudaStream_t st, int digit_cap,
-                     int items) {
+                     int items, bool words) {
   tj_stats stats = {};
   stats.groups = 1;
   const int tile = kSortThreads * items;
@@ -2806,6 +2824,7 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
       const int64_t a = side ? s_off[j] : r_off[j];
       const int64_t n = (side ? s_off[j + 1] : r_off[j + 1]) - a;
       x.keys = (side ? ks : kr) + a;
+      if (sizeof(K) == 8 && words) x.ids = (side ? is : ir) + a;
       x.n = n;
       x.tile0 = tiles;
       tiles += ceil_div(n, tile);
@@ -2835,7 +2854,8 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   // per-pair ranges; pairs that cannot match are dropped from the batch
   std::vector<uint64_t> plo((size_t)nj, 0), prange((size_t)nj, 0);
   std::vector<char> live((size_t)nj, 0);
-  int P = 0;
+  int P = 0, max_kb = 0;
+  unsigned long long id_lo = ~0ull, id_hi = 0ull;
   for (int64_t j = 0; j < nj; ++j) {
     const RadixJob<K>& xr = hj[(size_t)(2 * j)];
     const RadixJob<K>& xs = hj[(size_t)(2 * j + 1)];
@@ -2849,6 +2869,39 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
     prange[(size_t)j] = range_of<K>(lo, hi);
     live[(size_t)j] = 1;
     P = std::max(P, make_plan(plo[(size_t)j], prange[(size_t)j], false, digit_cap).passes);
+    max_kb = std::max(max_kb, bitlen(prange[(size_t)j]));
+    for (int side = 0; side < 2; ++side) {
+      id_lo = std::min(id_lo, hs[(size_t)(2 * j + side)].id_min_u);
+      id_hi = std::max(id_hi, ~hs[(size_t)(2 * j + side)].id_max_u);
+    }
+  }
+  // the word tile: the large one unless the arrays' last tiles waste more by it
+  // than it saves a pass (about a tenth); arrays that the small one pads by more
+  // than kPadShare stay columns, whose passes step over a tile's missing rows
+  int64_t pad_large = 0, pad_small = 0;
+  for (int64_t j = 0; words && j < 2 * nj; ++j) {
+    pad_large += ceil_div(hj[(size_t)j].n, kWThreads * kWItems) * (kWThreads * kWItems);
+    pad_small += ceil_div(hj[(size_t)j].n, kWThreads * kWItemsSmall) * (kWThreads * kWItemsSmall);
+  }
+  constexpr double kPadShare = 0.25;
+  words = words && (double)pad_small <= (1.0 + kPadShare) * (double)(R + S);
+  const Fold fold = words ? make_fold<K>(0, max_kb, id_lo, id_hi, true) : Fold();
+  words = fold.on || fold.wide;
+  const int witems = R + S >= kWSmallRows && pad_large * 10 <= pad_small * 11 ? kWItems
+                                                                             : kWItemsSmall;
+  const int64_t ptile = words ? (int64_t)kWThreads * witems : tile;  // rows of a pass's tile
+  auto pair_plan = [&](int64_t j) {
+    const uint64_t lo = plo[(size_t)j], range = prange[(size_t)j];
+    if (!words) return make_plan(lo, range, false, digit_cap, P);
+    if (bitlen(range) == 0) return make_plan(lo, range, false, digit_cap, 1);
+    if (R + S >= kCostRows) return make_word_plan(lo, range, false, digit_cap, 1);
+    return make_plan(lo, range, false, digit_cap);
+  };
+  if (words) {
+    P = 0;
+    for (int64_t j = 0; j < nj; ++j)
+      if (live[(size_t)j]) P = std::max(P, pair_plan(j).passes);
+    stats.tile_rows = (int32_t)ptile;
   }
   stats.radix_passes = P;
   // scratch: ping-pong copies of every live pair, histograms, look-back, join state
@@ -2857,9 +2910,11 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   int64_t hist_words = 0, lb_words = 0, jtiles = 0;
   std::vector<int64_t> hist_at((size_t)(2 * nj), 0), lb_at((size_t)(2 * nj), 0);
   tiles = 0;
+  int64_t ptiles = 0;
+  std::vector<int64_t> ptile_at((size_t)(2 * nj), 0);
   for (int64_t j = 0; j < nj; ++j) {
     Plan pl;
-    if (live[(size_t)j]) pl = make_plan(plo[(size_t)j], prange[(size_t)j], false, digit_cap, P);
+    if (live[(size_t)j]) pl = pair_plan(j);
     plans[(size_t)j] = pl;
     stats.key_bits = std::max(stats.key_bits, pl.key_bits);
     stats.digit_bits = std::max(stats.digit_bits, pl.max_bits);
@@ -2868,8 +2923,10 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
       RadixJob<K>& x = hj[(size_t)(2 * j + side)];
       if (!live[(size_t)j]) x.n = 0;
       x.tile0 = tiles;
-      const int64_t t = ceil_div(x.n, tile);
-      tiles += t;
+      tiles += ceil_div(x.n, tile);
+      const int64_t t = ceil_div(x.n, ptile);
+      ptile_at[(size_t)(2 * j + side)] = ptiles;
+      ptiles += t;
       hist_at[(size_t)(2 * j + side)] = hist_words;
       hist_words += (int64_t)std::max(P, 1) * bins;
       lb_at[(size_t)(2 * j + side)] = lb_words;
@@ -2878,8 +2935,12 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
     if (live[(size_t)j]) jtiles += ceil_div(s_off[j + 1] - s_off[j], kJTile);
   }
   Carve bc;
-  size_t o_r[4] = {0, 0, 0, 0}, o_s[4] = {0, 0, 0, 0};
-  for (int b = 0; b < nbuf; ++b) {
+  size_t o_r[4] = {0, 0, 0, 0}, o_s[4] = {0, 0, 0, 0}, o_w[2] = {0, 0}, o_wi[2] = {0, 0};
+  for (int b = 0; words && b < nbuf; ++b) {  // R's rows, then S's
+    o_w[b] = bc.add<uint64_t>((size_t)(R + S));
+    o_wi[b] = bc.add<uint32_t>(fold.wide ? (size_t)(R + S) : 0);
+  }
+  for (int b = 0; !words && b < nbuf; ++b) {
     o_r[2 * b] = bc.add<K>((size_t)R);
     o_r[2 * b + 1] = bc.add<K>((size_t)R);
     o_s[2 * b] = bc.add<K>((size_t)S);
@@ -2891,11 +2952,18 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   const size_t o_jlb = bc.add<uint64_t>((size_t)std::max<int64_t>(jtiles, 1));
   const size_t o_tmap = bc.add<int32_t>((size_t)std::max<int64_t>(tiles, 1));
   const size_t o_jmap = bc.add<int32_t>((size_t)std::max<int64_t>(jtiles, 1));
+  // (word passes: a second view of the jobs, digits of words, and its tile map)
+  const size_t o_pjobs = bc.add<RadixJob<K>>(words ? (size_t)(2 * nj) : 0);
+  const size_t o_pmap = bc.add<int32_t>(words ? (size_t)std::max<int64_t>(ptiles, 1) : 0);
   Block big;
   TJ_CUDA(big.alloc(bc.off, st));
   stats.scratch_peak = (int64_t)(bc.off + cc.off);
   int32_t* d_tmap = big.at<int32_t>(o_tmap);
   int32_t* d_jmap = big.at<int32_t>(o_jmap);
+
+  RadixJob<K>* d_pjobs = big.at<RadixJob<K>>(o_pjobs);
+  int32_t* d_pmap = big.at<int32_t>(o_pmap);
+  std::vector<RadixJob<K>> hp(words ? (size_t)(2 * nj) : 0);
 
   std::vector<JoinJob<K>> hjj((size_t)nj);
   int64_t jt = 0;
@@ -2904,11 +2972,28 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
     for (int side = 0; side < 2; ++side) {
       RadixJob<K>& x = hj[(size_t)(2 * j + side)];
       set_job_plan(x, plans[(size_t)j]);
-      x.passes = live[(size_t)j] ? P : 0;
+      if (!words) x.passes = live[(size_t)j] ? P : 0;
       x.hist_stride = 1 << plans[(size_t)j].max_bits;
       x.hist = big.at<uint32_t>(o_hist) + hist_at[(size_t)(2 * j + side)];
       x.lookback = big.at<uint32_t>(o_lb) + lb_at[(size_t)(2 * j + side)];
       const int64_t a = side ? s_off[j] : r_off[j];
+      if (words) {
+        RadixJob<K>& q = hp[(size_t)(2 * j + side)];
+        q = x;
+        Fold f = fold;
+        f.wlo = plo[(size_t)j];
+        set_word_plan(q, plans[(size_t)j], f, 0);
+        q.tile0 = ptile_at[(size_t)(2 * j + side)];
+        const int64_t w0 = side ? R + a : a;
+        uint64_t* buf[2] = {big.at<uint64_t>(o_w[0]) + w0,
+                            nbuf > 1 ? big.at<uint64_t>(o_w[1]) + w0 : nullptr};
+        res[2 * side] = reinterpret_cast<const K*>(
+            set_word_buffers(q, res[2 * side], res[2 * side + 1], buf[0], buf[1]));
+        for (int p = 0; fold.wide && p < q.passes; ++p)
+          q.dst_v[p] = reinterpret_cast<K*>(big.at<uint32_t>(o_wi[p & 1]) + w0);
+        if (fold.wide && q.passes > 0) res[2 * side + 1] = q.dst_v[q.passes - 1];
+        continue;
+      }
       const size_t* o = side ? o_s : o_r;
       K* ak = nbuf > 0 ? big.at<K>(o[0]) + a : nullptr;
       K* av = nbuf > 0 ? big.at<K>(o[1]) + a : nullptr;
@@ -2929,6 +3014,11 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   }
   TJ_CUDA(put_small(d_jobs, hj.data(), hj.size() * sizeof(RadixJob<K>), st));
   TJ_CUDA(put_small(d_jj, hjj.data(), hjj.size() * sizeof(JoinJob<K>), st));
+  if (words) TJ_CUDA(put_small(d_pjobs, hp.data(), hp.size() * sizeof(RadixJob<K>), st));
+  WordFmt fmt;
+  fmt.ib = fold.on ? fold.ib : 0;
+  fmt.wide = fold.wide;
+  fmt.ilo = fold.ilo;
 
   // the batch's device work, captured once as a graph (plain launches on the
   // legacy stream, which cannot be captured)
@@ -2941,6 +3031,7 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
     if (e == cudaSuccess) e = x;
   };
   step(launch_fill_tile_job<K>(d_jobs, (int)(2 * nj), d_tmap, st, tile));
+  if (words) step(launch_fill_tile_job<K>(d_pjobs, (int)(2 * nj), d_pmap, st, (int)ptile));
   step(launch_fill_join_tile_job<K>(d_jj, (int)nj, d_jmap, st));
   if (P > 0) {
     step(cudaMemsetAsync(big.at<uint32_t>(o_hist), 0,
@@ -2950,15 +3041,22 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
     for (int p = 0; p < P; ++p) {
       step(cudaMemsetAsync(big.at<uint32_t>(o_lb), 0,
                            (size_t)std::max<int64_t>(lb_words, 1) * sizeof(uint32_t), st));
+      if (words) {
+        step(word_pass<K>(d_pjobs, (int)(2 * nj), ptiles, p, stats.digit_bits, p == 0, fold,
+                          witems, d_counters + p, d_err, st, d_pmap));
+        continue;
+      }
       step(launch_onesweep<K>(d_jobs, (int)(2 * nj), tiles, p, stats.digit_bits, false, d_counters + p,
                               d_err, st, d_tmap, items));
     }
   }
-  step(launch_tile_ranges<K>(d_jj, (int)nj, jtiles, big.at<JTile<K>>(o_jt), st, d_jmap));
+  step(launch_tile_ranges<K>(d_jj, (int)nj, jtiles, big.at<JTile<K>>(o_jt), st, d_jmap, fmt,
+                             words ? d_err : nullptr));
   step(cudaMemsetAsync(big.at<uint64_t>(o_jlb), 0,
                        (size_t)std::max<int64_t>(jtiles, 1) * sizeof(uint64_t), st));
   step(launch_join<K>(jtiles, big.at<JTile<K>>(o_jt), big.at<uint64_t>(o_jlb),
-                      d_counters + kMaxPasses, out, cap, nullptr, d_out_off, d_total, d_err, st));
+                      d_counters + kMaxPasses, out, cap, nullptr, d_out_off, d_total, d_err, st,
+                      fmt));
   step(launch_fix_job_out<K>(d_jj, (int)nj, jtiles, d_out_off, d_total, st));
   if (use_graph) {
     cudaError_t e2 = cudaStreamEndCapture(st, &graph);
@@ -2976,6 +3074,7 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess)
     return set_err(TJ_ERR_CUDA, "batch launch: %s", cudaGetErrorString(e));
+  if (h_err == kErrFold) return kColumnsAgain;
   if (h_err) return set_err((tj_status)h_err, "device reported %d", h_err);
   *out_count = h_total;
   stats.out_count = h_total;
@@ -2986,11 +3085,25 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   return TJ_OK;
 }
 
+// ... with folded rows unless the tile choice asks for the small tile of the
+// column passes, and on columns when a row did not fold
+template <typename K>
+tj_status batch_run(int64_t nj, const int64_t* r_off, const int64_t* s_off, const K* kr,
+                    const K* ir, const K* ks, const K* is, K* out, int64_t cap,
+                    int64_t* d_out_off, int64_t* out_count, cudaStream_t st, int digit_cap,
+                    int items) {
+  tj_status s = batch_impl<K>(nj, r_off, s_off, kr, ir, ks, is, out, cap, d_out_off, out_count,
+                              st, digit_cap, items, items == kItems);
+  if (s == kColumnsAgain)
+    s = batch_impl<K>(nj, r_off, s_off, kr, ir, ks, is, out, cap, d_out_off, out_count, st,
+                      digit_cap, items, false);
+  return s;
+}
 
 // ---- autotuner of the batched join --------------------------------------------------
 // Choices: the widest radix digit (and so the number of passes and the fan-out
-// of each pass) and the onesweep tile (1536 or 3072 rows: small jobs waste
-// less of a smaller last tile).  A choice is cached per (dtype, log2 jobs,
+// of each pass) and the pass (folded rows, or columns in tiles of 1536 rows:
+// small jobs waste less of a smaller last tile).  A choice is cached per (dtype, log2 jobs,
 // log2 mean rows per array); TJ_TUNE_CACHE names a file that persists it.
 struct TuneChoice {
   int digit;
@@ -3052,7 +3165,7 @@ tj_status batch_tuned(int dt, int64_t nj, const int64_t* r_off, const int64_t* s
   TuneChoice c = {max_digit_bits<K>(), kItems};
   if (!tune) {
     tune_get(key, &c);
-    return batch_impl<K>(nj, r_off, s_off, kr, ir, ks, is, out, cap, d_out_off, out_count, st,
+    return batch_run<K>(nj, r_off, s_off, kr, ir, ks, is, out, cap, d_out_off, out_count, st,
                          c.digit, c.items);
   }
   // time every candidate on this batch (each run also produces the result)
@@ -3062,7 +3175,7 @@ tj_status batch_tuned(int dt, int64_t nj, const int64_t* r_off, const int64_t* s
     for (int it : {4, kItems}) {
       for (int rep = 0; rep < 2; ++rep) {  // the first run warms the pool
         const auto t0 = std::chrono::steady_clock::now();
-        tj_status s = batch_impl<K>(nj, r_off, s_off, kr, ir, ks, is, out, cap, d_out_off,
+        tj_status s = batch_run<K>(nj, r_off, s_off, kr, ir, ks, is, out, cap, d_out_off,
                                     out_count, st, d, it);
         const double dtm =
             std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
@@ -3074,7 +3187,7 @@ tj_status batch_tuned(int dt, int64_t nj, const int64_t* r_off, const int64_t* s
       }
     }
   tune_put(key, bc);
-  return batch_impl<K>(nj, r_off, s_off, kr, ir, ks, is, out, cap, d_out_off, out_count, st,
+  return batch_run<K>(nj, r_off, s_off, kr, ir, ks, is, out, cap, d_out_off, out_count, st,
                        bc.digit, bc.items);
 }
 
