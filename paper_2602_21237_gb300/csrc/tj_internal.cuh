@@ -62,11 +62,14 @@ constexpr int kMaxDigitBits = 10;           // widest radix digit
 constexpr int kMaxBins = 1 << kMaxDigitBits;
 constexpr int kMaxPasses = 8;               // 64-bit keys at 8 bits per pass
 #ifndef TJ_JTILE
-#define TJ_JTILE 4096
+#define TJ_JTILE 2048
 #endif
 constexpr int kJTile = TJ_JTILE;            // S rows per join tile (a power of two)
+#ifndef TJ_CHUNKS
+#define TJ_CHUNKS 4
+#endif
 constexpr int kRCap = kJTile / 2;           // R rows a join tile keeps on chip at once
-constexpr int kMaxChunks = 4;               // R chunks a join tile aligns on chip
+constexpr int kMaxChunks = TJ_CHUNKS;               // R chunks a join tile aligns on chip
 constexpr int kHTSlots = kJTile;            // on-chip hash table slots (load <= 0.5)
 static_assert((kJTile & (kJTile - 1)) == 0 && kJTile >= 1024, "join tile: a power of two");
 

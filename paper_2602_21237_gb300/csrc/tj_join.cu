@@ -9,9 +9,10 @@
 //                     1. read the tile's descriptor, stage its S rows and its
 //                        R range (in chunks of kRCap rows, up to 4) in shared
 //                        memory with cp.async;
-//                     2. build an open-addressing hash table of each chunk's
-//                        distinct keys with shared-memory atomicCAS: slot ->
-//                        (first, end) of the key's run of R rows;
+//                     2. build a table of each chunk's distinct keys, key ->
+//                        (first, end) of its run of R rows: by key value where
+//                        the chunk's keys are dense, else an open-addressing
+//                        hash table filled with shared-memory atomicCAS;
 //                     3. probe it once per S row -> match count, run start;
 //                     4. a decoupled look-back over all tiles of all jobs gives
 //                        the tile's first output index;
@@ -89,7 +90,14 @@ __device__ __forceinline__ K word_id(uint64_t w, const WordFmt& f) {
 }
 static_assert(kRCap < 0xFFFF, "run bounds are packed in 16 bits");
 
-constexpr uint32_t kHTEmpty = 0xFFFFFFFFu;
+constexpr uint32_t kHTEmpty = 0u;  // (no entry is 0: a run's end is at least 1)
+// Entries of the on-chip table: a chunk of R whose keys span fewer values than
+// that has one entry per value instead of a hash table of kHTSlots.
+// (Separate columns, W = 0, leave shared memory for half as many.)
+template <int W>
+__host__ __device__ constexpr int tab_slots() {
+  return W == 0 ? kHTSlots : 2 * kHTSlots;
+}
 
 __device__ __forceinline__ uint32_t lanemask_lt_j() {
   uint32_t m;
@@ -185,18 +193,22 @@ __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
 
 // ---------------------------------------------------------------------------
 #ifndef TJ_JTHREADS
-#define TJ_JTHREADS 512
+#define TJ_JTHREADS 256
 #endif
 #ifndef TJ_JMINB
-#define TJ_JMINB 2
+#define TJ_JMINB 4
 #endif
 constexpr int kJThreads = TJ_JTHREADS;          // threads per join CTA
 constexpr int kJWarps = kJThreads / 32;
 constexpr int kJItems = kJTile / kJThreads;     // S rows per thread
 static_assert(kJItems * kJThreads == kJTile, "join tile = threads x items");
+// Most matches a row may have for its thread to write them one after another
+// (the matches of neighbouring rows share sectors); beyond, every output index
+// of the tile finds its row by a binary search.
+constexpr uint32_t kJDirect = 16;
 
 // Shared memory: S keys | R keys | S ids | R ids (kJTile or kRCap elements and
-// kPad more each) | hash table[kHTSlots] u32; folded rows: S words | R words |
+// kPad more each) | hash table[tab_slots] u32; folded rows: S words | R words |
 // table.  Each staged array starts up to kPad
 // elements into its area (its first element keeps the source's address modulo
 // 16, so that all but a head and a tail move in 16-byte copies).  After the
@@ -213,7 +225,7 @@ constexpr size_t join_smem_bytes() {
   constexpr bool ids = W == 0 || W == 3;
   return sizeof(E) * (size_t)(kJTile + join_pad<E>() + kRCap + join_pad<E>()) +
          (ids ? sizeof(V) * (size_t)(kJTile + join_pad<V>() + kRCap + join_pad<V>()) : 0) +
-         sizeof(uint32_t) * kHTSlots;
+         sizeof(uint32_t) * tab_slots<W>();
 }
 static_assert(sizeof(uint64_t) * (kJTile + kRCap) >= (sizeof(uint64_t) + sizeof(uint32_t)) * kJTile,
               "offsets and run starts fit in the folded rows' shared memory");
@@ -254,18 +266,18 @@ __device__ __forceinline__ K* join_copy_async(K* dst, const K* __restrict__ src,
 // of sorted R whose keys lie between the tile's first and last key.
 //   1. S keys and ids and the first chunk of the R range go to shared memory
 //      (cp.async); warp w owns S rows [w*32*kJItems, ...), item u = 32 rows;
-//   2. per chunk of the R range (kRCap rows, at most kMaxChunks): an
-//      open-addressing table of the chunk's distinct keys is built with
-//      shared-memory atomicCAS (slot -> first and end of the key's run), and
-//      every S row probes it -> match count, run start and the R id of the
-//      first match; wider R ranges are searched through a strided sample
+//   2. per chunk of the R range (kRCap rows, at most kMaxChunks): a table of
+//      the chunk's distinct keys (entry: first and end of the key's run) by key
+//      value, or hashed, and every S row looks its key up -> match
+//      count and run start; wider R ranges are searched through a strided sample
 //      staged on chip, then within one stride in global memory;
 //   3. the tile's total goes to the decoupled look-back chain over all tiles
 //      (warp 0, 32 predecessors per round trip), which yields the tile's
 //      first output index;
-//   4. at most one match per row (a foreign-key join): each row's output index
-//      comes from ballots over the warp and the warps' totals; otherwise the
-//      tile's counts are scanned and each output index finds its S row.
+//   4. at most kJDirect matches a row: each row's first output index comes
+//      from ballots (one match at most, a foreign-key join) or shuffles over
+//      the warp and from the warps' totals; otherwise the tile's counts are
+//      scanned and each output index finds its S row.
 // Output order: key, then S position, then R position.
 template <typename K, int W>
 __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
@@ -280,6 +292,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   const int ib = f.ib;
   using V = typename Row::V;
   constexpr bool kIds = W == 0 || W == 3;  // an id column beside the keys
+  constexpr int kTabSlots = tab_slots<W>();
   constexpr int kPad = join_pad<E>(), kPadV = join_pad<V>();
   E* const b_sk = reinterpret_cast<E*>(smem);  // staging areas (16-byte aligned)
   E* const b_rk = b_sk + kJTile + kPad;
@@ -290,6 +303,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   // an id column's element as the caller's id
   auto id_of = [&](V v) -> K { return W == 3 ? (K)((uint64_t)v + f.ilo) : (K)v; };
   __shared__ uint64_t s_wsum[kJWarps];
+  __shared__ uint32_t s_wmax[kJWarps];
   __shared__ uint64_t s_base;
   __shared__ uint32_t s_t;
 
@@ -341,9 +355,36 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         if constexpr (kIds) s_rv = join_copy_async<V>(b_rv, rv_g + c0, nc);
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
-      for (int i = tid; i < kHTSlots; i += kJThreads) s_ht[i] = kHTEmpty;
+      for (int i = tid; i < kTabSlots / 4; i += kJThreads)
+        reinterpret_cast<uint4*>(s_ht)[i] = make_uint4(0u, 0u, 0u, 0u);
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();
+      const Key cf = Row::key(s_rk[0], ib), cl = Row::key(s_rk[nc - 1], ib);
+      if ((uint64_t)cl - (uint64_t)cf < (uint64_t)kTabSlots) {
+        // dense keys: entry key - cf holds the key's run (first | end << 16),
+        // each half written by the run's first or last row
+        uint16_t* const s_run = reinterpret_cast<uint16_t*>(s_ht);
+        for (int i = tid; i < nc; i += kJThreads) {
+          const Key key = Row::key(s_rk[i], ib);
+          const uint32_t d = (uint32_t)((uint64_t)key - (uint64_t)cf);
+          if (i == 0 || key != Row::key(s_rk[i - 1], ib)) s_run[2 * d] = (uint16_t)i;
+          if (i == nc - 1 || key != Row::key(s_rk[i + 1], ib))
+            s_run[2 * d + 1] = (uint16_t)(i + 1);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kJItems; ++u) {
+          const int q = wbase + u * 32 + lane;
+          if (q >= nv) continue;
+          const Key key = Row::key(s_sk[q], ib);
+          if (key < cf || cl < key) continue;
+          const uint32_t w = s_ht[(uint32_t)((uint64_t)key - (uint64_t)cf)];
+          if (w == 0u) continue;
+          if (cnt[u] == 0u) start[u] = (uint32_t)c0 + (w & 0xFFFFu);
+          cnt[u] += (w >> 16) - (w & 0xFFFFu);
+        }
+        continue;
+      }
       // insert the first row of every run of equal keys; keys are distinct, so
       // an occupied slot is never this key and insertion needs no comparison
       for (int i = tid; i < nc; i += kJThreads) {
@@ -371,7 +412,6 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         }
       }
       __syncthreads();
-      const Key cf = Row::key(s_rk[0], ib), cl = Row::key(s_rk[nc - 1], ib);
 #pragma unroll
       for (int u = 0; u < kJItems; ++u) {
         const int q = wbase + u * 32 + lane;
@@ -478,14 +518,19 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   }
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) mysum += __shfl_xor_sync(0xFFFFFFFFu, mysum, o);
-  if (lane == 0) s_wsum[warp] = mysum;
-  const bool multi = __syncthreads_or(mymax > 1u) != 0;  // also publishes s_wsum
+  mymax = __reduce_max_sync(0xFFFFFFFFu, mymax);
+  if (lane == 0) {
+    s_wsum[warp] = mysum;
+    s_wmax[warp] = mymax;
+  }
+  __syncthreads();
   uint64_t C = 0, wpre = 0;
 #pragma unroll
   for (int w = 0; w < kJWarps; ++w) {
     const uint64_t x = s_wsum[w];
     if (w < warp) wpre += x;
     C += x;
+    mymax = max(mymax, s_wmax[w]);  // the tile's largest match count
   }
   // chained scan over all tiles by warp 0: each round trip reads the 32 newest
   // predecessors not yet summed (lane l: tile k - l), sums the run of ready
@@ -540,39 +585,56 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   if (first + C > (uint64_t)capacity) return;  // the host reports TJ_ERR_CAPACITY
 
   // 4. write
-  if (!multi) {
+  if (mymax <= kJDirect) {
     using P = typename PairOf<K>::type;
     const bool vec = (((uintptr_t)out) & (2 * sizeof(K) - 1)) == 0;
     const uint32_t ltm = lanemask_lt_j();
     // R rows of the chunk still in shared memory (the last one) are read
     // there, earlier ones from global memory
-    const int64_t cres = onchip && nchunks > 0 ? (nchunks - 1) * kRCap : INT64_MAX;
-    uint64_t off = first + wpre;
+    const uint32_t cres = onchip && nchunks > 0 ? (uint32_t)((nchunks - 1) * kRCap) : ~0u;
+    const bool single = mymax <= 1u;
+    K* __restrict__ const o_w = out + 2 * (first + wpre);  // the warp's first pair
+    uint32_t off = 0;  // (a warp has at most 32 kJItems kJDirect pairs)
 #pragma unroll
     for (int u = 0; u < kJItems; ++u) {
-      const uint32_t m = __ballot_sync(0xFFFFFFFFu, cnt[u] != 0u);
-      if (cnt[u] != 0u) {
-        const uint64_t o = off + __popc(m & ltm);
-        const int64_t st0 = (int64_t)start[u];
-        K sid, rid;
-        if constexpr (!kIds) {
-          sid = word_id<K>(s_sk[wbase + u * 32 + lane], f);
-          rid = st0 >= cres ? word_id<K>(s_rk[st0 - cres], f) : rid_g(st0);
-        } else {
-          sid = id_of(s_sv[wbase + u * 32 + lane]);
-          rid = st0 >= cres ? id_of(s_rv[st0 - cres]) : rid_g(st0);
+      const uint32_t c = cnt[u];
+      uint32_t before, all;  // pairs of lower lanes, of the warp's 32 rows
+      if (single) {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, c != 0u);
+        before = __popc(m & ltm);
+        all = __popc(m);
+      } else {
+        uint32_t x = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+          if (lane >= o) x += y;
         }
-        if (vec) {
-          P pr;
-          pr.x = rid;
-          pr.y = sid;
-          *reinterpret_cast<P*>(out + 2 * o) = pr;
-        } else {
-          out[2 * o] = rid;
-          out[2 * o + 1] = sid;
+        before = x - c;
+        all = __shfl_sync(0xFFFFFFFFu, x, 31);
+      }
+      if (c != 0u) {
+        K* __restrict__ o = o_w + 2 * (off + before);
+        const uint32_t st0 = start[u];
+        K sid;
+        if constexpr (!kIds) sid = word_id<K>(s_sk[wbase + u * 32 + lane], f);
+        else sid = id_of(s_sv[wbase + u * 32 + lane]);
+        for (uint32_t r = st0; r < st0 + c; ++r, o += 2) {
+          K rid;
+          if constexpr (!kIds) rid = r >= cres ? word_id<K>(s_rk[r - cres], f) : rid_g(r);
+          else rid = r >= cres ? id_of(s_rv[r - cres]) : rid_g(r);
+          if (vec) {
+            P pr;
+            pr.x = rid;
+            pr.y = sid;
+            *reinterpret_cast<P*>(o) = pr;
+          } else {
+            o[0] = rid;
+            o[1] = sid;
+          }
         }
       }
-      off += __popc(m);
+      off += all;
     }
   } else {
     // many matches: per-row counts -> exclusive offsets, then each output
