@@ -517,13 +517,6 @@ void set_job_buffers(RadixJob<K>& j, const K* in_k, const K* in_v, K* ak, K* av,
 // rows: the ids' range is known from a sample (two rows a tile), so the window
 // the spare bits allow is centred on it; the folding pass checks every row, and
 // one outside sends the call back to separate columns (kErrFold).
-struct Fold {
-  bool on = false;
-  bool wide = false;  // wide rows instead: the key as it is and a 32-bit id
-  uint64_t wlo = 0, ilo = 0;
-  int ib = 0;
-};
-
 template <typename K>
 Fold make_fold(uint64_t lo, int key_bits, unsigned long long id_min_u,
                unsigned long long id_max_u, bool wide_too) {
@@ -572,6 +565,29 @@ Plan make_word_plan(uint64_t lo, uint64_t range, bool even, int max_digit, int m
     }
   }
   return make_plan(lo, range, false, max_digit, kb == 0 ? 0 : best);
+}
+
+// Sorts by a key prefix: three digits of the key's leading 24 or 27 bits, then
+// the runs of equal prefixes (k_runs). Worth it from five passes on; keys a
+// sample finds nearly unique by that prefix (kPrefPairs pairs among 2048 rows
+// mean runs of 1 + n / 10^6 rows or so as the average row sees them).
+constexpr int64_t kPrefMinRows = (int64_t)1 << 17;
+constexpr int kPrefMinBits = 37;
+constexpr uint32_t kPrefPairs = 2;
+int prefix_digit(int64_t n) { return n <= (int64_t)1 << 22 ? 8 : 9; }
+
+Plan make_prefix_plan(uint64_t lo, int key_bits, int64_t n) {
+  Plan p;
+  const int w = prefix_digit(n);
+  p.lo = lo;
+  p.key_bits = key_bits;
+  p.passes = 3;
+  p.max_bits = w;
+  for (int i = 0; i < 3; ++i) {
+    p.shift[i] = key_bits - (3 - i) * w;
+    p.bits[i] = w;
+  }
+  return p;
 }
 
 // A plan's digits as positions within words whose keys start at bit ib,
@@ -2495,8 +2511,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
 // do wide rows (a pass that unfolds does not run after a row failed to fold).
 template <typename K>
 tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f,
-                     RadixJob<K>* d_jobs, uint32_t* d_counters, int* d_err, size_t ctl_bytes,
-                     tj_stats& stats, Tracer& tr, cudaStream_t st) {
+                     bool prefix, RadixJob<K>* d_jobs, uint32_t* d_counters, int* d_err,
+                     size_t ctl_bytes, int* h_err, tj_stats& stats, Tracer& tr, cudaStream_t st) {
   const double w = (double)sizeof(K);
   const int P = plan.passes;
   const int items = word_items(n);
@@ -2527,7 +2543,9 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
   hj[1].lookback = big.at<uint32_t>(o_lb);
   hj[1].lb_stride = regions ? lb_words : 0;
   auto folds = [&](int p) { return p == 0 || (turns && (p & 1) == 0); };
-  auto unfolds = [&](int p) { return p == P - 1 || (turns && (p & 1) == 1); };
+  // (a prefix sort has an odd number of passes: its words end in scratch)
+  auto unfolds = [&](int p) { return prefix ? turns && (p & 1) == 1
+                                            : p == P - 1 || (turns && (p & 1) == 1); };
   uint64_t* a = big.at<uint64_t>(o_a);
   uint64_t* b = big.at<uint64_t>(o_b);
   for (int p = 0; p < P; ++p) {
@@ -2553,6 +2571,21 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
                              unfolds(p), f.ib >= 32, f.wide, items, false, d_counters + p, d_err,
                              st));
     tr.end();
+  }
+  if constexpr (sizeof(K) == 8) {
+    if (prefix) {
+      tr.begin("runs", ((f.wide ? 12.0 : 8.0) + 16.0) * n);
+      TJ_CUDA(launch_runs(a, big.at<uint32_t>(o_ai), n, f, plan.shift[0], true, keys, ids, d_err,
+                          st));
+      tr.end();
+    }
+  }
+  TJ_CUDA(get_small(h_err, d_err, sizeof(int), st));
+  TJ_CUDA(sync_stream(st));
+  if constexpr (sizeof(K) == 8) {
+    if (*h_err == kErrRuns)  // back into columns: a stable order by the prefix
+      TJ_CUDA(launch_runs(a, big.at<uint32_t>(o_ai), n, f, plan.shift[0], false, keys, ids, d_err,
+                          st));
   }
   return TJ_OK;
 }
@@ -2593,6 +2626,15 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
   TJ_CUDA(launch_stats<K>(d_jobs, 1, tiles, d_stats, st));
   tr.end();
   KeyStats hs;
+  uint32_t pref_pairs = ~0u;
+  if constexpr (sizeof(K) == 8) {
+    if (n >= kPrefMinRows) {
+      uint32_t* d_pairs = ctl.at<uint32_t>(o_misc + 128);
+      TJ_CUDA(launch_prefix_sample(keys, n, d_stats, 3 * prefix_digit(n), kPrefMinBits, d_pairs,
+                                   st));
+      TJ_CUDA(get_small(&pref_pairs, d_pairs, sizeof(pref_pairs), st));
+    }
+  }
   TJ_CUDA(get_small(&hs, d_stats, sizeof(hs), st));
   TJ_CUDA(sync_stream(st));
   tr.flush();
@@ -2613,24 +2655,29 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
                            ? make_word_plan(plan.lo, range_of<K>(lo, hi),
                                             sizeof(K) == 4 || fold.wide, max_digit_bits<K>(), 2)
                            : plan;
-    stats.radix_passes = wplan.passes;
-    stats.digit_bits = wplan.max_bits;
-    s = sort_words<K>(keys, ids, n, wplan, fold, d_jobs, d_counters, d_err, cc.off, stats, tr2,
-                      st);
-    if (s != TJ_OK) return s;
+    bool prefix = wplan.passes >= 5 && plan.key_bits >= kPrefMinBits && pref_pairs <= kPrefPairs;
     int h_err = 0;
-    TJ_CUDA(get_small(&h_err, d_err, sizeof(int), st));
-    TJ_CUDA(sync_stream(st));
-    if (h_err == 0) {
-      tr2.flush();
-      g_stats = stats;
-      return TJ_OK;
+    while (true) {
+      const Plan use = prefix ? make_prefix_plan(plan.lo, plan.key_bits, n) : wplan;
+      stats.radix_passes = use.passes;
+      stats.digit_bits = use.max_bits;
+      s = sort_words<K>(keys, ids, n, use, fold, prefix, d_jobs, d_counters, d_err, cc.off, &h_err,
+                        stats, tr2, st);
+      if (s != TJ_OK) return s;
+      if (h_err == 0) {
+        tr2.flush();
+        g_stats = stats;
+        return TJ_OK;
+      }
+      if (h_err != kErrFold && h_err != kErrRuns)
+        return set_err((tj_status)h_err, "device reported %d", h_err);
+      TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
+      if (h_err == kErrFold) break;
+      prefix = false;  // a long run was out of order
     }
-    if (h_err != kErrFold) return set_err((tj_status)h_err, "device reported %d", h_err);
     // an id outside the window of the sampled ones: the columns are untouched
     stats.radix_passes = plan.passes;
     stats.digit_bits = plan.max_bits;
-    TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
   }
   const int64_t bins_max = (int64_t)1 << plan.max_bits;
   // onesweep tiles (narrow digits: the wider tile); the histogram keeps kTile

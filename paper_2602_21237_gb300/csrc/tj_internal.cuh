@@ -170,6 +170,10 @@ struct RadixJob {
 // separate columns.
 constexpr int kErrFold = 101;
 
+// A long run of equal key prefixes is not in order (k_runs): the call sorts by
+// every digit.
+constexpr int kErrRuns = 102;
+
 // Kinds of onesweep pass: a sort digit of key - lo, a route by the cut table
 // (batch = number of cuts <= key), a route by equal-width ranges.
 constexpr int kModeSort = 0;
@@ -184,6 +188,14 @@ struct KeyStats {
   unsigned long long max_u;
   unsigned long long id_min_u;
   unsigned long long id_max_u;
+};
+
+// Folded rows (tj_word.cu), as the host lays them out: see make_fold.
+struct Fold {
+  bool on = false;
+  bool wide = false;  // wide rows instead: the key as it is and a 32-bit id
+  uint64_t wlo = 0, ilo = 0;
+  int ib = 0;
 };
 
 // Layout of the rows a join kernel reads: separate key and id columns (ib = 0)
@@ -392,6 +404,20 @@ cudaError_t launch_wsweep(const RadixJob<K>* d_jobs, int num_jobs, int64_t total
                           int max_bits, int mode, bool raw_in, bool raw_out, bool hi, bool wide,
                           int items, bool guard, uint32_t* d_tile_counter, int* d_err,
                           cudaStream_t st, const int32_t* d_tile_job = nullptr);
+
+// Sorts by a key prefix (k_prefix_sample, k_runs)
+constexpr int kPrefSample = 2048;  // rows of the sample
+constexpr int kRunThreads = 256;
+constexpr int kRunTile = 4096;     // rows a CTA writes
+constexpr int kRunMax = 256;       // longest run put in order
+static_assert((kRunTile + 2 * kRunMax) % kRunThreads == 0, "whole rounds of loads");
+// *d_pairs += pairs of equal `prefix_bits`-bit prefixes in a sample of the keys
+// (n >= kPrefSample), unless their range has fewer than min_bits bits
+cudaError_t launch_prefix_sample(const int64_t* keys, int64_t n, const KeyStats* d_stats,
+                                 int prefix_bits, int min_bits, uint32_t* d_pairs,
+                                 cudaStream_t st);
+cudaError_t launch_runs(const uint64_t* rows, const uint32_t* ids, int64_t n, const Fold& f, int s,
+                        bool fix, int64_t* out_k, int64_t* out_v, int* d_err, cudaStream_t st);
 
 // ---- launchers (tj_join.cu) -------------------------------------------------
 cudaError_t join_init_attributes();
