@@ -2,7 +2,8 @@
 // join aligns R(A, B, C) and S(B, D, E) on B and yields (r_id, s_id) pairs;
 // k_gather_pairs then reads, for every pair, each requested column of R at
 // r_id and of S at s_id and writes it to the pair's position of an output
-// column.  One pass over the pairs; up to kGatherCols columns per launch.
+// column.  Up to kGatherCols columns per pass over the pairs.
+// Launches follow what L2 can hold of the columns (launch_gather_pairs).
 //
 // Work per pair: one 2w-byte pair read (coalesced), and per column one
 // element read at a data-dependent row (a 32-byte sector per element unless
@@ -24,14 +25,14 @@ __device__ __forceinline__ void load_pair(const I* p, int64_t i, I& r, I& s);
 template <>
 __device__ __forceinline__ void load_pair<int32_t>(const int32_t* p, int64_t i, int32_t& r,
                                                    int32_t& s) {
-  const int2 v = __ldg(reinterpret_cast<const int2*>(p) + i);
+  const int2 v = __ldcs(reinterpret_cast<const int2*>(p) + i);  // (leaves L2 to the columns)
   r = v.x;
   s = v.y;
 }
 template <>
 __device__ __forceinline__ void load_pair<int64_t>(const int64_t* p, int64_t i, int64_t& r,
                                                    int64_t& s) {
-  const longlong2 v = __ldg(reinterpret_cast<const longlong2*>(p) + i);
+  const longlong2 v = __ldcs(reinterpret_cast<const longlong2*>(p) + i);
   r = v.x;
   s = v.y;
 }
@@ -46,7 +47,7 @@ __device__ __forceinline__ void gather_col(const GatherCol& c, const int64_t (&r
   for (int u = 0; u < kGatherRows; ++u) v[u] = row[u] >= 0 ? __ldg(src + row[u]) : E(0);
 #pragma unroll
   for (int u = 0; u < kGatherRows; ++u)
-    if (row[u] >= 0) dst[at[u]] = v[u];
+    if (row[u] >= 0) __stcs(dst + at[u], v[u]);
 }
 
 // pairs[i] = (r_id, s_id), i < n; an id outside [0, rows of its side) sets
@@ -100,7 +101,45 @@ cudaError_t launch_gather_pairs(const I* pairs, int64_t n, int64_t n_r, int64_t 
   const int64_t per_block = (int64_t)kGatherThreads * kGatherRows;
   const int64_t want = (n + per_block - 1) / per_block;
   const int64_t grid = std::min<int64_t>(want, (int64_t)std::max(1, sms) * 8);
-  k_gather_pairs<I><<<(unsigned)grid, kGatherThreads, 0, st>>>(pairs, n, n_r, n_s, a, d_err);
+  // Columns share a launch up to one and a half times L2 together; a larger one is
+  // gathered by itself, the pairs being read again, where L2 still holds a good
+  // part of it; columns beyond kFarL2 times L2 gain nothing from that and go
+  // together.  (4x10^7 random 8-byte elements take 0.20, 0.45, 0.72 and 1.04 ms
+  // from a column of 80, 160, 320 and 3200 MB, alone; L2 is 129 MB. Two payload
+  // columns of 8 and 4 bytes a row on either side of a join of 10^7 x 4x10^7 rows:
+  // 2.03 ms in one launch, now 1.81.)
+  constexpr int64_t kFarL2 = 4;
+  int dev = 0, l2 = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+  if (e != cudaSuccess) return e;
+  auto bytes = [&](const GatherCol& c) { return (c.side ? n_s : n_r) * c.bytes; };
+  GatherArgs g, far;  // the launch being filled, the columns that go together
+  g.n = far.n = 0;
+  int64_t held = 0;
+  auto flush = [&](GatherArgs& x) {
+    if (x.n > 0)
+      k_gather_pairs<I><<<(unsigned)grid, kGatherThreads, 0, st>>>(pairs, n, n_r, n_s, x, d_err);
+    x.n = 0;
+  };
+  // (one side's columns, then the other's)
+  for (int side = 0; side < 2; ++side)
+    for (int c = 0; c < a.n; ++c) {
+      if ((a.c[c].side != 0) != (side != 0)) continue;
+      const int64_t b = bytes(a.c[c]);
+      if (b > kFarL2 * l2) {
+        far.c[far.n++] = a.c[c];
+        continue;
+      }
+      if (2 * (held + b) > 3 * (int64_t)l2) {
+        flush(g);
+        held = 0;
+      }
+      g.c[g.n++] = a.c[c];
+      held += b;
+    }
+  flush(g);
+  flush(far);
   return cudaGetLastError();
 }
 
