@@ -808,7 +808,6 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
   const size_t o_hist = bc.add<uint32_t>(2 * kMaxPasses * kMaxBins);
   const size_t o_lb = bc.add<uint32_t>((size_t)(tiles_r + tiles_s) * bins_max);
   const size_t o_tiles = bc.add<JTile<K>>(jtiles);
-  const size_t o_jlb = bc.add<uint64_t>(jtiles);
   const size_t need = bc.off + cc.off;
   int router = opts.router;
   if (router == TJ_ROUTE_AUTO) {
@@ -850,7 +849,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     const int64_t wtile = (int64_t)kWThreads * items;
     const int64_t wt_r = ceil_div(nr, wtile), wt = wt_r + ceil_div(ns, wtile);
     const int64_t lb_words = wt << wp.max_bits;
-    size_t o_a, o_b, o_ai, o_bi, o_wt, o_whist, o_wjlb, o_wlb;
+    size_t o_a, o_b, o_ai, o_bi, o_wt, o_whist, o_wlb;
     auto lay_out = [&](bool per_pass) -> size_t {
       Carve wc;
       o_a = wc.add<uint64_t>((size_t)(nr + ns));
@@ -859,7 +858,6 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
       o_bi = wc.add<uint32_t>(fold.wide && wp.passes > 1 ? (size_t)(nr + ns) : 0);
       o_wt = wc.add<JTile<K>>(jtiles);
       o_whist = wc.add<uint32_t>((size_t)2 * wp.passes << wp.max_bits);
-      o_wjlb = wc.add<uint64_t>(jtiles);
       o_wlb = wc.add<uint32_t>((size_t)(per_pass ? wp.passes : 1) * lb_words);
       return wc.off;
     };
@@ -931,8 +929,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     JTile<K>* d_tiles = big.at<JTile<K>>(o_wt);
     TJ_CUDA(launch_tile_ranges<K>(d_jj, 1, jtiles, d_tiles, st, nullptr, fmt, d_err));
     tr.begin("join", rowb * (nr + ns));
-    TJ_CUDA(launch_join<K>(jtiles, d_tiles, big.at<uint64_t>(o_wjlb), d_counters + kMaxPasses,
-                           out, cap, nullptr, nullptr, d_total, d_err, st, fmt));
+    TJ_CUDA(launch_join<K>(jtiles, d_tiles, d_counters + kMaxPasses, out, cap, nullptr, nullptr, d_total, d_err, st, fmt));
     tr.end();
     int64_t h_total = 0;
     int h_err = 0;
@@ -1015,12 +1012,10 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
   jj.ns = ns;
   jj.tile0 = 0;
   JTile<K>* d_tiles = big.at<JTile<K>>(o_tiles);
-  uint64_t* d_jlb = big.at<uint64_t>(o_jlb);
   TJ_CUDA(put_small(d_jj, &jj, sizeof(jj), st));
   TJ_CUDA(launch_tile_ranges<K>(d_jj, 1, jtiles, d_tiles, st));
-  TJ_CUDA(cudaMemsetAsync(d_jlb, 0, jtiles * sizeof(uint64_t), st));
   tr.begin("join", 2.0 * w * (nr + ns));
-  TJ_CUDA(launch_join<K>(jtiles, d_tiles, d_jlb, d_counters + kMaxPasses, out, cap, nullptr,
+  TJ_CUDA(launch_join<K>(jtiles, d_tiles, d_counters + kMaxPasses, out, cap, nullptr,
                          nullptr, d_total, d_err, st));
   tr.end();
   int64_t h_misc[2] = {0, 0};
@@ -1848,7 +1843,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     q.lb = rtiles * bins * 4;
     const int64_t buf = (int64_t)std::min(q.plan.passes, 1) * (q.nr + q.ns);
     const int64_t rest =
-        ceil_div(q.ns, kJTile) * (int64_t)(sizeof(JTile<K>) + 12) + rtiles * 4 + 4096;
+        ceil_div(q.ns, kJTile) * (int64_t)(sizeof(JTile<K>) + 4) + rtiles * 4 + 4096;
     q.ask = buf * 2 * (int64_t)sizeof(K) + rest + q.lb * q.np;
     q.ws = buf * (words ? 8 : 2 * (int64_t)sizeof(K)) + rest;
   };
@@ -2100,7 +2095,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     int64_t items;        // fused
     bool any_multi;
     double rows;
-    size_t o_jlb, o_ilb, o_kbl, o_kbt, o_items;
+    size_t o_ilb, o_kbl, o_kbt, o_items;
     int base;  // index of its first output index in d_gbase
   };
   struct GroupPlan {
@@ -2219,8 +2214,6 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
         r.o_ilb = gc.add<uint64_t>((size_t)std::max<int64_t>(r.items, 1));
         r.o_kbl = gc.add<uint32_t>((size_t)std::max<int64_t>(kbt, 1) * kFKeys);
         r.o_kbt = gc.add<uint32_t>((size_t)std::max<int64_t>(kbs, 1) * kFKeys);
-      } else if (!r.cross) {
-        r.o_jlb = gc.add<uint64_t>((size_t)std::max<int64_t>(r.jtiles, 1));
       }
     }
     gp.zero_bytes = gc.off - gp.o_zero;
@@ -2473,7 +2466,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       } else {
         if (!whole) tr.begin("join", rowb * r.rows, gs);
         TJ_CUDA(launch_join<K>(r.jtiles, lw.at<JTile<K>>(gp.o_jt) + r.jt0,
-                               lw.at<uint64_t>(r.o_jlb), cnt, out, cap, d_gbase + r.base, nullptr,
+                               cnt, out, cap, d_gbase + r.base, nullptr,
                                d_gbase + r.base + 1, d_err, gs, fmt));
         if (!whole) tr.end();
       }
@@ -2996,7 +2989,6 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   const size_t o_hist = bc.add<uint32_t>((size_t)std::max<int64_t>(hist_words, 1));
   const size_t o_lb = bc.add<uint32_t>((size_t)std::max<int64_t>(lb_words, 1));
   const size_t o_jt = bc.add<JTile<K>>((size_t)std::max<int64_t>(jtiles, 1));
-  const size_t o_jlb = bc.add<uint64_t>((size_t)std::max<int64_t>(jtiles, 1));
   const size_t o_tmap = bc.add<int32_t>((size_t)std::max<int64_t>(tiles, 1));
   const size_t o_jmap = bc.add<int32_t>((size_t)std::max<int64_t>(jtiles, 1));
   // (word passes: a second view of the jobs, digits of words, and its tile map)
@@ -3099,10 +3091,7 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   }
   step(launch_tile_ranges<K>(d_jj, (int)nj, jtiles, big.at<JTile<K>>(o_jt), st, d_jmap, fmt,
                              words ? d_err : nullptr));
-  step(cudaMemsetAsync(big.at<uint64_t>(o_jlb), 0,
-                       (size_t)std::max<int64_t>(jtiles, 1) * sizeof(uint64_t), st));
-  step(launch_join<K>(jtiles, big.at<JTile<K>>(o_jt), big.at<uint64_t>(o_jlb),
-                      d_counters + kMaxPasses, out, cap, nullptr, d_out_off, d_total, d_err, st,
+  step(launch_join<K>(jtiles, big.at<JTile<K>>(o_jt), d_counters + kMaxPasses, out, cap, nullptr, d_out_off, d_total, d_err, st,
                       fmt));
   step(launch_fix_job_out<K>(d_jj, (int)nj, jtiles, d_out_off, d_total, st));
   if (use_graph) {

@@ -64,11 +64,6 @@ __device__ __forceinline__ void st_vol_v4(uint32_t* p, uint4 v) {
                "r"(v.z), "r"(v.w)
                : "memory");
 }
-__device__ __forceinline__ uint64_t ld_vol_u64(const uint64_t* p) {
-  uint64_t v;
-  asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ void st_vol_u64(uint64_t* p, uint64_t v) {
   asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -644,41 +639,11 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
   }
   // 4. chained scan over the group's items (warp 0): the tile's first pair
   if (warp == 0) {
-    uint64_t* mine = item_lb + ii;
-    uint64_t prefix = 0;
-    if (ii == 0) {
-      if (lane == 0) st_vol_u64(mine, kFlagInc64 | (cnt_tile & kValMask64));
-    } else {
-      if (lane == 0) st_vol_u64(mine, kFlagAgg64 | (cnt_tile & kValMask64));
-      int64_t k = ii - 1;
-      int spins = 0;
-      while (true) {
-        const int64_t idx = k - lane;
-        const uint64_t v = idx >= 0 ? ld_vol_u64(item_lb + idx) : kFlagInc64;
-        const uint64_t f = v & ~kValMask64;
-        const uint32_t notready = __ballot_sync(0xFFFFFFFFu, f == 0ull);
-        const uint32_t inc = __ballot_sync(0xFFFFFFFFu, f == kFlagInc64);
-        const int first_nr = notready ? __ffs(notready) - 1 : 32;
-        const int first_inc = inc ? __ffs(inc) - 1 : 32;
-        const int take = first_inc < first_nr ? first_inc + 1 : first_nr;
-        uint64_t y = lane < take ? (v & kValMask64) : 0ull;
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) y += __shfl_xor_sync(0xFFFFFFFFu, y, o);
-        prefix += y;
-        if (first_inc < first_nr) break;
-        k -= take;
-        if (take == 0) {
-          if (++spins > kSpinLimit) {
-            if (lane == 0) atomicExch(err, (int)TJ_ERR_TIMEOUT);
-            break;
-          }
-          __nanosleep(32);
-        } else {
-          spins = 0;
-        }
-      }
-      if (lane == 0) st_vol_u64(mine, kFlagInc64 | ((prefix + cnt_tile) & kValMask64));
-    }
+    if (lane == 0)
+      st_vol_u64(item_lb + ii, (ii == 0 ? kFlagInc64 : kFlagAgg64) | (cnt_tile & kValMask64));
+    const uint64_t prefix = chain_prefix<1>(item_lb, ii, err);
+    if (lane == 0 && ii != 0)
+      st_vol_u64(item_lb + ii, kFlagInc64 | ((prefix + cnt_tile) & kValMask64));
     if (lane == 0) {
       const int64_t gb = out_base ? *out_base : 0;
       S.s_base = (uint64_t)gb + prefix;

@@ -14,7 +14,8 @@
 //                        the chunk's keys are dense, else an open-addressing
 //                        hash table filled with shared-memory atomicCAS;
 //                     3. probe it once per S row -> match count, run start;
-//                     4. a decoupled look-back over all tiles of all jobs gives
+//                     4. a decoupled look-back over all tiles of all jobs
+//                        (the words in the tiles' descriptors) gives
 //                        the tile's first output index;
 //                     5. write the pairs, ordered by key, S position, R
 //                        position, if they fit the caller's capacity.
@@ -22,6 +23,7 @@
 //                   against R) search a strided sample of the range on chip,
 //                   then one stride of R in global memory.
 #include "tj_internal.cuh"
+#include "tj_warp.cuh"
 
 namespace tj {
 
@@ -99,17 +101,6 @@ __host__ __device__ constexpr int tab_slots() {
   return W == 0 ? kHTSlots : 2 * kHTSlots;
 }
 
-__device__ __forceinline__ uint32_t lanemask_lt_j() {
-  uint32_t m;
-  asm volatile("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-  return m;
-}
-
-__device__ __forceinline__ uint64_t ld_volatile_u64(const uint64_t* p) {
-  uint64_t v;
-  asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ void st_volatile_u64(uint64_t* p, uint64_t v) {
   asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -186,17 +177,17 @@ __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
     d.nrr = b - res;
     d.nv = (int32_t)(row1 - row0);
     d.j = j;
-    d.pad = 0;
+    d.chain = 0;
     tiles[t] = d;
   }
 }
 
 // ---------------------------------------------------------------------------
 #ifndef TJ_JTHREADS
-#define TJ_JTHREADS 256
+#define TJ_JTHREADS 512
 #endif
 #ifndef TJ_JMINB
-#define TJ_JMINB 4
+#define TJ_JMINB 2
 #endif
 constexpr int kJThreads = TJ_JTHREADS;          // threads per join CTA
 constexpr int kJWarps = kJThreads / 32;
@@ -281,8 +272,7 @@ __device__ __forceinline__ K* join_copy_async(K* dst, const K* __restrict__ src,
 // Output order: key, then S position, then R position.
 template <typename K, int W>
 __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
-    k_join(int64_t total_tiles, const JTile<K>* __restrict__ tiles, WordFmt f,
-           uint64_t* __restrict__ lookback, uint32_t* __restrict__ tile_counter,
+    k_join(int64_t total_tiles, JTile<K>* tiles, WordFmt f, uint32_t* __restrict__ tile_counter,
            K* __restrict__ out, int64_t capacity, const int64_t* __restrict__ out_base,
            int64_t* __restrict__ job_out, int64_t* __restrict__ total, int* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -532,45 +522,12 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
     C += x;
     mymax = max(mymax, s_wmax[w]);  // the tile's largest match count
   }
-  // chained scan over all tiles by warp 0: each round trip reads the 32 newest
-  // predecessors not yet summed (lane l: tile k - l), sums the run of ready
-  // words up to the first inclusive one, and stops there
+  // chained scan over all tiles by warp 0 (the first tile is inclusive at once)
   if (warp == 0) {
-    uint64_t* mine = lookback + t;
-    uint64_t prefix = 0;
-    if (t == 0) {
-      if (lane == 0) st_volatile_u64(mine, kFlagInc64 | (C & kValMask64));
-    } else {
-      if (lane == 0) st_volatile_u64(mine, kFlagAgg64 | (C & kValMask64));
-      int64_t k = t - 1;  // newest predecessor not yet summed
-      int spins = 0;
-      while (true) {
-        const int64_t idx = k - lane;
-        const uint64_t v = idx >= 0 ? ld_volatile_u64(lookback + idx) : kFlagInc64;
-        const uint64_t f = v & ~kValMask64;
-        const uint32_t notready = __ballot_sync(0xFFFFFFFFu, f == 0ull);
-        const uint32_t inc = __ballot_sync(0xFFFFFFFFu, f == kFlagInc64);
-        const int first_nr = notready ? __ffs(notready) - 1 : 32;
-        const int first_inc = inc ? __ffs(inc) - 1 : 32;
-        const int take = first_inc < first_nr ? first_inc + 1 : first_nr;  // lanes summed
-        uint64_t x = lane < take ? (v & kValMask64) : 0ull;
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-        prefix += x;
-        if (first_inc < first_nr) break;
-        k -= take;
-        if (take == 0) {
-          if (++spins > kSpinLimit) {
-            if (lane == 0) atomicExch(err, (int)TJ_ERR_TIMEOUT);
-            break;
-          }
-          __nanosleep(32);
-        } else {
-          spins = 0;
-        }
-      }
-      if (lane == 0) st_volatile_u64(mine, kFlagInc64 | ((prefix + C) & kValMask64));
-    }
+    uint64_t* const mine = &tiles[t].chain;
+    if (lane == 0) st_volatile_u64(mine, (t == 0 ? kFlagInc64 : kFlagAgg64) | (C & kValMask64));
+    const uint64_t prefix = chain_prefix<(int)(sizeof(JTile<K>) / 8)>(&tiles[0].chain, t, err);
+    if (lane == 0 && t != 0) st_volatile_u64(mine, kFlagInc64 | ((prefix + C) & kValMask64));
     if (lane == 0) {
       s_base = prefix;
       if (lt == 0 && job_out) job_out[j] = (int64_t)prefix;
@@ -588,7 +545,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   if (mymax <= kJDirect) {
     using P = typename PairOf<K>::type;
     const bool vec = (((uintptr_t)out) & (2 * sizeof(K) - 1)) == 0;
-    const uint32_t ltm = lanemask_lt_j();
+    const uint32_t ltm = lanemask_lt();
     // R rows of the chunk still in shared memory (the last one) are read
     // there, earlier ones from global memory
     const uint32_t cres = onchip && nchunks > 0 ? (uint32_t)((nchunks - 1) * kRCap) : ~0u;
@@ -768,14 +725,13 @@ cudaError_t launch_fill_join_tile_job(const JoinJob<K>* d_jobs, int num_jobs, in
 }
 
 template <typename K>
-cudaError_t launch_join(int64_t total_tiles, const JTile<K>* d_tiles, uint64_t* d_lookback,
-                        uint32_t* d_tile_counter, K* out, int64_t capacity,
+cudaError_t launch_join(int64_t total_tiles, JTile<K>* d_tiles, uint32_t* d_tile_counter, K* out, int64_t capacity,
                         const int64_t* d_out_base, int64_t* d_job_out, int64_t* d_total,
                         int* d_err, cudaStream_t st, WordFmt f) {
   if (total_tiles <= 0) return cudaSuccess;
 #define TJ_JOIN(W)                                                                            \
   k_join<K, W><<<(unsigned)total_tiles, kJThreads, join_smem_bytes<K, W>(), st>>>(            \
-      total_tiles, d_tiles, f, d_lookback, d_tile_counter, out, capacity, d_out_base,         \
+      total_tiles, d_tiles, f, d_tile_counter, out, capacity, d_out_base,         \
       d_job_out, d_total, d_err)
   if (f.wide) {
     if constexpr (sizeof(K) == 8) TJ_JOIN(3);
@@ -912,7 +868,7 @@ cudaError_t join_init_attributes() {
                                              cudaStream_t, const int32_t*, WordFmt, const int*); \
   template cudaError_t launch_fill_join_tile_job<K>(const JoinJob<K>*, int, int32_t*,            \
                                                     cudaStream_t);                              \
-  template cudaError_t launch_join<K>(int64_t, const JTile<K>*, uint64_t*, uint32_t*, K*,        \
+  template cudaError_t launch_join<K>(int64_t, JTile<K>*, uint32_t*, K*,        \
                                       int64_t, const int64_t*, int64_t*, int64_t*, int*,          \
                                       cudaStream_t, WordFmt);                                     \
   template cudaError_t launch_cross<K>(const CrossJob<K>*, int, int64_t, K*, int64_t,            \

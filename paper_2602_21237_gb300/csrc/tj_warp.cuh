@@ -194,4 +194,48 @@ __device__ __forceinline__ void wrank(const D& digit, Half<ITEMS>& rank, C* cnt,
   }
 }
 
+// Decoupled look-back over one 64-bit word a tile (STRIDE words apart), by one
+// warp: the sum of the words before tile t back to the first inclusive one. Each
+// round trip reads the 32 newest predecessors not yet summed and sums the run of
+// ready words; the sum of 62-bit words is three sums of 21 bits (redux), shorter
+// than ten shuffles in a wait that every later tile inherits. Bounded wait:
+// *err = TJ_ERR_TIMEOUT.
+template <int STRIDE>
+__device__ __forceinline__ uint64_t chain_prefix(const uint64_t* words, int64_t t, int* err) {
+  const int lane = threadIdx.x & 31;
+  uint64_t prefix = 0;
+  int64_t k = t - 1;  // newest predecessor not yet summed
+  int spins = 0;
+  bool done = t == 0;
+  while (!done) {
+    const int64_t i = k - lane;
+    uint64_t v = kFlagInc64;
+    if (i >= 0)
+      asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(words + i * STRIDE) : "memory");
+    const uint64_t f = v & ~kValMask64;
+    const uint32_t notready = __ballot_sync(0xFFFFFFFFu, f == 0ull);
+    const uint32_t inc = __ballot_sync(0xFFFFFFFFu, f == kFlagInc64);
+    const int first_nr = notready ? __ffs(notready) - 1 : 32;
+    const int first_inc = inc ? __ffs(inc) - 1 : 32;
+    done = first_inc < first_nr;
+    const int take = done ? first_inc + 1 : first_nr;  // lanes summed
+    const uint64_t x = lane < take ? v & kValMask64 : 0ull;
+    const uint32_t s0 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)x & 0x1FFFFFu);
+    const uint32_t s1 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(x >> 21) & 0x1FFFFFu);
+    const uint32_t s2 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(x >> 42));
+    prefix += (uint64_t)s0 + ((uint64_t)s1 << 21) + ((uint64_t)s2 << 42);
+    k -= take;
+    if (take != 0) {
+      spins = 0;
+    } else {
+      if (++spins > kSpinLimit) {
+        if (lane == 0) atomicExch(err, (int)TJ_ERR_TIMEOUT);
+        break;
+      }
+      __nanosleep(32);
+    }
+  }
+  return prefix;
+}
+
 }  // namespace tj

@@ -11,7 +11,7 @@ from gpu_util import DEV, assert_pairs_equal, np_of
 
 pytestmark = pytest.mark.gpu
 
-SMALL, LARGE = 3072, 8192  # rows of the two word tiles
+SMALL, LARGE = 4096, 8192  # rows of the two word tiles
 
 
 def sorted_as_oracle(keys, ids):
