@@ -381,24 +381,8 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         const Key key = Row::key(s_rk[i], ib);
         if (i == 0 || key != Row::key(s_rk[i - 1], ib)) {
           uint32_t h = ht_hash(key);
-          while (atomicCAS(&s_ht[h], kHTEmpty, (uint32_t)i | 0xFFFF0000u) != kHTEmpty)
+          while (atomicCAS(&s_ht[h], kHTEmpty, (uint32_t)i + 1u) != kHTEmpty)
             h = (h + 1) & (kHTSlots - 1);
-        }
-      }
-      __syncthreads();
-      // the last row of every run records the run's end
-      for (int i = tid; i < nc; i += kJThreads) {
-        const Key key = Row::key(s_rk[i], ib);
-        if (i == nc - 1 || key != Row::key(s_rk[i + 1], ib)) {
-          uint32_t h = ht_hash(key);
-          while (true) {
-            const uint32_t w = s_ht[h];
-            if (Row::key(s_rk[w & 0xFFFFu], ib) == key) {
-              s_ht[h] = (w & 0xFFFFu) | ((uint32_t)(i + 1) << 16);
-              break;
-            }
-            h = (h + 1) & (kHTSlots - 1);
-          }
         }
       }
       __syncthreads();
@@ -412,10 +396,13 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         while (true) {
           const uint32_t w = s_ht[h];
           if (w == kHTEmpty) break;
-          const uint32_t r0 = w & 0xFFFFu;
+          const int r0 = (int)w - 1;
           if (Row::key(s_rk[r0], ib) == key) {
-            if (cnt[u] == 0u) start[u] = (uint32_t)c0 + r0;
-            cnt[u] += (w >> 16) - r0;
+            // the run's end: as many steps as the row has matches here
+            int e = r0 + 1;
+            while (e < nc && Row::key(s_rk[e], ib) == key) ++e;
+            if (cnt[u] == 0u) start[u] = (uint32_t)(c0 + r0);
+            cnt[u] += (uint32_t)(e - r0);
             break;
           }
           h = (h + 1) & (kHTSlots - 1);
@@ -526,7 +513,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   if (warp == 0) {
     uint64_t* const mine = &tiles[t].chain;
     if (lane == 0) st_volatile_u64(mine, (t == 0 ? kFlagInc64 : kFlagAgg64) | (C & kValMask64));
-    const uint64_t prefix = chain_prefix<(int)(sizeof(JTile<K>) / 8)>(&tiles[0].chain, t, err);
+    const uint64_t prefix = chain_prefix<(int)(sizeof(JTile<K>) / 8), 1>(&tiles[0].chain, t, err);
     if (lane == 0 && t != 0) st_volatile_u64(mine, kFlagInc64 | ((prefix + C) & kValMask64));
     if (lane == 0) {
       s_base = prefix;

@@ -196,11 +196,11 @@ __device__ __forceinline__ void wrank(const D& digit, Half<ITEMS>& rank, C* cnt,
 
 // Decoupled look-back over one 64-bit word a tile (STRIDE words apart), by one
 // warp: the sum of the words before tile t back to the first inclusive one. Each
-// round trip reads the 32 newest predecessors not yet summed and sums the run of
+// round trip reads the 32 WORDS newest predecessors not yet summed and sums the run of
 // ready words; the sum of 62-bit words is three sums of 21 bits (redux), shorter
 // than ten shuffles in a wait that every later tile inherits. Bounded wait:
 // *err = TJ_ERR_TIMEOUT.
-template <int STRIDE>
+template <int STRIDE, int WORDS>
 __device__ __forceinline__ uint64_t chain_prefix(const uint64_t* words, int64_t t, int* err) {
   const int lane = threadIdx.x & 31;
   uint64_t prefix = 0;
@@ -208,18 +208,32 @@ __device__ __forceinline__ uint64_t chain_prefix(const uint64_t* words, int64_t 
   int spins = 0;
   bool done = t == 0;
   while (!done) {
-    const int64_t i = k - lane;
-    uint64_t v = kFlagInc64;
-    if (i >= 0)
-      asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(words + i * STRIDE) : "memory");
-    const uint64_t f = v & ~kValMask64;
-    const uint32_t notready = __ballot_sync(0xFFFFFFFFu, f == 0ull);
-    const uint32_t inc = __ballot_sync(0xFFFFFFFFu, f == kFlagInc64);
-    const int first_nr = notready ? __ffs(notready) - 1 : 32;
-    const int first_inc = inc ? __ffs(inc) - 1 : 32;
-    done = first_inc < first_nr;
-    const int take = done ? first_inc + 1 : first_nr;  // lanes summed
-    const uint64_t x = lane < take ? v & kValMask64 : 0ull;
+    uint64_t v[WORDS];
+#pragma unroll
+    for (int q = 0; q < WORDS; ++q) {
+      const int64_t i = k - 32 * q - lane;
+      v[q] = kFlagInc64;
+      if (i >= 0)
+        asm volatile("ld.volatile.global.u64 %0, [%1];"
+                     : "=l"(v[q])
+                     : "l"(words + i * STRIDE)
+                     : "memory");
+    }
+    uint64_t x = 0;
+    int take = 0;  // words summed
+#pragma unroll
+    for (int q = 0; q < WORDS; ++q) {
+      if (done || take != 32 * q) break;
+      const uint64_t f = v[q] & ~kValMask64;
+      const uint32_t notready = __ballot_sync(0xFFFFFFFFu, f == 0ull);
+      const uint32_t inc = __ballot_sync(0xFFFFFFFFu, f == kFlagInc64);
+      const int first_nr = notready ? __ffs(notready) - 1 : 32;
+      const int first_inc = inc ? __ffs(inc) - 1 : 32;
+      done = first_inc < first_nr;
+      const int n = done ? first_inc + 1 : first_nr;  // lanes summed
+      if (lane < n) x += v[q] & kValMask64;
+      take += n;
+    }
     const uint32_t s0 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)x & 0x1FFFFFu);
     const uint32_t s1 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(x >> 21) & 0x1FFFFFu);
     const uint32_t s2 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(x >> 42));
