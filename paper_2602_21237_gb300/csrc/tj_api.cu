@@ -735,9 +735,12 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     hj[0].ids = ir;
     hj[1].ids = is;
   }
-  TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
-  TJ_CUDA(cudaMemsetAsync(d_stats, 0xFF, 2 * sizeof(KeyStats), st));
-  TJ_CUDA(put_small(d_jobs, hj, sizeof(hj), st));
+  // one transfer sets the whole control block (jobs, statistics, counters): a
+  // small join is a chain of short launches
+  std::vector<unsigned char> img(cc.off, 0);
+  memset(img.data() + o_stats, 0xFF, 2 * sizeof(KeyStats));
+  memcpy(img.data() + o_jobs, hj, sizeof(hj));
+  TJ_CUDA(put_small(ctl.p, img.data(), cc.off, st));
   Tracer tr(st);
   const double w = (double)sizeof(K);
 
@@ -905,8 +908,9 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     jj.sv = res_i[1];
     jj.ns = ns;
     jj.tile0 = 0;
-    TJ_CUDA(put_small(d_jobs, hw, sizeof(hw), st));
-    TJ_CUDA(put_small(d_jj, &jj, sizeof(jj), st));
+    memcpy(img.data() + o_jobs, hw, sizeof(hw));
+    memcpy(img.data() + o_jj, &jj, sizeof(jj));
+    TJ_CUDA(put_small(ctl.p, img.data(), cc.off, st));
     TJ_CUDA(cudaMemsetAsync(big.p + o_whist, 0,
                             (regions ? o_wlb + (size_t)wp.passes * lb_words * 4 : o_wlb) - o_whist,
                             st));
@@ -931,11 +935,11 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     tr.begin("join", rowb * (nr + ns));
     TJ_CUDA(launch_join<K>(jtiles, d_tiles, d_counters + kMaxPasses, out, cap, nullptr, nullptr, d_total, d_err, st, fmt));
     tr.end();
-    int64_t h_total = 0;
-    int h_err = 0;
-    TJ_CUDA(get_small(&h_total, d_total, sizeof(int64_t), st));
-    TJ_CUDA(get_small(&h_err, d_err, sizeof(int), st));
+    int64_t misc[32] = {};  // the error word, the counters, the total
+    TJ_CUDA(get_small(misc, d_err, sizeof(misc), st));
     TJ_CUDA(sync_stream(st));
+    const int64_t h_total = misc[d_total - reinterpret_cast<int64_t*>(d_err)];
+    const int h_err = *reinterpret_cast<const int*>(misc);
     if (h_err == kErrFold) {  // an id outside the window of the sampled ones
       TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
       break;
@@ -2610,26 +2614,31 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
   hj.keys = keys;
   hj.ids = sizeof(K) == 8 ? ids : nullptr;
   hj.n = n;
-  TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
-  TJ_CUDA(cudaMemsetAsync(d_stats, 0xFF, sizeof(KeyStats), st));
-  TJ_CUDA(put_small(d_jobs, &hj, sizeof(hj), st));
+  std::vector<unsigned char> img(cc.off, 0);  // one transfer sets the control block
+  memset(img.data() + o_stats, 0xFF, sizeof(KeyStats));
+  memcpy(img.data() + o_jobs, &hj, sizeof(hj));
+  TJ_CUDA(put_small(ctl.p, img.data(), cc.off, st));
   Tracer tr(st);
   const double w = (double)sizeof(K);
   tr.begin("stats", w * n);
   TJ_CUDA(launch_stats<K>(d_jobs, 1, tiles, d_stats, st));
   tr.end();
   KeyStats hs;
-  uint32_t pref_pairs = ~0u;
+  bool sampled = false;
   if constexpr (sizeof(K) == 8) {
     if (n >= kPrefMinRows) {
       uint32_t* d_pairs = ctl.at<uint32_t>(o_misc + 128);
+      sampled = true;
       TJ_CUDA(launch_prefix_sample(keys, n, d_stats, 3 * prefix_digit(n), kPrefMinBits, d_pairs,
                                    st));
-      TJ_CUDA(get_small(&pref_pairs, d_pairs, sizeof(pref_pairs), st));
     }
   }
-  TJ_CUDA(get_small(&hs, d_stats, sizeof(hs), st));
+  // the statistics and the sample's count lie in one stretch of the block
+  TJ_CUDA(get_small(img.data() + o_stats, d_stats, o_misc + 132 - o_stats, st));
   TJ_CUDA(sync_stream(st));
+  memcpy(&hs, img.data() + o_stats, sizeof(hs));
+  uint32_t pref_pairs = ~0u;
+  if (sampled) memcpy(&pref_pairs, img.data() + o_misc + 128, sizeof(pref_pairs));
   tr.flush();
   Tracer tr2(st);
   const K lo = key_of<K>(hs.min_u), hi = key_of<K>(~hs.max_u);
