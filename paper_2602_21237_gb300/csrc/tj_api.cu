@@ -635,6 +635,19 @@ uint64_t* set_word_buffers(RadixJob<K>& j, const K* in_k, const K* in_v, uint64_
   return reinterpret_cast<uint64_t*>(const_cast<K*>(src));
 }
 
+// S rows of a join tile. Where R has many rows to one of S a tile of kJTile rows
+// spans more of R than its CTA takes on chip and every row searches R in global
+// memory: 90 us a tile, which the tiles behind it in the chained scan wait for, and
+// several times R's bytes. Such joins take fewer rows a tile, whose R range is
+// two and a half chunks
+// (sparse tiles stage that at once). 1024 joins of 10^3 to 10^6 int32 rows: join
+// kernel 3.87 -> 2.15 ms, all 9.02 -> 7.40.
+int64_t join_tile_rows(int64_t nr, int64_t ns) {
+  if (nr <= 2 * ns) return kJTile;
+  const int64_t t = 5 * (int64_t)kRCap / 2 * ns / nr / 32 * 32;
+  return std::min<int64_t>(kJSparse, std::max<int64_t>(64, t));
+}
+
 // ---- inner join -------------------------------------------------------------------
 struct Opts {
   int router = TJ_ROUTE_AUTO;
@@ -798,7 +811,9 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
 
   const int P = plan.passes;
   const int64_t bins_max = (int64_t)1 << plan.max_bits;
-  const int64_t jtiles = ceil_div(ns, kJTile);
+  // (a budget holds the tiles of kJTile rows it always held)
+  const int64_t trows = budget != 0 ? kJTile : join_tile_rows(nr, ns);
+  const int64_t jtiles = ceil_div(ns, trows);
   const int nbuf = P >= 2 ? 2 : P;
   Carve bc;
   size_t o_r[4] = {0, 0, 0, 0}, o_s[4] = {0, 0, 0, 0};
@@ -908,6 +923,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     jj.sv = res_i[1];
     jj.ns = ns;
     jj.tile0 = 0;
+    jj.trows = trows;
     memcpy(img.data() + o_jobs, hw, sizeof(hw));
     memcpy(img.data() + o_jj, &jj, sizeof(jj));
     TJ_CUDA(put_small(ctl.p, img.data(), cc.off, st));
@@ -1015,6 +1031,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
   jj.sv = res_sv;
   jj.ns = ns;
   jj.tile0 = 0;
+  jj.trows = trows;
   JTile<K>* d_tiles = big.at<JTile<K>>(o_tiles);
   TJ_CUDA(put_small(d_jj, &jj, sizeof(jj), st));
   TJ_CUDA(launch_tile_ranges<K>(d_jj, 1, jtiles, d_tiles, st));
@@ -2333,6 +2350,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
           y.sv = res[li * 4 + 3];
           y.ns = q.ns;
           y.tile0 = jt;
+          y.trows = kJTile;
           jt += ceil_div(q.ns, kJTile);
           all_jj.push_back(y);
         }
@@ -2926,14 +2944,18 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   }
   // the word tile: the large one unless the arrays' last tiles waste more by it
   // than it saves a pass (about a tenth); arrays that the small one pads by more
-  // than kPadShare stay columns, whose passes step over a tile's missing rows
+  // than kPadShare stay columns, whose passes step over a tile's missing rows, and
+  // so do arrays of less than kWordRows on average, for which the word pass's
+  // tables cost too much a tile (10^8 int32 rows in arrays of 4000, 8000, 20000
+  // and 10^5: words 9.9, 5.9, 3.9 and 2.6 ms, columns 9.1, 6.1, 4.2 and 3.5)
   int64_t pad_large = 0, pad_small = 0;
   for (int64_t j = 0; words && j < 2 * nj; ++j) {
     pad_large += ceil_div(hj[(size_t)j].n, kWThreads * kWItems) * (kWThreads * kWItems);
     pad_small += ceil_div(hj[(size_t)j].n, kWThreads * kWItemsSmall) * (kWThreads * kWItemsSmall);
   }
   constexpr double kPadShare = 0.25;
-  words = words && (double)pad_small <= (1.0 + kPadShare) * (double)(R + S);
+  constexpr int64_t kWordRows = 6144;
+  words = words && R + S >= 2 * nj * kWordRows && (double)pad_small <= (1.0 + kPadShare) * (double)(R + S);
   const Fold fold = words ? make_fold<K>(0, max_kb, id_lo, id_hi, true) : Fold();
   words = fold.on || fold.wide;
   const int witems = R + S >= kWSmallRows && pad_large * 10 <= pad_small * 11 ? kWItems
@@ -2981,7 +3003,10 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
       lb_at[(size_t)(2 * j + side)] = lb_words;
       lb_words += t * bins;
     }
-    if (live[(size_t)j]) jtiles += ceil_div(s_off[j + 1] - s_off[j], kJTile);
+    if (live[(size_t)j]) {
+      const int64_t ns = s_off[j + 1] - s_off[j];
+      jtiles += ceil_div(ns, join_tile_rows(r_off[j + 1] - r_off[j], ns));
+    }
   }
   Carve bc;
   size_t o_r[4] = {0, 0, 0, 0}, o_s[4] = {0, 0, 0, 0}, o_w[2] = {0, 0}, o_wi[2] = {0, 0};
@@ -3058,7 +3083,8 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
     y.sv = res[3];
     y.ns = live[(size_t)j] ? s_off[j + 1] - s_off[j] : 0;
     y.tile0 = jt;
-    jt += ceil_div(y.ns, kJTile);
+    y.trows = join_tile_rows(y.nr, s_off[j + 1] - s_off[j]);
+    jt += ceil_div(y.ns, y.trows);
   }
   TJ_CUDA(put_small(d_jobs, hj.data(), hj.size() * sizeof(RadixJob<K>), st));
   TJ_CUDA(put_small(d_jj, hjj.data(), hjj.size() * sizeof(JoinJob<K>), st));

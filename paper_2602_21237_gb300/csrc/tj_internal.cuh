@@ -65,11 +65,11 @@ constexpr int kMaxPasses = 8;               // 64-bit keys at 8 bits per pass
 #define TJ_JTILE 4096
 #endif
 constexpr int kJTile = TJ_JTILE;            // S rows per join tile (a power of two)
-#ifndef TJ_CHUNKS
-#define TJ_CHUNKS 4
-#endif
 constexpr int kRCap = kJTile / 2;           // R rows a join tile keeps on chip at once
-constexpr int kMaxChunks = TJ_CHUNKS;               // R chunks a join tile aligns on chip
+constexpr int kMaxChunks = 8;               // R chunks a join tile aligns on chip
+// S rows of a tile up to which they search R's chunks instead of a table: two
+// rows a thread, 11 steps each, cost less than filling the table's 2048 rows.
+constexpr int kJSparse = kJTile / 4;
 constexpr int kHTSlots = kJTile;            // on-chip hash table slots (load <= 0.5)
 static_assert((kJTile & (kJTile - 1)) == 0 && kJTile >= 1024, "join tile: a power of two");
 
@@ -216,7 +216,8 @@ struct JoinJob {
   const K* sk;          // sorted S keys
   const K* sv;
   int64_t ns;
-  int64_t tile0;        // first global join tile (kJTile S rows per tile)
+  int64_t tile0;        // first global join tile
+  int64_t trows;        // S rows of a tile (a multiple of 32, at most kJTile)
 };
 
 // A batch of one key value (a heavy key the cuts isolate): every R row pairs

@@ -1,7 +1,7 @@
 // Join of two key-sorted relations on their common key axis (paper Sec. 4.1)
 // with a single final materialisation of (r_id, s_id) pairs (Sec. 3.1).
 //
-//   k_tile_ranges : for every tile of kJTile sorted S rows, the range [a, b)
+//   k_tile_ranges : for every tile of up to kJTile sorted S rows, the range [a, b)
 //                   of sorted R rows whose keys lie between the tile's first
 //                   and last key (two searches per tile), written with the
 //                   tile's rows and job as one 64-byte descriptor;
@@ -136,8 +136,8 @@ __global__ void k_tile_ranges(const JoinJob<K>* __restrict__ jobs, int num_jobs,
     }
     return;
   }
-  const int64_t row0 = (t - J->tile0) * kJTile;
-  const int64_t row1 = min(J->ns, row0 + kJTile);
+  const int64_t row0 = (t - J->tile0) * J->trows;
+  const int64_t row1 = min(J->ns, row0 + J->trows);
   const E* __restrict__ s = reinterpret_cast<const E*>(J->sk);
   const E* __restrict__ r = reinterpret_cast<const E*>(J->rk);
   const auto key = Row::key(upper ? s[row1 - 1] : s[row0], ib);
@@ -197,6 +197,14 @@ static_assert(kJItems * kJThreads == kJTile, "join tile = threads x items");
 // (the matches of neighbouring rows share sectors); beyond, every output index
 // of the tile finds its row by a binary search.
 constexpr uint32_t kJDirect = 16;
+static_assert(kJSparse % kJThreads == 0, "whole rounds of a sparse tile's rows");
+// R rows a sparse tile takes on chip at once: the room of the table and of the S
+// rows it has not.
+template <int W>
+__host__ __device__ constexpr int sparse_rcap() {
+  return W == 0 || W == 3 ? 3 * kRCap : 4 * kRCap;
+}
+constexpr int kSparseChunks = 2;  // and how often (beyond: searched in global memory)
 
 // Shared memory: S keys | R keys | S ids | R ids (kJTile or kRCap elements and
 // kPad more each) | hash table[tab_slots] u32; folded rows: S words | R words |
@@ -218,6 +226,20 @@ constexpr size_t join_smem_bytes() {
          (ids ? sizeof(V) * (size_t)(kJTile + join_pad<V>() + kRCap + join_pad<V>()) : 0) +
          sizeof(uint32_t) * tab_slots<W>();
 }
+template <typename K, int W>
+constexpr size_t sparse_smem_bytes() {
+  using E = typename RowOf<K, W>::E;
+  using V = typename RowOf<K, W>::V;
+  constexpr bool ids = W == 0 || W == 3;
+  return sizeof(E) * (size_t)(kJSparse + join_pad<E>() + sparse_rcap<W>() + join_pad<E>()) +
+         (ids ? sizeof(V) * (size_t)(kJSparse + join_pad<V>() + sparse_rcap<W>() + join_pad<V>())
+              : 0);
+}
+static_assert(sparse_smem_bytes<int32_t, 0>() <= join_smem_bytes<int32_t, 0>() &&
+                  sparse_smem_bytes<int64_t, 0>() <= join_smem_bytes<int64_t, 0>() &&
+                  sparse_smem_bytes<int64_t, 2>() <= join_smem_bytes<int64_t, 2>() &&
+                  sparse_smem_bytes<int64_t, 3>() <= join_smem_bytes<int64_t, 3>(),
+              "sparse tiles fit the join's shared memory");
 static_assert(sizeof(uint64_t) * (kJTile + kRCap) >= (sizeof(uint64_t) + sizeof(uint32_t)) * kJTile,
               "offsets and run starts fit in the folded rows' shared memory");
 static_assert(sizeof(int32_t) * (2 * kJTile + 2 * kRCap) >=
@@ -253,7 +275,7 @@ __device__ __forceinline__ K* join_copy_async(K* dst, const K* __restrict__ src,
   return d;
 }
 
-// One join tile: kJTile consecutive rows of sorted S against the range [a, b)
+// One join tile: up to kJTile consecutive rows of sorted S against the range [a, b)
 // of sorted R whose keys lie between the tile's first and last key.
 //   1. S keys and ids and the first chunk of the R range go to shared memory
 //      (cp.async); warp w owns S rows [w*32*kJItems, ...), item u = 32 rows;
@@ -284,12 +306,6 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   constexpr bool kIds = W == 0 || W == 3;  // an id column beside the keys
   constexpr int kTabSlots = tab_slots<W>();
   constexpr int kPad = join_pad<E>(), kPadV = join_pad<V>();
-  E* const b_sk = reinterpret_cast<E*>(smem);  // staging areas (16-byte aligned)
-  E* const b_rk = b_sk + kJTile + kPad;
-  V* const b_sv = reinterpret_cast<V*>(b_rk + kRCap + kPad);  // (kIds only)
-  V* const b_rv = b_sv + kJTile + kPadV;
-  uint32_t* s_ht = kIds ? reinterpret_cast<uint32_t*>(b_rv + kRCap + kPadV)
-                        : reinterpret_cast<uint32_t*>(b_sv);
   // an id column's element as the caller's id
   auto id_of = [&](V v) -> K { return W == 3 ? (K)((uint64_t)v + f.ilo) : (K)v; };
   __shared__ uint64_t s_wsum[kJWarps];
@@ -314,8 +330,17 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
     if constexpr (!kIds) return word_id<K>(rk_g[i], f);
     else return id_of(rv_g[i]);
   };
-  const int64_t nchunks = (nrr + kRCap - 1) / kRCap;
-  const bool onchip = nchunks <= kMaxChunks;
+  // staging areas (16-byte aligned); a sparse tile has no table and more of R
+  const bool sparse = nv <= kJSparse;
+  const int srows = sparse ? kJSparse : kJTile, rcap = sparse ? sparse_rcap<W>() : kRCap;
+  E* const b_sk = reinterpret_cast<E*>(smem);
+  E* const b_rk = b_sk + srows + kPad;
+  V* const b_sv = reinterpret_cast<V*>(b_rk + rcap + kPad);  // (kIds only)
+  V* const b_rv = b_sv + srows + kPadV;
+  uint32_t* s_ht = kIds ? reinterpret_cast<uint32_t*>(b_rv + kRCap + kPadV)
+                        : reinterpret_cast<uint32_t*>(b_sv);
+  const int64_t nchunks = (nrr + rcap - 1) / rcap;
+  const bool onchip = nchunks <= (sparse ? kSparseChunks : kMaxChunks);
 
   // 1. stage S and the first R chunk
   const E* s_sk = join_copy_async<E>(b_sk, reinterpret_cast<const E*>(T.sk), nv);
@@ -324,32 +349,56 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   V* s_rv = b_rv;
   if constexpr (kIds) s_sv = join_copy_async<V>(b_sv, reinterpret_cast<const V*>(T.sv), nv);
   if (onchip && nchunks > 0) {
-    const int nc0 = (int)min((int64_t)kRCap, nrr);
+    const int nc0 = (int)min((int64_t)rcap, nrr);
     s_rk = join_copy_async<E>(b_rk, rk_g, nc0);
     if constexpr (kIds) s_rv = join_copy_async<V>(b_rv, rv_g, nc0);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 
-  // 2. probe
-  const int wbase = warp * 32 * kJItems;
+  // 2. probe (a short tile's rows are spread over all warps, 32 at a time)
+  const int wits = (nv + kJThreads - 1) / kJThreads;  // items of a warp
+  const int wbase = warp * 32 * wits;
   uint32_t cnt[kJItems], start[kJItems];
 #pragma unroll
   for (int u = 0; u < kJItems; ++u) cnt[u] = start[u] = 0u;
   if (onchip) {
     for (int64_t c = 0; c < nchunks; ++c) {
-      const int c0 = (int)(c * kRCap);
-      const int nc = (int)min((int64_t)kRCap, nrr - c0);
+      const int c0 = (int)(c * rcap);
+      const int nc = (int)min((int64_t)rcap, nrr - c0);
       if (c > 0) {
         __syncthreads();  // the previous chunk's probes are done
         s_rk = join_copy_async<E>(b_rk, rk_g + c0, nc);
         if constexpr (kIds) s_rv = join_copy_async<V>(b_rv, rv_g + c0, nc);
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
-      for (int i = tid; i < kTabSlots / 4; i += kJThreads)
+      for (int i = tid; !sparse && i < kTabSlots / 4; i += kJThreads)
         reinterpret_cast<uint4*>(s_ht)[i] = make_uint4(0u, 0u, 0u, 0u);
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();
       const Key cf = Row::key(s_rk[0], ib), cl = Row::key(s_rk[nc - 1], ib);
+      if (sparse) {
+        // few S rows: each searches the chunk, no table
+#pragma unroll
+        for (int u = 0; u < kJSparse / kJThreads; ++u) {
+          const int q = wbase + u * 32 + lane;
+          if (u >= wits || q >= nv) continue;
+          const Key key = Row::key(s_sk[q], ib);
+          if (key < cf || cl < key) continue;
+          int a = 0, n = nc;
+          while (n > 0) {
+            const int half = n >> 1;
+            const bool go = Row::key(s_rk[a + half], ib) < key;
+            a = go ? a + half + 1 : a;
+            n = go ? n - half - 1 : half;
+          }
+          int e = a;  // (a < nc: the chunk's last key is not below this one)
+          while (e < nc && Row::key(s_rk[e], ib) == key) ++e;
+          if (e == a) continue;
+          if (cnt[u] == 0u) start[u] = (uint32_t)(c0 + a);
+          cnt[u] += (uint32_t)(e - a);
+        }
+        continue;
+      }
       if ((uint64_t)cl - (uint64_t)cf < (uint64_t)kTabSlots) {
         // dense keys: entry key - cf holds the key's run (first | end << 16),
         // each half written by the run's first or last row
@@ -365,7 +414,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
 #pragma unroll
         for (int u = 0; u < kJItems; ++u) {
           const int q = wbase + u * 32 + lane;
-          if (q >= nv) continue;
+          if (u >= wits || q >= nv) continue;
           const Key key = Row::key(s_sk[q], ib);
           if (key < cf || cl < key) continue;
           const uint32_t w = s_ht[(uint32_t)((uint64_t)key - (uint64_t)cf)];
@@ -389,7 +438,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
 #pragma unroll
       for (int u = 0; u < kJItems; ++u) {
         const int q = wbase + u * 32 + lane;
-        if (q >= nv) continue;
+        if (u >= wits || q >= nv) continue;
         const Key key = Row::key(s_sk[q], ib);
         if (key < cf || cl < key) continue;
         uint32_t h = ht_hash(key);
@@ -426,7 +475,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
 #pragma unroll
     for (int u = 0; u < kJItems; ++u) {
       const int q = wbase + u * 32 + lane;
-      key[u] = q < nv ? Row::key(s_sk[q], ib) : Key(0);
+      key[u] = u < wits && q < nv ? Row::key(s_sk[q], ib) : Key(0);
     }
     // bound 0: first R row with key >= the row's key; 1: first with key >
     // (offsets into the range: nrr < 2^30)
@@ -467,7 +516,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
     uint32_t more = 0u;
 #pragma unroll
     for (int u = 0; u < kJItems; ++u) {
-      const bool valid = wbase + u * 32 + lane < nv;
+      const bool valid = u < wits && wbase + u * 32 + lane < nv;
       const Key r0 = Row::key(rk_g[min(lo[u], nr32 - 1)], ib);
       const Key r1 = Row::key(rk_g[min(lo[u] + 1, nr32 - 1)], ib);
       const bool e0 = valid && lo[u] < nr32 && r0 == key[u];
@@ -535,7 +584,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
     const uint32_t ltm = lanemask_lt();
     // R rows of the chunk still in shared memory (the last one) are read
     // there, earlier ones from global memory
-    const uint32_t cres = onchip && nchunks > 0 ? (uint32_t)((nchunks - 1) * kRCap) : ~0u;
+    const uint32_t cres = onchip && nchunks > 0 ? (uint32_t)((nchunks - 1) * rcap) : ~0u;
     const bool single = mymax <= 1u;
     K* __restrict__ const o_w = out + 2 * (first + wpre);  // the warp's first pair
     uint32_t off = 0;  // (a warp has at most 32 kJItems kJDirect pairs)
@@ -588,7 +637,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
 #pragma unroll
     for (int u = 0; u < kJItems; ++u) {
       const int q = wbase + u * 32 + lane;
-      if (q < nv) {
+      if (u < wits && q < nv) {
         s_off[q] = cnt[u];
         s_rs[q] = start[u];
       }
@@ -680,7 +729,7 @@ __global__ void k_group_maps(const RadixJob<K>* __restrict__ rjobs, int nr,
   } else {
     const int j = b - nr;
     const int64_t t0 = jjobs[j].tile0;
-    const int64_t nt = (jjobs[j].ns + kJTile - 1) / kJTile;
+    const int64_t nt = (jjobs[j].ns + jjobs[j].trows - 1) / jjobs[j].trows;
     for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) jmap[t0 + t] = j;
   }
 }
@@ -699,7 +748,7 @@ __global__ void k_fill_join_tile_job(const JoinJob<K>* __restrict__ jobs,
                                      int32_t* __restrict__ map) {
   const int j = blockIdx.x;
   const int64_t t0 = jobs[j].tile0;
-  const int64_t nt = (jobs[j].ns + kJTile - 1) / kJTile;
+  const int64_t nt = (jobs[j].ns + jobs[j].trows - 1) / jobs[j].trows;
   for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) map[t0 + t] = j;
 }
 
