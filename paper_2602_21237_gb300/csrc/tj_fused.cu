@@ -317,7 +317,7 @@ template <typename K>
 struct FusedSmem {
   uint16_t wh[kFWarps][kFKeys];
   union {
-    uint32_t wm[kFWarps][128 * kWMaskItems];  // dead before the R rows are sorted
+    uint32_t wm[kFWarps][128 * kFMaskItems];  // dead before the R rows are sorted
     struct {
       uint16_t r_pa[kFCapR];
       uint16_t r_pb[kFCapR];
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
     if constexpr (WORDS) return koff(skey[u], sublo);
     else return dig.get(u);
   };
-  wrank<kFKeyBits, kFItemsS>(row_digit, rank, S.wh[warp], S.wm[warp], ns - wrow);
+  wrank<kFKeyBits, kFItemsS, kFMaskItems>(row_digit, rank, S.wh[warp], S.wm[warp], ns - wrow);
   __syncthreads();  // counts complete, ranks done
 
   // 3. per key offset (four per thread, two 16-bit counters a word): the S rows

@@ -57,7 +57,8 @@ constexpr int kWWarps = kWThreads / 32;
 constexpr int kWMinB = TJ_W_MINB;
 constexpr int kWItems = TJ_W_ITEMS;
 constexpr int kWItemsSmall = 8;
-constexpr int kWMaskItems = 2;  // of four items ranked by the lane-mask tables
+constexpr int kWMaskItems = 3;  // of four items a word pass ranks by the lane-mask tables
+constexpr int kFMaskItems = 2;  // of three items the resident join does
 constexpr int kMaxDigitBits = 10;           // widest radix digit
 constexpr int kMaxBins = 1 << kMaxDigitBits;
 constexpr int kMaxPasses = 8;               // 64-bit keys at 8 bits per pass

@@ -139,20 +139,22 @@ __host__ __device__ constexpr int wrank_group() {
 // of 16 or 32 bits, and `masks` zero on entry; groups of items at or beyond row
 // nv are skipped, rows beyond it in the last group counted).  All
 // lanes read the warp's count of their digit and the digit's highest lane
-// stores the new one.  The lanes of equal digit are found for kWMaskItems of
+// stores the new one.  The lanes of equal digit are found for MAXM of
 // every G items through a table of lane masks by the digit's low 7 bits (each
 // lane ORs its bit in, reads the word back, and the group's highest lane
 // clears it) with a ballot per higher bit, for the others by a ballot per
 // digit bit.  Ballots cost issue slots, the table conflicting shared-memory
 // accesses, and each alone bounds the pass: 10^8 words by a 7-bit digit take
 // 526 us with ballots only, 527 with the table only, 500 with two of four
-// items each way (GB300, 512 threads x 16 words).
-template <int NB, int ITEMS, typename C, typename D>
+// items each way (GB300, 512 threads x 16 words). With 8 and 9 bits three of four
+// through the table are 1-2% better than two (sort of 10^8 int64 2.79 -> 2.76 ms,
+// 3x10^7 hashed keys 1.36 -> 1.34, join of 10^8 x 4x10^8 under 256 MiB 13.97 -> 13.86).
+template <int NB, int ITEMS, int MAXM, typename C, typename D>
 __device__ __forceinline__ void wrank(const D& digit, Half<ITEMS>& rank, C* cnt, uint32_t* masks,
                                       int nv = 32 * ITEMS) {
   const uint32_t bit = 1u << (threadIdx.x & 31), ltm = lanemask_lt(), gtm = lanemask_gt();
   constexpr int G = wrank_group<ITEMS>();
-  constexpr int MX = kWMaskItems < G ? kWMaskItems : G;
+  constexpr int MX = MAXM < G ? MAXM : G;
 #pragma unroll
   for (int i0 = 0; i0 < ITEMS; i0 += G) {
     if (nv < 32 * ITEMS && i0 * 32 >= nv) break;

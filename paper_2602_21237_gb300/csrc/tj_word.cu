@@ -127,16 +127,16 @@ __device__ __forceinline__ void wrank_bits(const D& digit, int nbits, Half<ITEMS
                                            uint32_t* cnt, uint32_t* masks) {
   switch (nbits) {
     case 0:  // one digit value
-    case 1: wrank<1, ITEMS>(digit, rank, cnt, masks); break;
-    case 2: wrank<2, ITEMS>(digit, rank, cnt, masks); break;
-    case 3: wrank<3, ITEMS>(digit, rank, cnt, masks); break;
-    case 4: wrank<4, ITEMS>(digit, rank, cnt, masks); break;
-    case 5: wrank<5, ITEMS>(digit, rank, cnt, masks); break;
-    case 6: wrank<6, ITEMS>(digit, rank, cnt, masks); break;
-    case 7: wrank<7, ITEMS>(digit, rank, cnt, masks); break;
-    case 8: wrank<8, ITEMS>(digit, rank, cnt, masks); break;
-    case 9: wrank<9, ITEMS>(digit, rank, cnt, masks); break;
-    default: wrank<10, ITEMS>(digit, rank, cnt, masks); break;
+    case 1: wrank<1, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    case 2: wrank<2, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    case 3: wrank<3, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    case 4: wrank<4, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    case 5: wrank<5, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    case 6: wrank<6, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    case 7: wrank<7, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    case 8: wrank<8, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    case 9: wrank<9, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
+    default: wrank<10, ITEMS, kWMaskItems>(digit, rank, cnt, masks); break;
   }
 }
 
