@@ -204,6 +204,15 @@ template <int W>
 __host__ __device__ constexpr int sparse_rcap() {
   return W == 0 || W == 3 ? 3 * kRCap : 4 * kRCap;
 }
+// Wide rows (W = 3) have no table in any tile: their keys are seldom dense, and
+// searching takes the whole R range of a tile of as many R rows at once.
+// Against 2048-row chunks hashed one after another: join of 2 x 2^26 rows of clustered
+// 40-bit keys 7.23 -> 6.22 ms (join kernel 1.8 -> 0.8). Dense keys stay with the table:
+// join of 10^7 x 4x10^7 rows 1.48 ms by table, 1.63 by search.
+template <int W>
+__host__ __device__ constexpr int search_rcap() {
+  return W == 3 ? 9 * kRCap / 4 : kRCap;
+}
 constexpr int kSparseChunks = 2;  // and how often (beyond: searched in global memory)
 
 // Shared memory: S keys | R keys | S ids | R ids (kJTile or kRCap elements and
@@ -235,6 +244,10 @@ constexpr size_t sparse_smem_bytes() {
          (ids ? sizeof(V) * (size_t)(kJSparse + join_pad<V>() + sparse_rcap<W>() + join_pad<V>())
               : 0);
 }
+static_assert(sizeof(int64_t) * (kJTile + 2 + search_rcap<3>() + 2) +
+                      sizeof(uint32_t) * (kJTile + 4 + search_rcap<3>() + 4) <=
+                  join_smem_bytes<int64_t, 3>(),
+              "searched tiles of wide rows fit the join's shared memory");
 static_assert(sparse_smem_bytes<int32_t, 0>() <= join_smem_bytes<int32_t, 0>() &&
                   sparse_smem_bytes<int64_t, 0>() <= join_smem_bytes<int64_t, 0>() &&
                   sparse_smem_bytes<int64_t, 2>() <= join_smem_bytes<int64_t, 2>() &&
@@ -332,7 +345,9 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
   };
   // staging areas (16-byte aligned); a sparse tile has no table and more of R
   const bool sparse = nv <= kJSparse;
-  const int srows = sparse ? kJSparse : kJTile, rcap = sparse ? sparse_rcap<W>() : kRCap;
+  const bool search = W == 3 || sparse;
+  const int srows = sparse ? kJSparse : kJTile;
+  const int rcap = sparse ? sparse_rcap<W>() : search_rcap<W>();
   E* const b_sk = reinterpret_cast<E*>(smem);
   E* const b_rk = b_sk + srows + kPad;
   V* const b_sv = reinterpret_cast<V*>(b_rk + rcap + kPad);  // (kIds only)
@@ -371,15 +386,15 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         if constexpr (kIds) s_rv = join_copy_async<V>(b_rv, rv_g + c0, nc);
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
-      for (int i = tid; !sparse && i < kTabSlots / 4; i += kJThreads)
+      for (int i = tid; !search && i < kTabSlots / 4; i += kJThreads)
         reinterpret_cast<uint4*>(s_ht)[i] = make_uint4(0u, 0u, 0u, 0u);
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();
       const Key cf = Row::key(s_rk[0], ib), cl = Row::key(s_rk[nc - 1], ib);
-      if (sparse) {
-        // few S rows: each searches the chunk, no table
+      if (search) {
+        // each S row searches the chunk
 #pragma unroll
-        for (int u = 0; u < kJSparse / kJThreads; ++u) {
+        for (int u = 0; u < (W == 3 ? kJItems : kJSparse / kJThreads); ++u) {
           const int q = wbase + u * 32 + lane;
           if (u >= wits || q >= nv) continue;
           const Key key = Row::key(s_sk[q], ib);
