@@ -20,24 +20,24 @@ namespace tj {
 constexpr int kGatherThreads = 256;
 constexpr int kGatherRows = 4;  // pairs per thread per round
 
-template <typename I>
-__device__ __forceinline__ void load_pair(const I* p, int64_t i, I& r, I& s);
-template <>
-__device__ __forceinline__ void load_pair<int32_t>(const int32_t* p, int64_t i, int32_t& r,
-                                                   int32_t& s) {
-  const int2 v = __ldcs(reinterpret_cast<const int2*>(p) + i);  // (leaves L2 to the columns)
+// NEAR: L2 holds a good part of the columns and is left to them, pairs and results
+// passing it as streams.
+template <bool NEAR>
+__device__ __forceinline__ void load_pair(const int32_t* p, int64_t i, int32_t& r, int32_t& s) {
+  const int2* q = reinterpret_cast<const int2*>(p) + i;
+  const int2 v = NEAR ? __ldcs(q) : __ldg(q);
   r = v.x;
   s = v.y;
 }
-template <>
-__device__ __forceinline__ void load_pair<int64_t>(const int64_t* p, int64_t i, int64_t& r,
-                                                   int64_t& s) {
-  const longlong2 v = __ldcs(reinterpret_cast<const longlong2*>(p) + i);
+template <bool NEAR>
+__device__ __forceinline__ void load_pair(const int64_t* p, int64_t i, int64_t& r, int64_t& s) {
+  const longlong2* q = reinterpret_cast<const longlong2*>(p) + i;
+  const longlong2 v = NEAR ? __ldcs(q) : __ldg(q);
   r = v.x;
   s = v.y;
 }
 
-template <typename E>
+template <typename E, bool NEAR>
 __device__ __forceinline__ void gather_col(const GatherCol& c, const int64_t (&row)[kGatherRows],
                                            const int64_t (&at)[kGatherRows]) {
   const E* __restrict__ src = reinterpret_cast<const E*>(c.src);
@@ -47,12 +47,15 @@ __device__ __forceinline__ void gather_col(const GatherCol& c, const int64_t (&r
   for (int u = 0; u < kGatherRows; ++u) v[u] = row[u] >= 0 ? __ldg(src + row[u]) : E(0);
 #pragma unroll
   for (int u = 0; u < kGatherRows; ++u)
-    if (row[u] >= 0) __stcs(dst + at[u], v[u]);
+    if (row[u] >= 0) {
+      if (NEAR) __stcs(dst + at[u], v[u]);
+      else dst[at[u]] = v[u];
+    }
 }
 
 // pairs[i] = (r_id, s_id), i < n; an id outside [0, rows of its side) sets
 // *err = TJ_ERR_INVALID and its row is not written.
-template <typename I>
+template <typename I, bool NEAR>
 __global__ void __launch_bounds__(kGatherThreads)
     k_gather_pairs(const I* __restrict__ pairs, int64_t n, int64_t n_r, int64_t n_s,
                    GatherArgs a, int* __restrict__ err) {
@@ -66,7 +69,7 @@ __global__ void __launch_bounds__(kGatherThreads)
       rr[u] = sr[u] = -1;
       if (at[u] < n) {
         I r, s;
-        load_pair<I>(pairs, at[u], r, s);
+        load_pair<NEAR>(pairs, at[u], r, s);
         const bool ok = (int64_t)r >= 0 && (int64_t)r < n_r && (int64_t)s >= 0 && (int64_t)s < n_s;
         if (ok) {
           rr[u] = (int64_t)r;
@@ -81,14 +84,14 @@ __global__ void __launch_bounds__(kGatherThreads)
       const GatherCol& col = a.c[c];
       if (col.bytes == 8) {
         if (col.side)
-          gather_col<unsigned long long>(col, sr, at);
+          gather_col<unsigned long long, NEAR>(col, sr, at);
         else
-          gather_col<unsigned long long>(col, rr, at);
+          gather_col<unsigned long long, NEAR>(col, rr, at);
       } else {
         if (col.side)
-          gather_col<unsigned int>(col, sr, at);
+          gather_col<unsigned int, NEAR>(col, sr, at);
         else
-          gather_col<unsigned int>(col, rr, at);
+          gather_col<unsigned int, NEAR>(col, rr, at);
       }
     }
   }
@@ -107,7 +110,7 @@ cudaError_t launch_gather_pairs(const I* pairs, int64_t n, int64_t n_r, int64_t 
   // together.  (4x10^7 random 8-byte elements take 0.20, 0.45, 0.72 and 1.04 ms
   // from a column of 80, 160, 320 and 3200 MB, alone; L2 is 129 MB. Two payload
   // columns of 8 and 4 bytes a row on either side of a join of 10^7 x 4x10^7 rows:
-  // 2.03 ms in one launch, now 1.81.)
+  // 2.03 ms in one launch, now 1.74.)
   constexpr int64_t kFarL2 = 4;
   int dev = 0, l2 = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -117,9 +120,12 @@ cudaError_t launch_gather_pairs(const I* pairs, int64_t n, int64_t n_r, int64_t 
   GatherArgs g, far;  // the launch being filled, the columns that go together
   g.n = far.n = 0;
   int64_t held = 0;
-  auto flush = [&](GatherArgs& x) {
-    if (x.n > 0)
-      k_gather_pairs<I><<<(unsigned)grid, kGatherThreads, 0, st>>>(pairs, n, n_r, n_s, x, d_err);
+  const unsigned blocks = (unsigned)grid;
+  auto flush = [&](GatherArgs& x, bool near) {
+    if (x.n > 0 && near)
+      k_gather_pairs<I, true><<<blocks, kGatherThreads, 0, st>>>(pairs, n, n_r, n_s, x, d_err);
+    else if (x.n > 0)
+      k_gather_pairs<I, false><<<blocks, kGatherThreads, 0, st>>>(pairs, n, n_r, n_s, x, d_err);
     x.n = 0;
   };
   // (one side's columns, then the other's)
@@ -132,14 +138,14 @@ cudaError_t launch_gather_pairs(const I* pairs, int64_t n, int64_t n_r, int64_t 
         continue;
       }
       if (2 * (held + b) > 3 * (int64_t)l2) {
-        flush(g);
+        flush(g, true);
         held = 0;
       }
       g.c[g.n++] = a.c[c];
       held += b;
     }
-  flush(g);
-  flush(far);
+  flush(g, true);
+  flush(far, false);
   return cudaGetLastError();
 }
 
