@@ -71,7 +71,6 @@ constexpr int kMaxChunks = 8;               // R chunks a join tile aligns on ch
 // S rows of a tile up to which they search R's chunks instead of a table: two
 // rows a thread, 11 steps each, cost less than filling the table's 2048 rows.
 constexpr int kJSparse = kJTile / 4;
-constexpr int kHTSlots = kJTile;            // on-chip hash table slots (load <= 0.5)
 static_assert((kJTile & (kJTile - 1)) == 0 && kJTile >= 1024, "join tile: a power of two");
 
 // ---- decoupled look-back words (30-bit counts) ----------------------------

@@ -7,13 +7,12 @@
 //                   tile's rows and job as one 64-byte descriptor;
 //   k_join        : per S tile, fused count -> scan -> write:
 //                     1. read the tile's descriptor, stage its S rows and its
-//                        R range (in chunks of kRCap rows, up to 4) in shared
+//                        R range (in chunks of kRCap rows, up to 8) in shared
 //                        memory with cp.async;
-//                     2. build a table of each chunk's distinct keys, key ->
-//                        (first, end) of its run of R rows: by key value where
-//                        the chunk's keys are dense, else an open-addressing
-//                        hash table filled with shared-memory atomicCAS;
-//                     3. probe it once per S row -> match count, run start;
+//                     2. look every S row's key up in each chunk: in a table key
+//                        -> (first, end) of its run of R rows where the chunk's
+//                        keys are dense, else by a search of its sorted rows;
+//                     3. which gives its match count and run start;
 //                     4. a decoupled look-back over all tiles of all jobs
 //                        (the words in the tiles' descriptors) gives
 //                        the tile's first output index;
@@ -39,18 +38,6 @@ __device__ __forceinline__ int find_job_j(const Job* jobs, int num_jobs, int64_t
   }
   return lo;
 }
-
-// multiplicative hashing onto the table's log2(kHTSlots) bits
-constexpr int kHTBits = kHTSlots == 1024 ? 10 : kHTSlots == 2048 ? 11 : kHTSlots == 4096 ? 12 : 13;
-static_assert((1 << kHTBits) == kHTSlots, "hash table slots: 2^10 .. 2^13");
-__device__ __forceinline__ uint32_t ht_hash(int32_t k) {
-  return ((uint32_t)k * 0x9E3779B9u) >> (32 - kHTBits);
-}
-__device__ __forceinline__ uint32_t ht_hash(int64_t k) {
-  return (uint32_t)(((uint64_t)k * 0x9E3779B97F4A7C15ull) >> (64 - kHTBits));
-}
-__device__ __forceinline__ uint32_t ht_hash(uint64_t k) { return ht_hash((int64_t)k); }
-__device__ __forceinline__ uint32_t ht_hash(uint32_t k) { return ht_hash((int32_t)k); }
 
 // How a join kernel reads rows: W = 0, separate columns (an element is a key);
 // W = 1, folded rows (tj_word.cu), keys of up to 63 bits; W = 2, folded rows
@@ -92,13 +79,14 @@ __device__ __forceinline__ K word_id(uint64_t w, const WordFmt& f) {
 }
 static_assert(kRCap < 0xFFFF, "run bounds are packed in 16 bits");
 
-constexpr uint32_t kHTEmpty = 0u;  // (no entry is 0: a run's end is at least 1)
-// Entries of the on-chip table: a chunk of R whose keys span fewer values than
-// that has one entry per value instead of a hash table of kHTSlots.
-// (Separate columns, W = 0, leave shared memory for half as many.)
+// Entries of the on-chip table: a chunk of R whose keys span at most that many
+// values has one entry per value. (Separate columns, W = 0, leave shared memory for
+// half as many.) In other chunks each S row searches the sorted R rows: filling a
+// hash table of them took longer (5x10^6 x 5x10^6 int32 rows over 31 bits 589 us,
+// now 537; 2^23 x 2^23 clustered rows 997, now 914; 2x10^6 x 8x10^6 516, now 525).
 template <int W>
 __host__ __device__ constexpr int tab_slots() {
-  return W == 0 ? kHTSlots : 2 * kHTSlots;
+  return W == 0 ? kJTile : 2 * kJTile;
 }
 
 __device__ __forceinline__ void st_volatile_u64(uint64_t* p, uint64_t v) {
@@ -204,7 +192,7 @@ template <int W>
 __host__ __device__ constexpr int sparse_rcap() {
   return W == 0 || W == 3 ? 3 * kRCap : 4 * kRCap;
 }
-// Wide rows (W = 3) have no table in any tile: their keys are seldom dense, and
+// Wide rows (W = 3) use no table in any tile: their keys are seldom dense, and
 // searching takes the whole R range of a tile of as many R rows at once.
 // Against 2048-row chunks hashed one after another: join of 2 x 2^26 rows of clustered
 // 40-bit keys 7.23 -> 6.22 ms (join kernel 1.8 -> 0.8). Dense keys stay with the table:
@@ -216,7 +204,7 @@ __host__ __device__ constexpr int search_rcap() {
 constexpr int kSparseChunks = 2;  // and how often (beyond: searched in global memory)
 
 // Shared memory: S keys | R keys | S ids | R ids (kJTile or kRCap elements and
-// kPad more each) | hash table[tab_slots] u32; folded rows: S words | R words |
+// kPad more each) | table[tab_slots] u32; folded rows: S words | R words |
 // table.  Each staged array starts up to kPad
 // elements into its area (its first element keeps the source's address modulo
 // 16, so that all but a head and a tail move in 16-byte copies).  After the
@@ -292,10 +280,10 @@ __device__ __forceinline__ K* join_copy_async(K* dst, const K* __restrict__ src,
 // of sorted R whose keys lie between the tile's first and last key.
 //   1. S keys and ids and the first chunk of the R range go to shared memory
 //      (cp.async); warp w owns S rows [w*32*kJItems, ...), item u = 32 rows;
-//   2. per chunk of the R range (kRCap rows, at most kMaxChunks): a table of
-//      the chunk's distinct keys (entry: first and end of the key's run) by key
-//      value, or hashed, and every S row looks its key up -> match
-//      count and run start; wider R ranges are searched through a strided sample
+//   2. per chunk of the R range (kRCap rows, at most kMaxChunks): every S
+//      row's match count and run start, from a table of the chunk's keys by value
+//      (entry: first and end of the key's run) where they are dense, else by a
+//      search; wider R ranges are searched through a strided sample
 //      staged on chip, then within one stride in global memory;
 //   3. the tile's total goes to the decoupled look-back chain over all tiles
 //      (warp 0, 32 predecessors per round trip), which yields the tile's
@@ -391,30 +379,7 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();
       const Key cf = Row::key(s_rk[0], ib), cl = Row::key(s_rk[nc - 1], ib);
-      if (search) {
-        // each S row searches the chunk
-#pragma unroll
-        for (int u = 0; u < (W == 3 ? kJItems : kJSparse / kJThreads); ++u) {
-          const int q = wbase + u * 32 + lane;
-          if (u >= wits || q >= nv) continue;
-          const Key key = Row::key(s_sk[q], ib);
-          if (key < cf || cl < key) continue;
-          int a = 0, n = nc;
-          while (n > 0) {
-            const int half = n >> 1;
-            const bool go = Row::key(s_rk[a + half], ib) < key;
-            a = go ? a + half + 1 : a;
-            n = go ? n - half - 1 : half;
-          }
-          int e = a;  // (a < nc: the chunk's last key is not below this one)
-          while (e < nc && Row::key(s_rk[e], ib) == key) ++e;
-          if (e == a) continue;
-          if (cnt[u] == 0u) start[u] = (uint32_t)(c0 + a);
-          cnt[u] += (uint32_t)(e - a);
-        }
-        continue;
-      }
-      if ((uint64_t)cl - (uint64_t)cf < (uint64_t)kTabSlots) {
+      if (!search && (uint64_t)cl - (uint64_t)cf < (uint64_t)kTabSlots) {
         // dense keys: entry key - cf holds the key's run (first | end << 16),
         // each half written by the run's first or last row
         uint16_t* const s_run = reinterpret_cast<uint16_t*>(s_ht);
@@ -439,38 +404,25 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
         }
         continue;
       }
-      // insert the first row of every run of equal keys; keys are distinct, so
-      // an occupied slot is never this key and insertion needs no comparison
-      for (int i = tid; i < nc; i += kJThreads) {
-        const Key key = Row::key(s_rk[i], ib);
-        if (i == 0 || key != Row::key(s_rk[i - 1], ib)) {
-          uint32_t h = ht_hash(key);
-          while (atomicCAS(&s_ht[h], kHTEmpty, (uint32_t)i + 1u) != kHTEmpty)
-            h = (h + 1) & (kHTSlots - 1);
-        }
-      }
-      __syncthreads();
+      // each S row searches the chunk
 #pragma unroll
       for (int u = 0; u < kJItems; ++u) {
         const int q = wbase + u * 32 + lane;
         if (u >= wits || q >= nv) continue;
         const Key key = Row::key(s_sk[q], ib);
         if (key < cf || cl < key) continue;
-        uint32_t h = ht_hash(key);
-        while (true) {
-          const uint32_t w = s_ht[h];
-          if (w == kHTEmpty) break;
-          const int r0 = (int)w - 1;
-          if (Row::key(s_rk[r0], ib) == key) {
-            // the run's end: as many steps as the row has matches here
-            int e = r0 + 1;
-            while (e < nc && Row::key(s_rk[e], ib) == key) ++e;
-            if (cnt[u] == 0u) start[u] = (uint32_t)(c0 + r0);
-            cnt[u] += (uint32_t)(e - r0);
-            break;
-          }
-          h = (h + 1) & (kHTSlots - 1);
+        int a = 0, n = nc;
+        while (n > 0) {
+          const int half = n >> 1;
+          const bool go = Row::key(s_rk[a + half], ib) < key;
+          a = go ? a + half + 1 : a;
+          n = go ? n - half - 1 : half;
         }
+        int e = a;  // (a < nc: the chunk's last key is not below this one)
+        while (e < nc && Row::key(s_rk[e], ib) == key) ++e;
+        if (e == a) continue;
+        if (cnt[u] == 0u) start[u] = (uint32_t)(c0 + a);
+        cnt[u] += (uint32_t)(e - a);
       }
     }
     if (nchunks == 0) asm volatile("cp.async.wait_all;" ::: "memory");
