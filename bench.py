@@ -480,7 +480,7 @@ def run_tj(args, ws, rank, local):
     peak, peak_kind = measured_peaks()
     roof = None
     launches = sum(v["launches"] for v in trace.values())
-    # k_onesweep dominates the step.  The groups of a budgeted join alternate
+    # k_wsweep (k_onesweep where rows do not fold) dominates the step.  The groups of a budgeted join alternate
     # between two streams and are traced per group ("group/lanes": sort passes
     # and join), since their launches overlap: the kernel's figure comes from
     # its launches that ran alone (the route passes, tj_sort's passes and the
@@ -500,7 +500,7 @@ def run_tj(args, ws, rank, local):
         step_bytes = sum(v["bytes"] for v in trace.values()) / len(step_ms)
         step_ach = step_bytes / (ms_step / 1e3) / 1e9
         roof = {"bound": "hbm",
-                "kernel": "k_onesweep (launches that ran alone: route passes, tj_sort, the "
+                "kernel": "k_wsweep (launches that ran alone: route passes, tj_sort, the "
                           "router's sample sorts)",
                 "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
                 "peak_kind": f"{peak_kind} hbm_gbs (copy, burst)",
