@@ -2955,7 +2955,9 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   }
   constexpr double kPadShare = 0.25;
   constexpr int64_t kWordRows = 6144;
-  words = words && R + S >= 2 * nj * kWordRows && (double)pad_small <= (1.0 + kPadShare) * (double)(R + S);
+  // (a batch whose pairs all hold one key value needs no pass at all)
+  words = words && max_kb > 0 && R + S >= 2 * nj * kWordRows &&
+          (double)pad_small <= (1.0 + kPadShare) * (double)(R + S);
   const Fold fold = words ? make_fold<K>(0, max_kb, id_lo, id_hi, true) : Fold();
   words = fold.on || fold.wide;
   const int witems = R + S >= kWSmallRows && pad_large * 10 <= pad_small * 11 ? kWItems

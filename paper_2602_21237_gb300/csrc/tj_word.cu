@@ -617,11 +617,20 @@ __global__ void __launch_bounds__(kRunThreads)
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+// Shared memory of a launch over jobs of several digit widths: the largest of their
+// layouts, from 0 bits on (a batched pair whose rows all have one key folds them in a
+// pass of no digit, which stages its tile like any other).
+template <int ITEMS>
+size_t wsweep_launch_smem(int max_bits, int mode, bool guard, bool wide) {
+  size_t m = wsweep_smem_bytes<ITEMS>(0, mode, guard, wide);
+  for (int b = 1; b <= max_bits; ++b)
+    m = std::max(m, wsweep_smem_bytes<ITEMS>(b, mode, guard, wide));
+  return m;
+}
+
 template <typename K, bool RI, bool RO, int MODE, bool HI, bool WIDE, int ITEMS>
 cudaError_t wsweep_attr() {
-  size_t m = 0;
-  for (int b = 1; b <= kMaxDigitBits; ++b)
-    m = std::max(m, wsweep_smem_bytes<ITEMS>(b, MODE, MODE != kModeSort, WIDE));
+  const size_t m = wsweep_launch_smem<ITEMS>(kMaxDigitBits, MODE, MODE != kModeSort, WIDE);
   return cudaFuncSetAttribute(k_wsweep<K, RI, RO, MODE, HI, WIDE, ITEMS>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m);
 }
@@ -631,10 +640,8 @@ cudaError_t wsweep_go(const RadixJob<K>* d_jobs, int num_jobs, int64_t tiles, in
                       int max_bits, bool guard, uint32_t* d_counter, int* d_err, cudaStream_t st,
                       const int32_t* d_tile_job) {
   if (tiles <= 0) return cudaSuccess;
-  // a launch over jobs of several digit widths takes the widest one's layout
-  size_t smem = 0;
-  for (int b = 1; b <= max_bits; ++b)
-    smem = std::max(smem, wsweep_smem_bytes<ITEMS>(b, MODE, guard, WIDE));
+  if (max_bits < 0 || max_bits > kMaxDigitBits) return cudaErrorInvalidValue;
+  const size_t smem = wsweep_launch_smem<ITEMS>(max_bits, MODE, guard, WIDE);
   k_wsweep<K, RI, RO, MODE, HI, WIDE, ITEMS><<<(unsigned)tiles, kWThreads, smem, st>>>(
       d_jobs, num_jobs, tiles, pass, d_counter, d_err, d_tile_job);
   return cudaGetLastError();
