@@ -1724,12 +1724,12 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     if (h_err == kErrFold || h_err == TJ_ERR_CAPACITY) return kColumnsAgain;
     if (h_err) return set_err((tj_status)h_err, "device reported %d during the route pass", h_err);
   }
+  int p_first = 0, p_last = nparts - 1;
   if (!range_known) {
     // the smallest key is in the first non-empty batch, the largest in the
     // last one (equal-width ranges over a sample's range may leave the top
     // ranges empty): their rows on both sides (about 2 / nparts of the data)
     // give the exact range
-    int p_first = 0, p_last = nparts - 1;
     while (p_first < nparts - 1 && pcount[(size_t)p_first] + pcount[(size_t)nparts + p_first] == 0)
       ++p_first;
     while (p_last > p_first && pcount[(size_t)p_last] + pcount[(size_t)nparts + p_last] == 0)
@@ -1819,7 +1819,9 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     q.s0 = rstart[(size_t)nparts + j];
     if (q.nr == 0 || q.ns == 0) continue;
     q.lo = j == 0 ? lo : std::max(lo, cuts[(size_t)j - 1]);
-    q.hi = j == ncuts ? hi : std::min(hi, (K)(cuts[(size_t)j] - 1));
+    // (the last batch that has rows holds every key from its cut on: a key above the
+    // sample's range goes to the batch of the sample's largest, past the next cut too)
+    q.hi = j >= p_last || j == ncuts ? hi : std::min(hi, (K)(cuts[(size_t)j] - 1));
     q.lsd = make_plan(lo_bits<K>(q.lo), range_of<K>(q.lo, q.hi), false, maxd, -1, q.nr + q.ns);
     const int bits = q.lsd.key_bits;
     // (narrower batches -- a heavy key's own batch above all -- need no sort
