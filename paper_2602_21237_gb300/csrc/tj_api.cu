@@ -542,6 +542,17 @@ Fold make_fold(uint64_t lo, int key_bits, unsigned long long id_min_u,
   return f;
 }
 
+// First key of a window of 2^kw keys (kw < 64) around a range read off a sample, the
+// spare keys half on either side, within int64's own keys: a window that ran past an
+// end of them would take in keys of the other end, whose offsets then fold and sort
+// them on the wrong side.
+uint64_t window_start(int64_t lo, uint64_t range, int kw) {
+  const uint64_t spare = ((((uint64_t)1 << kw) - 1) - range) / 2;
+  const uint64_t at = (uint64_t)lo ^ (1ull << 63);  // keys below lo
+  const uint64_t first = at < spare ? 0ull : at - spare;
+  return std::min<uint64_t>(first, ~0ull - (((uint64_t)1 << kw) - 1)) ^ (1ull << 63);
+}
+
 // Rows below which a word pass takes the small tile: the large one would
 // leave most of the chip without a CTA.
 constexpr int64_t kWSmallRows = (int64_t)1 << 22;
@@ -1373,8 +1384,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
       const uint64_t slack = range_known ? 0 : range / 32 + 1024;
       if (range + 2 * slack >= range && range + 2 * slack < ((uint64_t)1 << 62)) {
         const int kw = std::max(1, bitlen(range + 2 * slack));
-        const uint64_t spare = range_known ? 0 : ((((uint64_t)1 << kw) - 1) - range) / 2;
-        fold = make_fold<K>(lo_bits<K>(lo) - spare, kw, id_min_u, id_max_u, false);
+        const uint64_t wlo = range_known ? lo_bits<K>(lo) : window_start((int64_t)lo, range, kw);
+        fold = make_fold<K>(wlo, kw, id_min_u, id_max_u, false);
       }
     }
   }
