@@ -418,11 +418,24 @@ __global__ void __launch_bounds__(kJThreads, TJ_JMINB)
           a = go ? a + half + 1 : a;
           n = go ? n - half - 1 : half;
         }
-        int e = a;  // (a < nc: the chunk's last key is not below this one)
-        while (e < nc && Row::key(s_rk[e], ib) == key) ++e;
-        if (e == a) continue;
+        // (a < nc: the chunk's last key is not below this one)
+        if (Row::key(s_rk[a], ib) != key) continue;
+        // the run's end, by steps that double while it goes on, then by halving: a walk
+        // of it by one lane held up every later tile's chained scan (10^7 R rows of
+        // 5000 keys, 10^6 S rows of which 1000 match: 1049 us, now 505)
+        int in = 0, past = 1;  // rows of the run after row a, rows to probe next
+        while (a + past < nc && Row::key(s_rk[a + past], ib) == key) {
+          in = past;
+          past *= 2;
+        }
+        past = min(past, nc - a);
+        while (past - in > 1) {
+          const int mid = (in + past) >> 1;
+          if (Row::key(s_rk[a + mid], ib) == key) in = mid;
+          else past = mid;
+        }
         if (cnt[u] == 0u) start[u] = (uint32_t)(c0 + a);
-        cnt[u] += (uint32_t)(e - a);
+        cnt[u] += (uint32_t)past;
       }
     }
     if (nchunks == 0) asm volatile("cp.async.wait_all;" ::: "memory");
