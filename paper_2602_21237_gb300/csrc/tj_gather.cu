@@ -111,7 +111,13 @@ cudaError_t launch_gather_pairs(const I* pairs, int64_t n, int64_t n_r, int64_t 
   // from a column of 80, 160, 320 and 3200 MB, alone; L2 is 129 MB. Two payload
   // columns of 8 and 4 bytes a row on either side of a join of 10^7 x 4x10^7 rows:
   // 2.03 ms in one launch, now 1.74.)
+  // What a launch of its own saves is reading the column's 64-byte lines from
+  // memory more than once, so it takes about as many pairs as there are lines: from
+  // half as many on (four columns of 320 and 160 MB, one launch against four: 3x10^6
+  // pairs 323 and 312 us, 10^6 140 and 159), and kSplitPairs, below which the
+  // launches count (10^5 pairs 65 and 82 us).
   constexpr int64_t kFarL2 = 4;
+  constexpr int64_t kSplitPairs = (int64_t)1 << 20;
   int dev = 0, l2 = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
@@ -119,7 +125,9 @@ cudaError_t launch_gather_pairs(const I* pairs, int64_t n, int64_t n_r, int64_t 
   auto bytes = [&](const GatherCol& c) { return (c.side ? n_s : n_r) * c.bytes; };
   GatherArgs g, far;  // the launch being filled, the columns that go together
   g.n = far.n = 0;
-  int64_t held = 0;
+  const int64_t limit = 3 * (int64_t)l2 / 2;
+  int64_t held = 0, all = 0;
+  for (int c = 0; c < a.n; ++c) all += bytes(a.c[c]);
   const unsigned blocks = (unsigned)grid;
   auto flush = [&](GatherArgs& x, bool near) {
     if (x.n > 0 && near)
@@ -133,11 +141,11 @@ cudaError_t launch_gather_pairs(const I* pairs, int64_t n, int64_t n_r, int64_t 
     for (int c = 0; c < a.n; ++c) {
       if ((a.c[c].side != 0) != (side != 0)) continue;
       const int64_t b = bytes(a.c[c]);
-      if (b > kFarL2 * l2) {
+      if (b > kFarL2 * l2 || (all > limit && (n < kSplitPairs || b > 128 * n))) {
         far.c[far.n++] = a.c[c];
         continue;
       }
-      if (2 * (held + b) > 3 * (int64_t)l2) {
+      if (held + b > limit) {
         flush(g, true);
         held = 0;
       }
