@@ -359,8 +359,16 @@ size_t fused_smem_bytes() {
 // Eight warps a CTA, four CTAs a multiprocessor: the per-warp counter tables
 // are cleared and summed for every item, so few warps with many rows each pay
 // less for them, and four items in different phases hide each other's waits.
+// Separate columns hold key offsets beside the ids and keep half of a thread's 64-bit
+// S ids in registers at a time, three CTAs a multiprocessor: at 64 registers they
+// spilled 304 bytes a thread, now 44 at 80 (join of 10^8 x 4x10^8 rows whose ids do not
+// fold, under 256 MiB: 20.02 ms, now 18.70; 2x10^7 x 8x10^7 without a budget 3.62 and
+// 3.40; only the halves 19.78, only three CTAs 18.84).
 #ifndef TJ_FUSED_MINB
 #define TJ_FUSED_MINB 4
+#endif
+#ifndef TJ_FUSED_MINB_COLUMNS
+#define TJ_FUSED_MINB_COLUMNS 3
 #endif
 // An item's pair count needs only the R counts (each row has its key's), so it is
 // published before the ranking, half of an item's time, and the chained scan reads
@@ -369,7 +377,7 @@ size_t fused_smem_bytes() {
 constexpr int kFChainWords = 4;
 // WORDS: the rows are folded (tj_word.cu), R and S words at it.rk and it.sk.
 template <typename K, bool WORDS>
-__global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
+__global__ void __launch_bounds__(kFThreads, WORDS ? TJ_FUSED_MINB : TJ_FUSED_MINB_COLUMNS)
     k_fused_join(const FItem* __restrict__ items, WordFmt f,
                  int64_t n_items, uint32_t* __restrict__ item_counter,
                  uint64_t* __restrict__ item_lb, uint32_t* __restrict__ kb_lb,
@@ -426,6 +434,17 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
     const int row = wrow + u * 32 + lane;
     skey[u] = row < ns ? g_sk[row] : pad;
   }
+  // (columns keep the key offsets, 16 bits a row, from here on: their ids are read
+  // when the pairs are written, and folded rows give the offset again with the id)
+  Half<kFItemsS> rank, dig;
+  if constexpr (!WORDS) {
+#pragma unroll
+    for (int u = 0; u < kFItemsS; ++u) dig.set(u, koff(skey[u], sublo));
+  }
+  auto row_digit = [&](int u) -> uint32_t {
+    if constexpr (WORDS) return koff(skey[u], sublo);
+    else return dig.get(u);
+  };
   // R rows: counts per key offset, a key's first R id in the table
   bool dup = false;
 #pragma unroll 1
@@ -464,7 +483,7 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
 #pragma unroll
     for (int u = 0; u < kFItemsS; ++u)
       if (wrow + u * 32 + lane < ns)
-        c += reinterpret_cast<const uint16_t*>(S.cR)[koff(skey[u], sublo)];
+        c += reinterpret_cast<const uint16_t*>(S.cR)[row_digit(u)];
     c = __reduce_add_sync(0xFFFFFFFFu, c);
     if (lane == 0) {
       atomicAdd(&S.s_pairs, c);
@@ -474,15 +493,6 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
     }
   }
   //    S rows counted and ranked
-  Half<kFItemsS> rank, dig;
-  if constexpr (!WORDS) {  // folded rows give the offset again when they are read again
-#pragma unroll
-    for (int u = 0; u < kFItemsS; ++u) dig.set(u, koff(skey[u], sublo));
-  }
-  auto row_digit = [&](int u) -> uint32_t {
-    if constexpr (WORDS) return koff(skey[u], sublo);
-    else return dig.get(u);
-  };
   wrank<kFKeyBits, kFItemsS, kFMaskItems>(row_digit, rank, S.wh[warp], S.wm[warp], ns - wrow);
   __syncthreads();  // counts complete, ranks done
 
@@ -650,16 +660,25 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
   // the S ids (folded rows: the words again, from L2), needed when the pairs
   // are written: their loads in flight while warp 0 runs the chained scan
   using SRow = typename std::conditional<WORDS, uint64_t, K>::type;
-  SRow srow[kFItemsS];
-  {
-    const SRow* __restrict__ src =
-        WORDS ? reinterpret_cast<const SRow*>(it.sk) : reinterpret_cast<const SRow*>(g_sv);
+  // (64-bit columns, whose digits take registers too: half of them, and the other half
+  // after those are written, prefetched to L2)
+  constexpr int kHold = !WORDS && sizeof(K) == 8 ? kFItemsS / 2 : kFItemsS;
+  static_assert(kFItemsS % kHold == 0, "whole groups");
+  const SRow* __restrict__ g_srow =
+      WORDS ? reinterpret_cast<const SRow*>(it.sk) : reinterpret_cast<const SRow*>(g_sv);
+  SRow srow[kHold];
+  auto load_rows = [&](int u0) {
 #pragma unroll
-    for (int u = 0; u < kFItemsS; ++u) {
-      const int row = wrow + u * 32 + lane;
-      srow[u] = row < ns ? src[row] : SRow(0);
+    for (int h = 0; h < kHold; ++h) {
+      const int row = wrow + (u0 + h) * 32 + lane;
+      srow[h] = row < ns ? g_srow[row] : SRow(0);
     }
-  }
+  };
+  load_rows(0);
+#pragma unroll
+  for (int u = kHold; u < kFItemsS; ++u)
+    if (wrow + u * 32 + lane < ns)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(g_srow + (wrow + u * 32 + lane)));
   // 4. chained scan over the group's items (warp 0): the tile's first pair
   if (warp == 0) {
     const uint64_t prefix = chain_prefix<1, kFChainWords>(item_lb, ii, err);
@@ -684,15 +703,16 @@ __global__ void __launch_bounds__(kFThreads, TJ_FUSED_MINB)
   const uint16_t* wx = S.wh[warp];
 #pragma unroll
   for (int u = 0; u < kFItemsS; ++u) {
+    if (u > 0 && u % kHold == 0) load_rows(u);
     if (wrow + u * 32 + lane >= ns) continue;
     uint32_t k;
     K s_id;
     if constexpr (WORDS) {
-      k = koff(srow[u], sublo);
-      s_id = word_id(srow[u]);
+      k = koff(srow[u % kHold], sublo);
+      s_id = word_id(srow[u % kHold]);
     } else {
       k = dig.get(u);
-      s_id = srow[u];
+      s_id = srow[u % kHold];
     }
     const KeyEnt<K> en = S.ent[k];
     if (en.a == ~0ull) continue;  // no R row has the key
