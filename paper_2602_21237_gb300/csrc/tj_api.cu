@@ -514,16 +514,17 @@ void set_job_buffers(RadixJob<K>& j, const K* in_k, const K* in_v, K* ak, K* av,
 // A row is one 64-bit word, (key - wlo) << ib | (id - ilo), when the bits of
 // the key range and of the ids fit together; then every pass but the first and
 // the last moves 8 bytes a row.  32-bit rows always fit (ib = 32).  64-bit
-// rows: the ids' range is known from a sample (two rows a tile), so the window
-// the spare bits allow is centred on it; the folding pass checks every row, and
-// one outside sends the call back to separate columns (kErrFold).
+// rows: the ids' range is known from a sample (two rows a tile, or 32), so the window
+// the spare bits allow is centred on it and up to kFarIds ids outside get codes, where
+// there is a bit for them (see k_far_ids); the folding pass checks every row, and one
+// more sends the call back to separate columns (kErrFold).
 template <typename K>
 Fold make_fold(uint64_t lo, int key_bits, unsigned long long id_min_u,
                unsigned long long id_max_u, bool wide_too) {
   Fold f;
   f.wlo = lo;
   if (sizeof(K) == 4) {
-    f.ib = 32;
+    f.ib = f.cb = 32;
     f.on = true;
     return f;
   }
@@ -535,9 +536,9 @@ Fold make_fold(uint64_t lo, int key_bits, unsigned long long id_min_u,
     f.wide = true;
     avail = 32;
   }
-  const uint64_t window = ((uint64_t)1 << avail) - 1;
   f.ib = avail;
-  f.ilo = (uint64_t)key_of<int64_t>(id_min_u) - (window - range) / 2;
+  f.cb = bitlen(range) < avail && ((uint64_t)kFarIds >> (avail - 1)) == 0 ? avail - 1 : avail;
+  f.ilo = (uint64_t)key_of<int64_t>(id_min_u) - ((((uint64_t)1 << f.cb) - 1) - range) / 2;
   f.on = !f.wide;
   return f;
 }
@@ -608,11 +609,36 @@ void set_word_plan(RadixJob<K>& j, const Plan& p, const Fold& f, uint64_t lo) {
   set_job_plan(j, p);
   j.ilo = f.ilo;
   j.ib = f.ib;
+  j.cb = f.cb;
   j.wlo = f.wlo;
   j.dst_rows = j.n;
   if (f.wide) return;  // digits of the keys as they are
   for (int i = 0; i < p.passes; ++i) j.shift[i] += f.ib;
   j.lo = lo;
+}
+
+// The table of a job's far ids and their count, which lies kFarAt bytes into a call's
+// error word, counters and totals.
+constexpr size_t kFarAt = 192;
+template <typename K>
+void set_far(RadixJob<K>& j, uint64_t* far_ids, uint32_t* far_n) {
+  j.far_ids = far_ids;
+  j.far_n = far_n;
+}
+bool has_far(const Fold& f) { return f.cb < f.ib; }
+uint32_t far_count(const int64_t* misc) {
+  return reinterpret_cast<const uint32_t*>(misc)[kFarAt / sizeof(uint32_t)];
+}
+// ... back into a result's n ids (a call's results are complete when it returns)
+template <typename K>
+cudaError_t put_far_ids(K* ids, int64_t n, const Fold& f, const uint64_t* far_ids,
+                        uint32_t far_n, cudaStream_t st) {
+  if constexpr (sizeof(K) == 8) {  // (32-bit ids always fold)
+    if (far_n == 0) return cudaSuccess;
+    const cudaError_t e = launch_far_ids(ids, n, f, far_ids, far_n, st);
+    return e != cudaSuccess ? e : sync_stream(st);
+  }
+  return cudaSuccess;
 }
 
 // One word pass: from columns into words, or words to words (8 bytes a row
@@ -878,7 +904,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     const int64_t wtile = (int64_t)kWThreads * items;
     const int64_t wt_r = ceil_div(nr, wtile), wt = wt_r + ceil_div(ns, wtile);
     const int64_t lb_words = wt << wp.max_bits;
-    size_t o_a, o_b, o_ai, o_bi, o_wt, o_whist, o_wlb;
+    size_t o_a, o_b, o_ai, o_bi, o_wt, o_far, o_whist, o_wlb;
     auto lay_out = [&](bool per_pass) -> size_t {
       Carve wc;
       o_a = wc.add<uint64_t>((size_t)(nr + ns));
@@ -886,6 +912,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
       o_ai = wc.add<uint32_t>(fold.wide ? (size_t)(nr + ns) : 0);
       o_bi = wc.add<uint32_t>(fold.wide && wp.passes > 1 ? (size_t)(nr + ns) : 0);
       o_wt = wc.add<JTile<K>>(jtiles);
+      o_far = wc.add<uint64_t>(has_far(fold) ? kFarIds : 0);
       o_whist = wc.add<uint32_t>((size_t)2 * wp.passes << wp.max_bits);
       o_wlb = wc.add<uint32_t>((size_t)(per_pass ? wp.passes : 1) * lb_words);
       return wc.off;
@@ -915,6 +942,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
       x.hist_stride = h.hist_stride;
       x.hist = h.hist;
       set_word_plan(x, wp, fold, 0);
+      set_far(x, big.at<uint64_t>(o_far), ctl.at<uint32_t>(o_misc + kFarAt));
       x.tile0 = i ? wt_r : 0;
       x.lookback = big.at<uint32_t>(o_wlb) + ((i ? wt_r : 0) << wp.max_bits);
       x.lb_stride = regions ? lb_words : 0;
@@ -967,7 +995,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     TJ_CUDA(sync_stream(st));
     const int64_t h_total = misc[d_total - reinterpret_cast<int64_t*>(d_err)];
     const int h_err = *reinterpret_cast<const int*>(misc);
-    if (h_err == kErrFold) {  // an id outside the window of the sampled ones
+    if (h_err == kErrFold) {  // too many ids outside the window of the sampled ones
       TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
       break;
     }
@@ -983,6 +1011,7 @@ tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* 
     if (h_total > cap)
       return set_err(TJ_ERR_CAPACITY, "result has %lld pairs, capacity %lld", (long long)h_total,
                      (long long)cap);
+    TJ_CUDA(put_far_ids(out, 2 * h_total, fold, big.at<uint64_t>(o_far), far_count(misc), st));
     return TJ_OK;
   }
   Block big;
@@ -1538,6 +1567,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   };
   const size_t o_cuts = cc.add<K>(kMaxCuts);
   const size_t o_wcuts = words ? cc.add<uint64_t>(kMaxCuts) : 0;  // cuts as offsets
+  const size_t o_far = has_far(fold) ? cc.add<uint64_t>(kFarIds) : 0;
   const size_t o_tab = cc.add<uint16_t>(kRouteBuckets + 1);
   const size_t o_hist = cc.add<uint32_t>((size_t)nch * kMaxBins);
   const size_t o_rend = cc.add<uint32_t>(2 * (size_t)kMaxBins);  // regions' ends (est)
@@ -1609,6 +1639,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
         x.wlo = fold.wlo;
         x.ilo = fold.ilo;
         x.ib = fold.ib;
+        x.cb = fold.cb;
+        set_far(x, stg.at<uint64_t>(o_far), stg.at<uint32_t>(o_misc + kFarAt));
         x.dst_rows = side_rows[chunks[(size_t)c].side];
         if (!radix_route) x.cuts = reinterpret_cast<const K*>(stg.at<uint64_t>(o_wcuts));
       }
@@ -1678,7 +1710,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   // larger of the two blocks + tables.
   const int64_t control = (int64_t)(cc.off - staging);
   // what separate columns would need decides whether the budget suffices
-  const int64_t ask_control = control - (words ? (int64_t)(kMaxCuts * sizeof(uint64_t)) : 0);
+  const int64_t ask_control = control - (words ? (int64_t)(kMaxCuts * sizeof(uint64_t)) : 0) -
+                              (has_far(fold) ? (int64_t)(kFarIds * sizeof(uint64_t)) : 0);
   if (budget && ask_control + lb_max + 4096 > (int64_t)budget)
     return set_err(TJ_ERR_BUDGET, "budget %zu below the route pass's %lld bytes", budget,
                    (long long)(ask_control + lb_max + 4096));
@@ -2082,7 +2115,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     int64_t bad = -1;
     for (size_t i = 0; i < P.size() && bad < 0; ++i)
       if (P[i].ask > room) bad = (int64_t)i;
-    if (bad < 0 && make_groups(use) >= 0) return kColumnsAgain;  // (words always fit, but for 8 KB)
+    if (bad < 0 && make_groups(use) >= 0) return kColumnsAgain;  // (words always fit, but for 24 KB)
     if (bad >= 0)
       return set_err(TJ_ERR_BUDGET,
                      "batch of keys [%lld, %lld] needs %lld bytes of working set, budget "
@@ -2512,11 +2545,11 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   }
   back.now();
   stats.radix_passes = maxp;
-  int64_t h_total = 0;
-  int h_err = 0;
+  int64_t h_total = 0, misc[32] = {};
   TJ_CUDA(get_small(&h_total, d_gbase + n_bases, sizeof(int64_t), st));
-  TJ_CUDA(get_small(&h_err, d_err, sizeof(int), st));
+  TJ_CUDA(get_small(misc, d_err, sizeof(misc), st));
   TJ_CUDA(sync_stream(st));
+  const int h_err = *reinterpret_cast<const int*>(misc);
   if (h_total <= cap && !plans.empty())
     tr.add_bytes(lanes > 1 ? "group/lanes" : (plans.back().runs.back().fused ? "fused" : "join"),
                  2.0 * w * (double)h_total);
@@ -2527,6 +2560,8 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
   if (h_total > cap)
     return set_err(TJ_ERR_CAPACITY, "result has %lld pairs, capacity %lld", (long long)h_total,
                    (long long)cap);
+  if (words)
+    TJ_CUDA(put_far_ids(out, 2 * h_total, fold, stg.at<uint64_t>(o_far), far_count(misc), st));
   return TJ_OK;
 }
 
@@ -2554,6 +2589,7 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
   const size_t o_a = bc.add<uint64_t>((size_t)n);
   const size_t o_ai = bc.add<uint32_t>(f.wide ? (size_t)n : 0);
   const size_t o_b = bc.add<uint64_t>(!turns && P > 2 ? (size_t)n : 0);
+  const size_t o_far = bc.add<uint64_t>(has_far(f) ? kFarIds : 0);
   const size_t o_hist = bc.add<uint32_t>((size_t)P << plan.max_bits);
   const size_t o_lb = bc.add<uint32_t>((size_t)(regions ? P : 1) * lb_words);
   Block big;
@@ -2568,6 +2604,8 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
   hj[0].hist = big.at<uint32_t>(o_hist);
   hj[1] = hj[0];
   set_word_plan(hj[1], plan, f, 0);
+  set_far(hj[1], big.at<uint64_t>(o_far),
+          reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(d_err) + kFarAt));
   hj[1].lookback = big.at<uint32_t>(o_lb);
   hj[1].lb_stride = regions ? lb_words : 0;
   auto folds = [&](int p) { return p == 0 || (turns && (p & 1) == 0); };
@@ -2608,12 +2646,16 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
       tr.end();
     }
   }
-  TJ_CUDA(get_small(h_err, d_err, sizeof(int), st));
+  int64_t misc[32] = {};
+  TJ_CUDA(get_small(misc, d_err, sizeof(misc), st));
   TJ_CUDA(sync_stream(st));
+  *h_err = *reinterpret_cast<const int*>(misc);
   if constexpr (sizeof(K) == 8) {
     if (*h_err == kErrRuns)  // back into columns: a stable order by the prefix
       TJ_CUDA(launch_runs(a, big.at<uint32_t>(o_ai), n, f, plan.shift[0], false, keys, ids, d_err,
                           st));
+    if (*h_err == 0 || *h_err == kErrRuns)
+      TJ_CUDA(put_far_ids(ids, n, f, big.at<uint64_t>(o_far), far_count(misc), st));
   }
   return TJ_OK;
 }
@@ -2708,7 +2750,7 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
       if (h_err == kErrFold) break;
       prefix = false;  // a long run was out of order
     }
-    // an id outside the window of the sampled ones: the columns are untouched
+    // too many ids outside the window of the sampled ones: the columns are untouched
     stats.radix_passes = plan.passes;
     stats.digit_bits = plan.max_bits;
   }
@@ -3043,6 +3085,7 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   // (word passes: a second view of the jobs, digits of words, and its tile map)
   const size_t o_pjobs = bc.add<RadixJob<K>>(words ? (size_t)(2 * nj) : 0);
   const size_t o_pmap = bc.add<int32_t>(words ? (size_t)std::max<int64_t>(ptiles, 1) : 0);
+  const size_t o_far = bc.add<uint64_t>(has_far(fold) ? kFarIds : 0);
   Block big;
   TJ_CUDA(big.alloc(bc.off, st));
   stats.scratch_peak = (int64_t)(bc.off + cc.off);
@@ -3071,6 +3114,7 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
         Fold f = fold;
         f.wlo = plo[(size_t)j];
         set_word_plan(q, plans[(size_t)j], f, 0);
+        set_far(q, big.at<uint64_t>(o_far), ctl.at<uint32_t>(o_misc + kFarAt));
         q.tile0 = ptile_at[(size_t)(2 * j + side)];
         const int64_t w0 = side ? R + a : a;
         uint64_t* buf[2] = {big.at<uint64_t>(o_w[0]) + w0,
@@ -3150,12 +3194,11 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
     if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
     if (e == cudaSuccess) e = cudaGraphLaunch(exec, st);
   }
-  int64_t h_total = 0;
-  int h_err = 0;
-  if (e == cudaSuccess)
-    e = get_small(&h_total, d_total, sizeof(int64_t), st);
-  if (e == cudaSuccess) e = get_small(&h_err, d_err, sizeof(int), st);
+  int64_t misc[32] = {};  // the error word, the counters, the total
+  if (e == cudaSuccess) e = get_small(misc, d_err, sizeof(misc), st);
   if (e == cudaSuccess) e = sync_stream(st);
+  const int64_t h_total = misc[d_total - reinterpret_cast<int64_t*>(d_err)];
+  const int h_err = *reinterpret_cast<const int*>(misc);
   if (exec) cudaGraphExecDestroy(exec);
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess)
@@ -3168,6 +3211,8 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
   if (h_total > cap)
     return set_err(TJ_ERR_CAPACITY, "batch result has %lld pairs, capacity %lld",
                    (long long)h_total, (long long)cap);
+  if (words)
+    TJ_CUDA(put_far_ids(out, 2 * h_total, fold, big.at<uint64_t>(o_far), far_count(misc), st));
   return TJ_OK;
 }
 

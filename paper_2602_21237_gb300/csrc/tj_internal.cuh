@@ -133,7 +133,14 @@ struct RadixJob {
       const K* fold_v;  // the id column of passes that fold
       uint64_t wlo, ilo;
       int64_t dst_rows;  // room at dst_k (rows) of a pass that folds
-      const K* ids;      // statistics: ids sampled beside the keys (may be null)
+      const K* ids;      // statistics: ids sampled beside the keys (null in all jobs
+                         // of a launch, or in none)
+      // ids whose offset has more than cb bits, cb < ib (pass 0): the n-th of them
+      // becomes 2^cb + n, and its value far_ids[n]; the pairs or rows that come out
+      // get it back (k_far_ids). cb = ib: a row with such an id does not fold.
+      uint64_t* far_ids;
+      uint32_t* far_n;
+      int32_t cb;
     };
   };
   K* dst_k[kMaxPasses];
@@ -166,9 +173,10 @@ struct RadixJob {
   uint64_t route_hi;
 };
 
-// A row's key offset or id did not fit its word: the call runs again on
-// separate columns.
+// A row's key offset did not fit its word, or more than kFarIds ids did not: the
+// call runs again on separate columns.
 constexpr int kErrFold = 101;
+constexpr int kFarIds = 2048;
 
 // A long run of equal key prefixes is not in order (k_runs): the call sorts by
 // every digit.
@@ -196,6 +204,7 @@ struct Fold {
   bool wide = false;  // wide rows instead: the key as it is and a 32-bit id
   uint64_t wlo = 0, ilo = 0;
   int ib = 0;
+  int cb = 0;  // see RadixJob::far_ids
 };
 
 // Layout of the rows a join kernel reads: separate key and id columns (ib = 0)
@@ -420,6 +429,9 @@ static_assert((kRunTile + 2 * kRunMax) % kRunThreads == 0, "whole rounds of load
 cudaError_t launch_prefix_sample(const int64_t* keys, int64_t n, const KeyStats* d_stats,
                                  int prefix_bits, int min_bits, uint32_t* d_pairs,
                                  cudaStream_t st);
+// ids that stand for far ones -> their values
+cudaError_t launch_far_ids(int64_t* ids, int64_t n, const Fold& f, const uint64_t* far_ids,
+                           uint32_t far_n, cudaStream_t st);
 cudaError_t launch_runs(const uint64_t* rows, const uint32_t* ids, int64_t n, const Fold& f, int s,
                         bool fix, int64_t* out_k, int64_t* out_v, int* d_err, cudaStream_t st);
 
@@ -452,7 +464,7 @@ cudaError_t launch_group_maps(const RadixJob<K>* d_rjobs, int nr, int32_t* d_rma
 template <typename K>
 cudaError_t launch_sample_gather(const K* a, int64_t ma, int64_t off_a, const K* b, int64_t mb,
                                  int64_t off_b, int stride, K* out_k, K* out_v, cudaStream_t st);
-// *out's id fields: the range of about 8000 ids of each side (out filled with 0xFF before)
+// *out's id fields: the range of about 65000 ids of each side (out filled with 0xFF before)
 template <typename K>
 cudaError_t launch_id_range(const K* a, int64_t na, const K* b, int64_t nb, KeyStats* out,
                             cudaStream_t st);

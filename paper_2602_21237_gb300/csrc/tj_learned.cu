@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(256)
 template <typename K>
 cudaError_t launch_id_range(const K* a, int64_t na, const K* b, int64_t nb, KeyStats* out,
                             cudaStream_t st) {
-  k_id_range<K><<<32, 256, 0, st>>>(a, na, b, nb, out);
+  k_id_range<K><<<256, 256, 0, st>>>(a, na, b, nb, out);
   return cudaGetLastError();
 }
 template cudaError_t launch_id_range<int32_t>(const int32_t*, int64_t, const int32_t*, int64_t,

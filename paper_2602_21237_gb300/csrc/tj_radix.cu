@@ -142,19 +142,34 @@ __global__ void __launch_bounds__(kThreads, 8) k_stats(const RadixJob<K>* __rest
   // per job the run touches
   const int64_t per = (total_tiles + gridDim.x - 1) / gridDim.x;
   const int64_t t0 = (int64_t)blockIdx.x * per, t1 = min(total_tiles, t0 + per);
-  if (threadIdx.x == 0 && t0 < t1) {
-    // a sample of the ids' range: the run's first and last row (and the last
-    // row of the job it starts in)
-    auto sample = [&](int j, int64_t r) {
-      if (!jobs[j].ids) return;
-      const unsigned long long u = order_u(jobs[j].ids[r]);
-      atomicMin(&stats[j].id_min_u, u);
-      atomicMin(&stats[j].id_max_u, ~u);
-    };
-    const int j0 = find_job(jobs, num_jobs, t0), j1 = find_job(jobs, num_jobs, t1 - 1);
-    sample(j0, (t0 - jobs[j0].tile0) * tile);
-    sample(j1, min(jobs[j1].n, (t1 - jobs[j1].tile0) * tile) - 1);
-    if (j0 != j1) sample(j0, jobs[j0].n - 1);
+  if (!WORDS && jobs[0].ids) {
+    // a sample of the ids' range: the first and last row of every tile, of small
+    // inputs (a tile a CTA) 32 rows, whole warps at a time
+    const int lg = per > 1 ? 1 : 5;
+    const int rows = (int)max((int64_t)0, t1 - t0) << lg;
+    for (int b = 32 * warp; b < rows; b += kThreads) {
+      const int i = min(b + lane, rows - 1);
+      const int64_t t = t0 + (i >> lg);
+      const int j = find_job(jobs, num_jobs, t);
+      const int64_t first = (t - jobs[j].tile0) * tile;
+      const int nt = (int)min((int64_t)tile, jobs[j].n - first);  // rows of the tile
+      const int step = lg == 1 ? nt : (nt + 30) / 31;
+      const unsigned long long u =
+          order_u(jobs[j].ids[first + min(nt - 1, (i & ((1 << lg) - 1)) * step)]);
+      unsigned long long a = u, z = ~u;
+      if (__all_sync(0xFFFFFFFFu, j == __shfl_sync(0xFFFFFFFFu, j, 0))) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const unsigned long long x = __shfl_xor_sync(0xFFFFFFFFu, a, o);
+          const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, z, o);
+          a = x < a ? x : a;
+          z = y < z ? y : z;
+        }
+        if (lane != 0) continue;
+      }
+      atomicMin(&stats[j].id_min_u, a);
+      atomicMin(&stats[j].id_max_u, z);
+    }
   }
   int cur = -1;
   int64_t cur_end = 0;  // first tile after the current job

@@ -13,6 +13,10 @@
 // bits) travel as "wide" rows, the key as it is beside a 32-bit id, when their
 // ids' range fits 32 bits.
 //
+// The ids' range is a sample's.  The few ids outside it (a sentinel in some rows, say)
+// fold as codes, which have the id's top bit, their values go to a table beside the
+// words, and one pass over the result puts them back (k_far_ids).
+//
 // k_wsweep is one onesweep pass (decoupled look-back, as k_onesweep in
 // tj_radix.cu) over a tile of kWThreads * ITEMS rows: take the digits, rank
 // them inside the warp, move the words to their tile-sorted slots in shared
@@ -168,8 +172,9 @@ __device__ __forceinline__ int wlookback(const uint32_t (&v)[W], uint32_t& prefi
 //   1. digits, 16 bits a row in registers (from the key column, or the words'
 //      upper halves when the key is there), and stable ranks inside each warp;
 //   2. per digit: sum over the warps, publish to the look-back chain, scan;
-//   3. the rows are read again, from L2 (RAW_IN: keys and ids, folded; a row
-//      whose key offset or id does not fit sets *err = kErrFold), and move to
+//   3. the rows are read again, from L2 (RAW_IN: keys and ids, folded; far ids get
+//      a code; a row whose key offset does not fit, or one far id too many, sets
+//      *err = kErrFold), and move to
 //      their tile-sorted slots in shared memory, after the digits' threads have
 //      finished the look-back (bounded wait);
 //   4. slots in order -> global: each digit's run lands contiguously (RAW_OUT:
@@ -392,9 +397,19 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
   {
     const K* __restrict__ vp = RAW_IN ? J->fold_v + row0 : nullptr;
     const U wlo = (U)J->wlo, ilo = (U)J->ilo;
+    // bits that no row of a group should have: far ids, keys that do not fit (a later
+    // pass that folds meets far ids' codes, which are ids of the window to it)
     uint64_t out = 0;
-    // (pairs of 64-bit columns: half of the rows at a time, to spare registers)
-    constexpr int G = (RAW_IN && sizeof(K) == 8) || WIDE ? ITEMS / 2 : ITEMS;
+    constexpr bool kCheck = RAW_IN && sizeof(K) == 8;
+    const int cb = kCheck && pass == 0 ? J->cb : ib;
+    const uint32_t code_bit = WIDE && cb < 32 ? 1u << cb : 0u;  // (cb is 31 or 32)
+    uint32_t wide_out = 0;
+    bool misfit = false;  // a key that does not fit, or a far id too many
+    // (pairs of 64-bit columns: half of the rows at a time, wide ones a quarter, to
+    // spare registers)
+    constexpr int G = RAW_IN && WIDE                        ? ITEMS / 4
+                      : (RAW_IN && sizeof(K) == 8) || WIDE ? ITEMS / 2
+                                                            : ITEMS;
     static_assert(ITEMS % G == 0, "whole groups");
     const uint32_t* __restrict__ ip =
         WIDE && !RAW_IN ? reinterpret_cast<const uint32_t*>(J->dst_v[pass - 1]) + row0 : nullptr;
@@ -413,8 +428,8 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
 #pragma unroll
         for (int i = 0; i < G; ++i) {
           const uint64_t io = (uint64_t)(U)((U)v[i] - ilo);
-          out |= io >> 32;
           id[i] = (uint32_t)io;
+          wide_out |= (uint32_t)(io >> 32) | (id[i] & code_bit);
         }
       } else if constexpr (RAW_IN) {
         K v[G], k[G];
@@ -427,7 +442,7 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
 #pragma unroll
         for (int i = 0; i < G; ++i) {
           const uint64_t ko = (uint64_t)(U)((U)k[i] - wlo), io = (uint64_t)(U)((U)v[i] - ilo);
-          if (sizeof(K) == 8 && wbase + (i0 + i) * 32 < nvalid) out |= (io >> ib) | (ko >> (64 - ib));
+          if (kCheck && wbase + (i0 + i) * 32 < nvalid) out |= (io >> cb) | (ko >> (64 - ib));
           w[i] = (ko << ib) | (io & idm);
         }
       } else {
@@ -437,6 +452,31 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
           w[i] = r < nvalid ? wp[r] : 0ull;
           if constexpr (WIDE) id[i] = r < nvalid ? ip[r] : 0u;
         }
+      }
+      if (kCheck && (WIDE ? wide_out != 0u : out != 0ull)) {
+        // which rows: far ids get a code (here, before the rows move, it needs no
+        // register beyond the group's; after all groups it held their ranks, and wide
+        // folding passes took 2% more)
+#pragma unroll 1
+        for (int i = 0; i < G && !misfit; ++i) {
+          const int r = wbase + (i0 + i) * 32;
+          if (r >= nvalid) break;
+          const K v = vp[r];
+          if (!WIDE) misfit = ((uint64_t)(U)((U)kp[r] - wlo) >> (64 - ib)) != 0ull;
+          if (((uint64_t)(U)((U)v - ilo) >> cb) == 0ull) continue;
+          const uint32_t k = cb < ib ? atomicAdd(J->far_n, 1u) : (uint32_t)kFarIds;
+          misfit |= k >= (uint32_t)kFarIds;
+          if (misfit) break;
+          J->far_ids[k] = (uint64_t)v;
+#pragma unroll
+          for (int q = 0; q < G; ++q)
+            if (q == i) {
+              if constexpr (WIDE) id[q] = (1u << cb) + k;
+              else w[q] = (w[q] & ~idm) | ((1ull << cb) + k);
+            }
+        }
+        out = 0;
+        wide_out = 0;
       }
 #pragma unroll
       for (int i = 0; i < G; ++i) {
@@ -451,8 +491,7 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
         }
       }
     }
-    if (RAW_IN && sizeof(K) == 8 && out != 0ull &&
-        wld_volatile(reinterpret_cast<const uint32_t*>(err)) == 0u)
+    if (misfit && wld_volatile(reinterpret_cast<const uint32_t*>(err)) == 0u)
       atomicCAS(err, 0, kErrFold);
   }
   __syncthreads();
@@ -614,6 +653,28 @@ __global__ void __launch_bounds__(kRunThreads)
   if (bad) atomicCAS(err, 0, kErrRuns);
 }
 
+// Far ids back into a result: an id whose offset is a code takes the code's value. (No
+// other row has such an id: one that had was far itself.) A read of the ids and a write
+// of few: a sort of 10^8 rows with one far id takes 2.44 ms, 0.15 more than without
+// (4.34 when it went back to columns, 3.43 on columns from the start).
+__global__ void __launch_bounds__(256)
+    k_far_ids(int64_t* __restrict__ ids, int64_t n, uint64_t ilo, uint64_t esc,
+              const uint64_t* __restrict__ far_ids, uint32_t far_n) {  // esc: code 0
+  constexpr int kRows = 8;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x * kRows;
+  for (int64_t r0 = (int64_t)blockIdx.x * blockDim.x * kRows + threadIdx.x; r0 < n; r0 += step) {
+    uint64_t x[kRows];
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) {
+      const int64_t r = r0 + u * 256;
+      x[u] = r < n ? (uint64_t)ids[r] - ilo - esc : ~0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (x[u] < (uint64_t)far_n) ids[r0 + u * 256] = (int64_t)far_ids[x[u]];
+  }
+}
+
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
@@ -756,6 +817,15 @@ cudaError_t launch_prefix_sample(const int64_t* keys, int64_t n, const KeyStats*
                                  cudaStream_t st) {
   if (n < kPrefSample || prefix_bits > 32 || min_bits < prefix_bits) return cudaErrorInvalidValue;
   k_prefix_sample<<<1, kPrefSample / 2, 0, st>>>(keys, n, d_stats, prefix_bits, min_bits, d_pairs);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_far_ids(int64_t* ids, int64_t n, const Fold& f, const uint64_t* far_ids,
+                           uint32_t far_n, cudaStream_t st) {
+  if (n <= 0 || far_n == 0) return cudaSuccess;
+  const unsigned grid = (unsigned)std::min<int64_t>((n + 2047) / 2048, 152 * 16);
+  k_far_ids<<<grid, 256, 0, st>>>(ids, n, f.ilo, 1ull << f.cb, far_ids,
+                                  std::min<uint32_t>(far_n, kFarIds));
   return cudaGetLastError();
 }
 
