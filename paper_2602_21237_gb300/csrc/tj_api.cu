@@ -581,11 +581,13 @@ Plan make_word_plan(uint64_t lo, uint64_t range, bool even, int max_digit, int m
 
 // Sorts by a key prefix: three digits of the key's leading 24 or 27 bits, then
 // the runs of equal prefixes (k_runs). Worth it from five passes on; keys a
-// sample finds nearly unique by that prefix (kPrefPairs pairs among 2048 rows
-// mean runs of 1 + n / 10^6 rows or so as the average row sees them).
+// sample finds nearly unique by that prefix (2 pairs among 2048 rows mean runs of
+// 1 + n / 10^6 rows or so as the average row sees them; above 2^27 rows, where such
+// runs would near kRunMax, 4 pairs among 8192 mean 1 + n / 8x10^6). Long runs that the
+// sample misses are sorted by themselves where they are few.
 constexpr int64_t kPrefMinRows = (int64_t)1 << 17;
 constexpr int kPrefMinBits = 37;
-constexpr uint32_t kPrefPairs = 2;
+uint32_t prefix_pairs(int64_t n) { return prefix_sample(n) == 2048 ? 2u : 4u; }
 int prefix_digit(int64_t n) { return n <= (int64_t)1 << 22 ? 8 : 9; }
 
 Plan make_prefix_plan(uint64_t lo, int key_bits, int64_t n) {
@@ -618,8 +620,8 @@ void set_word_plan(RadixJob<K>& j, const Plan& p, const Fold& f, uint64_t lo) {
 }
 
 // The table of a job's far ids and their count, which lies kFarAt bytes into a call's
-// error word, counters and totals.
-constexpr size_t kFarAt = 192;
+// error word, counters and totals (a sort's two counts of long runs behind it).
+constexpr size_t kFarAt = 192, kRunsAt = 200;
 template <typename K>
 void set_far(RadixJob<K>& j, uint64_t* far_ids, uint32_t* far_n) {
   j.far_ids = far_ids;
@@ -742,7 +744,7 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
                          K* out, int64_t cap, int64_t* out_count, tj_stats& stats, Tracer& tr,
                          cudaStream_t st);
 template <typename K>
-tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st);
+tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st, bool prefix_ok = true);
 
 template <typename K>
 tj_status join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, const K* is, int64_t ns,
@@ -2566,6 +2568,51 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
 }
 
 // ---- sort ---------------------------------------------------------------------------
+// The long runs that k_runs listed, sorted by themselves (they ascend by prefix, so one
+// sort of all their rows leaves each in its place): 3x10^7 hashed keys with 15000 small
+// ones among them took 3.70 ms by sorting all rows again, by every digit, now 1.65.
+// *done = false: too many to be listed, or a quarter of the rows and more.
+tj_status sort_long_runs(int64_t* keys, int64_t* ids, int64_t n, const uint32_t* d_runs,
+                         const uint32_t* runs_n, bool* done, tj_stats& stats, cudaStream_t st) {
+  *done = false;
+  const size_t m = runs_n[0];
+  if (m == 0 || m > (size_t)kLongRuns || runs_n[1] != m) return TJ_OK;
+  std::vector<uint32_t> at(2 * (size_t)kLongRuns), off(m + 1, 0u);
+  TJ_CUDA(get_small(at.data(), d_runs, at.size() * sizeof(uint32_t), st));
+  TJ_CUDA(sync_stream(st));
+  std::sort(at.begin(), at.begin() + m);
+  std::sort(at.begin() + kLongRuns, at.begin() + kLongRuns + m);
+  int64_t rows = 0;
+  for (size_t r = 0; r < m; ++r) {
+    off[r] = (uint32_t)rows;
+    rows += (int64_t)at[kLongRuns + r] - at[r] + 1;
+  }
+  off[m] = (uint32_t)rows;
+  if (rows > n / 4) return TJ_OK;
+  Carve c;
+  const size_t o_k = c.add<int64_t>((size_t)rows), o_v = c.add<int64_t>((size_t)rows);
+  const size_t o_first = c.add<uint32_t>(m), o_off = c.add<uint32_t>(m + 1);
+  Block b;
+  TJ_CUDA(b.alloc(c.off, st));
+  TJ_CUDA(put_small(b.at<uint32_t>(o_first), at.data(), m * sizeof(uint32_t), st));
+  TJ_CUDA(put_small(b.at<uint32_t>(o_off), off.data(), (m + 1) * sizeof(uint32_t), st));
+  int64_t* const pk = b.at<int64_t>(o_k);
+  int64_t* const pv = b.at<int64_t>(o_v);
+  TJ_CUDA(launch_long_rows(b.at<uint32_t>(o_first), b.at<uint32_t>(o_off), (int)m, rows, keys, ids,
+                           pk, pv, false, st));
+  const tj_stats keep = g_stats;
+  const tj_status s = sort_impl<int64_t>(pk, pv, rows, st, false);
+  stats.radix_passes += g_stats.radix_passes;  // (of those rows)
+  stats.scratch_peak += (int64_t)c.off + g_stats.scratch_peak;
+  g_stats = keep;
+  if (s != TJ_OK) return s;
+  TJ_CUDA(launch_long_rows(b.at<uint32_t>(o_first), b.at<uint32_t>(o_off), (int)m, rows, keys, ids,
+                           pk, pv, true, st));
+  TJ_CUDA(sync_stream(st));
+  *done = true;
+  return TJ_OK;
+}
+
 // The passes over folded rows.  64-bit rows: columns -> words -> ... -> columns,
 // the words alternating between two scratch arrays, so the caller's columns
 // stay as they are until the last pass (which does not run if a row failed to
@@ -2590,6 +2637,7 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
   const size_t o_ai = bc.add<uint32_t>(f.wide ? (size_t)n : 0);
   const size_t o_b = bc.add<uint64_t>(!turns && P > 2 ? (size_t)n : 0);
   const size_t o_far = bc.add<uint64_t>(has_far(f) ? kFarIds : 0);
+  const size_t o_runs = bc.add<uint32_t>(prefix ? 2 * kLongRuns : 0);
   const size_t o_hist = bc.add<uint32_t>((size_t)P << plan.max_bits);
   const size_t o_lb = bc.add<uint32_t>((size_t)(regions ? P : 1) * lb_words);
   Block big;
@@ -2638,22 +2686,35 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
                              st));
     tr.end();
   }
-  if constexpr (sizeof(K) == 8) {
-    if (prefix) {
-      tr.begin("runs", ((f.wide ? 12.0 : 8.0) + 16.0) * n);
-      TJ_CUDA(launch_runs(a, big.at<uint32_t>(o_ai), n, f, plan.shift[0], true, keys, ids, d_err,
-                          st));
-      tr.end();
-    }
+  uint32_t* const d_runs_n =
+      reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(d_err) + kRunsAt);
+  auto runs = [&](bool fix) -> cudaError_t {
+    if constexpr (sizeof(K) == 8)
+      return launch_runs(a, big.at<uint32_t>(o_ai), n, f, plan.shift[0], fix, keys, ids,
+                         big.at<uint32_t>(o_runs), d_runs_n, d_err, st);
+    return cudaErrorInvalidValue;  // (32-bit keys have too few bits)
+  };
+  if (prefix) {
+    tr.begin("runs", ((f.wide ? 12.0 : 8.0) + 16.0) * n);
+    TJ_CUDA(runs(true));
+    tr.end();
   }
   int64_t misc[32] = {};
   TJ_CUDA(get_small(misc, d_err, sizeof(misc), st));
   TJ_CUDA(sync_stream(st));
   *h_err = *reinterpret_cast<const int*>(misc);
   if constexpr (sizeof(K) == 8) {
-    if (*h_err == kErrRuns)  // back into columns: a stable order by the prefix
-      TJ_CUDA(launch_runs(a, big.at<uint32_t>(o_ai), n, f, plan.shift[0], false, keys, ids, d_err,
-                          st));
+    if (*h_err == kErrRuns) {
+      bool done = false;
+      const uint32_t* runs_n = reinterpret_cast<const uint32_t*>(misc) + kRunsAt / sizeof(uint32_t);
+      const tj_status s =
+          sort_long_runs(keys, ids, n, big.at<uint32_t>(o_runs), runs_n, &done, stats, st);
+      if (s != TJ_OK) return s;
+      if (done)
+        *h_err = 0;
+      else  // back into columns: a stable order by the prefix
+        TJ_CUDA(runs(false));
+    }
     if (*h_err == 0 || *h_err == kErrRuns)
       TJ_CUDA(put_far_ids(ids, n, f, big.at<uint64_t>(o_far), far_count(misc), st));
   }
@@ -2661,7 +2722,7 @@ tj_status sort_words(K* keys, K* ids, int64_t n, const Plan& plan, const Fold& f
 }
 
 template <typename K>
-tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
+tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st, bool prefix_ok) {
   tj_stats stats = {};
   stats.groups = 1;
   if (n <= 1) {
@@ -2699,7 +2760,7 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
   KeyStats hs;
   bool sampled = false;
   if constexpr (sizeof(K) == 8) {
-    if (n >= kPrefMinRows) {
+    if (prefix_ok && n >= kPrefMinRows) {
       uint32_t* d_pairs = ctl.at<uint32_t>(o_misc + 128);
       sampled = true;
       TJ_CUDA(launch_prefix_sample(keys, n, d_stats, 3 * prefix_digit(n), kPrefMinBits, d_pairs,
@@ -2730,7 +2791,7 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
                            ? make_word_plan(plan.lo, range_of<K>(lo, hi),
                                             sizeof(K) == 4 || fold.wide, max_digit_bits<K>(), 2)
                            : plan;
-    bool prefix = wplan.passes >= 5 && plan.key_bits >= kPrefMinBits && pref_pairs <= kPrefPairs;
+    bool prefix = wplan.passes >= 5 && plan.key_bits >= kPrefMinBits && pref_pairs <= prefix_pairs(n);
     int h_err = 0;
     while (true) {
       const Plan use = prefix ? make_prefix_plan(plan.lo, plan.key_bits, n) : wplan;
@@ -2748,7 +2809,7 @@ tj_status sort_impl(K* keys, K* ids, int64_t n, cudaStream_t st) {
         return set_err((tj_status)h_err, "device reported %d", h_err);
       TJ_CUDA(cudaMemsetAsync(ctl.p + o_misc, 0, 32 * sizeof(int64_t), st));
       if (h_err == kErrFold) break;
-      prefix = false;  // a long run was out of order
+      prefix = false;  // long runs out of order, many rows of them
     }
     // too many ids outside the window of the sampled ones: the columns are untouched
     stats.radix_passes = plan.passes;

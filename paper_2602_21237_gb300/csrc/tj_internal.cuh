@@ -178,8 +178,8 @@ struct RadixJob {
 constexpr int kErrFold = 101;
 constexpr int kFarIds = 2048;
 
-// A long run of equal key prefixes is not in order (k_runs): the call sorts by
-// every digit.
+// A long run of equal key prefixes is not in order (k_runs): the call sorts such runs
+// by themselves, or all rows by every digit.
 constexpr int kErrRuns = 102;
 
 // Kinds of onesweep pass: a sort digit of key - lo, a route by the cut table
@@ -419,21 +419,30 @@ cudaError_t launch_wsweep(const RadixJob<K>* d_jobs, int num_jobs, int64_t total
                           cudaStream_t st, const int32_t* d_tile_job = nullptr);
 
 // Sorts by a key prefix (k_prefix_sample, k_runs)
-constexpr int kPrefSample = 2048;  // rows of the sample
+// rows of the sample
+constexpr int prefix_sample(int64_t n) { return n <= (int64_t)1 << 27 ? 2048 : 8192; }
 constexpr int kRunThreads = 256;
 constexpr int kRunTile = 4096;     // rows a CTA writes
 constexpr int kRunMax = 256;       // longest run put in order
 static_assert((kRunTile + 2 * kRunMax) % kRunThreads == 0, "whole rounds of loads");
+constexpr int kLongRuns = 1024;    // longer runs listed
 // *d_pairs += pairs of equal `prefix_bits`-bit prefixes in a sample of the keys
-// (n >= kPrefSample), unless their range has fewer than min_bits bits
+// (n >= prefix_sample(n)), unless their range has fewer than min_bits bits
 cudaError_t launch_prefix_sample(const int64_t* keys, int64_t n, const KeyStats* d_stats,
                                  int prefix_bits, int min_bits, uint32_t* d_pairs,
                                  cudaStream_t st);
 // ids that stand for far ones -> their values
 cudaError_t launch_far_ids(int64_t* ids, int64_t n, const Fold& f, const uint64_t* far_ids,
                            uint32_t far_n, cudaStream_t st);
+// (d_runs: the first rows of the runs longer than kRunMax, then, from kLongRuns on, their
+// last ones, in no order; d_runs_n: how many of either)
 cudaError_t launch_runs(const uint64_t* rows, const uint32_t* ids, int64_t n, const Fold& f, int s,
-                        bool fix, int64_t* out_k, int64_t* out_v, int* d_err, cudaStream_t st);
+                        bool fix, int64_t* out_k, int64_t* out_v, uint32_t* d_runs,
+                        uint32_t* d_runs_n, int* d_err, cudaStream_t st);
+// rows [first[r], first[r] + off[r + 1] - off[r]) of run r <-> the same rows packed
+cudaError_t launch_long_rows(const uint32_t* d_first, const uint32_t* d_off, int runs, int64_t n,
+                             int64_t* keys, int64_t* ids, int64_t* packed_k, int64_t* packed_v,
+                             bool back, cudaStream_t st);
 
 // ---- launchers (tj_join.cu) -------------------------------------------------
 cudaError_t join_init_attributes();

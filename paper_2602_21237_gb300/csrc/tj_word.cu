@@ -553,16 +553,22 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
 // 0.84 GB) are 1.35 ms.
 //
 // k_prefix_sample decides from the statistics and a sample whether that will
-// do: *pairs = the number of pairs of equal prefixes among kPrefSample rows.
-// Prefixes that n rows share evenly among D values give kPrefSample^2 / 2 D.
-__global__ void __launch_bounds__(kPrefSample / 2)
+// do: *pairs = the number of pairs of equal prefixes among SAMPLE rows.
+// Prefixes that n rows share evenly among D values give SAMPLE^2 / 2 D.
+template <int SAMPLE>
+__host__ __device__ constexpr size_t sample_smem_bytes() {
+  return 2 * SAMPLE * (sizeof(unsigned long long) + sizeof(uint32_t));
+}
+template <int SAMPLE>
+__global__ void __launch_bounds__(1024)
     k_prefix_sample(const int64_t* __restrict__ keys, int64_t n,
                     const KeyStats* __restrict__ stats, int prefix_bits, int min_bits,
                     uint32_t* __restrict__ pairs) {
-  constexpr int kSlots = 2 * kPrefSample;
+  constexpr int kSlots = 2 * SAMPLE;
   constexpr unsigned long long kNone = ~0ull;  // (prefixes have at most 32 bits)
-  __shared__ unsigned long long s_key[kSlots];
-  __shared__ uint32_t s_cnt[kSlots];
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned long long* const s_key = reinterpret_cast<unsigned long long*>(smem);
+  uint32_t* const s_cnt = reinterpret_cast<uint32_t*>(s_key + kSlots);
   const unsigned long long lo = stats->min_u, range = ~stats->max_u - lo;
   const int kb = 64 - __clzll((long long)range);
   if (kb < min_bits) return;
@@ -571,10 +577,10 @@ __global__ void __launch_bounds__(kPrefSample / 2)
     s_cnt[i] = 0u;
   }
   __syncthreads();
-  const int64_t step = n / kPrefSample;
+  const int64_t step = n / SAMPLE;
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const uint32_t i = threadIdx.x + u * (kPrefSample / 2);
+  for (int u = 0; u < SAMPLE / 1024; ++u) {
+    const uint32_t i = threadIdx.x + u * 1024;
     // one row of every stretch of `step`, not always the same one
     const int64_t r = i * step + (int64_t)((i * 0x9E3779B97F4A7C15ull >> 33) % (uint64_t)step);
     const unsigned long long k = (unsigned long long)keys[r] ^ 0x8000000000000000ull;
@@ -594,15 +600,15 @@ __global__ void __launch_bounds__(kPrefSample / 2)
 // keys and kRunMax rows on either side come to shared memory; a row finds the
 // ends of its run (rows of the same prefix) and counts the run's rows that come
 // before it. A run of more than kRunMax rows is left as it is, which is right
-// when its keys are in order already (one repeated key, say); where they are
-// not, *err = kErrRuns and the caller sorts by every digit. fix = false only
-// writes the rows out as columns, in the order they have.
+// when its keys are in order already (one repeated key, say), and its ends are listed;
+// where one is not, *err = kErrRuns and the caller sorts the listed runs by themselves.
+// fix = false only writes the rows out as columns, in the order they have.
 // WIDE: keys as they are and ids as 32-bit offsets; otherwise folded rows.
 template <bool WIDE>
 __global__ void __launch_bounds__(kRunThreads)
     k_runs(const uint64_t* __restrict__ rows, const uint32_t* __restrict__ ids, int64_t n, Fold f,
            int s, bool fix, int64_t* __restrict__ out_k, int64_t* __restrict__ out_v,
-           int* __restrict__ err) {
+           uint32_t* __restrict__ runs, uint32_t* __restrict__ runs_n, int* __restrict__ err) {
   constexpr int kSpan = kRunTile + 2 * kRunMax;
   __shared__ uint64_t s_row[kSpan];
   const int tid = threadIdx.x;
@@ -644,9 +650,12 @@ __global__ void __launch_bounds__(kRunThreads)
       }
       if (e - a <= kRunMax)
         pos = a + before;
-      else if (i > 0) {  // a long run: rows in order stay where they are
-        const uint64_t x = key(s_row[i - 1]);
-        bad |= (x >> s) == pre && k < x;
+      else {  // a long run: rows in order stay where they are
+        if (i > a) bad |= k < key(s_row[i - 1]);
+        if (i == a || e == i + 1) {  // its first row, its last one
+          const uint32_t q = atomicAdd(&runs_n[i != a], 1u);
+          if (q < (uint32_t)kLongRuns) runs[(i == a ? 0 : kLongRuns) + q] = (uint32_t)(b0 + i);
+        }
       }
     }
     const int64_t g = b0 + pos;
@@ -680,6 +689,30 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
     for (int u = 0; u < kRows; ++u)
       if (x[u] < (uint64_t)far_n) ids[r0 + u * 256] = (int64_t)far_ids[x[u]];
+  }
+}
+
+// Long runs packed one after another, to be sorted, and back: run r's rows start at row
+// first[r] of the columns and at off[r] of the packed ones.
+__global__ void __launch_bounds__(256)
+    k_long_rows(const uint32_t* __restrict__ first, const uint32_t* __restrict__ off, int runs,
+                int64_t n, int64_t* __restrict__ keys, int64_t* __restrict__ ids,
+                int64_t* __restrict__ packed_k, int64_t* __restrict__ packed_v, bool back) {
+  for (int64_t x = (int64_t)blockIdx.x * 256 + threadIdx.x; x < n; x += (int64_t)gridDim.x * 256) {
+    int lo = 0, hi = runs - 1;  // last run with off <= x
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if ((int64_t)off[mid] <= x) lo = mid;
+      else hi = mid - 1;
+    }
+    const int64_t r = (int64_t)first[lo] + (x - (int64_t)off[lo]);
+    if (back) {
+      keys[r] = packed_k[x];
+      ids[r] = packed_v[x];
+    } else {
+      packed_k[x] = keys[r];
+      packed_v[x] = ids[r];
+    }
   }
 }
 
@@ -823,8 +856,23 @@ cudaError_t wsweep_attrs() {
 cudaError_t launch_prefix_sample(const int64_t* keys, int64_t n, const KeyStats* d_stats,
                                  int prefix_bits, int min_bits, uint32_t* d_pairs,
                                  cudaStream_t st) {
-  if (n < kPrefSample || prefix_bits > 32 || min_bits < prefix_bits) return cudaErrorInvalidValue;
-  k_prefix_sample<<<1, kPrefSample / 2, 0, st>>>(keys, n, d_stats, prefix_bits, min_bits, d_pairs);
+  if (n < prefix_sample(n) || prefix_bits > 32 || min_bits < prefix_bits)
+    return cudaErrorInvalidValue;
+  if (prefix_sample(n) == 2048)
+    k_prefix_sample<2048><<<1, 1024, sample_smem_bytes<2048>(), st>>>(keys, n, d_stats, prefix_bits,
+                                                                      min_bits, d_pairs);
+  else
+    k_prefix_sample<8192><<<1, 1024, sample_smem_bytes<8192>(), st>>>(keys, n, d_stats, prefix_bits,
+                                                                      min_bits, d_pairs);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_long_rows(const uint32_t* d_first, const uint32_t* d_off, int runs, int64_t n,
+                             int64_t* keys, int64_t* ids, int64_t* packed_k, int64_t* packed_v,
+                             bool back, cudaStream_t st) {
+  if (n <= 0 || runs <= 0) return cudaSuccess;
+  const unsigned grid = (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8);
+  k_long_rows<<<grid, 256, 0, st>>>(d_first, d_off, runs, n, keys, ids, packed_k, packed_v, back);
   return cudaGetLastError();
 }
 
@@ -838,19 +886,29 @@ cudaError_t launch_far_ids(int64_t* ids, int64_t n, const Fold& f, const uint64_
 }
 
 cudaError_t launch_runs(const uint64_t* rows, const uint32_t* ids, int64_t n, const Fold& f, int s,
-                        bool fix, int64_t* out_k, int64_t* out_v, int* d_err, cudaStream_t st) {
+                        bool fix, int64_t* out_k, int64_t* out_v, uint32_t* d_runs,
+                        uint32_t* d_runs_n, int* d_err, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const unsigned grid = (unsigned)((n + kRunTile - 1) / kRunTile);
   if (f.wide)
-    k_runs<true><<<grid, kRunThreads, 0, st>>>(rows, ids, n, f, s, fix, out_k, out_v, d_err);
+    k_runs<true><<<grid, kRunThreads, 0, st>>>(rows, ids, n, f, s, fix, out_k, out_v, d_runs,
+                                                 d_runs_n, d_err);
   else
-    k_runs<false><<<grid, kRunThreads, 0, st>>>(rows, ids, n, f, s, fix, out_k, out_v, d_err);
+    k_runs<false><<<grid, kRunThreads, 0, st>>>(rows, ids, n, f, s, fix, out_k, out_v, d_runs,
+                                                 d_runs_n, d_err);
   return cudaGetLastError();
 }
 
 cudaError_t word_init_attributes() {
   cudaError_t e = wsweep_attrs<int32_t>();
-  return e != cudaSuccess ? e : wsweep_attrs<int64_t>();
+  if (e == cudaSuccess) e = wsweep_attrs<int64_t>();
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_prefix_sample<2048>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sample_smem_bytes<2048>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_prefix_sample<8192>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sample_smem_bytes<8192>());
+  return e;
 }
 
 #define TJ_INSTANTIATE_WORD(K)                                                                  \
