@@ -3059,21 +3059,23 @@ tj_status batch_impl(int64_t nj, const int64_t* r_off, const int64_t* s_off, con
     }
   }
   // the word tile: the large one unless the arrays' last tiles waste more by it
-  // than it saves a pass (about a tenth); arrays that the small one pads by more
-  // than kPadShare stay columns, whose passes step over a tile's missing rows, and
-  // so do arrays of less than kWordRows on average, for which the word pass's
-  // tables cost too much a tile (10^8 int32 rows in arrays of 4000, 8000, 20000
-  // and 10^5: words 9.9, 5.9, 3.9 and 2.6 ms, columns 9.1, 6.1, 4.2 and 3.5)
+  // than it saves a pass (about a tenth)
   int64_t pad_large = 0, pad_small = 0;
   for (int64_t j = 0; words && j < 2 * nj; ++j) {
     pad_large += ceil_div(hj[(size_t)j].n, kWThreads * kWItems) * (kWThreads * kWItems);
     pad_small += ceil_div(hj[(size_t)j].n, kWThreads * kWItemsSmall) * (kWThreads * kWItemsSmall);
   }
-  constexpr double kPadShare = 0.25;
-  constexpr int64_t kWordRows = 6144;
-  // (a batch whose pairs all hold one key value needs no pass at all)
-  words = words && max_kb > 0 && R + S >= 2 * nj * kWordRows &&
-          (double)pad_small <= (1.0 + kPadShare) * (double)(R + S);
+  // Short arrays stay columns, whose passes step over a tile's missing rows and set up
+  // less a tile. Fitted to 1000 and 8000 arrays of 3000 to 30000 rows, a batch takes
+  // 0.34 us an array and 19 ns (20 ns int64) per 1000 rows of its padded tiles as words,
+  // 0.27 us and 27 ns (31) per 1000 rows as columns: 8000 arrays of 4096 rows 3.64 ms
+  // (3.79) and 3.13 (3.35), of 6000 to 9000 4.19 (4.33) and 3.83 (4.17), of 12500 to 16384
+  // 5.08 (5.26) and 5.26 (5.81), of 28700 to 30000 7.58 (7.88) and 8.36 (9.48).
+  // (A batch whose pairs all hold one key value needs no pass at all.)
+  constexpr double kRowGain = sizeof(K) == 8 ? 1.58 : 1.42;
+  constexpr double kArrayRows = sizeof(K) == 8 ? 3500 : 4000;
+  words = words && max_kb > 0 &&
+          kRowGain * (double)(R + S) >= (double)pad_small + kArrayRows * 2.0 * (double)nj;
   const Fold fold = words ? make_fold<K>(0, max_kb, id_lo, id_hi, true) : Fold();
   words = fold.on || fold.wide;
   const int witems = R + S >= kWSmallRows && pad_large * 10 <= pad_small * 11 ? kWItems

@@ -1,6 +1,5 @@
 """GPU parity of batched joins whose live pairs all hold one key value each: no digit
-to sort by, on the word path's sizes (arrays of 6144 rows and more on average, little
-padding), also beside pairs that cannot match and beside one pair of two values."""
+to sort by, on the word path's sizes (long arrays), also beside pairs that cannot match and beside one pair of two values."""
 import numpy as np
 import pytest
 import torch
@@ -13,11 +12,12 @@ pytestmark = pytest.mark.gpu
 
 # (R rows, S rows, R's key, S's key) a job
 JOBS = {
-    "one_job": [(10, 20_000, 7, 7)],
-    "single_row": [(1, 30_000, -3, -3)],
-    "equal_sides": [(300, 16_384, 5, 5), (16_384, 300, 1, 1)],
-    "with_dead_pairs": [(40, 20_000, 7, 7), (12_000, 12_000, 7, 8), (0, 9_000, 1, 1),
-                        (64, 40_000, -(1 << 30), -(1 << 30))],
+    "short": [(10, 20_000, 7, 7)],
+    "one_job": [(10, 200_000, 7, 7)],
+    "single_row": [(1, 130_000, -3, -3)],
+    "either_side": [(30, 160_000, 5, 5), (160_000, 30, 1, 1)],
+    "with_dead_pairs": [(40, 100_000, 7, 7), (60_000, 60_000, 7, 8), (0, 90_000, 1, 1),
+                        (20, 140_000, -(1 << 30), -(1 << 30))],
 }
 
 
@@ -52,5 +52,5 @@ def test_pairs_of_one_key(jobs, dtype, ids):
 
 @pytest.mark.parametrize("dtype", [torch.int32, torch.int64])
 def test_one_pair_of_two_values(dtype):
-    run(JOBS["equal_sides"], dtype, "near", second=12_345)
+    run(JOBS["either_side"], dtype, "near", second=12_345)
     assert api.stats()["radix_passes"] == 1
