@@ -325,7 +325,9 @@ __global__ void __launch_bounds__(kWThreads, kWMinB)
   {
     const uint32_t npad = (uint32_t)(TILE - nvalid);
     uint32_t* const lb_mine = J->lookback + pass * J->lb_stride + (int64_t)lt * bins;
-    const uint32_t dpad = npad ? (MODE == kModeCuts ? (uint32_t)J->ncuts : digit(pad)) : ~0u;
+    // (by the cut table not always the last batch: a cut after the largest key of a
+    // range of 2^k keys lies past every key that folds)
+    const uint32_t dpad = npad ? digit(pad) : ~0u;
 #pragma unroll 1
     for (int d = d0; d < d1; ++d) {
       uint32_t c = 0;
