@@ -1475,7 +1475,9 @@ tj_status part_join_impl(const K* kr, const K* ir, int64_t nr, const K* ks, cons
     std::vector<uint16_t> utab(kRouteBuckets + 1, (uint16_t)ncuts);
     for (int bkt = 0; bkt <= ub; ++bkt) {
       const uint64_t start = (uint64_t)bkt << us;
-      if (start > krange) break;
+      // (a range of nearly 2^64 keys ends where the last bucket does, and there the
+      // shift is back at 0)
+      if (start > krange || start >> us != (uint64_t)bkt) break;
       const K sk = (K)(lo_bits<K>(lo) + start);
       utab[(size_t)bkt] = (uint16_t)(std::lower_bound(cuts.begin(), cuts.end(), sk) - cuts.begin());
     }
