@@ -155,7 +155,8 @@ typedef struct {
  *   then by the R row's input position.
  * out_count : HOST pointer; receives |J|.  If |J| > out_capacity the call
  *   returns TJ_ERR_CAPACITY, *out_count = |J| and out_pairs holds garbage.
- * The call synchronises `stream` twice (plan statistics, final count).
+ * The call synchronises `stream` for the plan statistics and the final count,
+ * and between the steps of a partitioned join.
  */
 tj_status tj_join_inner(tj_dtype dt, const void* keys_r, const void* ids_r, int64_t n_r,
                         const void* keys_s, const void* ids_s, int64_t n_s,
@@ -178,7 +179,8 @@ tj_status tj_join_inner_ex(tj_dtype dt, const void* keys_r, const void* ids_r, i
 /*
  * ORDER BY key (Sec. 4.2): stable sort of the rows (keys[i], ids[i]) by key
  * ascending, in place.  n rows; keys and ids are device arrays (read-write).
- * Synchronises `stream` once (key statistics for the digit plan).
+ * Synchronises `stream` for the key statistics and at the end, and once or
+ * twice more where its rows turn out not to suit the path it took.
  */
 tj_status tj_sort(tj_dtype dt, void* keys, void* ids, int64_t n, void* stream);
 
@@ -212,8 +214,9 @@ tj_status tj_sort_multi(tj_dtype dt, void* const* cols, int32_t n_cols, void* id
  * counterpart).  Some callers cannot call cudaMalloc, cudaMallocAsync or any
  * allocator when they sort: code that runs while an outer framework owns the
  * device's memory pool, allocation-free real-time paths, or processes that
- * must not grow device memory after start-up.  This entry point runs the same
- * kernels as tj_sort and allocates nothing, on the device or on the host (no
+ * must not grow device memory after start-up.  This entry point sorts by the
+ * column passes that tj_sort takes for rows which do not fold into one word
+ * (the result is the same) and allocates nothing, on the device or on the host (no
  * cudaMalloc*, no pool allocation, no pinned host memory): its scratch is one
  * file-scope device array of about 18 MB that every GPU loading this library
  * holds until the process exits; its job table travels as a kernel argument

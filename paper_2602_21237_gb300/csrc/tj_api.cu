@@ -559,9 +559,11 @@ uint64_t window_start(int64_t lo, uint64_t range, int kw) {
 constexpr int64_t kWSmallRows = (int64_t)1 << 22;
 int word_items(int64_t rows) { return rows < kWSmallRows ? kWItemsSmall : kWItems; }
 
-// Time of one word pass by digit width, relative to one of at most 7 bits
-// (GB300, 10^8 words: 500, 538, 618 and 770 us for 7 to 10 bits), and the plan
-// of fewest such units: 27 bits take 3 passes of 9 instead of 4 of 7.
+// Time of one word pass by digit width, relative to one of at most 7 bits, and the plan
+// of fewest such units: 27 bits take 3 passes of 9 instead of 4 of 7.  (GB300, sorts of
+// 10^8 int32 rows: 502, 536, 604 and 792 us a pass for 7 to 10 bits. The table is from
+// passes of 500, 538, 618 and 770; 1.07, 1.20 and 1.58 would take a pass less at 41, 42
+// and 57 to 63 bits.)
 double word_pass_cost(int w) { return w <= 7 ? 1.0 : w == 8 ? 1.08 : w == 9 ? 1.24 : 1.55; }
 
 Plan make_word_plan(uint64_t lo, uint64_t range, bool even, int max_digit, int min_passes) {
@@ -3393,9 +3395,10 @@ bool bad_ptr(const void* p, int64_t n) { return n > 0 && p == nullptr; }
 // Some callers cannot call cudaMalloc (or any allocator) at the point they
 // sort: code running while an outer framework owns the device memory pool,
 // allocation-free real-time paths, or hosts that must not grow device memory
-// after start-up.  For them, tj_sort_noalloc runs the same kernels as tj_sort
-// with its scratch in one file-scope device array of a fixed size, held by
-// every GPU that loads this library until the process exits.
+// after start-up.  For them, tj_sort_noalloc sorts by the column passes of
+// tj_radix.cu (rows that tj_sort would fold too) with its scratch in one
+// file-scope device array of a fixed size, held by every GPU that loads this
+// library until the process exits.
 constexpr int64_t kNoAllocMaxRows = (int64_t)1 << 20;  // rows per call
 constexpr int64_t kNoAllocTiles = (kNoAllocMaxRows + kTile - 1) / kTile;
 constexpr size_t kNoAllocBytes = 2 * (size_t)kNoAllocMaxRows * 8           // B keys, B ids

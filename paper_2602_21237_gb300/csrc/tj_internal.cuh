@@ -41,8 +41,8 @@ constexpr int kTileWide = kSortThreads * kItemsWide;
 #endif
 constexpr int kItemsRoute = TJ_ROUTE_ITEMS;
 constexpr int kTileRoute = kSortThreads * kItemsRoute;
-// onesweep passes over folded rows (tj_word.cu): words a thread holds in
-// registers, and fewer for arrays too small to fill the chip with big tiles
+// onesweep passes over folded rows (tj_word.cu): rows of a thread, and fewer for
+// arrays too small to fill the chip with big tiles
 #ifndef TJ_W_THREADS
 #define TJ_W_THREADS 512
 #endif
