@@ -130,4 +130,4 @@ def test_one_far_id_costs_no_second_run(n, op):
     call = (lambda ids: api.sort(keys.clone(), ids.clone())) if op == "sort" else \
         (lambda ids: api.join_inner(kr, ir, keys, ids, out=out))
     t_any, t_one = best(lambda: call(any_)), best(lambda: call(one))
-    assert t_one < 1.15 * t_any, (t_one, t_any)
+    assert t_one < 1.2 * t_any, (t_one, t_any)
